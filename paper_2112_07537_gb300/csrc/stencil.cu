@@ -6,57 +6,97 @@
 
 namespace mr {
 
-// One CTA per leaf: rhs from the padded block P (shell Gi >= 3), then the RK
-// stage combination (or the bare rhs).  u: u^n (stages 1, 2), may alias out.
+// Right-hand side from the padded block P (shell Gi >= 3), then the RK stage
+// combination (or the bare rhs).  u: u^n (stages 1, 2), may alias out.
+// One CTA per slab of nz z-planes of a leaf.  The x and y grid lines of the
+// slab, cut into segments of seg cells, are walked first (walk_line: every
+// interface flux once, differences shared along the line), their flux
+// differences left in shared memory; the z lines of the slab then add theirs
+// and finish their cells.  FP64 is bound by the FP64 pipe: about 45 of its
+// instructions per interface, so the walk (each flux once, one division
+// instead of four) is what counts; slabs and segments only spread small grids
+// over the chip (see rhs_dispatch) and change no value: point fluxes are
+// rounded products and the sums of walk_line leave nothing to contract, so a
+// flux does not depend on where its line was cut.  Measured (WENO-Z5, velocity
+// fields, 1 408 leaves of 24^3 = 19.5 M points): 23.9 ms per launch with both
+// fluxes of every point evaluated per thread and four divisions each, 6.35 ms
+// so (the FP64 pipe's floor for 147 instructions a point is 4.6 ms); 15 leaves
+// of 16^3: 680 us in 15 CTAs, 39 us.
 template <typename T, int SCHEME>
-__global__ void __launch_bounds__(256) k_rhs_stage(Tree t, const T *__restrict__ P, int Gi,
-                                                   const T *u, T *out, int stage, T dt, T ux, T uy,
-                                                   T uz, int rhs_only, const T *__restrict__ vpad, T nu,
-                                                   int diff, T vscale) {
+__global__ void __launch_bounds__(256) k_rhs_stage(Tree t, const T *__restrict__ P, int Gi, const T *u, T *out,
+                                                   int stage, T dt, T ux, T uy, T uz, int rhs_only,
+                                                   const T *__restrict__ vpad, T nu, int diff, T vscale, int nz,
+                                                   int nslab, int seg) {
   // vpad: ghost-filled velocity components (shell 3) or null for constant u
-  const int b = blockIdx.x;
-  const int nb = t.nb, Wd = nb + 2 * Gi;
-  const size_t np = (size_t)Wd * Wd * Wd;
-  const T h = T(t.tree_len / ((double)nb * (double)(1 << __ldg(t.lev + b))));
-  const T *Pb = P + (size_t)b * np;
-  const T uc[3] = {ux, uy, uz};
-  const int stride[3] = {1, Wd, Wd * Wd};
-  for (int p = threadIdx.x; p < nb * nb * nb; p += blockDim.x) {
-    const int i = p % nb, j = (p / nb) % nb, k = p / (nb * nb);
-    const size_t c = (i + Gi) + Wd * ((j + Gi) + (size_t)Wd * (k + Gi));
-    T acc = T(0);
-    const int Wv = nb + 6;
-    const size_t vblk = (size_t)Wv * Wv * Wv, vcomp = (size_t)t.nleaf * vblk;
-    const size_t cv = (size_t)b * vblk + (i + 3) + Wv * ((j + 3) + (size_t)Wv * (k + 3));
-    const int vstride[3] = {1, Wv, Wv * Wv};
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      if (!vpad && uc[d] == T(0)) continue;
-      T f[7], uu[7];
-#pragma unroll
-      for (int m = 0; m < 7; ++m) {
-        uu[m] = vpad ? vscale * vpad[d * vcomp + cv + (ptrdiff_t)(m - 3) * vstride[d]] : uc[d];
-        f[m] = uu[m] * Pb[c + (ptrdiff_t)(m - 3) * stride[d]];
-      }
-      const bool lp = uu[3] + uu[4] >= T(0), lm = uu[2] + uu[3] >= T(0);
-      acc += iface_flux<T, SCHEME>(f + 1, lp) - iface_flux<T, SCHEME>(f, lm);
-    }
-    T r = -acc / h;
-    if (diff) r += nu * lap_at<T>(Pb + c, stride, diff) / (h * h);
-    const size_t q = (size_t)b * nb * nb * nb + p;
-    if (rhs_only) {
-      out[q] = r;
+  const int b = blockIdx.x / nslab, k0 = (blockIdx.x - b * nslab) * nz;
+  const int nb = t.nb, Wd = nb + 2 * Gi, Wv = nb + 6, nzs = min(nz, nb - k0), RS = nb + 1;
+  const size_t np = (size_t)Wd * Wd * Wd, vblk = (size_t)Wv * Wv * Wv, vcomp = (size_t)t.nleaf * vblk;
+  const T *Pb = P + (size_t)b * np + Gi + Wd * (Gi + (size_t)Wd * (Gi + k0));  // cell (0, 0, k0)
+  const T *Vb = vpad ? vpad + (size_t)b * vblk + 3 + Wv * (3 + (size_t)Wv * (3 + k0)) : nullptr;
+  const T hscale = T(0.5) * vscale;
+  extern __shared__ double smd[];
+  T *R0 = reinterpret_cast<T *>(smd), *R1 = R0 + (size_t)nz * nb * RS;  // x and y flux differences
+  auto walk = [&](int d, const T *p, const T *v, int st, int sv, int n, auto emit) {
+    if (vpad) {
+      v += d * vcomp;
+      walk_line<T, SCHEME>(
+          n, [&](int m) { return rmul(rmul(hscale, v[m * sv]), p[m * st]); },
+          [&](int m) { return rmul(hscale, v[m * sv]); }, emit);
     } else {
-      const T v = Pb[c] + dt * r;
-      T o;
-      if (stage == 0) o = v;
-      else if (stage == 1) o = T(0.75) * u[q] + T(0.25) * v;
-      else o = T(1.0 / 3) * u[q] + T(2.0 / 3) * v;
-      out[q] = o;
+      const T ud = d == 0 ? ux : d == 1 ? uy : uz, hu = T(0.5) * ud;
+      walk_line<T, SCHEME>(
+          n, [&](int m) { return rmul(hu, p[m * st]); }, [&](int) { return ud; }, emit);
     }
+  };
+  const bool xon = vpad || ux != T(0), yon = vpad || uy != T(0), zon = vpad || uz != T(0);
+  // x segments, then y segments: nseg per line, lines (other axis, plane)
+  const int nseg = (nb + seg - 1) / seg, nx = nb * nzs * nseg;
+  for (int idx = threadIdx.x; idx < 2 * nx; idx += blockDim.x) {
+    const bool yd = idx >= nx;
+    const int q = yd ? idx - nx : idx, l = q % nb, r = q / nb, s = r % nseg, k = r / nseg;
+    const int m0 = s * seg, n = min(seg, nb - m0);
+    if (yd ? !yon : !xon) continue;
+    const int i = yd ? l : m0, j = yd ? m0 : l;
+    const size_t o = i + Wd * (j + (size_t)Wd * k), ov = i + Wv * (j + (size_t)Wv * k);
+    T *rr = (yd ? R1 : R0) + i + RS * (j + nb * k);
+    const int rs = yd ? RS : 1;
+    walk(yd ? 1 : 0, Pb + o, Vb + (vpad ? ov : 0), yd ? Wd : 1, yd ? Wv : 1, n,
+         [&](int m, T dF) { rr[m * rs] = dF; });
+  }
+  __syncthreads();
+  const T h = T(t.tree_len / ((double)nb * (double)(1 << __ldg(t.lev + b)))), inv2 = T(2) / h, invh2 = T(1) / (h * h);
+  const int stride[3] = {1, Wd, Wd * Wd};
+  for (int c = threadIdx.x; c < nb * nb; c += blockDim.x) {
+    const int j = c / nb, i = c - j * nb;
+    const T *p = Pb + i + Wd * j;
+    const size_t q0 = (size_t)b * nb * nb * nb + c + (size_t)nb * nb * k0;
+    auto finish = [&](int m, T dz) {
+      const int ro = i + RS * (j + nb * m);
+      T acc = T(0);
+      if (xon) acc = R0[ro];
+      if (yon) acc += R1[ro];
+      if (zon) acc += dz;
+      T r = -acc * inv2;
+      const T *pc = p + (size_t)m * Wd * Wd;
+      if (diff) r += nu * lap_at<T>(pc, stride, diff) * invh2;
+      const size_t q = q0 + (size_t)m * nb * nb;
+      if (rhs_only) {
+        out[q] = r;
+      } else {
+        const T v = pc[0] + dt * r;
+        T o;
+        if (stage == 0) o = v;
+        else if (stage == 1) o = T(0.75) * u[q] + T(0.25) * v;
+        else o = T(1.0 / 3) * u[q] + T(2.0 / 3) * v;
+        out[q] = o;
+      }
+    };
+    if (zon)
+      walk(2, p, Vb + (vpad ? i + Wv * j : 0), Wd * Wd, Wv * Wv, nzs, finish);
+    else
+      for (int m = 0; m < nzs; ++m) finish(m, T(0));
   }
 }
-
 
 template <typename T>
 static int rhs_dispatch(mr_grid *g, const T *P, int Gi, const T *u, T *out, int stage, double dt,
@@ -66,15 +106,31 @@ static int rhs_dispatch(mr_grid *g, const T *P, int Gi, const T *u, T *out, int 
   static const double zero3[3] = {0.0, 0.0, 0.0};
   if (!uc) uc = zero3;
   const T ux = T(uc[0]), uy = T(uc[1]), uz = T(uc[2]);
-  if (scheme == MR_CONS3)
-    MR_LAUNCH(g, MRK_RHS, k_rhs_stage<T, MR_CONS3><<<n, 256, 0, g->stream>>>(t, P, Gi, u, out, stage, T(dt), ux, uy, uz, rhs_only, vpad, T(g->diff_nu), g->diff_order, T(g->vel_scale)));
-  else if (scheme == MR_CONS5)
-    MR_LAUNCH(g, MRK_RHS, k_rhs_stage<T, MR_CONS5><<<n, 256, 0, g->stream>>>(t, P, Gi, u, out, stage, T(dt), ux, uy, uz, rhs_only, vpad, T(g->diff_nu), g->diff_order, T(g->vel_scale)));
-  else if (scheme == MR_WENOZ5)
-    MR_LAUNCH(g, MRK_RHS, k_rhs_stage<T, MR_WENOZ5><<<n, 256, 0, g->stream>>>(t, P, Gi, u, out, stage, T(dt), ux, uy, uz, rhs_only, vpad, T(g->diff_nu), g->diff_order, T(g->vel_scale)));
-  else
-    return MR_ERR_INVALID;
-  return check_cuda(cudaGetLastError(), "k_rhs_stage") ? MR_ERR_CUDA : MR_OK;
+  // Slabs of 8 planes (a z line of 8 cells evaluates 9 fluxes; its sums take
+  // 77 KB of shared memory at nb = 24 in FP64, two CTAs per SM).  Grids too
+  // small to give every SM two such slabs get thinner ones, down to 2 planes,
+  // and x/y lines cut until the CTA's threads all have a segment.
+  const int nb = g->desc.nb;
+  int nslab = (nb + 7) / 8;
+  while (nslab * 2 <= nb / 2 && (long)n * nslab < 2 * 152) nslab *= 2;
+  const int nz = (nb + nslab - 1) / nslab;
+  nslab = (nb + nz - 1) / nz;
+  int seg = nb;
+  if ((long)n * nslab < 4 * 152)
+    while (seg > 4 && 2 * nb * nz * ((nb + seg - 1) / seg) < 256) seg = (seg + 1) / 2;
+  const size_t sm = 2 * sizeof(T) * (size_t)nz * nb * (nb + 1);
+  auto go = [&](auto kern) -> int {
+    if (check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), "rhs smem"))
+      return MR_ERR_CUDA;
+    MR_LAUNCH(g, MRK_RHS, kern<<<n * nslab, 256, sm, g->stream>>>(t, P, Gi, u, out, stage, T(dt), ux, uy, uz, rhs_only,
+                                                                  vpad, T(g->diff_nu), g->diff_order, T(g->vel_scale),
+                                                                  nz, nslab, seg));
+    return check_cuda(cudaGetLastError(), "k_rhs_stage") ? MR_ERR_CUDA : MR_OK;
+  };
+  if (scheme == MR_CONS3) return go(k_rhs_stage<T, MR_CONS3>);
+  if (scheme == MR_CONS5) return go(k_rhs_stage<T, MR_CONS5>);
+  if (scheme == MR_WENOZ5) return go(k_rhs_stage<T, MR_WENOZ5>);
+  return MR_ERR_INVALID;
 }
 
 int launch_rhs_stage(mr_grid *g, const void *P, int Gi, const void *u, void *out, int stage,
