@@ -637,12 +637,9 @@ int launch_writeback32(mr_grid *g, int Gi, void *phi);
 int launch_substitute(mr_grid *g, void *phi, const int *need = nullptr, bool in_side_buffer = false,
                       bool f32 = false);
 int launch_ghost_adapt32(mr_grid *g, const float *phi, int G, const int *need, void **P, int *Gi);
+// stage.cu
 int launch_fused(mr_grid *g, const void *phi, const void *P, const void *Q, int Gi, const void *u, void *out,
                  int stage, double dt, const double *uc, int scheme, bool rhs_only, const void *vpad = nullptr);
-// stage_kernels.cuh (instantiated in stage_i_*.cu)
-template <int N, int NT>
-int fused_launch(mr_grid *g, const float *phi, const float *P, const float *Q, int Gi, const float *u, float *out,
-                 int stage, double dt, const double *uc, int scheme, bool rhs_only, const float *vpad);
 int adapt_shell(int N, int Nt);
 // boundary.cu: grids with physical boundaries (the general point-wise path)
 int ghost_bounded(mr_grid *g, const void *phi_in, void *phi_out, int G, bool fp64, void *P, void *Q, int Gi);

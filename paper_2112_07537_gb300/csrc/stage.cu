@@ -1,0 +1,556 @@
+// stage.cu -- the FP32 stage kernels: ghost faces + advection right-hand side
+// + RK3 stage in one launch.  Two kernels compute the same values with the
+// same arithmetic; the autotuner picks the faster:
+//   k_fused  one CTA per slab of a leaf: the slab with its ghosts in shared
+//            memory, one thread per grid line and direction;
+//   k_march  one CTA per leaf marching through the block's z-planes: the six
+//            face slabs in shared memory, one thread per (x, y) column with a
+//            register window along z, x/y fluxes of one plane at a time.
+#include <algorithm>
+
+#include "stage_kernels.cuh"
+
+namespace mr {
+
+// ---------------------------------------------------------------------------
+// Where the three ghost layers behind each face f = 2*axis + (0: -side, 1:
+// +side) of leaf b come from:
+//   same-level face  the neighbour's field;
+//   coarser face     b's padded block: the pre-pass (k_prep) of every leaf next
+//                    to a coarser one has refined the coarse values there;
+//   finer face       the Part-2 coarsening pushed by the finer leaves into Q
+//                    (lifted wavelets), or the coincident values of the finer
+//                    leaves (N.0): one sub-block per face quadrant.
+// ---------------------------------------------------------------------------
+struct FaceSrc {
+  int kind;              // 0: block stride, 1: padded stride, 2: finer leaves
+  const float *base[4];  // address of the (virtual) block point (0, 0, 0)
+};
+
+__device__ __forceinline__ void face_sources(const Tree &t, int b, int L, const int *a, const float *phi,
+                                             const float *P, const float *Q, int Gi, int lifted, FaceSrc *fs) {
+  if (threadIdx.x >= 6) return;
+  const int f = threadIdx.x, ax = f >> 1, sg = f & 1, nb = t.nb, Wd = nb + 2 * Gi;
+  const long long nb3 = (long long)nb * nb * nb, np = (long long)Wd * Wd * Wd, org = Gi * (1 + Wd + (long long)Wd * Wd);
+  const int st[3] = {1, nb, nb * nb};
+  int g[3] = {a[0], a[1], a[2]};
+  g[ax] += sg ? nb : -1;
+  const int o = owner(t, L, g[0], g[1], g[2], b), Lo = __ldg(t.lev + o);
+  FaceSrc s;
+  s.base[1] = s.base[2] = s.base[3] = nullptr;
+  if (Lo == L) {
+    s.kind = 0, s.base[0] = phi + o * nb3 + (sg ? -nb : nb) * st[ax];
+  } else if (Lo < L || lifted) {
+    s.kind = 1, s.base[0] = (Lo < L ? P : Q) + b * np + org;
+  } else {
+    s.kind = 2;
+    const int e1 = ax == 0 ? 1 : 0, e2 = ax == 2 ? 1 : 2;
+    for (int q = 0; q < 4; ++q) {
+      int h[3], gf[3];
+      h[ax] = sg ? 0 : 1, h[e1] = q & 1, h[e2] = q >> 1;
+      long long off = 0;
+      for (int d = 0; d < 3; ++d) {
+        const int dd = d == ax ? (sg ? 1 : -1) : 0;
+        gf[d] = 2 * (a[d] + dd * nb) + h[d] * nb;
+        off -= (long long)st[d] * (2 * dd + h[d]) * nb;
+      }
+      s.base[q] = phi + owner(t, L + 1, gf[0], gf[1], gf[2], b) * nb3 + off;
+    }
+  }
+  fs[f] = s;
+}
+
+// ghost value behind face f at block-local point (i, j, k)
+__device__ __forceinline__ const float *face_ptr(const FaceSrc &s, int ax, int i, int j, int k, int nb, int Wd) {
+  if (s.kind == 0) return s.base[0] + i + nb * (j + nb * k);
+  if (s.kind == 1) return s.base[0] + i + Wd * (j + Wd * k);
+  const int hb = nb / 2, p = ax == 0 ? j : i, q = ax == 2 ? j : k;
+  return s.base[(p >= hb) + 2 * (q >= hb)] + 2 * (i + nb * (j + nb * k));
+}
+
+// one float from global to shared memory, asynchronously
+__device__ __forceinline__ void copy_async(float *dst, const float *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+struct StageArgs {
+  const float *phi, *P, *Q;
+  int Gi, lifted;
+  const int *cmask;
+  const float *u;   // u^n (stages 1, 2), may alias out
+  float *out;
+  int stage, rhs_only;
+  float dt, ux, uy, uz;
+  const float *vpad;  // ghost-filled velocity components (shell 3) or null
+  float nu, vscale;
+  int diff;
+};
+
+// RK3-TVD stage (or the bare rhs r) of one cell with value c
+__device__ __forceinline__ float stage_value(const StageArgs &s, float c, float r, float uo) {
+  if (s.rhs_only) return r;
+  const float v = c + s.dt * r;
+  return s.stage == 0 ? v : s.stage == 1 ? 0.75f * uo + 0.25f * v : (1.0f / 3) * uo + (2.0f / 3) * v;
+}
+
+// ---------------------------------------------------------------------------
+// k_fused: one CTA per slab of nz z-planes.  Shared memory (floats):
+//   T  [nz][nb+6][nb+7]  the slab's planes with their x and y ghosts
+//   H  [6][nb][nb]       three planes below and above the slab
+//   X  [nz][nb][nb+7]    half velocity u_x on the x rows (velocity fields);
+//                        each row's walk leaves its flux differences there
+//   Y  [nz][nb+6][nb]    likewise u_y on the y columns
+// (odd row pitch: threads on neighbouring x rows hit different banks).  The x
+// and y lines of the slab are walked first, one thread each with the same
+// code, then the z lines, whose thread finishes its cells (u_z and u^n are
+// read once, along x, straight from memory).  Bound by issued instructions
+// (ncu: 390 per point with velocity fields, issue slots 61 % busy, DRAM 27 %),
+// so every difference and smoothness term is evaluated once along a line;
+// slabs of a quarter block keep three CTAs (27 warps at nb = 24) on an SM, the
+// z walks' extra interface per slab costs 5 %.  Measured against the whole
+// block in one CTA (WENO-Z5, 6.2 ghosts): 3 424 leaves of 24^3 with velocity
+// fields 1 660 -> 755 us per launch, 42 400 leaves with a constant velocity
+// 15.35 -> 6.06 ms, 11 019 leaves of 16^3 with velocity fields 1 333 -> 843 us.
+// k_march takes 1 070 us, 8.5 ms and 1 047 us there.
+// ---------------------------------------------------------------------------
+__host__ __device__ constexpr int fused_smem_floats(int nb, int nz, bool vel) {
+  return nz * (nb + 6) * (nb + 7) + 6 * nb * nb + (vel ? nz * nb * (nb + 7) + nz * (nb + 6) * nb
+                                                        : nz * nb * (nb + 1) + nz * nb * nb);
+}
+
+template <int SCHEME, bool VEL, bool LAP>
+__global__ void __launch_bounds__(288, 3) k_fused(Tree t, StageArgs s, int nz, int nslab) {
+  const int b = blockIdx.x / nslab, k0 = (blockIdx.x - b * nslab) * nz;
+  const int nb = t.nb, nb2 = nb * nb, Ws = nb + 6, RS = nb + 7, Wd = nb + 2 * s.Gi, nzs = min(nz, nb - k0);
+  const int tid = threadIdx.x, bd = blockDim.x;
+  const int L = __ldg(t.lev + b);
+  const int a[3] = {__ldg(t.anc + 3 * b) * nb, __ldg(t.anc + 3 * b + 1) * nb, __ldg(t.anc + 3 * b + 2) * nb};
+  extern __shared__ float sm[];
+  float *T = sm, *H = T + nz * Ws * RS, *X = H + 6 * nb2, *Y = X + nz * nb * (VEL ? RS : nb + 1);
+  __shared__ FaceSrc fs[6];
+  face_sources(t, b, L, a, s.phi, s.P, s.Q, s.Gi, s.lifted, fs);
+  const DivM dnb = t.dnb;
+  __shared__ float sh_h;
+  if (tid == 32) sh_h = (float)(t.tree_len / ((double)nb * (double)(1 << L)));
+  // Every value goes to shared memory by an asynchronous copy of its own (all
+  // in flight at once; nothing waits for memory before the barrier).  Each
+  // thread keeps its (x, y) and steps through the planes.
+  // Interior planes of the slab and of its z neighbourhood inside the leaf:
+  // the field, or the substituted block that the pre-pass wrote.
+  {
+    const int ka = max(k0 - 3, 0), kb = min(k0 + nzs + 3, nb);
+    const bool pad = s.cmask[b] != 0;
+    const int sy = pad ? Wd : nb, sz = pad ? Wd * Wd : nb2;
+    const float *src = (pad ? s.P + (size_t)b * Wd * Wd * Wd + s.Gi * (1 + Wd + Wd * Wd)
+                            : s.phi + (size_t)b * nb2 * nb) + (size_t)ka * sz;
+    for (int c = tid; c < nb2; c += bd) {
+      const int j = divq(c, dnb), i = c - j * nb;
+      const float *p = src + i + sy * j;
+      float *tp = T + (j + 3) * RS + i + 3, *hp = H + c;
+      for (int z = ka - k0; z < kb - k0; ++z, p += sz)
+        copy_async(z < 0 ? hp + (z + 3) * nb2 : z < nzs ? tp + z * Ws * RS : hp + (z - nzs + 3) * nb2, p);
+    }
+  }
+  const float hscale = 0.5f * s.vscale;
+  const size_t vblk = (size_t)Ws * Ws * Ws;
+  const float *vb = VEL ? s.vpad + (size_t)b * vblk : nullptr;
+  const size_t vcomp = (size_t)t.nleaf * vblk;
+  if (VEL) {
+    const DivM dws = divm(Ws);
+    const float *vx = vb + (size_t)Ws * Ws * (k0 + 3) + 3 * Ws, *vy = vb + vcomp + (size_t)Ws * Ws * (k0 + 3) + 3;
+    for (int c = tid; c < nb * Ws; c += bd) {
+      const int j = divq(c, dws), x = c - j * Ws, jy = divq(c, dnb), i = c - jy * nb;
+      float *xp = X + j * RS + x, *yp = Y + c;
+      const float *px = vx + c, *py = vy + i + Ws * jy;
+      for (int k = 0; k < nzs; ++k) {
+        copy_async(xp + k * nb * RS, px + k * Ws * Ws);
+        copy_async(yp + k * Ws * nb, py + k * Ws * Ws);
+      }
+    }
+  }
+  __syncthreads();  // fs
+  // ghosts: x and y of the slab's planes, z planes beyond the leaf
+  for (int c = tid; c < nb * 6; c += bd) {
+    const int j = c / 6, m = c - 6 * j, i = m < 3 ? m - 3 : nb + m - 3;
+    const FaceSrc &f = fs[m < 3 ? 0 : 1];
+    float *tp = T + (j + 3) * RS + i + 3;
+    for (int k = 0; k < nzs; ++k) copy_async(tp + k * Ws * RS, face_ptr(f, 0, i, j, k0 + k, nb, Wd));
+  }
+  for (int c = tid; c < 6 * nb; c += bd) {
+    const int m = divq(c, dnb), i = c - m * nb, j = m < 3 ? m - 3 : nb + m - 3;
+    const FaceSrc &f = fs[m < 3 ? 2 : 3];
+    float *tp = T + (j + 3) * RS + i + 3;
+    for (int k = 0; k < nzs; ++k) copy_async(tp + k * Ws * RS, face_ptr(f, 1, i, j, k0 + k, nb, Wd));
+  }
+  for (int h = 0; h < 6; ++h) {
+    const int z = h < 3 ? k0 + h - 3 : k0 + nzs + h - 3;
+    if (z >= 0 && z < nb) continue;
+    for (int c = tid; c < nb2; c += bd) {
+      const int j = divq(c, dnb), i = c - j * nb;
+      copy_async(H + h * nb2 + c, face_ptr(fs[z < 0 ? 4 : 5], 2, i, j, z, nb, Wd));
+    }
+  }
+  copy_wait();
+  __syncthreads();
+  const float invh = 1.0f / sh_h;
+  const float lk = LAP ? 0.5f * s.nu * invh : 0.f;  // rhs = -2/h (dF - lk lap)
+  const bool xon = VEL || LAP || s.ux != 0.f, yon = VEL || LAP || s.uy != 0.f, zon = VEL || LAP || s.uz != 0.f;
+  // x lines, then y lines: base and pitch of the line in T and in X / Y.  A
+  // constant velocity u < 0 is walked in the other direction with |u|: the
+  // right-biased flux of u phi is minus the left-biased one of |u| phi on the
+  // mirrored line, and the order of the difference reverses with it.  So
+  // neither sign selects an upwind side.
+  const int nl = nb * nzs;
+  for (int idx = tid; idx < 2 * nl; idx += bd) {
+    const bool yd = idx >= nl;
+    if (yd ? !yon : !xon) continue;
+    const int q = yd ? idx - nl : idx, k = divq(q, dnb), l = q - k * nb;
+    const float *p = T + (yd ? (k * Ws + 3) * RS + l + 3 : (k * Ws + l + 3) * RS + 3);
+    const int st = yd ? RS : 1;
+    if (VEL) {
+      float *v = yd ? Y + (k * Ws + 3) * nb + l : X + q * RS + 3;
+      const int sv = yd ? nb : 1;
+      walk_line<float, SCHEME, LAP, false>(
+          nb, s.diff, [&](int m) { return p[m * st]; }, [&](int m) { return rmul(hscale, v[m * sv]); },
+          [&](int m, float dF, float, float lap) { v[m * sv] = LAP ? fmaf(-lk, lap, dF) : dF; });
+    } else {
+      float *v = yd ? Y + k * nb2 + l : X + q * (nb + 1);
+      const float uu = yd ? s.uy : s.ux, hu = 0.5f * fabsf(uu);
+      const int e = uu >= 0.f ? 0 : nb - 1, sv = yd ? nb : 1, d = uu >= 0.f ? 1 : -1;
+      const float *pe = p + e * st;
+      float *ve = v + e * sv;
+      walk_line<float, SCHEME, LAP, true>(
+          nb, s.diff, [&](int m) { return pe[m * d * st]; }, [&](int) { return hu; },
+          [&](int m, float dF, float, float lap) { ve[m * d * sv] = LAP ? fmaf(-lk, lap, dF) : dF; });
+    }
+  }
+  __syncthreads();
+  const bool rk_u = !s.rhs_only && s.stage > 0;
+  for (int c = tid; c < nb2; c += bd) {
+    const int j = divq(c, dnb), i = c - j * nb;
+    const float *tp = T + (j + 3) * RS + i + 3, *hp = H + c;
+    const int tst = Ws * RS;
+    const float *xp = VEL ? X + j * RS + i + 3 : X + j * (nb + 1) + i;
+    const float *yp = VEL ? Y + (j + 3) * nb + i : Y + c;
+    const int xst = VEL ? nb * RS : nb * (nb + 1), yst = VEL ? Ws * nb : nb2;
+    const size_t q0 = (size_t)b * nb2 * nb + (size_t)k0 * nb2 + c;
+    const float *up = s.u + q0;
+    auto phi = [&](int m) { return m < 0 ? hp[(m + 3) * nb2] : m < nzs ? tp[m * tst] : hp[(m - nzs + 3) * nb2]; };
+    const int e = !VEL && s.uz < 0.f ? nzs - 1 : 0, d = !VEL && s.uz < 0.f ? -1 : 1;  // walk direction
+    float un = rk_u ? up[(size_t)e * nb2] : 0.f;  // u^n one cell ahead
+    auto finish = [&](int m, float dF, float ph, float lap) {
+      const float uo = un;
+      const int z = e + d * m;
+      if (rk_u && m + 1 < nzs) un = up[(size_t)(z + d) * nb2];
+      float acc = LAP ? fmaf(-lk, lap, dF) : dF;
+      acc = (xon ? xp[z * xst] : 0.f) + (yon ? yp[z * yst] : 0.f) + acc;
+      s.out[q0 + (size_t)z * nb2] = stage_value(s, ph, -2.f * (acc * invh), uo);
+    };
+    if (VEL) {
+      const float *vz = vb + 2 * vcomp + (size_t)Ws * Ws * k0 + Ws * (j + 3) + i + 3;  // plane k0 - 3
+      float nxt = __ldg(vz);
+      auto hv = [&](int m) {
+        const float v = nxt;
+        if (m + 1 < nzs + 3) nxt = __ldg(vz + (size_t)Ws * Ws * (m + 4));  // one plane ahead
+        return rmul(hscale, v);
+      };
+      walk_line<float, SCHEME, LAP, false>(nzs, s.diff, phi, hv, finish);
+    } else if (zon) {
+      const float hu = 0.5f * fabsf(s.uz);
+      walk_line<float, SCHEME, LAP, true>(nzs, s.diff, [&](int m) { return phi(e + d * m); },
+                                          [&](int) { return hu; }, finish);
+    } else {
+      for (int m = 0; m < nzs; ++m) finish(m, 0.f, phi(e + d * m), 0.f);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// k_march: blockDim = nb*nb threads (12 <= nb, nb*nb <= 576); thread (ti, tj)
+// owns the grid column (ti, tj, 0..nb-1).  Shared memory: the six face slabs
+// (face f at F + f*3nb^2), then plane buffers laid out like one z-plane of a
+// block with a 3-point shell, (y+3)*Ws + x+3 (the layout of a velocity plane):
+//   XP[2]  u_x phi / 2 on the x rows of a plane, x ghosts included
+//   YP[2]  u_y phi / 2 on the y columns, y ghosts included
+//   PH[3]  phi of the plane with its x/y ghosts (diffusion only)
+//   UX[2], UY[2]  u_x / 2 on the x rows, u_y / 2 on the y columns (velocity
+//          fields: the interface velocity that picks the upwind side)
+//   FX[2][nb][nb+1], FY[2][nb+1][nb]  halved x and y interface fluxes.
+// The column's phi and u_z at planes k-2..k+3 stay in registers, so the z fluxes need no
+// shared memory.  Interval t of the march (one barrier each) evaluates the
+// x/y fluxes of plane t, completes plane t-1 (z flux, rhs, RK stage,
+// coalesced store) and assembles plane t+1: XP/YP/FX/FY are double-buffered,
+// PH triple-buffered (plane t-1 is read while plane t+1 is written).  Every
+// flux is computed with the operations of k_fused (the point fluxes u*phi are
+// rounded products in both, never contracted; where the compiler fuses another
+// multiply-add differently the two may differ in the last bit).
+// ---------------------------------------------------------------------------
+// faces, XP..FY, PH[3], and (velocity fields) UX[2], UY[2]
+__host__ __device__ constexpr int march_smem_floats(int nb, bool vel) {
+  return 18 * nb * nb + 4 * nb * (nb + 1) + (vel ? 11 : 7) * (nb + 6) * (nb + 6);
+}
+
+template <int SCHEME, bool VEL>
+__global__ void __launch_bounds__(576, 2) k_march(Tree t, StageArgs s) {
+  constexpr int GS = 3;
+  const int b = blockIdx.x, nb = t.nb, Ws = nb + 2 * GS, W2 = Ws * Ws, nb1 = nb + 1, nth = nb * nb;
+  const int fs = 3 * nb * nb, Gi = s.Gi, diff = s.diff;
+  const float ux = 0.5f * s.ux, uy = 0.5f * s.uy, uz = 0.5f * s.uz, vscale = 0.5f * s.vscale;  // halved point fluxes
+  const float *const phi = s.phi;
+  const int tid = threadIdx.x, tj = tid / nb, ti = tid - tj * nb;
+  const int L = __ldg(t.lev + b);
+  const size_t nb3 = (size_t)nb * nb * nb;
+  extern __shared__ float sm[];
+  float *F = sm;
+  float *XP = F + 6 * fs;
+  float *YP = XP + 2 * W2;
+  float *FX = YP + 2 * W2;
+  float *FY = FX + 2 * nb * nb1;
+  float *PH = FY + 2 * nb * nb1;
+  float *UX = PH + 3 * W2, *UY = UX + 2 * W2;  // velocity fields only
+  // prologue: the face slabs
+  {
+    const int a[3] = {__ldg(t.anc + 3 * b) * nb, __ldg(t.anc + 3 * b + 1) * nb, __ldg(t.anc + 3 * b + 2) * nb};
+    __shared__ FaceSrc src[6];
+    face_sources(t, b, L, a, phi, s.P, s.Q, Gi, s.lifted, src);
+    __syncthreads();
+    const int Wd = nb + 2 * Gi;
+    for (int f = 0; f < 6; ++f)
+      for (int p = tid; p < fs; p += nth) {
+        // F index: the face's axis runs over 3 layers, the others over nb
+        const int n0 = f < 2 ? 3 : nb, n1 = f == 2 || f == 3 ? 3 : nb, r = p / n0, c2 = r / n1;
+        int c[3] = {p - r * n0, r - c2 * n1, c2};
+        c[f >> 1] += (f & 1) ? nb : -GS;
+        F[f * fs + p] = __ldg(face_ptr(src[f], f >> 1, c[0], c[1], c[2], nb, Wd));
+      }
+  }
+  // the column: interior from the field, or from the substituted padded block
+  // that k_prep wrote for leaves next to a coarser leaf
+  const float *col;
+  int cst;
+  if (s.cmask[b]) {
+    const int Wd = nb + 2 * Gi;
+    col = s.P + (size_t)b * Wd * Wd * Wd + (ti + Gi) + (size_t)Wd * ((tj + Gi) + (size_t)Wd * Gi);
+    cst = Wd * Wd;
+  } else {
+    col = phi + (size_t)b * nb3 + ti + nb * tj;
+    cst = nb * nb;
+  }
+  // velocity components: ghost-filled blocks with shell GS; the plane-buffer
+  // offset o of a point of plane z is o + W2*(z+GS) in them
+  const size_t vblk = (size_t)Ws * W2;
+  const float *vbx = VEL ? s.vpad + (size_t)b * vblk : nullptr;
+  const float *vby = VEL ? vbx + (size_t)t.nleaf * vblk : nullptr;
+  const float *vbz = VEL ? vby + (size_t)t.nleaf * vblk : nullptr;
+  const int cidx = (tj + GS) * Ws + ti + GS;  // the column's plane offset
+  // a velocity component at plane offset o of plane z
+  auto vat = [&](const float *vb, int o, int z) -> float { return vscale * __ldg(vb + o + W2 * (z + GS)); };
+  const bool xon = VEL || ux != 0.f, yon = VEL || uy != 0.f, zon = VEL || uz != 0.f;
+  // ghost columns/rows of a plane: thread tid < 12 nb fetches one of them
+  // (face index hsrc at plane 0, plane offset hdst; hy: a y ghost)
+  int hsrc = -1, hdst = 0, hy = 0;
+  if (tid < 6 * nb) {
+    const int j = tid / 6, m = tid - 6 * j, x = m < 3 ? m - GS : nb + m - GS;
+    hsrc = (m < 3 ? 0 : fs) + (m < 3 ? m : m - 3) + 3 * j;
+    hdst = (j + GS) * Ws + x + GS;
+  } else if (tid < 12 * nb) {
+    const int h = tid - 6 * nb, m = h / nb, i = h - m * nb, y = m < 3 ? m - GS : nb + m - GS;
+    hsrc = (m < 3 ? 2 * fs : 3 * fs) + i + nb * (m < 3 ? m : m - 3);
+    hdst = (y + GS) * Ws + i + GS;
+    hy = 1;
+  }
+  // x interfaces of a plane: flattened index tid, and tid + nth for tid < nb;
+  // interface i of row r is F_{i-1/2}, stored at FX[r*(nb+1) + i] = FX[index]
+  int xo0, xo1;
+  {
+    const int r0 = tid / nb1, r1 = (tid + nth) / nb1;
+    xo0 = (r0 + GS) * Ws + tid - r0 * nb1;  // plane offset of x = i-3 on row r
+    xo1 = (r1 + GS) * Ws + tid + nth - r1 * nb1;
+  }
+  auto xflux = [&](int buf, int z, int o, int fi) {
+    const float *p = XP + buf * W2 + o;
+    const float f6[6] = {p[0], p[1], p[2], p[3], p[4], p[5]};
+    const float *v = UX + buf * W2 + o;
+    const bool left = VEL ? (v[2] + v[3] >= 0.f) : ux >= 0.f;
+    FX[buf * nb * nb1 + fi] = half_flux6<float, SCHEME>(f6, left);
+  };
+  // y interfaces: F_{r-1/2} of column ti for r = tj, and r = nb for the last
+  // row of threads, stored at FY[r*nb + ti]
+  auto yflux = [&](int buf, int z, int r) {
+    const int o = r * Ws + ti + GS;  // plane offset of y = r-3
+    const float *p = YP + buf * W2 + o;
+    const float f6[6] = {p[0], p[Ws], p[2 * Ws], p[3 * Ws], p[4 * Ws], p[5 * Ws]};
+    const float *v = UY + buf * W2 + o;
+    const bool left = VEL ? (v[2 * Ws] + v[3 * Ws] >= 0.f) : uy >= 0.f;
+    FY[buf * nb1 * nb + r * nb + ti] = half_flux6<float, SCHEME>(f6, left);
+  };
+  // plane z into the buffers (z & 1) and z % 3; ph = phi at (ti, tj, z)
+  auto assemble = [&](int z, float ph, float vxv, float vyv) {
+    const int xb = (z & 1) * W2;
+    XP[xb + cidx] = __fmul_rn(vxv, ph);
+    YP[xb + cidx] = __fmul_rn(vyv, ph);
+    if (VEL) UX[xb + cidx] = vxv, UY[xb + cidx] = vyv;
+    if (diff) PH[(z % 3) * W2 + cidx] = ph;
+    if (hsrc >= 0) {
+      const float fv = F[hsrc + 3 * nb * z];
+      const float hu = VEL ? vat(hy ? vby : vbx, hdst, z) : (hy ? uy : ux);
+      (hy ? YP : XP)[xb + hdst] = __fmul_rn(hu, fv);
+      if (VEL) (hy ? UY : UX)[xb + hdst] = hu;
+      if (diff) PH[(z % 3) * W2 + hdst] = fv;
+    }
+  };
+  __syncthreads();
+  auto phi_at = [&](int m) -> float {
+    if (m < 0) return F[4 * fs + ti + nb * (tj + nb * (m + GS))];
+    if (m >= nb) return F[5 * fs + ti + nb * (tj + nb * (m - nb))];
+    return __ldg(col + (size_t)m * cst);
+  };
+  auto velz = [&](int z) -> float { return VEL ? vat(vbz, cidx, z) : uz; };
+  // register windows: phi and u_z at planes k-2..k+3 (k: the plane the next
+  // completion finishes); F_{k-1/2} along z
+  float pw[6], uw[6];
+#pragma unroll
+  for (int m = 0; m < 6; ++m) {
+    pw[m] = phi_at(m - 2);
+    uw[m] = velz(m - 2);
+  }
+  float Fzm = 0.f;
+  if (zon) {
+    const float u3 = velz(-3);
+    const float f6[6] = {__fmul_rn(u3, phi_at(-3)), __fmul_rn(uw[0], pw[0]), __fmul_rn(uw[1], pw[1]),
+                         __fmul_rn(uw[2], pw[2]),     __fmul_rn(uw[3], pw[3]), __fmul_rn(uw[4], pw[4])};
+    Fzm = half_flux6<float, SCHEME>(f6, VEL ? (uw[1] + uw[2] >= 0.f) : uz >= 0.f);
+  }
+  assemble(0, pw[2], VEL ? vat(vbx, cidx, 0) : ux, VEL ? vat(vby, cidx, 0) : uy);
+  __syncthreads();
+  const float h = (float)(t.tree_len / ((double)nb * (double)(1 << L)));
+  const float invh = 1.0f / h;
+  const bool rk_u = !s.rhs_only && s.stage > 0;
+  for (int tt = 0; tt <= nb; ++tt) {
+    // loads of this interval: the column's next window entries, the velocity
+    // of plane tt+1 and u^n of plane tt-1
+    const bool shift = tt >= 1 && tt < nb, asmb = tt + 1 < nb;
+    float pn = 0.f, uzn = 0.f, vxn = ux, vyn = uy, uo = 0.f;
+    if (shift) {
+      pn = phi_at(tt + 3);
+      uzn = velz(tt + 3);
+    }
+    if (VEL && asmb) {
+      vxn = vat(vbx, cidx, tt + 1);
+      vyn = vat(vby, cidx, tt + 1);
+    }
+    const size_t q = (size_t)b * nb3 + ti + nb * (tj + (size_t)nb * (tt - 1));
+    if (tt >= 1 && rk_u) uo = s.u[q];
+    // fluxes of plane tt
+    if (tt < nb) {
+      const int buf = tt & 1;
+      if (xon) {
+        xflux(buf, tt, xo0, tid);
+        if (tid < nb) xflux(buf, tt, xo1, tid + nth);
+      }
+      if (yon) {
+        yflux(buf, tt, tj);
+        if (tj == nb - 1) yflux(buf, tt, nb);
+      }
+    }
+    // completion of plane k = tt-1
+    if (tt >= 1) {
+      const int k = tt - 1, fb = k & 1;
+      float acc = 0.f;
+      if (xon) acc = FX[fb * nb * nb1 + tj * nb1 + ti + 1] - FX[fb * nb * nb1 + tj * nb1 + ti];
+      if (yon) acc += FY[fb * nb1 * nb + (tj + 1) * nb + ti] - FY[fb * nb1 * nb + tj * nb + ti];
+      if (zon) {
+        const float f6[6] = {__fmul_rn(uw[0], pw[0]), __fmul_rn(uw[1], pw[1]), __fmul_rn(uw[2], pw[2]),
+                             __fmul_rn(uw[3], pw[3]), __fmul_rn(uw[4], pw[4]), __fmul_rn(uw[5], pw[5])};
+        const float Fzp = half_flux6<float, SCHEME>(f6, VEL ? (uw[2] + uw[3] >= 0.f) : uz >= 0.f);
+        acc += Fzp - Fzm;
+        Fzm = Fzp;
+      }
+      float r = -2.f * (acc * invh);
+      if (diff) {
+        const float *pc = PH + (k % 3) * W2 + cidx;
+        float lp = 0.f;
+        lp += lap_term<float>(pc[-2], pc[-1], pc[0], pc[1], pc[2], diff);
+        lp += lap_term<float>(pc[-2 * Ws], pc[-Ws], pc[0], pc[Ws], pc[2 * Ws], diff);
+        lp += lap_term<float>(pw[0], pw[1], pw[2], pw[3], pw[4], diff);
+        r += s.nu * invh * invh * lp;
+      }
+      s.out[q] = stage_value(s, pw[2], r, uo);
+      if (shift) {
+#pragma unroll
+        for (int m = 0; m < 5; ++m) pw[m] = pw[m + 1], uw[m] = uw[m + 1];
+        pw[5] = pn;
+        uw[5] = uzn;
+      }
+    }
+    // plane tt+1 (the window now holds planes tt-2..tt+3)
+    if (asmb) assemble(tt + 1, pw[3], vxn, vyn);
+    __syncthreads();
+  }
+}
+
+// Host side: the variant (mr_set_stage_kernel: 0 tuned, 1 k_fused, 2
+// k_march) and, for k_fused, the slab height, tuned on launches that do not
+// overwrite their input (the bare right-hand side, stage 0).
+int launch_fused(mr_grid *g, const void *phi, const void *P, const void *Q, int Gi, const void *u, void *out,
+                 int stage, double dt, const double *uc, int scheme, bool rhs_only, const void *vpad) {
+  static const double zero3[3] = {0.0, 0.0, 0.0};
+  if (!uc) uc = zero3;
+  Tree t = tree_view(g);
+  const bool vel = vpad != nullptr;
+  const int nb = g->desc.nb, N = g->desc.wav_N, NT = g->desc.wav_Nt;
+  if (nb > 26) {  // the block with its ghosts and flux differences exceeds an SM's shared memory
+    set_error("FP32 stage: blocks of more than 26 points per edge");
+    return MR_ERR_CUDA;
+  }
+  StageArgs s{(const float *)phi, (const float *)P, (const float *)Q, Gi, NT != 0, g->cmask, (const float *)u,
+              (float *)out, stage, rhs_only ? 1 : 0, (float)dt, (float)uc[0], (float)uc[1], (float)uc[2],
+              (const float *)vpad, (float)g->diff_nu, (float)g->vel_scale, g->diff_order};
+  const bool march_ok = nb >= 12 && nb * nb <= 576;
+  const size_t smm = sizeof(float) * (size_t)march_smem_floats(nb, vel);
+  // slab heights: a quarter of the block (at least four planes), or four planes
+  // of a large and half of a small block
+  const int hq = nb > 16 ? (nb + 3) / 4 : 4, ht = nb > 16 ? 4 : std::max(6, nb / 2);
+  auto threads_of = [&](int nz) { return std::min(288, (2 * nb * nz + 31) / 32 * 32); };
+  const int cand[2] = {threads_of(hq), threads_of(ht)};
+  const int ncand = cand[0] != cand[1] ? 2 : 1;
+  const int vcand[2] = {1, 2};
+  const bool can_tune = rhs_only || stage == 0;
+  auto run = [&](auto kf, auto km) -> int {
+    const int smf_max = (int)sizeof(float) * fused_smem_floats(nb, std::max(hq, ht), vel);
+    if (check_cuda(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, smf_max), "fused smem"))
+      return MR_ERR_CUDA;
+    if (march_ok &&
+        check_cuda(cudaFuncSetAttribute(km, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smm), "march smem"))
+      return MR_ERR_CUDA;
+    const int mode = 2 * scheme + (vel ? 1 : 0);
+    auto fused = [&](int th) {
+      const int nz = th == cand[0] ? hq : ht, ns = (nb + nz - 1) / nz;
+      kf<<<g->nleaf * ns, th, sizeof(float) * fused_smem_floats(nb, nz, vel), g->stream>>>(t, s, nz, ns);
+    };
+    auto march = [&]() { km<<<g->nleaf, nb * nb, smm, g->stream>>>(t, s); };
+    const int threads = tune_threads(g, TuneKey{3, N, NT, nb, 4, Gi, mode}, cand, can_tune ? ncand : 1, fused);
+    int variant = march_ok ? g->stage_kernel : 1;
+    if (variant == 0)
+      variant = tune_threads(g, TuneKey{6, N, NT, nb, 4, Gi, mode}, vcand, can_tune ? 2 : 1,
+                             [&](int v) { v == 2 ? march() : fused(threads); });
+    if (variant == 2) MR_LAUNCH(g, MRK_RHS, march());
+    else MR_LAUNCH(g, MRK_RHS, fused(threads));
+    return check_cuda(cudaGetLastError(), variant == 2 ? "k_march" : "k_fused") ? MR_ERR_CUDA : MR_OK;
+  };
+#define MR_FV(S)                                                                                         \
+  do {                                                                                                   \
+    if (g->diff_order)                                                                                   \
+      return vel ? run(k_fused<S, true, true>, k_march<S, true>) : run(k_fused<S, false, true>, k_march<S, false>); \
+    return vel ? run(k_fused<S, true, false>, k_march<S, true>) : run(k_fused<S, false, false>, k_march<S, false>); \
+  } while (0)
+  if (scheme == MR_CONS3) MR_FV(MR_CONS3);
+  if (scheme == MR_CONS5) MR_FV(MR_CONS5);
+  if (scheme == MR_WENOZ5) MR_FV(MR_WENOZ5);
+#undef MR_FV
+  return MR_ERR_INVALID;
+}
+
+}  // namespace mr

@@ -39,13 +39,12 @@ __global__ void __launch_bounds__(256) k_rhs_stage(Tree t, const T *__restrict__
   auto walk = [&](int d, const T *p, const T *v, int st, int sv, int n, auto emit) {
     if (vpad) {
       v += d * vcomp;
-      walk_line<T, SCHEME>(
-          n, [&](int m) { return rmul(rmul(hscale, v[m * sv]), p[m * st]); },
-          [&](int m) { return rmul(hscale, v[m * sv]); }, emit);
+      walk_line<T, SCHEME, false, false>(
+          n, 0, [&](int m) { return p[m * st]; }, [&](int m) { return rmul(hscale, v[m * sv]); }, emit);
     } else {
-      const T ud = d == 0 ? ux : d == 1 ? uy : uz, hu = T(0.5) * ud;
-      walk_line<T, SCHEME>(
-          n, [&](int m) { return rmul(hu, p[m * st]); }, [&](int) { return ud; }, emit);
+      const T hu = T(0.5) * (d == 0 ? ux : d == 1 ? uy : uz);
+      walk_line<T, SCHEME, false, false>(
+          n, 0, [&](int m) { return p[m * st]; }, [&](int) { return hu; }, emit);
     }
   };
   const bool xon = vpad || ux != T(0), yon = vpad || uy != T(0), zon = vpad || uz != T(0);
@@ -61,7 +60,7 @@ __global__ void __launch_bounds__(256) k_rhs_stage(Tree t, const T *__restrict__
     T *rr = (yd ? R1 : R0) + i + RS * (j + nb * k);
     const int rs = yd ? RS : 1;
     walk(yd ? 1 : 0, Pb + o, Vb + (vpad ? ov : 0), yd ? Wd : 1, yd ? Wv : 1, n,
-         [&](int m, T dF) { rr[m * rs] = dF; });
+         [&](int m, T dF, T, T) { rr[m * rs] = dF; });
   }
   __syncthreads();
   const T h = T(t.tree_len / ((double)nb * (double)(1 << __ldg(t.lev + b)))), inv2 = T(2) / h, invh2 = T(1) / (h * h);
@@ -70,7 +69,7 @@ __global__ void __launch_bounds__(256) k_rhs_stage(Tree t, const T *__restrict__
     const int j = c / nb, i = c - j * nb;
     const T *p = Pb + i + Wd * j;
     const size_t q0 = (size_t)b * nb * nb * nb + c + (size_t)nb * nb * k0;
-    auto finish = [&](int m, T dz) {
+    auto finish = [&](int m, T dz, T ph, T) {
       const int ro = i + RS * (j + nb * m);
       T acc = T(0);
       if (xon) acc = R0[ro];
@@ -83,7 +82,7 @@ __global__ void __launch_bounds__(256) k_rhs_stage(Tree t, const T *__restrict__
       if (rhs_only) {
         out[q] = r;
       } else {
-        const T v = pc[0] + dt * r;
+        const T v = ph + dt * r;
         T o;
         if (stage == 0) o = v;
         else if (stage == 1) o = T(0.75) * u[q] + T(0.25) * v;
@@ -94,7 +93,7 @@ __global__ void __launch_bounds__(256) k_rhs_stage(Tree t, const T *__restrict__
     if (zon)
       walk(2, p, Vb + (vpad ? i + Wv * j : 0), Wd * Wd, Wv * Wv, nzs, finish);
     else
-      for (int m = 0; m < nzs; ++m) finish(m, T(0));
+      for (int m = 0; m < nzs; ++m) finish(m, T(0), p[(size_t)m * Wd * Wd], T(0));
   }
 }
 
@@ -155,29 +154,6 @@ __global__ void k_rk_combine(size_t n, int stage, T dt, const T *u, const T *y, 
   }
 }
 
-
-// fused_launch<N, NT> is instantiated in stage_i_*.cu
-#define MR_FEXT(n_, nt_)                                                                                      \
-  extern template int fused_launch<n_, nt_>(mr_grid *, const float *, const float *, const float *, int,     \
-                                            const float *, float *, int, double, const double *, int, bool,  \
-                                            const float *);
-MR_FEXT(2, 0) MR_FEXT(2, 2) MR_FEXT(4, 0) MR_FEXT(4, 2) MR_FEXT(6, 0) MR_FEXT(6, 2)
-#undef MR_FEXT
-
-int launch_fused(mr_grid *g, const void *phi, const void *P, const void *Q, int Gi, const void *u, void *out,
-                 int stage, double dt, const double *uc, int scheme, bool rhs_only, const void *vpad) {
-  const int N = g->desc.wav_N, Nt = g->desc.wav_Nt;
-  const float *a = (const float *)phi, *p = (const float *)P, *q = (const float *)Q, *uu = (const float *)u;
-  const float *vp = (const float *)vpad;
-  float *o = (float *)out;
-  static const double zero3[3] = {0.0, 0.0, 0.0};
-  if (!uc) uc = zero3;
-#define MR_FCASE(n_, nt_) \
-  if (N == n_ && Nt == nt_) return fused_launch<n_, nt_>(g, a, p, q, Gi, uu, o, stage, dt, uc, scheme, rhs_only, vp);
-  MR_FCASE(2, 0) MR_FCASE(2, 2) MR_FCASE(4, 0) MR_FCASE(4, 2) MR_FCASE(6, 0) MR_FCASE(6, 2)
-#undef MR_FCASE
-  return MR_ERR_UNSUPPORTED;
-}
 
 int launch_rk_combine(mr_grid *g, int stage, double dt, const void *u, const void *y, const void *r,
                       void *out) {
