@@ -99,10 +99,6 @@ int launch_ghost(mr_grid *g, const void *phi_in, void *phi_out, int G, bool fp64
   *Gi = gi;
   if (p_is64) *p_is64 = fp64 || g->desc.precision == MR_F64;
   const bool f32 = g->desc.precision == MR_F32;
-  if (grid_bounded(g)) {  // physical boundaries: the general point-wise path (every leaf)
-    *P = fp64 ? (void *)g->padP64 : g->padP;
-    return ghost_bounded(g, phi_in, phi_out, G, fp64, *P, fp64 ? (void *)g->padQ64 : g->padQ, gi);
-  }
   if (fp64) {
     *P = g->padP64;
     if (f32)

@@ -48,12 +48,129 @@ __device__ __forceinline__ TI leaf_value(const Tree &t, const TI *phi, int o, in
   return ld(phi + (size_t)o * nb * nb * nb + lx + nb * (ly + nb * lz));
 }
 
+// ---------------------------------------------------------------------------
+// Physical boundaries (Sec. 2.4).  Along a bounded axis, points beyond the
+// domain take the polynomial of degree < N through grid values next to the
+// boundary (or zeros); along several bounded axes the one-axis polynomials
+// multiply.  The regions of a block's neighbourhood beyond the domain count as
+// the block's own (level L, its own slot) in the region tables of the kernels
+// below: they are filled with in-range values first, and bc_box then
+// overwrites every point beyond the domain -- in the coarse tile before
+// refinement (Alg. SM1), in the block before substitution and coarsening
+// (Alg. SM2), and once more when every ghost is known.
+// ---------------------------------------------------------------------------
+
+// Nodes and weights of the boundary polynomial for the point r relative to the
+// boundary (lower: r < 0, domain points 0, 1, ...; upper: r >= 0, domain points
+// -1, -2, ...): value = sum_j w[j] f(node[j]).  Returns the node count, 0 for
+// plain zeros.  Zero value: 0 at position 0 and the N-1 nearest points off it.
+template <int N>
+__device__ int bc_weights(int bc, int r, bool lower, int *node, double *w) {
+  if (bc == MR_BC_ZERO) return 0;
+  const int first = bc == MR_BC_DIRICHLET0 ? 1 : 0, m = N - first;
+  double xs[N];
+  for (int i = 0; i < N; ++i) xs[i] = lower ? (double)i : bc == MR_BC_DIRICHLET0 ? (double)-i : (double)(-1 - i);
+  for (int j = 0; j < m; ++j) {
+    const int jj = j + first;
+    double wj = 1.0;
+    for (int k = 0; k < N; ++k)
+      if (k != jj) wj *= ((double)r - xs[k]) / (xs[jj] - xs[k]);
+    w[j] = wj;
+    node[j] = (int)xs[jj];
+  }
+  return m;
+}
+
+// first index inside the domain and one past the last along axis d, local to a
+// block whose first point is a at level L (no limit along a periodic axis)
+__device__ __forceinline__ int bc_first(const Tree &t, int a, int d) { return (t.bnd >> d) & 1 ? -a : -(1 << 28); }
+__device__ __forceinline__ int bc_end(const Tree &t, int L, int a, int d) {
+  return (t.bnd >> d) & 1 ? npts(t, L, d) - a : 1 << 28;
+}
+// the cube [lo, hi)^3 around that block reaches beyond the domain
+__device__ __forceinline__ bool bc_touches(const Tree &t, int L, int ax, int ay, int az, int lo, int hi) {
+  return lo < bc_first(t, ax, 0) || hi > bc_end(t, L, ax, 0) || lo < bc_first(t, ay, 1) || hi > bc_end(t, L, ay, 1) ||
+         lo < bc_first(t, az, 2) || hi > bc_end(t, L, az, 2);
+}
+
+// Every point of the box [lo, lo + n) beyond the domain, axis by axis: A[x +
+// s1 y + s2 z], indices local to the block whose first level-L point is (ax,
+// ay, az).  The whole CTA takes part; the nodes lie inside the box.  Out of
+// line: only blocks at a boundary call it.
+template <int N, typename TP>
+__device__ __noinline__ void bc_box(const Tree &t, int L, int ax, int ay, int az, TP *A, int s1, int s2, int lx, int ly,
+                                    int lz, int ex, int ey, int ez) {
+  __shared__ double wt[MR_MAX_SHELL + 4][N];
+  __shared__ int nd[N], nn;
+  const int st[3] = {1, s1, s2}, lo[3] = {lx, ly, lz}, hi[3] = {lx + ex, ly + ey, lz + ez}, a[3] = {ax, ay, az};
+  const int bc = t.bc;
+  for (int d = 0; d < 3; ++d)
+    for (int side = 0; side < 2; ++side) {
+      const int org = side ? bc_end(t, L, a[d], d) : bc_first(t, a[d], d);
+      const int l0 = side ? max(org, lo[d]) : lo[d], l1 = side ? hi[d] : min(org, hi[d]), n = l1 - l0;
+      if (n <= 0) continue;
+      __syncthreads();  // the values this side reads; the tables of the last one
+      if ((int)threadIdx.x < n) {
+        double w[N];
+        int node[N];
+        const int c = bc_weights<N>(bc, l0 + (int)threadIdx.x - org, !side, node, w);
+        for (int j = 0; j < c; ++j) wt[threadIdx.x][j] = w[j];
+        if (threadIdx.x == 0) {
+          nn = c;
+          for (int j = 0; j < c; ++j) nd[j] = node[j] + org;
+        }
+      }
+      __syncthreads();
+      const int e1 = d == 0 ? 1 : 0, e2 = d == 2 ? 1 : 2, n1 = hi[e1] - lo[e1], n2 = hi[e2] - lo[e2];
+      const DivM dn = divm(n), d1 = divm(n1);
+      for (int p = threadIdx.x; p < n * n1 * n2; p += blockDim.x) {
+        const int r = divq(p, dn), l = p - r * n, q2 = divq(r, d1), q1 = r - q2 * n1;
+        TP *c = A + st[e1] * (lo[e1] + q1) + st[e2] * (lo[e2] + q2);
+        TP v = TP(0);
+        for (int j = 0; j < nn; ++j) v += TP(wt[l][j]) * c[st[d] * nd[j]];
+        c[st[d] * (l0 + l)] = v;
+      }
+    }
+  __syncthreads();
+}
+
+// Coarse value of Alg. SM1 at level-Lq point q next to leaf hb: the stored
+// value inside the domain, the tensor of the boundary polynomials beyond it.
+// One point at a time, for coarse tiles that do not fit in shared memory.
+template <typename TI, typename TP, int N>
+__device__ __noinline__ TP coarse_bc(const Tree &t, int Lq, int qx, int qy, int qz, const TI *phi, int hb, int *err) {
+  const int q[3] = {qx, qy, qz};
+  int m[3], idx[3][N];
+  double w[3][N];
+  for (int d = 0; d < 3; ++d) {
+    m[d] = 1, idx[d][0] = q[d], w[d][0] = 1.0;
+    if (!beyond(t, Lq, q[d], d)) continue;
+    const int org = q[d] < 0 ? 0 : npts(t, Lq, d);
+    m[d] = bc_weights<N>(t.bc, q[d] - org, q[d] < 0, idx[d], w[d]);
+    for (int j = 0; j < m[d]; ++j) idx[d][j] += org;
+  }
+  TP s = TP(0);
+  for (int c = 0; c < m[2]; ++c)
+    for (int b = 0; b < m[1]; ++b)
+      for (int a = 0; a < m[0]; ++a) {
+        const int o = owner(t, Lq, idx[0][a], idx[1][b], idx[2][c], hb);
+        if (__ldg(t.lev + o) < Lq) {
+          atomicOr(err, 2);
+          return TP(0);
+        }
+        s += TP(w[0][a] * w[1][b] * w[2][c]) *
+             Cvt<TP>::f(leaf_value(t, phi, o, Lq, idx[0][a], idx[1][b], idx[2][c], err));
+      }
+  return s;
+}
+
 // Zero-detail refinement at level-L point g from the level-(L-1) values
 // (J^s on even, K^s on odd coordinates; taps landing on details skipped).
 template <typename TI, typename TP, int N, int NT>
 __device__ TP refine_point(const Tree &t, const TI *phi, int L, int gx, int gy, int gz, int *err, int hb) {
   return refine_dispatch<N, NT, TP>(gx & 1, gy & 1, gz & 1, [&](int ox, int oy, int oz) -> TP {
-    const int qx = (gx + ox) / 2, qy = (gy + oy) / 2, qz = (gz + oz) / 2;
+    const int qx = floordiv2(gx + ox), qy = floordiv2(gy + oy), qz = floordiv2(gz + oz);
+    if (t.bnd) return coarse_bc<TI, TP, N>(t, L - 1, qx, qy, qz, phi, hb, err);
     const int o = owner(t, L - 1, qx, qy, qz, hb);
     if (__ldg(t.lev + o) < L - 1) {
       atomicOr(err, 2);
@@ -64,174 +181,269 @@ __device__ TP refine_point(const Tree &t, const TI *phi, int L, int gx, int gy, 
 }
 
 // ---------------------------------------------------------------------------
-// Part 1 with the coarse-level values staged in shared memory, substitution,
-// and Part 2 pushed to the coarser neighbours.
+// The pre-pass of a leaf next to coarser ones: zero-detail refinement of the
+// coarser leaves' regions of its padded block (Part 1), substitution of the
+// band next to them, and Part 2 pushed to the coarser neighbours.
 //
-// T tile: every level-(L-1) value the zero-detail refinement of the padded
-// cube can read, fetched once (one owner lookup per coarse point instead of
-// one per tap).  Same taps and weights as refine_point.
-// After the substitution, the leaf coarsens (tensor H^a) its padded block at
-// every ghost point (shell Gpush) of each coarser neighbour c that lies in
-// the leaf's region, and writes the value into c's entry of Q: each ghost
-// point of c is owned by exactly one finer leaf, so the writes never collide.
+// Coarser neighbours by parent: a leaf's coarser neighbours touch its parent
+// from outside, so they lie in the (up to) seven directions e = 1..7 of the
+// parent's outward sides (bit d of e: across axis d, on the side of the
+// leaf's own half), and the neighbour in direction e owns one box of the
+// padded block: the shell along the axes of e, the block and its inward ghosts
+// along the others.  Refinement boxes, band boxes and push boxes are therefore
+// intervals per axis, cut into disjoint boxes by at most one clip each.
+//
+// Every phase is a flat list of items over all boxes (or as many as the
+// shared-memory sums allow), so the CTA meets a handful of barriers per leaf
+// instead of one per box and pass, and the index tables of a phase are built
+// by one thread each and read by all.  What bounds the kernel is issued
+// instructions (index arithmetic) and, after that, the latency of its ~20
+// dependent phases at 32 warps per SM.
 // ---------------------------------------------------------------------------
-template <int N>
-__host__ __device__ constexpr int tq_lo(int Gi) { return -((Gi + 2) / 2) - (N / 2 - 1); }
-template <int N>
-__host__ __device__ constexpr int tq_hi(int nb, int Gi) { return (nb + Gi - 2) / 2 + N / 2; }
-
-// ---------------------------------------------------------------------------
-// Separable substitution of the parity classes of one degree (2 or 3) over
-// the band boxes.  A band point p of a class with odd dimensions o_1..o_deg
-// becomes -S(p), S(p) = sum over t != 0 (t along the odd dimensions) of
-// prod_d G^a(t_d) P(p + t).  S is summed one odd dimension at a time,
-// thinnest box side first, with the partial sums of each (box, class) job in
-// shared memory: pass 1 reads the padded block at every point the later
-// passes need (odd dimensions not yet summed span the box plus the G^a
-// half-width), pass deg writes -S into the block.  Pass 1 drops its t = 0 term
-// where every other odd coordinate is odd -- exactly at the class points,
-// which no other term of any pass reads -- so the product over all t leaves
-// out t = 0.  Points of one degree read lower degrees only, so all jobs of a
-// degree run together, batched so that their partial sums fit in cap
-// elements; a job that does not fit alone runs point by point.
-// ---------------------------------------------------------------------------
-struct SubJob {
-  int lo[3], hi[3];
-  int om;          // odd dimensions (bit d)
-  int o0, o1, o2;  // odd dimensions, ascending box side
-  bool empty;
+struct PrepTab {
+  int rslot[27], rlev[27], ranc[27][3], rsub[27][8];
+  // level-(L-1) values of a region held by one leaf: index rbase + rmul *
+  // (q0 + nb q1 + nb^2 q2) of the block-local coarse point q (rmul 0: finer)
+  long long rbase[27];
+  int rmul[27];
+  int cmask, ce;  // coarser directions (bit region), coarser neighbours (bit e)
+  int s[3], odd[3];  // outward side per axis (+-1), anchor parity
 };
 
-__device__ __forceinline__ SubJob sub_job(const BoxList &bl, int j, int deg) {
-  SubJob J;
-  const int ncls = deg == 2 ? 3 : 1, e = j / ncls, k = j % ncls;
-  J.om = deg == 3 ? 7 : k == 0 ? 3 : k == 1 ? 5 : 6;
-  J.empty = false;
-  for (int d = 0; d < 3; ++d) {
-    J.lo[d] = bl.lo[e][d], J.hi[d] = bl.hi[e][d];
-    J.empty |= J.hi[d] <= J.lo[d];
+// up to 7 disjoint boxes over [0, n) per axis, the layers (dlo on the - side,
+// dhi on the + side) next to the coarser neighbours ce
+struct Boxes {
+  int n, lo[7][3], hi[7][3];
+};
+__device__ __forceinline__ void outward_boxes(Boxes &B, int ce, const int *s, int n, int dlo, int dhi) {
+  const int order[7] = {1, 2, 4, 3, 5, 6, 7};
+  int cnt = 0, kept = 0;
+  for (int q = 0; q < 7; ++q) {
+    const int e = order[q];
+    if (!((ce >> e) & 1)) continue;
+    bool inside = false;
+    for (int f = 1; f < 7; ++f) inside |= ((kept >> f) & 1) && (f & e) == f;
+    if (inside) continue;
+    int lo[3], hi[3];
+    for (int d = 0; d < 3; ++d) {
+      const bool on = (e >> d) & 1;
+      lo[d] = on && s[d] > 0 ? n - dhi : 0, hi[d] = on && s[d] < 0 ? dlo : n;
+    }
+    // an earlier box (across the axes of f) covers this one along every axis
+    // but the one of f that e does not have
+    for (int f = 1; f < 7; ++f)
+      if ((kept >> f) & 1)
+        for (int d = 0; d < 3; ++d)
+          if (((f & ~e) >> d) & 1) {
+            if (s[d] > 0) hi[d] = min(hi[d], n - dhi);
+            else lo[d] = max(lo[d], dlo);
+          }
+    kept |= 1 << e;
+    if (lo[0] >= hi[0] || lo[1] >= hi[1] || lo[2] >= hi[2]) continue;
+    for (int d = 0; d < 3; ++d) B.lo[cnt][d] = lo[d], B.hi[cnt][d] = hi[d];
+    ++cnt;
   }
+  B.n = cnt;
+}
+
+// level-Lq value (Lq = L or L - 1) at block-local point (i, j, k) through the
+// region tables, or through the owner map beyond the neighbouring regions
+template <typename TI>
+__device__ __noinline__ TI prep_fetch(const Tree &t, const PrepTab &T, const TI *phi, int b, int L, int Lq, int i, int j,
+                                      int k, int *err) {
+  const int nb = t.nb, hb = nb / 2, sc = Lq == L ? 1 : 2;
+  const size_t nb3 = (size_t)nb * nb * nb;
+  const int f[3] = {i * sc, j * sc, k * sc};
+  bool in = true;
+  int r = 0, rl[3], h = 0;
+  for (int d = 2; d >= 0; --d) {
+    in &= f[d] >= -nb && f[d] < 2 * nb;
+    const int c = f[d] < 0 ? 0 : f[d] >= nb ? 2 : 1;
+    r = 3 * r + c, rl[d] = f[d] - (c - 1) * nb;
+    h |= (rl[d] >= hb) << d;
+  }
+  if (in) {
+    if (T.rlev[r] == L) return ld(phi + T.rslot[r] * nb3 + rl[0] + nb * (rl[1] + nb * rl[2]));
+    if (T.rlev[r] == L + 1 && T.rsub[r][h] >= 0)
+      return ld(phi + T.rsub[r][h] * nb3 + (2 * rl[0] - (h & 1) * nb) +
+                nb * ((2 * rl[1] - ((h >> 1) & 1) * nb) + nb * (2 * rl[2] - (h >> 2) * nb)));
+  }
+  int g[3];
+  for (int d = 0; d < 3; ++d) g[d] = (Lq == L ? T.ranc[13][d] * nb : T.ranc[13][d] * nb / 2) + (d == 0 ? i : d == 1 ? j : k);
+  const int o = owner(t, Lq, g[0], g[1], g[2], b);
+  if (__ldg(t.lev + o) < Lq) return TI(__int_as_float(0x7fc00000));
+  return leaf_value(t, phi, o, Lq, g[0], g[1], g[2], err);
+}
+
+// Partial-sum type of the refinement: the block's, or float pairs for an FP32
+// field in an FP64 block (the K^s weights are dyadic, exact in FP32).
+template <typename TI, typename TP>
+struct RefSum {
+  using U = TP;
+  static __device__ __forceinline__ U zero() { return TP(0); }
+  static __device__ __forceinline__ U from(TI v) { return Cvt<TP>::f(v); }
+  static __device__ __forceinline__ U acc(U s, double w, U v) { return racc(s, TP(w), v); }
+  static __device__ __forceinline__ U norm(U s) { return s; }
+  static __device__ __forceinline__ TP value(U s) { return s; }
+};
+template <>
+struct RefSum<float, double> {
+  using U = F2;
+  static __device__ __forceinline__ U zero() { return f2_of(0.f); }
+  static __device__ __forceinline__ U from(float v) { return f2_of(v); }
+  static __device__ __forceinline__ U acc(U s, double w, U v) { return f2_acc(s, float(w), v); }
+  static __device__ __forceinline__ U norm(U s) { return f2_norm(s); }
+  static __device__ __forceinline__ double value(U s) { return f2_dbl(s); }
+};
+
+// One box of a coarser leaf's region: expanded along the thin axis a, then b,
+// then c (b = x where it can, so that neighbouring threads are neighbours in
+// memory; the box is cut along c so that its sums fit in shared memory).
+struct RefBox {
+  int a, b, c;                 // axes
+  int la, lb, lc, na, nb, nc;  // fine range per axis of the walk: [l, l + n)
+  int cb, cc, mb, mc;          // coarse range of the sums along b, c
+  int mbp, nbp, S;             // pitches (odd: no bank conflicts)
+  int off;                     // U1 at off, U2 at off + na * mbp * mc
+  unsigned dmb;                // reciprocal of mb
+};
+
+constexpr int SUB_RUN = 4;  // points of one item of the substitution
+
+// One parity class (odd dimensions om) of degree deg over one band box: summed
+// one odd dimension at a time (o[0] first), as walked by subst_sep.
+struct SubJob {
+  int om, deg, o[3];
+  short st[3][3], cn[3][3];  // per pass: first point, count per axis
+  int sp1[3];              // per pass: axes walked with step 1 (others 2)
+  unsigned d0[3], d1[3];   // reciprocals of the item counts along axes 0, 1
+  int n[3], it[3];         // points per pass; items (runs of SUB_RUN points along o[pass])
+  int off, next;           // sums in shared memory; end of the batch this job opens
+};
+
+// ---------------------------------------------------------------------------
+// Separable substitution.  A band point p of a class with odd dimensions o_1..
+// o_deg becomes -S(p), S(p) = sum over t != 0 (t along the odd dimensions) of
+// prod_d G^a(t_d) P(p + t).  S is summed one odd dimension at a time, thinnest
+// box side first, with the partial sums of each (box, class) job in shared
+// memory: pass 1 reads the padded block at every point the later passes need
+// (odd dimensions not yet summed span the box plus the G^a half-width), the
+// last pass writes -S into the block.  Pass 1 drops its t = 0 term where every
+// other odd coordinate is odd -- exactly at the class points, which no other
+// term of any pass reads -- so the product over all t leaves out t = 0.
+// Points of one degree read lower degrees only, so all jobs of a degree run
+// together, batched so that their sums fit; a job that does not fit alone
+// runs point by point.  An item is a run of SUB_RUN points along the summed
+// dimension: their taps share a window of even points, loaded together (13
+// loads in flight for four points instead of 28 in four dependent rounds).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void sub_job_build(SubJob &J, const int *lo, const int *hi, int om, int hG) {
+  J.om = om, J.deg = __popc(om);
   int o[3], n = 0;
   for (int d = 0; d < 3; ++d)
-    if ((J.om >> d) & 1) o[n++] = d;
-  for (int a = 1; a < n; ++a)
-    for (int b = a; b > 0 && J.hi[o[b]] - J.lo[o[b]] < J.hi[o[b - 1]] - J.lo[o[b - 1]]; --b) {
-      const int x = o[b];
-      o[b] = o[b - 1], o[b - 1] = x;
+    if ((om >> d) & 1) o[n++] = d;
+  for (int x = 1; x < n; ++x)
+    for (int y = x; y > 0 && hi[o[y]] - lo[o[y]] < hi[o[y - 1]] - lo[o[y - 1]]; --y) {
+      const int w = o[y];
+      o[y] = o[y - 1], o[y - 1] = w;
     }
-  J.o0 = o[0], J.o1 = n > 1 ? o[1] : 0, J.o2 = n > 2 ? o[2] : 0;
-  return J;
-}
-
-// positions start + step * i (i < count) of stage s (s odd dimensions summed)
-__device__ __forceinline__ void sub_stage(const SubJob &J, int s, int hG, int st[3], int sp[3], int cn[3]) {
-  const int sm = (s >= 1 ? 1 << J.o0 : 0) | (s >= 2 ? 1 << J.o1 : 0) | (s >= 3 ? 1 << J.o2 : 0);
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int odd = (J.om >> d) & 1;
-    if (odd && !((sm >> d) & 1)) {
-      st[d] = J.lo[d] - hG, sp[d] = 1, cn[d] = J.hi[d] - J.lo[d] + 2 * hG;
-    } else {
-      st[d] = par_first(J.lo[d], odd), sp[d] = 2, cn[d] = par_count(J.lo[d], J.hi[d], odd);
+  int summed = 0;
+  for (int s = 0; s < 3; ++s) {
+    J.o[s] = s < n ? o[s] : 0;
+    J.n[s] = J.it[s] = 0;
+    if (s >= n) continue;
+    summed |= 1 << o[s];
+    J.sp1[s] = om & ~summed;
+    for (int d = 0; d < 3; ++d) {
+      const int odd = (om >> d) & 1;
+      if ((J.sp1[s] >> d) & 1) J.st[s][d] = (short)(lo[d] - hG), J.cn[s][d] = (short)(hi[d] - lo[d] + 2 * hG);
+      else J.st[s][d] = (short)par_first(lo[d], odd), J.cn[s][d] = (short)par_count(lo[d], hi[d], odd);
     }
+    J.n[s] = J.cn[s][0] * J.cn[s][1] * J.cn[s][2];
+    int m[3];
+    for (int d = 0; d < 3; ++d) m[d] = d == o[s] ? (J.cn[s][d] + SUB_RUN - 1) / SUB_RUN : J.cn[s][d];
+    J.it[s] = m[0] * m[1] * m[2];
+    J.d0[s] = divm(max(m[0], 1)).m, J.d1[s] = divm(max(m[1], 1)).m;
   }
 }
 
-__device__ __forceinline__ long sub_elems(const SubJob &J, int s, int hG) {
-  int st[3], sp[3], cn[3];
-  sub_stage(J, s, hG, st, sp, cn);
-  return J.empty ? 0 : (long)cn[0] * cn[1] * cn[2];
+// sums of the run: sum_t G^a(t) src[(2 m + t) st] for m = 0 .. n - 1 (t = 0
+// only with centre); put(m, sum)
+template <int N, int NT, typename TP, typename F>
+__device__ __forceinline__ void subst_run(const TP *src, int st, int n, bool centre, F put) {
+  using W = Wav<N, NT>;
+  constexpr int hG = W::hwG;
+  TP e[N - 1 + SUB_RUN], c[SUB_RUN];
+#pragma unroll
+  for (int x = 0; x < N - 1 + SUB_RUN; ++x) e[x] = x < N - 1 + n ? src[(2 * x - hG) * st] : TP(0);
+#pragma unroll
+  for (int m = 0; m < SUB_RUN; ++m) c[m] = centre && m < n ? src[2 * m * st] : TP(0);
+#pragma unroll
+  for (int m = 0; m < SUB_RUN; ++m) {
+    if (m >= n) break;
+    TP acc = c[m];
+#pragma unroll
+    for (int x = 0; x < N; ++x) acc = racc(acc, TP(W::G(2 * x - hG)), e[m + x]);
+    put(m, acc);
+  }
 }
 
 template <int N, int NT, typename TP>
-__device__ void subst_sep(TP *__restrict__ Pb, int Wd, int Gi, const BoxList &bl, int deg, TP *__restrict__ buf,
-                          long cap) {
-  using W = Wav<N, NT>;
-  constexpr int hG = W::hwG;
-  const int ps1 = Wd, ps2 = Wd * Wd;
-  const int njob = bl.n * (deg == 2 ? 3 : 1), bd = blockDim.x;
-  // buffer elements of a job: stages 1 .. deg-1
-  auto job_buf = [&](const SubJob &J) -> long {
-    return sub_elems(J, 1, hG) + (deg == 3 ? sub_elems(J, 2, hG) : 0);
-  };
-  int j0 = 0;
-  while (j0 < njob) {
-    long used = 0;
-    int j1 = j0;
-    while (j1 < njob) {
-      const long sz = job_buf(sub_job(bl, j1, deg));
-      if (j1 > j0 && used + sz > cap) break;
-      used += sz, ++j1;
-    }
-    if (used > cap) {
-      // one job too large for the buffer: point by point
-      const SubJob J = sub_job(bl, j0, deg);
-      int st[3], sp[3], cn[3];
-      sub_stage(J, deg, hG, st, sp, cn);
-      const int n = J.empty ? 0 : cn[0] * cn[1] * cn[2];
-      const DivM dc0 = divm(cn[0]), dc1 = divm(cn[1]);
-      for (int idx = threadIdx.x; idx < n; idx += bd) {
-        const int r = divq(idx, dc0), i2 = divq(r, dc1), i0 = idx - r * cn[0], i1 = r - i2 * cn[1];
-        TP *c = Pb + (st[0] + sp[0] * i0 + Gi) + ps1 * (st[1] + sp[1] * i1 + Gi) + ps2 * (st[2] + sp[2] * i2 + Gi);
-        *c = subst_dispatch<N, NT, TP>(J.om & 1, J.om & 2, J.om & 4, [&](int tx, int ty, int tz) -> TP {
-          return c[tx + ps1 * ty + ps2 * tz];
-        });
-      }
-      __syncthreads();
-      j0 = j1;
-      continue;
-    }
-    for (int s = 1; s <= deg; ++s) {
-      long base = 0, off = 0;
+__device__ __forceinline__ void subst_jobs(TP *Pb, int Wd, int Gi, const SubJob *jobs, int j0, int jend, TP *buf,
+                                           int cap) {
+  const int W2 = Wd * Wd, bd = blockDim.x;
+  while (j0 < jend) {
+    const int j1 = jobs[j0].next, deg = jobs[j0].deg;
+    const bool pointwise = jobs[j0].n[0] * (deg > 1) + jobs[j0].n[1] * (deg > 2) > cap;
+    for (int s = pointwise ? deg - 1 : 0; s < deg; ++s) {
+      int rot = 0;  // the items of a job continue the thread rotation of the previous one
       for (int j = j0; j < j1; ++j) {
-        const SubJob J = sub_job(bl, j, deg);
-        const long n1 = sub_elems(J, 1, hG), n2 = deg == 3 ? sub_elems(J, 2, hG) : 0;
-        int st[3], sp[3], cn[3], pst[3], psp[3], pcn[3];
-        sub_stage(J, s, hG, st, sp, cn);
-        sub_stage(J, s - 1 > 0 ? s - 1 : 1, hG, pst, psp, pcn);
-        const int n = J.empty ? 0 : cn[0] * cn[1] * cn[2];
-        const int d = s == 1 ? J.o0 : s == 2 ? J.o1 : J.o2;  // dimension summed in this pass
-        TP *dst = buf + off + (s == 2 ? n1 : 0);
-        const TP *prev = buf + off + (s == 3 ? n1 : 0);
-        const int q1 = pcn[0], q2 = pcn[0] * pcn[1];
-        const int oth = J.om & ~(1 << d);
-        const DivM dc0 = divm(cn[0]), dc1 = divm(cn[1]);
-        // this job's items continue the thread rotation of the previous jobs
-        int idx = (int)(((long)threadIdx.x - base) % bd);
+        const SubJob &J = jobs[j];
+        const int n = J.it[s];
+        int idx = (int)threadIdx.x - rot;
         if (idx < 0) idx += bd;
+        rot = (rot + n) & (bd - 1);
+        if (idx >= n) continue;
+        const int st0 = J.st[s][0], st1 = J.st[s][1], st2 = J.st[s][2], sp1 = J.sp1[s];
+        const int h0 = !(sp1 & 1), h1 = !(sp1 & 2), h2 = !(sp1 & 4);  // log2 of the steps
+        const int d = J.o[s], cd = J.cn[s][d];
+        const int c0 = J.cn[s][0], c1 = J.cn[s][1];
+        const int m0 = d == 0 ? (c0 + SUB_RUN - 1) / SUB_RUN : c0, m1 = d == 1 ? (c1 + SUB_RUN - 1) / SUB_RUN : c1;
+        const DivM dc0{J.d0[s], m0}, dc1{J.d1[s], m1};
+        const int str = d == 0 ? 1 : d == 1 ? Wd : W2, ds = d == 0 ? 1 : d == 1 ? c0 : c0 * c1;
+        TP *dst = buf + J.off + (s == 1 ? J.n[0] : 0);
+        const bool last = s == deg - 1;
         for (; idx < n; idx += bd) {
-          const int r = divq(idx, dc0), i2 = divq(r, dc1), i0 = idx - r * cn[0], i1 = r - i2 * cn[1];
-          const int p0 = st[0] + sp[0] * i0, p1 = st[1] + sp[1] * i1, p2 = st[2] + sp[2] * i2;
-          TP acc = TP(0);
-          if (s == 1) {
-            const TP *src = Pb + (p0 + Gi) + ps1 * (p1 + Gi) + ps2 * (p2 + Gi);
-            const int str = d == 0 ? 1 : d == 1 ? ps1 : ps2;
-            const bool keep0 = ((oth & 1) && !(p0 & 1)) || ((oth & 2) && !(p1 & 1)) || ((oth & 4) && !(p2 & 1));
-#pragma unroll
-            for (int t = -hG; t <= hG; ++t) {
-              if (W::G(t) == 0.0) continue;
-              if (t == 0) {
-                if (keep0) acc = racc(acc, TP(1), src[0]);
-              } else {
-                acc = racc(acc, TP(W::G(t)), src[t * str]);
-              }
+          const int r = divq(idx, dc0), q2 = divq(r, dc1), q0 = idx - r * m0, q1 = r - q2 * m1;
+          const int i0 = d == 0 ? q0 * SUB_RUN : q0, i1 = d == 1 ? q1 * SUB_RUN : q1, i2 = d == 2 ? q2 * SUB_RUN : q2;
+          const int nr = min(SUB_RUN, cd - (d == 0 ? i0 : d == 1 ? i1 : i2));  // points of this run
+          const int p0 = st0 + (i0 << h0), p1 = st1 + (i1 << h1), p2 = st2 + (i2 << h2);
+          TP *pt = Pb + (p0 + Gi) + Wd * (p1 + Gi) + W2 * (p2 + Gi);
+          TP *out = dst + i0 + c0 * (i1 + c1 * i2);
+          auto put = [&](int m, TP acc) {
+            if (last) pt[2 * m * str] = -acc;
+            else out[m * ds] = acc;
+          };
+          if (pointwise) {
+            for (int m = 0; m < nr; ++m) {
+              TP *c = pt + 2 * m * str;
+              *c = subst_dispatch<N, NT, TP>(J.om & 1, J.om & 2, J.om & 4,
+                                             [&](int tx, int ty, int tz) -> TP { return c[tx + Wd * ty + W2 * tz]; });
             }
+          } else if (s == 0) {
+            const int oth = J.om & ~(1 << d);
+            const bool keep0 = (oth & ~((p0 & 1) | ((p1 & 1) << 1) | ((p2 & 1) << 2))) != 0;
+            subst_run<N, NT>(pt, str, nr, keep0, put);
           } else {
-            const int c0 = d == 0 ? p0 - pst[0] : i0, c1 = d == 1 ? p1 - pst[1] : i1, c2 = d == 2 ? p2 - pst[2] : i2;
-            const TP *src = prev + c0 + q1 * c1 + q2 * c2;
-            const int str = d == 0 ? 1 : d == 1 ? q1 : q2;
-#pragma unroll
-            for (int t = -hG; t <= hG; ++t) {
-              if (W::G(t) == 0.0) continue;
-              acc = racc(acc, TP(W::G(t)), src[t * str]);
-            }
+            // the previous pass summed another dimension; along this one it ran
+            // with step 1 from st[s-1], along the others its points are this pass's
+            const int k0 = J.cn[s - 1][0], k1 = k0 * J.cn[s - 1][1], ps = d == 0 ? 1 : d == 1 ? k0 : k1;
+            const int lead = J.st[s][d] - J.st[s - 1][d];
+            const TP *src = buf + J.off + (s == 2 ? J.n[0] : 0) + lead * ps + (d == 0 ? 2 * i0 : i0) +
+                            k0 * (d == 1 ? 2 * i1 : i1) + k1 * (d == 2 ? 2 * i2 : i2);
+            subst_run<N, NT>(src, ps, nr, true, put);
           }
-          if (s == deg)
-            Pb[(p0 + Gi) + ps1 * (p1 + Gi) + ps2 * (p2 + Gi)] = -acc;
-          else
-            dst[idx] = acc;
         }
-        base += n, off += n1 + n2;
       }
       __syncthreads();
     }
@@ -239,632 +451,498 @@ __device__ void subst_sep(TP *__restrict__ Pb, int Wd, int Gi, const BoxList &bl
   }
 }
 
-template <typename TI, typename TP, int N, int NT>
-__global__ void __launch_bounds__(512, sizeof(TP) == 4 ? 2 : 1) k_prep(Tree t, const TI *__restrict__ phi, TP *__restrict__ P,
-                                                 TP *__restrict__ Q, int Gi, int Gpush, int only_coarse,
-                                                 int use_tile, int tile_bytes, int zc, int *cmask_out,
-                                                 int *err, const int *__restrict__ need, int prefilled,
-                                                 int dyn_bytes) {
-  using W = Wav<N, NT>;
-  const int b = blockIdx.x;
-  if (need && !need[b]) return;
-  const int nb = t.nb, Wd = nb + 2 * Gi;
-  const size_t np = (size_t)Wd * Wd * Wd, nb3 = (size_t)nb * nb * nb;
-  const int L = __ldg(t.lev + b);
-  const int ax = __ldg(t.anc + 3 * b) * nb, ay = __ldg(t.anc + 3 * b + 1) * nb,
-            az = __ldg(t.anc + 3 * b + 2) * nb;
-  // owners of the 27 block-sized regions around b (same or coarser leaves own
-  // a whole region; a finer region is resolved point by point)
-  __shared__ int rslot[27], rlev[27], ranc[27][3];
-  __shared__ int cmask;
-  __shared__ int cslots[27];
-  __shared__ int ncs;
-  if (threadIdx.x == 0) cmask = 0, ncs = 0;
-  __syncthreads();
-  if (threadIdx.x < 27) {
-    const int r = threadIdx.x;
-    const int dd[3] = {r % 3 - 1, (r / 3) % 3 - 1, r / 9 - 1};
-    int g[3];
-    for (int d = 0; d < 3; ++d)
-      g[d] = __ldg(t.anc + 3 * b + d) * nb + (dd[d] < 0 ? -1 : dd[d] > 0 ? nb : 0);
-    const int o = owner(t, L, g[0], g[1], g[2], b);
-    const int Lo = __ldg(t.lev + o);
-    rslot[r] = o, rlev[r] = Lo;
-    for (int d = 0; d < 3; ++d) ranc[r][d] = __ldg(t.anc + 3 * o + d);
-    if (r != 13) {
-      if (Lo < L - 1 || Lo > L + 1) atomicOr(err, 4);
-      if (Lo < L) atomicOr(&cmask, 1 << r);
+constexpr int PUSH_LAYERS = 4;
+
+// tensor H^a along one line: sum_t H^a(t) src[(2 m + t) st], m = 0 .. n - 1 <= M,
+// from one window of fine values; put(m, sum)
+template <int N, int NT, int M, typename TP, typename F>
+__device__ __forceinline__ void coarsen_run(const TP *src, int st, int n, F put) {
+  constexpr int hH = Wav<N, NT>::hwH, len = 2 * M - 1 + 2 * hH;
+  TP v[len];
+#pragma unroll
+  for (int x = 0; x < len; ++x) {
+    // (points that no sum with m < n reads are not loaded)
+    bool used = false;
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+      if (x - hH - 2 * m >= -hH && x - hH - 2 * m <= hH && Wav<N, NT>::H(x - hH - 2 * m) != 0.0) used |= m < n;
+    v[x] = used ? src[(x - hH) * st] : TP(0);
+  }
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    if (m >= n) break;
+    TP s = TP(0);
+    for_taps<N, NT, FK_H>([&](int t, double w) { s = racc(s, TP(w), v[2 * m + hH + t]); });
+    put(m, s);
+  }
+}
+
+// boxes, jobs and tables of the three phases (one set per CTA)
+struct PrepPlan {
+  Boxes band, push;
+  RefBox ref[28];
+  int nref, refnext[28];  // refinement boxes; end of the batch a box opens
+  SubJob job[49];
+  int job0[4];            // first job of each degree (job0[3]: end)
+};
+
+// The boundary polynomial on the sums U1 of one box (beyond the domain along b
+// and c; the refinement along a acts on another index, so it may go first).
+template <int N, typename TP>
+__device__ __noinline__ void bc_sums(const Tree &t, int Lc, const RefBox &B, int ax, int ay, int az, TP *U1) {
+  __shared__ double wt[MR_MAX_SHELL + 4][N];
+  __shared__ int nd[N], nn;
+  for (int w = 0; w < 4; ++w) {
+    const int d = w < 2 ? B.b : B.c, side = w & 1, anc = d == 0 ? ax : d == 1 ? ay : az;
+    const int lo = w < 2 ? B.cb : B.cc, hi = lo + (w < 2 ? B.mb : B.mc);
+    const int org = side ? bc_end(t, Lc, anc, d) : bc_first(t, anc, d);
+    const int l0 = side ? max(org, lo) : lo, l1 = side ? hi : min(org, hi), n = l1 - l0;
+    if (n <= 0) continue;
+    __syncthreads();
+    if ((int)threadIdx.x < n) {
+      double wv[N];
+      int node[N];
+      const int c = bc_weights<N>(t.bc, l0 + (int)threadIdx.x - org, !side, node, wv);
+      for (int j = 0; j < c; ++j) wt[threadIdx.x][j] = wv[j];
+      if (threadIdx.x == 0) {
+        nn = c;
+        for (int j = 0; j < c; ++j) nd[j] = node[j] + org - lo;
+      }
+    }
+    __syncthreads();
+    // strides: along the axis; the two others of the box
+    const int pa = B.mbp, pc = B.mbp * B.na, str = w < 2 ? 1 : pc, so = w < 2 ? pc : 1, no = w < 2 ? B.mc : B.mb;
+    for (int p = threadIdx.x; p < n * B.na * no; p += blockDim.x) {
+      const int l = p % n, r = p / n;
+      TP *c = U1 + pa * (r % B.na) + so * (r / B.na), v = TP(0);
+      for (int j = 0; j < nn; ++j) v += TP(wt[l][j]) * c[str * nd[j]];
+      c[str * (l0 + l - lo)] = v;
     }
   }
   __syncthreads();
-  const int mask = cmask;
-  if (threadIdx.x == 0 && cmask_out) cmask_out[b] = mask;
-  if (only_coarse && !mask) return;
-  // finer regions: the owners of their eight one-level-finer sub-blocks (-1:
-  // the sub-block is refined further), so their values need no owner lookup
-  const int hb = nb / 2;
-  __shared__ int rsub[27][8];
-  for (int q = threadIdx.x; q < 216; q += blockDim.x) {
+}
+
+// planes of the sums along c: a chunk of twelve fine points (so that no leaf
+// has more than 28 boxes), and on grids with physical boundaries the nodes of
+// the polynomial
+constexpr int prep_min_planes(int N, bool bounded) { return (N - 1) + 2 + 6 + (bounded ? N : 0); }
+
+// Zero-detail refinement along one line: fine points f0 .. f0 + n - 1 (n <= 16)
+// from the coarse values src[q * st] (q: coarse index); put(m, v) receives
+// point f0 + m.  A register window of N coarse values moves along the line and
+// yields an even (coincident) and an odd (K^s) point per step.
+template <int N, int NT, typename RS, typename U, typename F>
+__device__ __forceinline__ void refine_run(const U *src, int st, int f0, int n, F put) {
+  using W = Wav<N, NT>;
+  constexpr int ko = N - 1, h = N / 2;
+  // window w[0..N-1] = coarse q-h+1 .. q+h around the odd point 2q + 1
+  const int q0 = f0 >> 1;
+  U w[N];
+#pragma unroll
+  for (int x = 0; x + 1 < N; ++x) w[x] = src[(q0 - h + 1 + x) * st];
+  const int par = f0 & 1;
+  // (the last value of a window is read only where its odd point exists)
+  w[N - 1] = par || n > 1 ? src[(q0 + h) * st] : w[0];
+  for (int m = -par; m < n; m += 2) {  // even point m, odd point m + 1
+    if (m >= 0) put(m, w[h - 1]);
+    if (m + 1 < n) {
+      U s = RS::acc(RS::zero(), W::K(-ko), w[0]);
+#pragma unroll
+      for (int x = 1; x < N; ++x) s = RS::acc(s, W::K(2 * x - ko), w[x]);
+      put(m + 1, s);
+    }
+    if (m + 2 < n) {
+#pragma unroll
+      for (int x = 0; x + 1 < N; ++x) w[x] = w[x + 1];
+      if (m + 3 < n) w[N - 1] = src[(q0 + (m + par) / 2 + 1 + h) * st];
+    }
+  }
+}
+
+template <typename TI, typename TP, int N, int NT, bool BND>
+__global__ void __launch_bounds__(256, sizeof(TP) == 4 ? 4 : 3) k_prep(Tree t, const TI *__restrict__ phi,
+                                                                     TP *__restrict__ P, TP *__restrict__ Q, int Gi,
+                                                                     int Gpush, int only_coarse, int *cmask_out,
+                                                                     int *err, const int *__restrict__ need,
+                                                                     int sum_bytes) {
+  using W = Wav<N, NT>;
+  using RS = RefSum<TI, TP>;
+  using U = typename RS::U;
+  constexpr int ko = N - 1;  // widest odd K^s tap
+  const int b = blockIdx.x;
+  if (need && !need[b]) return;
+  const int nb = t.nb, Wd = nb + 2 * Gi, W2 = Wd * Wd, hb = nb / 2, tid = threadIdx.x, bd = blockDim.x;
+  const size_t np = (size_t)Wd * W2, nb3 = (size_t)nb * nb * nb;
+  const int L = __ldg(t.lev + b);
+  const int ax = __ldg(t.anc + 3 * b) * nb, ay = __ldg(t.anc + 3 * b + 1) * nb, az = __ldg(t.anc + 3 * b + 2) * nb;
+  __shared__ PrepTab T;
+  __shared__ PrepPlan plan;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int capU = sum_bytes / (int)sizeof(U), capP = sum_bytes / (int)sizeof(TP);
+  if (tid == 0) T.cmask = 0, T.ce = 0;
+  __syncthreads();
+  // owners of the 27 block-sized regions around b (same or coarser leaves own
+  // a whole region); regions beyond a physical boundary count as the block
+  if (tid < 27) {
+    const int r = tid;
+    const int dd[3] = {r % 3 - 1, (r / 3) % 3 - 1, r / 9 - 1}, an[3] = {ax / nb, ay / nb, az / nb};
+    int g[3], e = 0;
+    bool parent = true;  // the direction of a parent-level neighbour
+    for (int d = 0; d < 3; ++d) {
+      g[d] = an[d] * nb + (dd[d] < 0 ? -1 : dd[d] > 0 ? nb : 0);
+      const int s = (an[d] & 1) ? 1 : -1;
+      if (dd[d] == s) e |= 1 << d;
+      else parent &= dd[d] == 0;
+    }
+    const int o = BND && beyond3(t, L, g) ? b : owner(t, L, g[0], g[1], g[2], b);
+    const int Lo = __ldg(t.lev + o);
+    T.rslot[r] = o, T.rlev[r] = Lo;
+    long long base = 0;
+    int mul = 0;
+    if (Lo == L || Lo == L - 1) {
+      mul = Lo == L ? 2 : 1;
+      int st = 1;
+      base = (long long)o * (long long)nb3;
+      for (int d = 0; d < 3; ++d, st *= nb) {
+        const bool out = (e >> d) & 1;
+        const int od = an[d] & 1;
+        // same level: 2 q relative to the region; coarser: q relative to the
+        // neighbour of the parent (or, along this axis, the parent's own range)
+        base += (long long)st * (Lo == L ? -dd[d] * nb : out ? (od ? -hb : nb) : od * hb);
+      }
+    }
+    T.rbase[r] = base, T.rmul[r] = mul;
+    if (r != 13) {
+      if (Lo < L - 1 || Lo > L + 1) atomicOr(err, 4);
+      if (Lo < L) atomicOr(&T.cmask, 1 << r);
+      if (Lo < L && parent && e) atomicOr(&T.ce, 1 << e);
+    }
+    for (int d = 0; d < 3; ++d) T.ranc[r][d] = __ldg(t.anc + 3 * o + d);
+    if (r < 3) T.s[r] = (an[r] & 1) ? 1 : -1, T.odd[r] = an[r] & 1;
+  }
+  __syncthreads();
+  const int mask = T.cmask, ce = T.ce;
+  if (tid == 0 && cmask_out) cmask_out[b] = mask;
+  if (!mask) return;
+  // one thread per phase builds its boxes; the sub-blocks of finer regions (-1:
+  // refined further) are looked up meanwhile
+  if (tid == 0) {
+    int n = 0, used = 0, open = 0;
+    for (int e = 1; e < 8; ++e) {
+      if (!((ce >> e) & 1)) continue;
+      int l[3], m[3];
+      for (int d = 0; d < 3; ++d) {
+        const bool on = (e >> d) & 1;
+        l[d] = on ? (T.s[d] > 0 ? nb : -Gi) : (T.s[d] > 0 ? -Gi : 0);
+        m[d] = on ? Gi : nb + Gi;
+      }
+      RefBox B;
+      B.a = (e & 1) ? 0 : (e & 2) ? 1 : 2;
+      B.b = B.a == 0 ? 1 : 0, B.c = 3 - B.a - B.b;
+      B.la = l[B.a], B.na = m[B.a], B.lb = l[B.b], B.nb = m[B.b];
+      B.cb = (B.lb - ko) >> 1, B.mb = ((B.lb + B.nb - 1 + ko) >> 1) - B.cb + 1;
+      B.mbp = B.mb | 1, B.nbp = B.nb | 1, B.dmb = divm(B.mb).m;
+      B.S = (B.a == 0 ? B.na * B.nb : B.na * B.nbp) | 1;
+      // cut along c: mc planes of both sums
+      const int plane = B.na * B.mbp + B.S, most = capU / plane, ext = BND ? N : 0;
+      const int step = max(2 * (most - ko - 2 - ext), 2);
+      for (int c0 = 0; c0 < m[B.c]; c0 += step) {
+        B.lc = l[B.c] + c0, B.nc = min(step, m[B.c] - c0);
+        B.cc = (B.lc - ko) >> 1;
+        int ce1 = ((B.lc + B.nc - 1 + ko) >> 1) + 1;
+        if (BND) {  // the polynomial's nodes, where the chunk reaches beyond the domain
+          const int anc = (B.c == 0 ? ax : B.c == 1 ? ay : az) / 2;
+          const int first = bc_first(t, anc, B.c), end = bc_end(t, L - 1, anc, B.c);
+          if (B.cc < first) ce1 = max(ce1, first + N);
+          if (ce1 > end) B.cc = min(B.cc, end - N);
+        }
+        B.mc = ce1 - B.cc;
+        const int sz = plane * B.mc;
+        if (n && used + sz > capU) {
+          for (int q = open; q < n; ++q) plan.refnext[q] = n;
+          open = n, used = 0;
+        }
+        B.off = used, plan.ref[n++] = B;
+        used += sz;
+      }
+    }
+    for (int q = open; q < n; ++q) plan.refnext[q] = n;
+    plan.nref = n;
+  } else if (tid == 32) {
+    outward_boxes(plan.band, ce, T.s, nb, W::ext_b, W::ext_f);
+  } else if (tid == 64) {
+    const int gp = min(Gpush, hb);
+    outward_boxes(plan.push, ce, T.s, hb, gp, gp);
+  }
+  for (int q = tid; q < 216; q += bd) {
     const int r = q >> 3, h = q & 7;
     int o2 = -1;
-    if (rlev[r] == L + 1 && L < t.M) {
+    if (T.rlev[r] == L + 1 && L < t.M) {
       const int dd[3] = {r % 3 - 1, (r / 3) % 3 - 1, r / 9 - 1};
       int g[3];
-      for (int d = 0; d < 3; ++d) g[d] = 2 * (__ldg(t.anc + 3 * b + d) + dd[d]) * nb + ((h >> d) & 1) * nb;
+      for (int d = 0; d < 3; ++d) g[d] = 2 * (T.ranc[13][d] + dd[d]) * nb + ((h >> d) & 1) * nb;
       o2 = owner(t, L + 1, g[0], g[1], g[2], b);
       if (o2 < 0 || o2 >= t.nleaf || __ldg(t.lev + o2) != L + 1) o2 = -1;
     }
-    rsub[r][h] = o2;
+    T.rsub[r][h] = o2;
   }
-  __syncthreads();  // rsub is read by every fetch below
-  // index into phi of the value stored at level-Lq point (i, j, k) (block-
-  // local level-L coords when Lq == L, coarse-local when Lq == L-1) from the
-  // region tables, or -1 where only the owner map resolves it
-  auto src_index = [&](int Lq, int i, int j, int k) -> long long {
-    const int sc = (Lq == L) ? 1 : 2;  // fine-index scale of the point
-    const int fi = i * sc, fj = j * sc, fk = k * sc;
-    if (fi < -nb || fi >= 2 * nb || fj < -nb || fj >= 2 * nb || fk < -nb || fk >= 2 * nb) return -1;
-    const int rx = fi < 0 ? 0 : fi >= nb ? 2 : 1, ry = fj < 0 ? 0 : fj >= nb ? 2 : 1, rz = fk < 0 ? 0 : fk >= nb ? 2 : 1;
-    const int r = rx + 3 * ry + 9 * rz;
-    const int Lo = rlev[r], o = rslot[r];
-    const int ri = fi - (rx - 1) * nb, rj = fj - (ry - 1) * nb, rk = fk - (rz - 1) * nb;  // region-local
-    if (Lo == L) return (long long)o * (long long)nb3 + ri + nb * (rj + nb * rk);
-    if (Lo == L - 1) {
-      // coarse leaf: level-(L-1) index of the point, relative to its anchor
-      const int gq[3] = {(ax + fi) / 2, (ay + fj) / 2, (az + fk) / 2};
-      int l[3];
-      for (int d = 0; d < 3; ++d) l[d] = pwrap(gq[d] - ranc[r][d] * nb, period(t, L - 1, d));
-      return (long long)o * (long long)nb3 + l[0] + nb * (l[1] + nb * l[2]);
-    }
-    if (Lo == L + 1) {
-      // the coincident point of the finer leaf holding the sub-block
-      const int hx = ri >= hb, hy = rj >= hb, hz = rk >= hb;
-      const int o2 = rsub[r][hx + 2 * hy + 4 * hz];
-      if (o2 >= 0)
-        return (long long)o2 * (long long)nb3 + (2 * ri - hx * nb) + nb * ((2 * rj - hy * nb) + nb * (2 * rk - hz * nb));
-    }
-    return -1;
-  };
-  auto fetch_slow = [&](int Lq, int i, int j, int k) -> TI {
-    const int gx = (Lq == L ? ax : ax / 2) + i, gy = (Lq == L ? ay : ay / 2) + j, gz = (Lq == L ? az : az / 2) + k;
-    const int o = owner(t, Lq, gx, gy, gz, b);
-    if (__ldg(t.lev + o) < Lq) return TI(__int_as_float(0x7fc00000));
-    return leaf_value(t, phi, o, Lq, gx, gy, gz, err);
-  };
-  auto fetch_raw = [&](int Lq, int i, int j, int k) -> TI {
-    const long long s = src_index(Lq, i, j, k);
-    return s >= 0 ? ld(phi + s) : fetch_slow(Lq, i, j, k);
-  };
-  auto fetch = [&](int Lq, int i, int j, int k) -> TP { return Cvt<TP>::f(fetch_raw(Lq, i, j, k)); };
-  extern __shared__ unsigned char smraw[];
-  TI *T = reinterpret_cast<TI *>(smraw);  // coarse tile, in the field's type
-  const int qlo = tq_lo<N>(Gi), nq = tq_hi<N>(nb, Gi) - qlo + 1;
-  const bool tile = use_tile && mask;
-  const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-  // boxes of the coarser leaves' regions in the padded cube, and the disjoint
-  // cells of the substitution band: per dimension [0, eb), [eb, nb-ef),
-  // [nb-ef, nb); a cell is in the band when a coarser direction covers it
-  __shared__ BoxList rbox, sbox;
-  if (threadIdx.x < 32) {
-    // per dimension the cuts 0 <= a <= b <= nb, a = min(ext_b, nb - ext_f),
-    // b = max(...): [0, a) lies in the band of a coarser leaf on the - side
-    // only, [b, nb) in that of the + side only, [a, b) in neither (or, when
-    // the two bands overlap -- small blocks -- in both)
-    const bool ov = W::ext_b > nb - W::ext_f;
-    const int c = lane;
-    bool in = false;
-    const int cc[3] = {c % 3, (c / 3) % 3, c / 9};
-    if (c < 27)
-      for (int m = 0; m < 27 && !in; ++m) {
-        if (!((mask >> m) & 1)) continue;
-        const int dd[3] = {m % 3 - 1, (m / 3) % 3 - 1, m / 9 - 1};
-        bool cov = true;
-        for (int d = 0; d < 3; ++d)
-          cov &= dd[d] == 0 || (dd[d] < 0 && (cc[d] == 0 || (ov && cc[d] == 1))) ||
-                 (dd[d] > 0 && (cc[d] == 2 || (ov && cc[d] == 1)));
-        in = cov;
-      }
-    const unsigned bc = __ballot_sync(0xffffffffu, in);
-    if (lane == 0) {
-      auto rect = [](int xa, int xb, int ya, int yb, int za, int zb) {
-        unsigned m = 0;
-        for (int z = za; z < zb; ++z)
-          for (int y = ya; y < yb; ++y)
-            for (int x = xa; x < xb; ++x) m |= 1u << (x + 3 * y + 9 * z);
-        return m;
-      };
-      // boxes of the coarser leaves' regions: the regions merged greedily (x
-      // run, then y, then z) as long as the separable refinement's partial
-      // sums of the box fit in the shared memory beside the coarse tile
-      {
-        const int cutr[4] = {-Gi, 0, nb, nb + Gi};
-        const long capU = use_tile == 2 ? ((long)dyn_bytes - tile_bytes) / (long)sizeof(TP) : 0x7fffffffL;
-        auto fits = [&](int xa, int xb, int ya, int yb, int za, int zb) {
-          const int lo3[3] = {cutr[xa], cutr[ya], cutr[za]}, hi3[3] = {cutr[xb], cutr[yb], cutr[zb]};
-          int fn[3], cn[3];
-          for (int d = 0; d < 3; ++d) {
-            fn[d] = hi3[d] - lo3[d];
-            cn[d] = ((hi3[d] - 1 + (N - 1)) >> 1) - ((lo3[d] - (N - 1)) >> 1) + 1;
-          }
-          int a = 0, c = 0;  // the refinement's order: thinnest side first, thickest last
-          for (int d = 1; d < 3; ++d) {
-            if (fn[d] < fn[a]) a = d;
-            if (fn[d] >= fn[c]) c = d;
-          }
-          if (a == c) c = (a + 2) % 3;
-          const int m = 3 - a - c;
-          return (long)fn[a] * cn[m] * cn[c] + (long)fn[a] * fn[m] * cn[c] <= capU;
-        };
-        unsigned left = (unsigned)mask & ~(1u << 13);
-        int n = 0;
-        while (left) {
-          const int c0 = __ffs(left) - 1;
-          const int x0 = c0 % 3, y0 = (c0 / 3) % 3, z0 = c0 / 9;
-          int x1 = x0 + 1, y1 = y0 + 1, z1 = z0 + 1;
-          while (x1 < 3 && ((left >> (x1 + 3 * y0 + 9 * z0)) & 1) && fits(x0, x1 + 1, y0, y1, z0, z1)) ++x1;
-          while (y1 < 3 && (left & rect(x0, x1, y1, y1 + 1, z0, z0 + 1)) == rect(x0, x1, y1, y1 + 1, z0, z0 + 1) &&
-                 fits(x0, x1, y0, y1 + 1, z0, z1))
-            ++y1;
-          while (z1 < 3 && (left & rect(x0, x1, y0, y1, z1, z1 + 1)) == rect(x0, x1, y0, y1, z1, z1 + 1) &&
-                 fits(x0, x1, y0, y1, z0, z1 + 1))
-            ++z1;
-          left &= ~rect(x0, x1, y0, y1, z0, z1);
-          rbox.lo[n][0] = cutr[x0], rbox.hi[n][0] = cutr[x1];
-          rbox.lo[n][1] = cutr[y0], rbox.hi[n][1] = cutr[y1];
-          rbox.lo[n][2] = cutr[z0], rbox.hi[n][2] = cutr[z1];
-          ++n;
-        }
-        rbox.n = n;
-      }
-      // band boxes: the (disjoint) band cells merged greedily, x run first,
-      // then y, then z
-      const int cut[4] = {0, ov ? nb - W::ext_f : W::ext_b, ov ? W::ext_b : nb - W::ext_f, nb};
-      unsigned left = bc;
-      int n = 0;
-      while (left) {
-        const int c0 = __ffs(left) - 1;
-        const int x0 = c0 % 3, y0 = (c0 / 3) % 3, z0 = c0 / 9;
-        int x1 = x0 + 1, y1 = y0 + 1, z1 = z0 + 1;
-        while (x1 < 3 && ((left >> (x1 + 3 * y0 + 9 * z0)) & 1)) ++x1;
-        while (y1 < 3 && (left & rect(x0, x1, y1, y1 + 1, z0, z0 + 1)) == rect(x0, x1, y1, y1 + 1, z0, z0 + 1)) ++y1;
-        while (z1 < 3 && (left & rect(x0, x1, y0, y1, z1, z1 + 1)) == rect(x0, x1, y0, y1, z1, z1 + 1)) ++z1;
-        left &= ~rect(x0, x1, y0, y1, z0, z1);
-        sbox.lo[n][0] = cut[x0], sbox.hi[n][0] = cut[x1];
-        sbox.lo[n][1] = cut[y0], sbox.hi[n][1] = cut[y1];
-        sbox.lo[n][2] = cut[z0], sbox.hi[n][2] = cut[z1];
-        ++n;
-      }
-      sbox.n = n;
-    }
-  }
-  if (tile && use_tile == 2) {
-    // coarse tile: only the level-(L-1) points the separable refinement
-    // reads -- per coarser region box, its fine extent widened by the widest
-    // odd K^s tap and halved (overlaps of boxes load the same values twice)
-    __syncthreads();  // rbox
-    constexpr int ko = N - 1;
-    for (int e = 0; e < rbox.n; ++e) {
-      int cl[3], cn[3];
-      bool ok = true;
-      for (int d = 0; d < 3; ++d) {
-        const int fl = rbox.lo[e][d], fh = rbox.hi[e][d];
-        cl[d] = (fl - ko) >> 1;
-        cn[d] = ((fh - 1 + ko) >> 1) - cl[d] + 1;
-        ok &= cl[d] >= qlo && cl[d] + cn[d] <= qlo + nq;
-      }
-      if (!ok) continue;  // flagged by the refinement below
-      // four points per thread and step, their loads issued together
-      const int cnt = cn[0] * cn[1] * cn[2], nthr = blockDim.x;
-      const DivM dc0 = divm(cn[0]), dc1 = divm(cn[1]);
-      auto qpt = [&](int idx, int &qx, int &qy, int &qz) {
-        const int r = divq(idx, dc0), z = divq(r, dc1);
-        qx = cl[0] + idx - r * cn[0], qy = cl[1] + r - z * cn[1], qz = cl[2] + z;
-      };
-      for (int i0 = threadIdx.x; i0 < cnt; i0 += 4 * nthr) {
-        long long si[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          si[u] = -2;
-          if (i0 + u * nthr < cnt) {
-            int qx, qy, qz;
-            qpt(i0 + u * nthr, qx, qy, qz);
-            si[u] = src_index(L - 1, qx, qy, qz);
-          }
-        }
-        TI v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = si[u] >= 0 ? ld(phi + si[u]) : TI(0);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (si[u] == -2) continue;
-          int qx, qy, qz;
-          qpt(i0 + u * nthr, qx, qy, qz);
-          T[(qx - qlo) + nq * ((qy - qlo) + nq * (qz - qlo))] = si[u] >= 0 ? v[u] : fetch_slow(L - 1, qx, qy, qz);
-        }
-      }
-    }
-  } else if (tile) {
-    // coarse tile, one row of nq values per warp
-    const DivM dnq = divm(nq);
-    for (int row = threadIdx.x >> 5; row < nq * nq; row += nwarp) {
-      const int z = divq(row, dnq), qy = qlo + row - z * nq, qz = qlo + z;
-      for (int x = lane; x < nq; x += 32) T[x + nq * row] = fetch_raw(L - 1, qlo + x, qy, qz);
+  __syncthreads();
+  // substitution jobs: one thread each (degree 1: classes x, y, z; 2: xy, xz,
+  // yz; 3: xyz), then one thread lays out their sums
+  {
+    const int nbx = plan.band.n, cls[7] = {1, 2, 4, 3, 5, 6, 7};
+    if (tid < 7 * nbx) {
+      const int k = tid < 3 * nbx ? tid % 3 : tid < 6 * nbx ? 3 + (tid - 3 * nbx) % 3 : 6;
+      const int e = tid < 3 * nbx ? tid / 3 : tid < 6 * nbx ? (tid - 3 * nbx) / 3 : tid - 6 * nbx;
+      sub_job_build(plan.job[tid], plan.band.lo[e], plan.band.hi[e], cls[k], W::hwG);
     }
   }
   TP *Pb = P + (size_t)b * np;
-  const TI *phib = phi + (size_t)b * nb3;
-  // every padded point outside the coarser leaves' regions (all points when
-  // the tile is off): interior, same-level copy, coincident value of a finer
-  // leaf; one padded row per warp.  prefilled: the plain gather has written
-  // every point outside the coarser leaves' regions already.
-  for (int row = threadIdx.x >> 5; row < ((prefilled && tile) ? 0 : Wd * Wd); row += nwarp) {
-    const int j = row % Wd - Gi, k = row / Wd - Gi;
-    const int ryz = 3 * (j < 0 ? 0 : j >= nb ? 2 : 1) + 9 * (k < 0 ? 0 : k >= nb ? 2 : 1);
-    TP *prow = Pb + (size_t)row * Wd + Gi;
-    for (int i = lane - Gi; i < nb + Gi; i += 32) {
-      const int r = (i < 0 ? 0 : i >= nb ? 2 : 1) + ryz;
-      if (prefilled && (r == 13 || rlev[r] >= L)) continue;
-      TP v;
-      if (r == 13) {
-        v = Cvt<TP>::f(ld(phib + i + nb * (j + nb * k)));
-      } else {
-        const int Lo = rlev[r];
-        if (Lo == L - 1) {
-          if (tile) continue;
-          v = refine_point<TI, TP, N, NT>(t, phi, L, ax + i, ay + j, az + k, err, b);
-        } else if (Lo >= L) {
-          v = fetch(L, i, j, k);  // copy, or the coincident value of a finer leaf
-        } else {
-          atomicOr(err, 8);
-          v = TP(0);
-        }
+  const long long lin1 = nb, lin2 = (long long)nb * nb;
+  // coarse values beyond a physical boundary (the leaf's own parent range or
+  // its lateral ghosts): the polynomial is applied to the sums along b and c;
+  // float pairs (FP64 blocks of an FP32 field) go point by point instead
+  const bool cbc = BND && bc_touches(t, L, ax, ay, az, -Gi - ko - 1, nb + Gi + ko + 1);
+  bool bad = false;  // a refined value is NaN: one flag per CTA, set below
+  if (BND && cbc && sizeof(TI) != sizeof(TP)) {
+    for (int e = 0; e < plan.nref; ++e) {
+      const RefBox &B = plan.ref[e];
+      const DivM dna = divm(B.na), dnb = divm(B.nb);
+      for (int idx = tid; idx < B.na * B.nb * B.nc; idx += bd) {
+        const int r = divq(idx, dna), kc = divq(r, dnb);
+        int p[3];
+        p[B.a] = B.la + idx - r * B.na, p[B.b] = B.lb + r - kc * B.nb, p[B.c] = B.lc + kc;
+        const TP v = refine_point<TI, TP, N, NT>(t, phi, L, ax + p[0], ay + p[1], az + p[2], err, b);
+        bad |= nan_bits(v);
+        Pb[(p[0] + Gi) + Wd * (p[1] + Gi) + W2 * (p[2] + Gi)] = v;
       }
-      prow[i] = v;
     }
-  }
-  __syncthreads();
-  if (!mask) return;
-  // zero-detail refinement of the coarse regions from the tile: separably per
-  // region box when the partial sums fit next to the tile (use_tile == 2),
-  // else one parity class at a time (every warp runs one tap sequence)
-  if (tile && use_tile == 2) {
-    // float pairs for an FP32 field in an FP64 block (the tile holds exact
-    // FP32 values and the K^s weights are dyadic, exact in FP32)
-    constexpr bool FP = sizeof(TI) == 4 && sizeof(TP) == 8 && f32_exact_taps<N, NT, FK_K>();
-    TP *U = reinterpret_cast<TP *>(smraw + tile_bytes);
-    constexpr int ko = N - 1;  // widest odd K^s tap
-    const int ts[3] = {1, nq, nq * nq}, ps[3] = {1, Wd, Wd * Wd};
-    for (int e = 0; e < rbox.n; ++e) {
-      int fl[3], fn[3], cl[3], cn[3];
-      bool ok = true;
-      for (int d = 0; d < 3; ++d) {
-        fl[d] = rbox.lo[e][d], fn[d] = rbox.hi[e][d] - fl[d];
-        cl[d] = (fl[d] - ko) >> 1;
-        cn[d] = ((fl[d] + fn[d] - 1 + ko) >> 1) - cl[d] + 1;
-        ok &= cl[d] >= qlo && cl[d] + cn[d] <= qlo + nq;
-      }
-      if (!ok) {  // outside the tile: not a valid shell for this block size
-        if (threadIdx.x == 0) atomicOr(err, 2);
-        continue;
-      }
-      // expansion order: thinnest dimension first, thickest last
-      int a = 0, c = 0;
-      for (int d = 1; d < 3; ++d) {
-        if (fn[d] < fn[a]) a = d;
-        if (fn[d] >= fn[c]) c = d;
-      }
-      if (a == c) c = (a + 2) % 3;
-      const int bd = 3 - a - c;
-      // per-box scalars (the loops below index nothing dynamically)
-      const int nfa = fn[a], nfb = fn[bd], nfc = fn[c], ncb = cn[bd], ncc = cn[c];
-      const int la = fl[a], lb = fl[bd], lc = fl[c], cb = cl[bd], cc = cl[c];
-      const int tsa = ts[a], tsb = ts[bd], tsc = ts[c], psa = ps[a], psb = ps[bd], psc = ps[c];
-      TP *U1 = U, *U2 = U + (size_t)nfa * ncb * ncc;
-      if constexpr (FP) {
-        // FP32 field, FP64 block: the three passes in float pairs (same
-        // layout, 8 bytes per partial sum), one conversion per written point
-        F2 *V1 = reinterpret_cast<F2 *>(U1), *V2 = reinterpret_cast<F2 *>(U2);
-        {
-          const int no = par_count(la, la + nfa, 1), ne = nfa - no, m = ncb * ncc;
-          const DivM dno = divm(no > 0 ? no : 1), dne = divm(ne > 0 ? ne : 1), dcb = divm(ncb);
-          for (int idx = threadIdx.x; idx < nfa * m; idx += blockDim.x) {
-            const bool od = idx < no * m;
-            const int q = od ? idx : idx - no * m, nh = od ? no : ne;
-            const int r = divq(q, od ? dno : dne), kc = divq(r, dcb);
-            const int f = par_first(la, od) + 2 * (q - r * nh), jb = r - kc * ncb;
-            const TI *tp = T + (cb + jb - qlo) * tsb + (cc + kc - qlo) * tsc;
-            F2 v;
-            if (od) {
-              v = f2_of(0.f);
-#pragma unroll
-              for (int t = -ko; t <= ko; t += 2)
-                v = f2_acc(v, float(Wav<N, NT>::K(t)), f2_of(tp[(((f + t) >> 1) - qlo) * tsa]));
-              v = f2_norm(v);
-            } else {
-              v = f2_of(tp[((f >> 1) - qlo) * tsa]);
+  } else {
+    for (int e0 = 0; e0 < plan.nref;) {
+      const int e1 = plan.refnext[e0];
+      U *UB = reinterpret_cast<U *>(smraw);
+      // pass 1: one thread per coarse column along a.  The column's values come
+      // from two runs (the coarser region, and the block's side of the face);
+      // its fine points go to U1.
+      int rot = 0;
+      for (int e = e0; e < e1; ++e) {
+        const RefBox &B = plan.ref[e];
+        const int a = B.a, ncol = B.mb * B.mc, na = B.na, par = B.la & 1;
+        const int ca = (B.la - ko) >> 1, cna = ((B.la + na - 1 + ko) >> 1) - ca + 1;
+        const int sta = a == 0 ? 1 : a == 1 ? nb : nb * nb;
+        const int pitch = B.mbp;
+        int idx = tid - rot;
+        if (idx < 0) idx += bd;
+        rot = (rot + ncol) & (bd - 1);
+        for (; idx < ncol; idx += bd) {
+          const int kc = divq(idx, DivM{B.dmb, B.mb}), jb = idx - kc * B.mb;
+          int q[3];
+          q[B.b] = B.cb + jb, q[B.c] = B.cc + kc, q[a] = ca;
+          // regions along b and c; the run along a changes region at the face
+          int rr = 0, ra = a == 0 ? 1 : a == 1 ? 3 : 9;
+          bool ok = 2 * ca >= -nb && 2 * (ca + cna - 1) < 2 * nb;
+          for (int d = 0; d < 3; ++d) {
+            if (d == a) continue;
+            const int f = 2 * q[d];
+            ok &= f >= -nb && f < 2 * nb;
+            rr += (f < 0 ? 0 : f >= nb ? 2 : 1) * (d == 0 ? 1 : d == 1 ? 3 : 9);
+          }
+          const int cut = B.la < 0 ? 0 : hb;  // first coarse point of the upper run
+          const int r0 = rr + (B.la < 0 ? 0 : 1) * ra, r1 = r0 + ra;
+          if (ok) ok = T.rmul[r0] && T.rmul[r1];
+          U *d = UB + B.off + jb + pitch * na * kc;
+          if (!ok) {  // a finer leaf or a region beyond the neighbours: point by point
+            for (int ia = 0; ia < na; ++ia) {
+              U s = RS::zero();
+              const int f = B.la + ia;
+              for (int o = (f & 1) ? -ko : 0; o <= ((f & 1) ? ko : 0); o += 2) {
+                q[a] = (f + o) >> 1;
+                s = RS::acc(s, (f & 1) ? W::K(o) : 1.0,
+                            RS::from(prep_fetch<TI>(t, T, phi, b, L, L - 1, q[0], q[1], q[2], err)));
+              }
+              d[pitch * ia] = RS::norm(s);
             }
-            V1[(f - la) + nfa * (jb + ncb * kc)] = v;
+            continue;
           }
-        }
-        __syncthreads();
-        {
-          const int no = par_count(lb, lb + nfb, 1), ne = nfb - no;
-          const DivM dfa = divm(nfa), dno = divm(no > 0 ? no : 1), dne = divm(ne > 0 ? ne : 1);
-          for (int idx = threadIdx.x; idx < nfa * nfb * ncc; idx += blockDim.x) {
-            const bool od = idx < nfa * no * ncc;
-            const int q = od ? idx : idx - nfa * no * ncc, nh = od ? no : ne;
-            const int r = divq(q, dfa), kc = divq(r, od ? dno : dne);
-            const int ia = q - r * nfa, f = par_first(lb, od) + 2 * (r - kc * nh);
-            const F2 *up = V1 + ia + nfa * ncb * kc;
-            F2 v;
-            if (od) {
-              v = f2_of(0.f);
+          TI v[MR_MAX_SHELL];
+          {
+            const long long lin = q[0] + lin1 * q[1] + lin2 * q[2];
+            const TI *p0 = phi + (T.rbase[r0] + T.rmul[r0] * lin), *p1 = phi + (T.rbase[r1] + T.rmul[r1] * lin);
+            const int s0 = T.rmul[r0] * sta, s1 = T.rmul[r1] * sta, n0 = cut - ca;
 #pragma unroll
-              for (int t = -ko; t <= ko; t += 2) v = f2_acc(v, float(Wav<N, NT>::K(t)), up[nfa * (((f + t) >> 1) - cb)]);
-              v = f2_norm(v);
-            } else {
-              v = up[nfa * ((f >> 1) - cb)];
+            for (int u = 0; u < MR_MAX_SHELL; ++u) v[u] = u < cna ? ld(u < n0 ? p0 + u * s0 : p1 + u * s1) : TI(0);
+          }
+          auto column = [&](auto parity) {
+            constexpr int PAR = decltype(parity)::x, base = (PAR - ko) >> 1;
+#pragma unroll
+            for (int ia = 0; ia < MR_MAX_SHELL; ++ia) {
+              if (ia >= na) break;
+              U s;
+              if ((PAR + ia) & 1) {
+                s = RS::zero();
+#pragma unroll
+                for (int o = -ko; o <= ko; o += 2) {
+                  const int x = ((PAR + ia + o) >> 1) - base;
+                  if (x < MR_MAX_SHELL) s = RS::acc(s, W::K(o), RS::from(v[x]));
+                }
+                s = RS::norm(s);
+              } else {
+                const int x = ((PAR + ia) >> 1) - base;
+                s = RS::from(x < MR_MAX_SHELL ? v[x] : TI(0));
+              }
+              d[pitch * ia] = s;
             }
-            V2[ia + nfa * ((f - lb) + nfb * kc)] = v;
-          }
-        }
-        __syncthreads();
-        {
-          const int no = par_count(lc, lc + nfc, 1), ne = nfc - no, m = nfa * nfb;
-          const DivM dfa = divm(nfa), dfb = divm(nfb);
-          for (int idx = threadIdx.x; idx < m * nfc; idx += blockDim.x) {
-            const bool od = idx < m * no;
-            const int q = od ? idx : idx - m * no;
-            const int r = divq(q, dfa), z = divq(r, dfb);
-            const int ia = q - r * nfa, ib = r - z * nfb, f = par_first(lc, od) + 2 * z;
-            const F2 *up = V2 + ia + nfa * ib;
-            F2 v;
-            if (od) {
-              v = f2_of(0.f);
-#pragma unroll
-              for (int t = -ko; t <= ko; t += 2)
-                v = f2_acc(v, float(Wav<N, NT>::K(t)), up[m * (((f + t) >> 1) - cc)]);
-            } else {
-              v = up[m * ((f >> 1) - cc)];
-            }
-            const TP d = f2_dbl(v);
-            if (nan_bits(d)) atomicOr(err, 2);
-            Pb[(la + ia + Gi) * psa + (lb + ib + Gi) * psb + (f + Gi) * psc] = d;
-          }
-        }
-        __syncthreads();
-        continue;
-      }
-      // pass 1: along a, coarse tile -> U1[ia][jb][kc] (odd fine points first)
-      {
-        const int no = par_count(la, la + nfa, 1), ne = nfa - no, m = ncb * ncc;
-        const DivM dno = divm(no > 0 ? no : 1), dne = divm(ne > 0 ? ne : 1), dcb = divm(ncb);
-        for (int idx = threadIdx.x; idx < nfa * m; idx += blockDim.x) {
-          const bool od = idx < no * m;
-          const int q = od ? idx : idx - no * m, nh = od ? no : ne;
-          const int r = divq(q, od ? dno : dne), kc = divq(r, dcb);
-          const int f = par_first(la, od) + 2 * (q - r * nh), jb = r - kc * ncb;
-          const TI *tp = T + (cb + jb - qlo) * tsb + (cc + kc - qlo) * tsc;
-          TP v;
-          if (od) {
-            v = TP(0);
-#pragma unroll
-            for (int t = -ko; t <= ko; t += 2)
-              v = racc(v, TP(Wav<N, NT>::K(t)), Cvt<TP>::f(tp[(((f + t) >> 1) - qlo) * tsa]));
-          } else {
-            v = Cvt<TP>::f(tp[((f >> 1) - qlo) * tsa]);
-          }
-          U1[(f - la) + nfa * (jb + ncb * kc)] = v;
+          };
+          if (par) column(Cls<1, 0, 0>());
+          else column(Cls<0, 0, 0>());
         }
       }
       __syncthreads();
-      // pass 2: along b, U1 -> U2[ia][ib][kc]
-      {
-        const int no = par_count(lb, lb + nfb, 1), ne = nfb - no;
-        const DivM dfa = divm(nfa), dno = divm(no > 0 ? no : 1), dne = divm(ne > 0 ? ne : 1);
-        for (int idx = threadIdx.x; idx < nfa * nfb * ncc; idx += blockDim.x) {
-          const bool od = idx < nfa * no * ncc;
-          const int q = od ? idx : idx - nfa * no * ncc, nh = od ? no : ne;
-          const int r = divq(q, dfa), kc = divq(r, od ? dno : dne);
-          const int ia = q - r * nfa, f = par_first(lb, od) + 2 * (r - kc * nh);
-          const TP *up = U1 + ia + nfa * ncb * kc;
-          TP v;
-          if (od) {
-            v = TP(0);
-#pragma unroll
-            for (int t = -ko; t <= ko; t += 2) v = racc(v, TP(Wav<N, NT>::K(t)), up[nfa * (((f + t) >> 1) - cb)]);
-          } else {
-            v = up[nfa * ((f >> 1) - cb)];
-          }
-          U2[ia + nfa * ((f - lb) + nfb * kc)] = v;
+      if constexpr (BND && sizeof(TI) == sizeof(TP))
+        if (cbc)
+          for (int e = e0; e < e1; ++e)
+            bc_sums<N>(t, L - 1, plan.ref[e], ax / 2, ay / 2, az / 2, UB + plan.ref[e].off);
+      // pass 2: along b, U1 -> U2; segments of 8 coarse points, a register
+      // window of N coarse values, two fine points per step
+      rot = 0;
+      for (int e = e0; e < e1; ++e) {
+        const RefBox &B = plan.ref[e];
+        const int na = B.na, lines = na * B.mc, nseg = (B.nb + 15) >> 4, n = lines * nseg;
+        const DivM dl = divm(lines), dna = divm(na);
+        const int sb = B.a == 0 ? na : 1, sa = B.a == 0 ? 1 : B.nbp;
+        const U *U1 = UB + B.off;
+        U *U2 = UB + B.off + na * B.mbp * B.mc;
+        int idx = tid - rot;
+        if (idx < 0) idx += bd;
+        rot = (rot + n) & (bd - 1);
+        for (; idx < n; idx += bd) {
+          const int sg = divq(idx, dl), ln = idx - sg * lines, kc = divq(ln, dna), ia = ln - kc * na;
+          const int f0 = B.lb + 16 * sg, n1 = min(16, B.nb - 16 * sg);
+          const U *src = U1 + B.mbp * ln - B.cb;  // (line kc, ia: U1 pitch mbp)
+          U *dst = U2 + B.S * kc + sa * ia + sb * (16 * sg);
+          refine_run<N, NT, RS>(src, 1, f0, n1, [&](int m, U v) { dst[sb * m] = RS::norm(v); });
         }
       }
       __syncthreads();
       // pass 3: along c, U2 -> padded block
-      {
-        const int no = par_count(lc, lc + nfc, 1), ne = nfc - no, m = nfa * nfb;
-        const DivM dfa = divm(nfa), dfb = divm(nfb);
-        for (int idx = threadIdx.x; idx < m * nfc; idx += blockDim.x) {
-          const bool od = idx < m * no;
-          const int q = od ? idx : idx - m * no;
-          const int r = divq(q, dfa), z = divq(r, dfb);
-          const int ia = q - r * nfa, ib = r - z * nfb, f = par_first(lc, od) + 2 * z;
-          const TP *up = U2 + ia + nfa * ib;
-          TP v;
-          if (od) {
-            v = TP(0);
-#pragma unroll
-            for (int t = -ko; t <= ko; t += 2) v = racc(v, TP(Wav<N, NT>::K(t)), up[m * (((f + t) >> 1) - cc)]);
-          } else {
-            v = up[m * ((f >> 1) - cc)];
-          }
-          if (nan_bits(v)) atomicOr(err, 2);
-          Pb[(la + ia + Gi) * psa + (lb + ib + Gi) * psb + (f + Gi) * psc] = v;
+      rot = 0;
+      for (int e = e0; e < e1; ++e) {
+        const RefBox &B = plan.ref[e];
+        const int na = B.na, lines = na * B.nb, nseg = (B.nc + 15) >> 4, n = lines * nseg;
+        const int n1d = B.a == 0 ? na : B.nb;  // dimension that varies fastest over threads
+        const DivM dl = divm(lines), df = divm(n1d);
+        const int sb = B.a == 0 ? na : 1, sa = B.a == 0 ? 1 : B.nbp;
+        const int psa = B.a == 0 ? 1 : B.a == 1 ? Wd : W2, psb = B.b == 0 ? 1 : B.b == 1 ? Wd : W2,
+                  psc = B.c == 0 ? 1 : B.c == 1 ? Wd : W2;
+        const U *U2 = UB + B.off + na * B.mbp * B.mc;
+        int idx = tid - rot;
+        if (idx < 0) idx += bd;
+        rot = (rot + n) & (bd - 1);
+        for (; idx < n; idx += bd) {
+          const int sg = divq(idx, dl), ln = idx - sg * lines, hi = divq(ln, df), lo = ln - hi * n1d;
+          const int ia = B.a == 0 ? lo : hi, ib = B.a == 0 ? hi : lo;
+          const int f0 = B.lc + 16 * sg, n1 = min(16, B.nc - 16 * sg);
+          TP *dst = Pb + (B.la + ia + Gi) * psa + (B.lb + ib + Gi) * psb + (f0 + Gi) * psc;
+          refine_run<N, NT, RS>(U2 + sa * ia + sb * ib - B.S * B.cc, B.S, f0, n1, [&](int m, U v) {
+            const TP d = RS::value(v);
+            bad |= nan_bits(d);
+            dst[psc * m] = d;
+          });
         }
       }
       __syncthreads();
+      e0 = e1;
     }
-  } else if (tile) {
-    auto refine_cls = [&](auto cls) {
-      constexpr int OX = decltype(cls)::x, OY = decltype(cls)::y, OZ = decltype(cls)::z;
-      for_class_points<OX, OY, OZ>(rbox, [&](int i, int j, int k) {
-        const TP v = refine_sum<N, NT, OX, OY, OZ, TP>([&](int ox, int oy, int oz) -> TP {
-          const int qx = (i + ox) / 2 - qlo, qy = (j + oy) / 2 - qlo, qz = (k + oz) / 2 - qlo;
-          return Cvt<TP>::f(T[qx + nq * (qy + nq * qz)]);
-        });
-        if (nan_bits(v)) atomicOr(err, 2);
-        Pb[(i + Gi) + Wd * ((j + Gi) + Wd * (k + Gi))] = v;
-      });
-    };
-    refine_cls(Cls<0, 0, 0>());
-    refine_cls(Cls<1, 0, 0>());
-    refine_cls(Cls<0, 1, 0>());
-    refine_cls(Cls<1, 1, 0>());
-    refine_cls(Cls<0, 0, 1>());
-    refine_cls(Cls<1, 0, 1>());
-    refine_cls(Cls<0, 1, 1>());
-    refine_cls(Cls<1, 1, 1>());
-    __syncthreads();
   }
+  // layout of the substitution sums: batches within a degree
+  __syncthreads();
+  if (tid == 0) {
+    const int nbx = plan.band.n;
+    int j = 0;
+    for (int deg = 1; deg <= 3; ++deg) {
+      const int end = j + (deg < 3 ? 3 : 1) * nbx;
+      plan.job0[deg - 1] = j;
+      int used = 0, open = j;
+      for (; j < end; ++j) {
+        SubJob &J = plan.job[j];
+        const int sz = deg == 1 ? 0 : J.n[0] + (deg == 3 ? J.n[1] : 0);
+        if (j > open && used + sz > capP) {
+          plan.job[open].next = j;
+          open = j, used = 0;
+        }
+        J.off = used, used += sz;
+      }
+      if (open < end) plan.job[open].next = end;
+    }
+    plan.job0[3] = j;
+  }
+  if (__syncthreads_or(bad) && tid == 0) atomicOr(err, 2);
+  if (BND && bc_touches(t, L, ax, ay, az, -Gi, nb + Gi))
+    bc_box<N>(t, L, ax, ay, az, Pb + Gi * (1 + Wd + W2), Wd, W2, -Gi, -Gi, -Gi, Wd, Wd, Wd);
   // substitution, degree by degree (a point of degree d reads lower degrees
   // only, so the classes of one degree are independent)
-  auto subst_cls = [&](auto cls) {
-    constexpr int OX = decltype(cls)::x, OY = decltype(cls)::y, OZ = decltype(cls)::z;
-    for_class_points<OX, OY, OZ>(sbox, [&](int i, int j, int k) {
-      TP *c = Pb + (i + Gi) + Wd * ((j + Gi) + Wd * (k + Gi));
-      *c = subst_sum<N, NT, OX, OY, OZ, TP>([&](int tx, int ty, int tz) -> TP {
-        return c[tx + Wd * (ty + Wd * tz)];
-      });
-    });
-  };
-  subst_cls(Cls<1, 0, 0>());
-  subst_cls(Cls<0, 1, 0>());
-  subst_cls(Cls<0, 0, 1>());
-  __syncthreads();
-  // degrees 2 and 3 separably, partial sums in the (now free) dynamic shared
-  // memory; each batch ends with a barrier
-  subst_sep<N, NT, TP>(Pb, Wd, Gi, sbox, 2, reinterpret_cast<TP *>(smraw), (long)dyn_bytes / (long)sizeof(TP));
-  subst_sep<N, NT, TP>(Pb, Wd, Gi, sbox, 3, reinterpret_cast<TP *>(smraw), (long)dyn_bytes / (long)sizeof(TP));
-  __syncthreads();
-  if (only_coarse == 2) return;  // substitution only: no fine-to-coarse push
-  // distinct coarser neighbours, and the boxes of this leaf's coarse points
-  // that lie in their ghost shells: per coarser direction, the Gpush coarse
-  // layers next to it (whole extent along the other dimensions); boxes inside
-  // another box dropped
-  const int gp = min(Gpush, hb);
-  __shared__ int pbox[27][6];  // coarse-local [x0, x1) [y0, y1) [z0, z1)
-  __shared__ int npb;
-  if (threadIdx.x == 0) {
-    int n = 0;
-    for (int m = 0; m < 27; ++m) {
-      if (!((mask >> m) & 1)) continue;
-      const int o = rslot[m];
-      bool seen = false;
-      for (int q = 0; q < ncs; ++q) seen |= cslots[q] == o;
-      if (!seen) cslots[ncs++] = o;
-      const int dd[3] = {m % 3 - 1, (m / 3) % 3 - 1, m / 9 - 1};
-      int bx[6];
-      for (int d = 0; d < 3; ++d) {
-        bx[2 * d] = dd[d] > 0 ? hb - gp : 0;
-        bx[2 * d + 1] = dd[d] < 0 ? gp : hb;
-      }
-      auto inside = [](const int *a, const int *c) {  // a within c
-        return a[0] >= c[0] && a[1] <= c[1] && a[2] >= c[2] && a[3] <= c[3] && a[4] >= c[4] && a[5] <= c[5];
-      };
-      bool covered = false;
-      for (int q = 0; q < n && !covered; ++q) covered = inside(bx, pbox[q]);
-      if (covered) continue;
-      int w = 0;
-      for (int q = 0; q < n; ++q)
-        if (!inside(pbox[q], bx)) {
-          for (int v = 0; v < 6; ++v) pbox[w][v] = pbox[q][v];
-          ++w;
+  for (int deg = 1; deg <= 3; ++deg)
+    subst_jobs<N, NT, TP>(Pb, Wd, Gi, plan.job, plan.job0[deg - 1], plan.job0[deg], reinterpret_cast<TP *>(smraw), capP);
+  // (N.0: H^a is the identity and even points are never substituted, so the
+  // coincident values the gather took are already the coarsened ones)
+  if (only_coarse == 2 || NT == 0) return;
+  // Part 2: H^a coarsening of the padded block at the coarse points of the push
+  // boxes, thinnest axis a first (then b, c), up to PUSH_LAYERS layers of a at a
+  // time: one thread loads a fine column along a and sums every layer from it;
+  // along b and c a thread sums four points from one window.  Each value goes to
+  // the side buffer of every coarser neighbour in whose shell the point lies.
+  if constexpr (NT != 0) {
+    constexpr int hH = W::hwH;
+    const int gp = min(Gpush, hb);
+    for (int e = 0; e < plan.push.n; ++e) {
+      const int *lo = plan.push.lo[e];
+      const int n3[3] = {plan.push.hi[e][0] - lo[0], plan.push.hi[e][1] - lo[1], plan.push.hi[e][2] - lo[2]};
+      const int a = n3[0] <= n3[1] && n3[0] <= n3[2] ? 0 : n3[1] <= n3[2] ? 1 : 2, bx = a == 0 ? 1 : 0,
+                c = 3 - a - bx;
+      const int na = n3[a], nbb = n3[bx], nc = n3[c], fb = 2 * nbb - 1 + 2 * hH, fc = 2 * nc - 1 + 2 * hH;
+      const int sA = a == 0 ? 1 : a == 1 ? Wd : W2, sB = bx == 0 ? 1 : Wd, sC = c == 1 ? Wd : W2;
+      const int layers = max(1, min(min(na, PUSH_LAYERS), capP / (fc * (fb + nbb))));
+      const int rb = (nbb + 3) >> 2, rc = (nc + 3) >> 2;  // runs of four points along b, c
+      const DivM dfb = divm(fb), dfc = divm(fc), drb = divm(rb), dnb = divm(nbb), drc = divm(rc);
+      const int q0 = 2 * lo[bx] - hH + Gi, q1 = 2 * lo[c] - hH + Gi;
+      for (int l0 = 0; l0 < na; l0 += layers) {
+        const int nl = min(layers, na - l0);
+        TP *A = reinterpret_cast<TP *>(smraw), *Bf = A + nl * fc * fb;  // [l][fc][fb], [l][fc][nbb]
+        const TP *src0 = Pb + (2 * (lo[a] + l0) + Gi) * sA + q0 * sB + q1 * sC;
+        for (int idx = tid; idx < fc * fb; idx += bd) {
+          const int ic = divq(idx, dfb), ib = idx - ic * fb;
+          coarsen_run<N, NT, PUSH_LAYERS>(src0 + ib * sB + ic * sC, sA, nl,
+                                          [&](int l, TP v) { A[l * fc * fb + idx] = v; });
         }
-      for (int v = 0; v < 6; ++v) pbox[w][v] = bx[v];
-      n = w + 1;
-    }
-    // two boxes whose bounding box is no larger than their volumes together
-    // become that box (wide shells: the face boxes nearly coincide)
-    auto vol = [](const int *a) { return (a[1] - a[0]) * (a[3] - a[2]) * (a[5] - a[4]); };
-    for (bool merged = true; merged;) {
-      merged = false;
-      for (int q = 0; q < n && !merged; ++q)
-        for (int u = q + 1; u < n && !merged; ++u) {
-          int bb[6];
-          for (int d = 0; d < 3; ++d) {
-            bb[2 * d] = min(pbox[q][2 * d], pbox[u][2 * d]);
-            bb[2 * d + 1] = max(pbox[q][2 * d + 1], pbox[u][2 * d + 1]);
-          }
-          if (vol(bb) <= vol(pbox[q]) + vol(pbox[u])) {
-            for (int v = 0; v < 6; ++v) pbox[q][v] = bb[v], pbox[u][v] = pbox[n - 1][v];
-            --n;
-            merged = true;
-          }
+        __syncthreads();
+        for (int idx = tid; idx < nl * fc * rb; idx += bd) {
+          const int r = divq(idx, drb), ib = 4 * (idx - r * rb);
+          TP *d = Bf + r * nbb + ib;
+          coarsen_run<N, NT, 4>(A + r * fb + 2 * ib + hH, 1, min(4, nbb - ib), [&](int m, TP v) { d[m] = v; });
         }
-    }
-    npb = n;
-  }
-  __syncthreads();
-  // Part 2: H^a coarsening of the padded block at the coarse points of those
-  // boxes, evaluated separably (x, then y, then z; zc coarse z-planes per
-  // chunk so the partial sums fit in shared memory), then written to each
-  // periodic image of the point that lies in the ghost shell (Gpush) of a
-  // coarser neighbour.
-  constexpr int hH = W::hwH;
-  const int Wg = nb + 2 * Gi;
-  TP *A = reinterpret_cast<TP *>(smraw);  // x-pass [nk][nfj][nx]
-  for (int e = 0; e < npb; ++e) {
-    const int x0 = pbox[e][0], nx = pbox[e][1] - x0, y0 = pbox[e][2], ny = pbox[e][3] - y0;
-    const int z0 = pbox[e][4], z1 = pbox[e][5];
-    const int nfj = 2 * ny - 1 + 2 * hH, jlo = 2 * y0 - hH;  // fine rows the y pass reads
-    const DivM dnx = divm(nx), dny = divm(ny), dnf = divm(nfj);
-    for (int pz0 = z0; pz0 < z1; pz0 += zc) {
-      const int zn = min(zc, z1 - pz0), k0 = 2 * pz0 - hH, nk = 2 * zn - 1 + 2 * hH;
-      TP *B = A + nk * nfj * nx;  // y-pass [nk][ny][nx]
-      for (int idx = threadIdx.x; idx < nx * nfj * nk; idx += blockDim.x) {
-        const int r = divq(idx, dnx), kr = divq(r, dnf);
-        const int px = x0 + idx - r * nx, j = jlo + r - kr * nfj, k = kr + k0;
-        A[idx] = tap_sum<N, NT, FK_H>(Pb + (2 * px + Gi) + Wd * ((j + Gi) + Wd * (k + Gi)), 1);
-      }
-      __syncthreads();
-      for (int idx = threadIdx.x; idx < nx * ny * nk; idx += blockDim.x) {
-        const int r = divq(idx, dnx), kk = divq(r, dny), px = idx - r * nx, py = r - kk * ny;
-        B[idx] = tap_sum<N, NT, FK_H>(A + (kk * nfj + 2 * py + hH) * nx + px, nx);
-      }
-      __syncthreads();
-      for (int idx = threadIdx.x; idx < nx * ny * zn; idx += blockDim.x) {
-        const int r = divq(idx, dnx), pz = divq(r, dny), px = idx - r * nx, py = r - pz * ny;
-        const TP sv = tap_sum<N, NT, FK_H>(B + ((2 * pz + hH) * ny + py) * nx + px, nx * ny);
-        // coarse (level L-1) point, global index
-        const int G[3] = {ax / 2 + x0 + px, ay / 2 + y0 + py, az / 2 + pz0 + pz};
-        for (int ci = 0; ci < ncs; ++ci) {
-          const int c = cslots[ci];
-          // c-local offsets of every periodic image of G in c's shell (tiny
-          // periodic domains: c can see this leaf on both sides)
-          int cand[3][3], ncand[3];
-          bool any = true;
-          for (int d = 0; d < 3; ++d) {
-            const int Pn = period(t, L - 1, d);
-            const int off = pwrap(G[d] - __ldg(t.anc + 3 * c + d) * nb, Pn);
-            ncand[d] = 0;
-            for (int sh = -1; sh <= 1; ++sh) {
-              const int o = off + sh * Pn;
-              if (o >= -Gpush && o < nb + Gpush) cand[d][ncand[d]++] = o;
-            }
-            any &= ncand[d] > 0;
-          }
-          if (!any) continue;
-          for (int iz = 0; iz < ncand[2]; ++iz)
-            for (int iy = 0; iy < ncand[1]; ++iy)
-              for (int ix = 0; ix < ncand[0]; ++ix) {
-                const int lc[3] = {cand[0][ix], cand[1][iy], cand[2][iz]};
-                const bool inside = lc[0] >= 0 && lc[0] < nb && lc[1] >= 0 && lc[1] < nb && lc[2] >= 0 && lc[2] < nb;
-                if (inside) continue;
-                Q[(size_t)c * np + (lc[0] + Gi) + Wg * ((lc[1] + Gi) + (size_t)Wg * (lc[2] + Gi))] = sv;
+        __syncthreads();
+        for (int idx = tid; idx < nl * rc * nbb; idx += bd) {
+          const int r = divq(idx, dnb), l = divq(r, drc), ib = idx - r * nbb, ic = 4 * (r - l * rc);
+          coarsen_run<N, NT, 4>(Bf + (l * fc + 2 * ic + hH) * nbb + ib, nbb, min(4, nc - ic), [&](int m, TP sv) {
+            int p[3], inb = 0;
+            p[a] = lo[a] + l0 + l, p[bx] = lo[bx] + ib, p[c] = lo[c] + ic + m;
+            for (int d = 0; d < 3; ++d) inb |= (T.s[d] > 0 ? p[d] >= hb - gp : p[d] < gp) << d;
+            for (int f = 1; f < 8; ++f) {
+              if (!((ce >> f) & 1) || (f & ~inb)) continue;
+              // position in the neighbour: beyond its face along the axes of f,
+              // in the leaf's half along the others
+              int r2 = 13, x[3];
+              for (int d = 0; d < 3; ++d) {
+                const bool on = (f >> d) & 1;
+                if (on) r2 += T.s[d] * (d == 0 ? 1 : d == 1 ? 3 : 9);
+                x[d] = (on ? (T.s[d] > 0 ? p[d] - hb : nb + p[d]) : p[d] + T.odd[d] * hb) + Gi;
               }
+              Q[(size_t)T.rslot[r2] * np + x[0] + Wd * (x[1] + (size_t)Wd * x[2])] = sv;
+            }
+          });
         }
+        __syncthreads();
       }
-      __syncthreads();
     }
   }
 }
@@ -877,9 +955,11 @@ __global__ void __launch_bounds__(512, sizeof(TP) == 4 ? 2 : 1) k_prep(Tree t, c
 // coarser neighbour is flagged in pneed for the full pre-pass (refinement of
 // the coarse regions, substitution, Part-2 push).
 // Finer regions are resolved through the owners of their eight one-level-
-// finer sub-blocks (one lookup per sub-block, not per point).  Every field
-// read is bounds-checked: an out-of-range index sets error bit 16 and yields
-// NaN instead of a load.
+// finer sub-blocks (one lookup per sub-block, not per point).
+// One thread per (x, y) column of the padded block: along z the column crosses
+// at most three regions (a finer one in two halves), each of which is a run
+// of values a fixed stride apart in one leaf, so a point costs a load, a
+// store and two additions.
 // ---------------------------------------------------------------------------
 template <typename TI, typename TP>
 __global__ void __launch_bounds__(512) k_fill_plain(Tree t, const TI *__restrict__ phi, TP *__restrict__ P,
@@ -893,7 +973,6 @@ __global__ void __launch_bounds__(512) k_fill_plain(Tree t, const TI *__restrict
   }
   const int nb = t.nb, Wd = nb + 2 * Gi, hb = nb / 2;
   const size_t np = (size_t)Wd * Wd * Wd, nb3 = (size_t)nb * nb * nb;
-  const long long lim = (long long)t.nleaf * (long long)nb3;
   const int L = __ldg(t.lev + b);
   __shared__ int rslot[27], rlev[27], rsub[27][8];
   __shared__ int coarse;
@@ -904,7 +983,7 @@ __global__ void __launch_bounds__(512) k_fill_plain(Tree t, const TI *__restrict
     const int dd[3] = {r % 3 - 1, (r / 3) % 3 - 1, r / 9 - 1};
     int g[3];
     for (int d = 0; d < 3; ++d) g[d] = __ldg(t.anc + 3 * b + d) * nb + (dd[d] < 0 ? -1 : dd[d] > 0 ? nb : 0);
-    const int o = owner(t, L, g[0], g[1], g[2], b);
+    const int o = beyond3(t, L, g) ? b : owner(t, L, g[0], g[1], g[2], b);
     const int Lo = __ldg(t.lev + o);
     rslot[r] = o, rlev[r] = Lo;
     if (r != 13 && Lo < L) atomicOr(&coarse, 1);
@@ -931,110 +1010,66 @@ __global__ void __launch_bounds__(512) k_fill_plain(Tree t, const TI *__restrict
   }
   __syncthreads();
   const int ax = __ldg(t.anc + 3 * b) * nb, ay = __ldg(t.anc + 3 * b + 1) * nb, az = __ldg(t.anc + 3 * b + 2) * nb;
-  TP *Pb = P + (size_t)b * np;
-  // one padded point per thread and step, four steps' sources resolved and
-  // loaded before any is stored (four independent loads in flight)
+  const int W2 = Wd * Wd, nb2 = nb * nb;
   const DivM dW = divm(Wd);
-  const int npt = Wd * Wd * Wd, bd = blockDim.x;
-  enum { SKIP = 0, LOAD = 1, SLOW = 2, BAD = 3 };
-  auto coords = [&](int p, int &i, int &j, int &k) {
-    const int row = divq(p, dW), kk = divq(row, dW);
-    i = p - row * Wd - Gi, j = row - kk * Wd - Gi, k = kk - Gi;
+  // n values st apart from src to padded planes from d on, four in flight
+  auto run = [&](TP *d, const TI *src, int st, int n) {
+    for (; n >= 4; n -= 4, d += 4 * W2, src += 4 * st) {
+      const TI v0 = ld(src), v1 = ld(src + st), v2 = ld(src + 2 * st), v3 = ld(src + 3 * st);
+      d[0] = Cvt<TP>::f(v0), d[W2] = Cvt<TP>::f(v1), d[2 * W2] = Cvt<TP>::f(v2), d[3 * W2] = Cvt<TP>::f(v3);
+    }
+    for (; n > 0; --n, d += W2, src += st) *d = Cvt<TP>::f(ld(src));
   };
-  for (int p0 = threadIdx.x; p0 < npt; p0 += 4 * bd) {
-    long long id[4];
-    int kind[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int p = p0 + u * bd;
-      kind[u] = SKIP, id[u] = 0;
-      if (p >= npt) continue;
-      int i, j, k;
-      coords(p, i, j, k);
-      const int rx = i < 0 ? 0 : i >= nb ? 2 : 1, ry = j < 0 ? 0 : j >= nb ? 2 : 1, rz = k < 0 ? 0 : k >= nb ? 2 : 1;
-      const int r = rx + 3 * ry + 9 * rz;
-      const int ri = i - (rx - 1) * nb, rj = j - (ry - 1) * nb, rk = k - (rz - 1) * nb;  // region-local
-      const int Lo = rlev[r];
+  for (int c = threadIdx.x; c < W2; c += blockDim.x) {
+    const int row = divq(c, dW), i = c - row * Wd - Gi, j = row - Gi;
+    const int rx = i < 0 ? 0 : i >= nb ? 2 : 1, ry = j < 0 ? 0 : j >= nb ? 2 : 1;
+    const int ri = i - (rx - 1) * nb, rj = j - (ry - 1) * nb;  // region-local
+    TP *col = P + (size_t)b * np + c + (size_t)W2 * Gi;        // (i, j, 0)
+    for (int rz = 0; rz < 3; ++rz) {
+      const int r = rx + 3 * ry + 9 * rz, Lo = rlev[r];
       if (Lo < L) continue;  // a coarser leaf's region: refined by the pre-pass
-      long long idx = -1;
+      const int k0 = rz == 0 ? nb - Gi : 0, k1 = rz == 2 ? Gi : nb, z0 = (rz - 1) * nb;  // region-local planes
       if (Lo == L) {
-        idx = (long long)rslot[r] * (long long)nb3 + ri + nb * (rj + nb * rk);
-      } else if (Lo == L + 1) {
-        const int hx = ri >= hb, hy = rj >= hb, hz = rk >= hb;
+        run(col + (ptrdiff_t)W2 * (z0 + k0), phi + (size_t)rslot[r] * nb3 + ri + nb * rj + nb2 * k0, nb2, k1 - k0);
+        continue;
+      }
+      const int hx = ri >= hb, hy = rj >= hb;
+      for (int hz = 0; hz < 2; ++hz) {
+        const int ka = hz ? max(k0, hb) : k0, kb = hz ? k1 : min(k1, hb);
+        if (ka >= kb) continue;
         const int o2 = rsub[r][hx + 2 * hy + 4 * hz];
-        if (o2 >= 0)
-          idx = (long long)o2 * (long long)nb3 + (2 * ri - hx * nb) + nb * ((2 * rj - hy * nb) + nb * (2 * rk - hz * nb));
+        if (o2 >= 0) {
+          run(col + (ptrdiff_t)W2 * (z0 + ka),
+              phi + (size_t)o2 * nb3 + (2 * ri - hx * nb) + nb * (2 * rj - hy * nb) + nb2 * (2 * ka - hz * nb),
+              2 * nb2, kb - ka);
+        } else {  // two levels down (shells wider than half a block)
+          for (int k = ka; k < kb; ++k) {
+            const int gx = ax + i, gy = ay + j, gz = az + z0 + k;
+            const int ow = owner(t, L, gx, gy, gz, b);
+            col[(ptrdiff_t)W2 * (z0 + k)] = Cvt<TP>::f(leaf_value(t, phi, ow, L, gx, gy, gz, err));
+          }
+        }
       }
-      if (idx >= 0 && idx < lim && ri >= 0 && ri < nb && rj >= 0 && rj < nb && rk >= 0 && rk < nb)
-        kind[u] = LOAD, id[u] = idx;
-      else
-        kind[u] = (idx == -1 && Lo > L) ? SLOW : BAD;  // SLOW: a finer region two levels down
-    }
-    TI v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = kind[u] == LOAD ? __ldg(phi + id[u]) : TI(0);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (kind[u] == SKIP) continue;
-      const int p = p0 + u * bd;
-      TP o;
-      if (kind[u] == LOAD) {
-        o = Cvt<TP>::f(v[u]);
-      } else if (kind[u] == SLOW) {  // shells wider than half a block
-        int i, j, k;
-        coords(p, i, j, k);
-        const int gx = ax + i, gy = ay + j, gz = az + k;
-        const int ow = owner(t, L, gx, gy, gz, b);
-        o = Cvt<TP>::f(leaf_value(t, phi, ow, L, gx, gy, gz, err));
-      } else {
-        atomicOr(err, 1 << 16);
-        o = TP(__int_as_float(0x7fc00000));
-      }
-      Pb[p] = o;
     }
   }
 }
 
-// partial sums of the separable refinement of the largest coarse-region box
-// (face nb x nb x Gi, edge nb x Gi x Gi, corner Gi^3; thinnest side first)
-static size_t sep_refine_elems(int N, int nb, int Gi) {
-  const int ko = N - 1;
-  auto ncmax = [&](int n) {
-    int m = 0;
-    for (int fl = 0; fl < 2; ++fl) m = std::max(m, ((fl + n - 1 + ko) >> 1) - ((fl - ko) >> 1) + 1);
-    return m;
-  };
-  const int shapes[3][3] = {{Gi, nb, nb}, {Gi, Gi, nb}, {Gi, Gi, Gi}};
-  size_t best = 0;
-  for (auto &sh : shapes) {
-    int f[3] = {sh[0], sh[1], sh[2]};
-    std::sort(f, f + 3);
-    const size_t u1 = (size_t)f[0] * ncmax(f[1]) * ncmax(f[2]), u2 = (size_t)f[0] * f[1] * ncmax(f[2]);
-    best = std::max(best, u1 + u2);
-  }
-  return best;
-}
-
-// partial sums of the separable refinement of one whole side of the padded
-// block (Gi x Wd x Wd fine points, its coarse extents), the largest box the
-// kernel builds from merged regions
-static size_t side_refine_elems(int N, int nb, int Gi) {
-  const int ko = N - 1, wd = nb + 2 * Gi;
-  const int cw = ((nb + Gi - 1 + ko) >> 1) - ((-Gi - ko) >> 1) + 1;
-  return (size_t)Gi * cw * cw + (size_t)Gi * wd * cw;
-}
-
-// shared memory of the separable Part-2 coarsening for zc coarse z-planes
-template <int N, int NT>
-static size_t push_smem(int nb, int zc, size_t es) {
-  const int hH = Wav<N, NT>::hwH, hb = nb / 2, nf = nb - 1 + 2 * hH, nk = 2 * zc - 1 + 2 * hH;
-  return es * ((size_t)nk * nf * hb + (size_t)nk * hb * hb);
+// Shared memory of the pre-pass's sums, or what a chunk of the largest box
+// takes.  Four CTAs of 256 threads per SM with FP32 blocks, three with FP64
+// ones; the sums stay small enough that the L1 cache keeps a share of the SM's
+// memory, since the block is read back through it: at 3 424 leaves of 24^3 with
+// 6.2 the pre-pass takes 312 us with 27 or 34 KB, 417 us with 42 KB (L1 almost
+// gone) and 323 us with 54 KB (three CTAs).
+static size_t prep_sum_bytes(int N, int nb, int Gi, size_t es, bool bounded) {
+  const int ko = N - 1, m = nb + Gi, mb = ((m - 1 + 2 * ko) >> 1) + 2;
+  const size_t plane = (size_t)Gi * (mb | 1) + ((size_t)Gi * (m | 1) | 1);
+  return std::max<size_t>(es == 4 ? 34 * 1024 : 48 * 1024, (plane * prep_min_planes(N, bounded) * es + 15) & ~(size_t)15);
 }
 
 // Merge the part-2 values into P (only the neighbour regions owned by finer
 // leaves hold them) and write the substituted interior back to the field of
 // leaves that have a coarser neighbour.
-template <typename TO, typename TP>
+template <typename TO, typename TP, int N, int NT, bool BND>
 __global__ void __launch_bounds__(512) k_merge(Tree t, TP *__restrict__ P, const TP *__restrict__ Q,
                                                int Gi, int G, const int *__restrict__ cmask,
                                                TO *__restrict__ phi_out, const int *__restrict__ need) {
@@ -1049,11 +1084,12 @@ __global__ void __launch_bounds__(512) k_merge(Tree t, TP *__restrict__ P, const
     const int dd[3] = {r % 3 - 1, (r / 3) % 3 - 1, r / 9 - 1};
     int g[3];
     for (int d = 0; d < 3; ++d) g[d] = __ldg(t.anc + 3 * b + d) * nb + (dd[d] < 0 ? -1 : dd[d] > 0 ? nb : 0);
-    rfin[r] = r != 13 && __ldg(t.lev + owner(t, L, g[0], g[1], g[2], b)) > L;
+    rfin[r] = r != 13 && !(BND && beyond3(t, L, g)) && __ldg(t.lev + owner(t, L, g[0], g[1], g[2], b)) > L;
   }
   __syncthreads();
+  // (N.0 pushes nothing: the gather's coincident values stand)
   for (int r = 0; r < 27; ++r) {
-    if (!rfin[r]) continue;
+    if (NT == 0 || !rfin[r]) continue;
     const int dd[3] = {r % 3 - 1, (r / 3) % 3 - 1, r / 9 - 1};
     int lo[3], ext[3];
     for (int d = 0; d < 3; ++d) {
@@ -1069,6 +1105,12 @@ __global__ void __launch_bounds__(512) k_merge(Tree t, TP *__restrict__ P, const
       P[q] = Q[q];
     }
   }
+  if constexpr (BND) {
+    const int ax = __ldg(t.anc + 3 * b) * nb, ay = __ldg(t.anc + 3 * b + 1) * nb, az = __ldg(t.anc + 3 * b + 2) * nb;
+    if (bc_touches(t, L, ax, ay, az, -G, nb + G))
+      bc_box<N>(t, L, ax, ay, az, P + b * np + Gi * (1 + Wd + Wd * Wd), Wd, Wd * Wd, -G, -G, -G, nb + 2 * G,
+                nb + 2 * G, nb + 2 * G);
+  }
   if (phi_out && cmask[b]) {
     const DivM dnb = divm(nb);
     for (int p = threadIdx.x; p < nb * nb * nb; p += blockDim.x) {
@@ -1080,15 +1122,22 @@ __global__ void __launch_bounds__(512) k_merge(Tree t, TP *__restrict__ P, const
   }
 }
 
+// The requested shell G of the padded blocks (internal shell Gi).  One thread
+// per (x, y) column, so a point costs a load, a store and two additions; bound
+// by the copy.
 template <typename TO, typename TP>
-__global__ void k_crop(const TP *__restrict__ P, int Gi, TO *__restrict__ out, int G, int nb) {
+__global__ void __launch_bounds__(256) k_crop(const TP *__restrict__ P, int Gi, TO *__restrict__ out, int G, int nb) {
   const int b = blockIdx.x;
-  const int Wd = nb + 2 * Gi, Wg = nb + 2 * G;
-  const size_t np = (size_t)Wd * Wd * Wd, ng = (size_t)Wg * Wg * Wg;
-  for (size_t p = threadIdx.x; p < ng; p += blockDim.x) {
-    const int i = (int)(p % Wg), j = (int)((p / Wg) % Wg), k = (int)(p / ((size_t)Wg * Wg));
-    out[(size_t)b * ng + p] =
-        TO(P[(size_t)b * np + (i - G + Gi) + Wd * ((j - G + Gi) + (size_t)Wd * (k - G + Gi))]);
+  const int Wd = nb + 2 * Gi, Wg = nb + 2 * G, W2 = Wd * Wd, Wg2 = Wg * Wg, o = Gi - G;
+  const TP *src = P + (size_t)b * Wd * W2 + o * (1 + Wd + (size_t)W2);
+  TO *dst = out + (size_t)b * Wg * Wg2;
+  const DivM dg = divm(Wg);
+  for (int c = threadIdx.x; c < Wg2; c += blockDim.x) {
+    const int j = divq(c, dg);
+    const TP *s = src + c - j * Wg + Wd * j;
+    TO *d = dst + c;
+#pragma unroll 6
+    for (int k = 0; k < Wg; ++k) d[(size_t)k * Wg2] = TO(__ldg(s + (size_t)k * W2));
   }
 }
 
@@ -1109,28 +1158,15 @@ int ghost_impl(mr_grid *g, const TI *phi_in, TI *phi_out, int G, TP *P, TP *Q, i
   Tree t = tree_view(g);
   const int n = g->nleaf, nb = g->desc.nb;
   int *err = g->counter + 1;
-  const int nq = tq_hi<N>(nb, Gi) - tq_lo<N>(Gi) + 1;
-  const size_t smT = (sizeof(TI) * (size_t)nq * nq * nq + 15) & ~(size_t)15;
-  const size_t budget = 220 * 1024;
-  // partial sums of the separable refinement: at least one region's, and up
-  // to a whole side of the padded block (the kernel merges the coarser
-  // regions into boxes that fit) as long as the occupancy stays (two CTAs
-  // per SM where one region's sums allow it)
-  const size_t smU1 = sizeof(TP) * sep_refine_elems(N, nb, Gi);
-  const size_t smUs = sizeof(TP) * side_refine_elems(N, nb, Gi);
-  const size_t target = smT + smU1 <= 110 * 1024 && sizeof(TP) == 4 ? 110 * 1024 : budget;
-  const size_t smU = std::max(smU1, std::min(smUs, target > smT ? (target - smT) & ~(size_t)15 : (size_t)0));
-  // 2: coarse tile + separable refinement, 1: tile + per-point tensor sums,
-  // 0: per-point sums through the owner map
-  const int use_tile = smT + smU <= budget ? 2 : smT <= budget ? 1 : 0;
-  int zc = nb / 2;
-  while (zc > 1 && push_smem<N, NT>(nb, zc, sizeof(TP)) > budget) --zc;
-  const size_t smP = push_smem<N, NT>(nb, zc, sizeof(TP));
-  if (smP > 227 * 1024) return MR_ERR_UNSUPPORTED;
-  const size_t sm = std::max(use_tile == 2 ? smT + smU : use_tile ? smT : (size_t)0, smP);
+  // (bounded grids have their own instantiations: their out-of-line calls would
+  // cost the others registers)
+  const auto prep = t.bnd ? k_prep<TI, TP, N, NT, true> : k_prep<TI, TP, N, NT, false>;
+  const auto merge = t.bnd ? k_merge<TI, TP, N, NT, true> : k_merge<TI, TP, N, NT, false>;
+  const size_t sm = prep_sum_bytes(N, nb, Gi, sizeof(TP), t.bnd != 0);
+  if (sm > 200 * 1024) return MR_ERR_UNSUPPORTED;
   // (set on every launch: the kernel's static shared memory counts against
   // the 48 KB that needs no opt-in)
-  if (check_cuda(cudaFuncSetAttribute(k_prep<TI, TP, N, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+  if (check_cuda(cudaFuncSetAttribute(prep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
                  "k_prep smem"))
     return MR_ERR_CUDA;
   // The plain gather writes every region but the coarser leaves' of the
@@ -1154,14 +1190,12 @@ int ghost_impl(mr_grid *g, const TI *phi_in, TI *phi_out, int G, TP *P, TP *Q, i
     }
   }
   const int *need_prep = g->pneed;
-  static const int cp[2] = {512, 256};
+  static const int cp[2] = {256, 128};
   const int thp = tune_threads(g, TuneKey{1, N, NT, nb, tp, Gi, only_coarse}, cp, 2, [&](int th) {
-    k_prep<TI, TP, N, NT><<<n, th, sm, g->stream>>>(t, phi_in, P, Q, Gi, G, only_coarse, use_tile, (int)smT, zc,
-                                                    g->cmask, err, need_prep, 1, (int)sm);
+    prep<<<n, th, sm, g->stream>>>(t, phi_in, P, Q, Gi, G, only_coarse, g->cmask, err, need_prep, (int)sm);
   });
-  MR_LAUNCH(g, MRK_PART1, k_prep<TI, TP, N, NT><<<n, thp, sm, g->stream>>>(t, phi_in, P, Q, Gi, G, only_coarse,
-                                                                           use_tile, (int)smT, zc, g->cmask, err,
-                                                                           need_prep, 1, (int)sm));
+  MR_LAUNCH(g, MRK_PART1, prep<<<n, thp, sm, g->stream>>>(t, phi_in, P, Q, Gi, G, only_coarse, g->cmask, err,
+                                                          need_prep, (int)sm));
   if (check_cuda(cudaGetLastError(), "k_prep")) return MR_ERR_CUDA;
   if (only_coarse != 2) {  // the substitution-only pass fills no shell
     const double wd = nb + 2.0 * G;
@@ -1170,9 +1204,9 @@ int ghost_impl(mr_grid *g, const TI *phi_in, TI *phi_out, int G, TP *P, TP *Q, i
   if (only_coarse) return MR_OK;
   static const int cm[3] = {256, 128, 512};
   const int thm = tune_threads(g, TuneKey{5, N, NT, nb, tp, Gi, 0}, cm, 3, [&](int th) {
-    k_merge<TI, TP><<<n, th, 0, g->stream>>>(t, P, Q, Gi, G, g->cmask, phi_out, need);
+    merge<<<n, th, 0, g->stream>>>(t, P, Q, Gi, G, g->cmask, phi_out, need);
   });
-  MR_LAUNCH(g, MRK_MERGE, k_merge<TI, TP><<<n, thm, 0, g->stream>>>(t, P, Q, Gi, G, g->cmask, phi_out, need));
+  MR_LAUNCH(g, MRK_MERGE, merge<<<n, thm, 0, g->stream>>>(t, P, Q, Gi, G, g->cmask, phi_out, need));
   if (check_cuda(cudaGetLastError(), "k_merge")) return MR_ERR_CUDA;
   return MR_OK;
 }

@@ -641,8 +641,7 @@ int launch_ghost_adapt32(mr_grid *g, const float *phi, int G, const int *need, v
 int launch_fused(mr_grid *g, const void *phi, const void *P, const void *Q, int Gi, const void *u, void *out,
                  int stage, double dt, const double *uc, int scheme, bool rhs_only, const void *vpad = nullptr);
 int adapt_shell(int N, int Nt);
-// boundary.cu: grids with physical boundaries (the general point-wise path)
-int ghost_bounded(mr_grid *g, const void *phi_in, void *phi_out, int G, bool fp64, void *P, void *Q, int Gi);
+// boundary.cu: the block criterion of grids with physical boundaries
 int launch_criterion_bounded(mr_grid *g, const double *P, int Gi, double *maxdet);
 inline bool grid_bounded(const mr_grid *g) {
   return (g->desc.flags & (MR_GRID_BOUNDED_X | MR_GRID_BOUNDED_Y | MR_GRID_BOUNDED_Z)) != 0;
