@@ -192,24 +192,30 @@ __global__ void k_field_set(Tree t, T *f, int kind, InitParams ip) {
     a[d] = __ldg(t.anc + 3 * b + d);
     if (t.indep) a[d] &= (1 << L) - 1;  // anchor within the leaf's tree
   }
+  // kinds that depend on the distance from one centre: the squared distance
+  // along each axis, once per block (a point adds three of them; the divisions
+  // and roundings of the nearest image took 40 % of the FP64 instructions)
+  const bool radial = kind == MR_INIT_GAUSSIAN || kind == MR_INIT_TANH_SPHERE || kind == MR_INIT_COMPACT_GAUSSIAN;
+  __shared__ double sq[3][32];
+  if (radial) {
+    for (int q = threadIdx.x; q < 3 * nb; q += blockDim.x) {
+      const int d = q / nb, i = q - d * nb;
+      const double dd = pdelta((a[d] * nb + i) * h, ip.p[d], ext[d]);
+      sq[d][i] = dd * dd;
+    }
+    __syncthreads();
+  }
   for (int p = threadIdx.x; p < nb * nb * nb; p += blockDim.x) {
-    const int i = p % nb, j = (p / nb) % nb, k = p / (nb * nb);
+    const int rr = divq(p, t.dnb), k = divq(rr, t.dnb), i = p - rr * nb, j = rr - k * nb;
     const double x[3] = {(a[0] * nb + i) * h, (a[1] * nb + j) * h, (a[2] * nb + k) * h};
+    const double r2 = radial ? sq[0][i] + sq[1][j] + sq[2][k] : 0.0;
     double v = 0.0;
     if (kind == MR_INIT_GAUSSIAN) {
-      double r2 = 0.0;
-      for (int d = 0; d < 3; ++d) {
-        const double dd = pdelta(x[d], ip.p[d], ext[d]);
-        r2 += dd * dd;
-      }
       v = ip.p[4] * exp(-r2 / (ip.p[3] * ip.p[3]));
     } else if (kind == MR_INIT_TANH_SPHERE) {
-      double r2 = 0.0;
-      for (int d = 0; d < 3; ++d) {
-        const double dd = pdelta(x[d], ip.p[d], ext[d]);
-        r2 += dd * dd;
-      }
-      v = 0.5 * (1.0 - tanh((sqrt(r2) - ip.p[3]) / ip.p[4]));
+      // tanh(x) rounds to +-1 from |x| = 19.1 on
+      const double y = (sqrt(r2) - ip.p[3]) / ip.p[4];
+      v = y > 22.0 ? 0.0 : y < -22.0 ? 1.0 : 0.5 * (1.0 - tanh(y));
     } else if (kind == MR_INIT_GAUSSIAN_SUM || kind == MR_INIT_GAUSSIAN_SUM_ADD) {
       const int ng = (int)ip.p[0];
       for (int q = 0; q < ng; ++q) {
@@ -222,11 +228,6 @@ __global__ void k_field_set(Tree t, T *f, int kind, InitParams ip) {
         v += c[4] * exp(-r2 / (c[3] * c[3]));
       }
     } else if (kind == MR_INIT_COMPACT_GAUSSIAN) {
-      double r2 = 0.0;
-      for (int d = 0; d < 3; ++d) {
-        const double dd = pdelta(x[d], ip.p[d], ext[d]);
-        r2 += dd * dd;
-      }
       const double s2 = ip.p[3] * ip.p[3], b2 = ip.p[4] * ip.p[4];
       v = r2 < b2 ? ip.p[5] * exp(-(r2 / s2) / (1.0 - r2 / b2)) : 0.0;
     } else if (kind == MR_INIT_DEFORMATION) {
@@ -267,29 +268,38 @@ template <typename T>
 __global__ void k_mass_leaf(Tree t, const T *f, double *part) {
   const int b = blockIdx.x, nb = t.nb;
   const double h = t.tree_len / ((double)nb * (double)(1 << __ldg(t.lev + b)));
-  double s = 0.0;
-  for (int p = threadIdx.x; p < nb * nb * nb; p += blockDim.x) s += (double)f[(size_t)b * nb * nb * nb + p];
-  __shared__ double red[256];
-  red[threadIdx.x] = s;
+  // one FP64 addition per value (the pipe's floor); the widening runs on the
+  // integer pipe, two sums per thread hide the addition's latency
+  const T *fb = f + (size_t)b * nb * nb * nb;
+  const int n = nb * nb * nb, bd = blockDim.x;
+  double s0 = 0.0, s1 = 0.0;
+  int p = threadIdx.x;
+#pragma unroll 4
+  for (; p + bd < n; p += 2 * bd) s0 += Cvt<double>::f(__ldg(fb + p)), s1 += Cvt<double>::f(__ldg(fb + p + bd));
+  if (p < n) s0 += Cvt<double>::f(__ldg(fb + p));
+  double s = s0 + s1;
+  for (int w = 16; w > 0; w >>= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
+  __shared__ double red[8];
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (bd >> 5); ++w) s += red[w];
+    part[b] = s * h * h * h;
   }
-  if (threadIdx.x == 0) part[b] = red[0] * h * h * h;
 }
 
-__global__ void k_sum_serial(const double *part, int n, double *out) {
-  __shared__ double red[256];
+__global__ void __launch_bounds__(1024) k_sum_serial(const double *part, int n, double *out) {
   double s = 0.0;
+#pragma unroll 4
   for (int i = threadIdx.x; i < n; i += blockDim.x) s += part[i];
-  red[threadIdx.x] = s;
+  for (int w = 16; w > 0; w >>= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
+  __shared__ double red[32];
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) s += red[w];
+    *out = s;
   }
-  if (threadIdx.x == 0) *out = red[0];
 }
 
 int launch_mass(mr_grid *g, const void *f, double *host_out) {
@@ -298,7 +308,7 @@ int launch_mass(mr_grid *g, const void *f, double *host_out) {
     MR_LAUNCH(g, MRK_MASS, k_mass_leaf<float><<<g->nleaf, 256, 0, g->stream>>>(t, (const float *)f, g->maxdet));
   else
     MR_LAUNCH(g, MRK_MASS, k_mass_leaf<double><<<g->nleaf, 256, 0, g->stream>>>(t, (const double *)f, g->maxdet));
-  MR_LAUNCH(g, MRK_MASS, k_sum_serial<<<1, 256, 0, g->stream>>>(g->maxdet, g->nleaf, g->dscratch));
+  MR_LAUNCH(g, MRK_MASS, k_sum_serial<<<1, 1024, 0, g->stream>>>(g->maxdet, g->nleaf, g->dscratch));
   if (check_cuda(cudaGetLastError(), "k_mass")) return MR_ERR_CUDA;
   if (check_cuda(cudaMemcpyAsync(host_out, g->dscratch, sizeof(double), cudaMemcpyDeviceToHost, g->stream),
                  "mass copy"))
@@ -316,9 +326,33 @@ __global__ void __launch_bounds__(256) k_umax_leaf(int nb, const T *__restrict__
   const int b = blockIdx.x;
   const size_t nb3 = (size_t)nb * nb * nb, o = (size_t)b * nb3;
   unsigned long long m = 0;
-  for (size_t p = threadIdx.x; p < nb3; p += blockDim.x) {
+  auto exact = [&](size_t p) {
     const double s = fabs((double)u0[o + p]) + fabs((double)u1[o + p]) + fabs((double)u2[o + p]);
     m = max(m, abs_key(s));
+  };
+  if constexpr (sizeof(T) == 4) {
+    // FP32 sums rounded down and up enclose the FP64 sum (rounding is monotone
+    // and every FP32 number is an FP64 one), so only points whose upper bound
+    // reaches the block's largest lower bound need it: the two FP64 additions
+    // and three conversions of every point were what bound this kernel.
+    float lo = 0.f;
+#pragma unroll 4
+    for (size_t p = threadIdx.x; p < nb3; p += blockDim.x)
+      lo = fmaxf(lo, __fadd_rd(__fadd_rd(fabsf(u0[o + p]), fabsf(u1[o + p])), fabsf(u2[o + p])));
+    __shared__ unsigned best;
+    if (threadIdx.x == 0) best = 0;
+    __syncthreads();
+    for (int w = 16; w > 0; w >>= 1) lo = fmaxf(lo, __shfl_xor_sync(0xffffffffu, lo, w));
+    if ((threadIdx.x & 31) == 0) atomicMax(&best, __float_as_uint(lo));  // lo >= 0: ordered as integers
+    __syncthreads();
+    const float top = __uint_as_float(best);
+#pragma unroll 4
+    for (size_t p = threadIdx.x; p < nb3; p += blockDim.x) {
+      const float hi = __fadd_ru(__fadd_ru(fabsf(u0[o + p]), fabsf(u1[o + p])), fabsf(u2[o + p]));
+      if (!(hi < top)) exact(p);  // (NaN included)
+    }
+  } else {
+    for (size_t p = threadIdx.x; p < nb3; p += blockDim.x) exact(p);
   }
   for (int w = 16; w > 0; w >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, w));
   __shared__ unsigned long long red[8];
