@@ -37,7 +37,7 @@ def _stale(obj, deps):
 
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OUT, exist_ok=True)
-    hdrs = [os.path.join(SRC, "mr_internal.cuh"), os.path.join(SRC, "ghost_kernels.cuh"),
+    hdrs = [os.path.join(SRC, "mr_internal.cuh"), os.path.join(SRC, "wavelet_runs.cuh"), os.path.join(SRC, "ghost_kernels.cuh"),
             os.path.join(SRC, "stage_kernels.cuh"),
             os.path.join(os.path.dirname(HERE), "include", "mrgb.h")]
     nvcc = _nvcc()

@@ -5,7 +5,9 @@
 // fixed point) -> new leaves in Morton order (scan + emit) -> owner map of
 // the new tree -> per field: ghost fill, refinement / coarsening / copy into
 // the second pool, update step next to newly coarsened leaves.
-#include "mr_internal.cuh"
+#include <algorithm>
+
+#include "wavelet_runs.cuh"
 
 namespace mr {
 
@@ -13,275 +15,309 @@ enum { KIND_COPY = 0, KIND_CHILD = 1, KIND_PARENT = 2 };
 enum { ST_COARSER = -1, ST_SAME = 0, ST_FINER = 1 };
 
 // ------------------------------------------------------------- criterion
-// Details gamma over the extended region [-ext_f, nb-1+ext_b]^3 of one padded
-// block: 1D filters x, then y, then z, G^a on odd and H^a on even
-// coordinates; points with only even coordinates carry no detail and get 0.
-// Each 1D pass uses the lifting form of the pair: the G^a output at an odd
-// point is the point minus the K^s-weighted prediction from its even
-// neighbours (odd taps only), and the H^a output at an even point is the
-// point plus 1/4 of the two neighbouring G^a outputs (N.2; H^a is the
+// Arithmetic of the details: the block's type TP, or float pairs (about 48
+// significant bits on the FP32 pipe) from FP64 blocks.
+template <typename TP, bool PAIRS>
+struct DetOps {
+  using E = TP;
+  static __device__ __forceinline__ E zero() { return TP(0); }
+  static __device__ __forceinline__ E load(TP v) { return v; }
+  static __device__ __forceinline__ E acc(E s, double w, E v) { return racc(s, TP(w), v); }
+  static __device__ __forceinline__ E norm(E s) { return s; }
+  static __device__ __forceinline__ E lift(E v, E a, E b) { return racc(v, TP(0.25), a + b); }
+  static __device__ __forceinline__ TP value(E s) { return s; }
+};
+template <>
+struct DetOps<double, true> {
+  using E = F2;
+  static __device__ __forceinline__ E zero() { return {0.f, 0.f}; }
+  static __device__ __forceinline__ E load(double v) { return f2_split(v); }
+  static __device__ __forceinline__ E acc(E s, double w, E v) { return f2_acc(s, float(w), v); }
+  static __device__ __forceinline__ E norm(E s) { return f2_norm(s); }
+  static __device__ __forceinline__ E lift(E v, E a, E b) { return f2_norm(f2_acc(v, 0.25f, f2_add(a, b))); }
+  static __device__ __forceinline__ double value(E s) { return f2_dbl(s); }
+};
+
+// Details gamma over a box of the extended region [-ext_f, nb-1+ext_b]^3 of one
+// padded block: 1D filters x, then y, then z, G^a on odd and H^a on even
+// coordinates; points with only even coordinates carry no detail and get 0.  Each 1D pass uses the lifting form of the pair:
+// the G^a output at an odd point is the point minus the K^s-weighted prediction
+// from its even neighbours (odd taps only), and the H^a output at an even point
+// is the point plus 1/4 of the two neighbouring G^a outputs (N.2; H^a is the
 // identity for N.0) -- the same filters, about half the multiply-adds.
-// The z-planes of the y-pass results live in a ring of 2(N-1)+1 planes and the
-// z-details of the last two odd planes in a second ring.  emit(i, j, k, idx,
-// gamma) is called once per point of the region (idx = i-r0 + nR*(j-r0)).
-// T: the padded blocks' type and the working precision.
-template <int N, int NT, typename T, typename F>
-__device__ __forceinline__ void detail_planes(const T *__restrict__ Pb, int nb, int Gi, T *sm, F emit) {
+// Planes march along z: the y-pass results live in a ring of 2(N-1)+1 planes,
+// the z-details of the last two odd planes in a second ring (written and read
+// by the same thread).  Four barriers per plane; the next plane is staged while
+// the y pass runs.  A block is cut into column tiles so that two or three CTAs
+// share an SM and one computes while another waits at a barrier.  Bound by issued
+// instructions of the FP32 pipe (float pairs) and by the barriers: 2 080 leaves
+// of 24^3, 6.2, took 2.79 ms whole (163 KB, one CTA per SM), 2.25 ms in tiles.
+// emit(i, j, k, gamma) is called once per point of the box (gamma unconverted).
+struct DetBox {  // inclusive
+  int lo[3], hi[3];
+};
+struct DetTile {  // computed points [c0, c0 + w) of one axis: the lift of an even edge point reads one more
+  int c0, w;
+};
+template <int NT>
+__host__ __device__ __forceinline__ DetTile det_tile(int i0, int i1) {
+  const int c0 = NT && !(i0 & 1) ? i0 - 1 : i0, c1 = NT && !(i1 & 1) ? i1 + 1 : i1;
+  return {c0, c1 - c0 + 1};
+}
+// elements of shared memory for w computed columns and nR computed rows
+template <int N>
+__host__ __device__ __forceinline__ size_t det_elems(int nR, int w) {
+  const int ko = N - 1, nA = nR + 2 * ko;
+  return (size_t)(2 * ko + 3) * nR * w + (size_t)nA * w + (size_t)nA * (w + 2 * ko);
+}
+
+// threads of a CTA, and items per thread and pass (det_tiles cuts accordingly):
+// the index arithmetic of a pass is done once, not once per plane
+constexpr int DET_THREADS = 512, DET_ITEMS = 2;
+
+template <int N, int NT, bool PAIRS, typename TP, typename F>
+__device__ __forceinline__ void detail_planes(const TP *__restrict__ Pb, int nb, int Gi, const DetBox &B,
+                                              typename DetOps<TP, PAIRS>::E *sm, F emit) {
   using W = Wav<N, NT>;
-  constexpr int ko = N - 1, R = 2 * ko + 1;
-  constexpr T U = NT ? T(0.25) : T(0);  // lifting update weight
-  const int Wd = nb + 2 * Gi;
-  const int r0 = -W::ext_f, r1 = nb - 1 + W::ext_b, nR = r1 - r0 + 1, nA = nR + 2 * ko;
+  using D = DetOps<TP, PAIRS>;
+  using E = typename D::E;
+  constexpr int ko = N - 1, R = 2 * ko + 1, K = DET_ITEMS;
+  const int Wd = nb + 2 * Gi, tid = threadIdx.x, bd = blockDim.x;
+  const DetTile tx = det_tile<NT>(B.lo[0], B.hi[0]), ty = det_tile<NT>(B.lo[1], B.hi[1]),
+                tz = det_tile<NT>(B.lo[2], B.hi[2]);
+  const int c0 = tx.c0, w = tx.w, wS = w + 2 * ko;               // columns
+  const int r0 = ty.c0, nR = ty.w, r1 = r0 + nR - 1, nA = nR + 2 * ko;  // rows
+  const int z0 = tz.c0, z1 = z0 + tz.w - 1, pl = nR * w;          // planes
   const int lo = -Gi, hi = nb - 1 + Gi;  // stored padded range
-  const int nodd = par_count(r0, r1 + 1, 1), nev = nR - nodd;
-  const int fo = par_first(r0, 1), fe = par_first(r0, 0);
-  const int pl = nR * nR;
-  const DivM dO = divm(nodd), dE = divm(nev), dR = divm(nR);
-  T *ring = sm;             // [R][nR][nR]  y-pass planes
-  T *dz = sm + R * pl;      // [2][nR][nR]  z-details of odd planes
-  T *A = dz + 2 * pl;       // [nA][nR]     x-pass of one plane
-  // G^a output: v[0] - sum_{t odd} K(t) v[t*stride]
-  auto gsum = [](const T *v, int stride) {
-    T s = v[0];
-#pragma unroll
-    for (int t = -ko; t <= ko; t += 2) s = racc(s, T(-Wav<N, NT>::K(t)), v[t * stride]);
-    return s;
+  E *ring = sm;             // [R][nR][w]     y-pass planes
+  E *dz = sm + R * pl;      // [2][nR][w]     z-details of odd planes
+  E *A = dz + 2 * pl;       // [nA][w]        x-pass of one plane
+  E *S = A + nA * w;        // [nA][wS]       the staged plane
+  // Beyond the region a pass reads even points only (the K^s taps of odd points):
+  // rows and planes there with odd coordinates are left out.  Row jr of the
+  // nE rows in use: the region's, then the even ones below and above it.
+  const int eb = ko / 2 + 1, nE = nR + 2 * eb;
+  auto row = [&](int q) {
+    return q < nR ? ko + q : q < nR + eb ? (r0 & 1 ? ko - 1 : ko - 2) - 2 * (q - nR)
+                                         : ko + nR + (r1 & 1 ? 0 : 1) + 2 * (q - nR - eb);
   };
-  for (int kk = r0 - ko; kk <= r1 + ko + 1; ++kk) {
-    const int slot = (kk - (r0 - ko)) % R;
+  // the thread's items of every pass, the same on all planes (-1: none).  x
+  // passes: (row, column) of A, packed; y and z passes: offset in a plane
+  int xo[K], xe[K], yo[K], ye[K];
+  const int fz = par_first(z0, 1);  // first odd plane
+  {
+    const int fo = par_first(c0, 1), nxo = par_count(c0, c0 + w, 1);
+    // even columns: those whose odd neighbours are computed (N.0: all)
+    const int fe = NT && par_first(c0, 0) == c0 ? c0 + 2 : par_first(c0, 0);
+    const int nxe = par_count(fe, NT ? c0 + w - 1 : c0 + w, 0);
+    const int fy = par_first(r0, 1), ge = par_first(r0, 0), nyo = par_count(r0, r1 + 1, 1), nye = nR - nyo;
+    const DivM dxo = divm(nxo > 0 ? nxo : 1), dxe = divm(nxe > 0 ? nxe : 1), dw = divm(w);
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+      const int idx = tid + u * bd, qo = divq(idx, dxo), qe = divq(idx, dxe), qw = divq(idx, dw);
+      const int ro = row(qo), re = row(qe);
+      xo[u] = idx < nxo * nE && ro >= 0 && ro < nA ? ro << 16 | (fo - c0 + 2 * (idx - qo * nxo)) : -1;
+      xe[u] = idx < nxe * nE && re >= 0 && re < nA ? re << 16 | (fe - c0 + 2 * (idx - qe * nxe)) : -1;
+      yo[u] = idx < w * nyo ? idx - qw * w + w * (fy - r0 + 2 * qw) : -1;
+      ye[u] = idx < w * nye ? idx - qw * w + w * (ge - r0 + 2 * qw) : -1;
+    }
+  }
+  // G^a output: v[0] - sum_{t odd} K(t) v[t*stride]
+  auto gsum = [](const E *v, int stride) {
+    E s = v[0];
+#pragma unroll
+    for (int t = -ko; t <= ko; t += 2) s = D::acc(s, -W::K(t), v[t * stride]);
+    return D::norm(s);
+  };
+  // rows r0-ko .. r1+ko of plane kk, columns c0-ko .. c0+w-1+ko, one row per warp
+  auto stage = [&](int kk) {
     const bool kin = kk >= lo && kk <= hi;
-    const T *pk = Pb + (size_t)(kk + Gi) * Wd * Wd;
-    // x pass: odd columns, then even columns (rows jj = r0-ko .. r1+ko)
-    for (int idx = threadIdx.x; idx < nodd * nA; idx += blockDim.x) {
-      const int q = divq(idx, dO), i = fo + 2 * (idx - q * nodd), jj = r0 - ko + q;
-      const bool in = kin && jj >= lo && jj <= hi;
-      A[(i - r0) + nR * (jj - (r0 - ko))] = in ? gsum(pk + (jj + Gi) * Wd + (i + Gi), 1) : T(0);
+    const TP *pk = Pb + (ptrdiff_t)(kk + Gi) * Wd * Wd + Gi;
+    for (int x = tid & 31; x < wS; x += 32) {
+      const int ii = c0 - ko + x;
+      const bool cin = kin && ii >= lo && ii <= hi;
+      for (int q = tid >> 5; q < nE; q += bd >> 5) {
+        const int jr = row(q), jj = r0 - ko + jr;
+        if (jr < 0 || jr >= nA) continue;
+        S[jr * wS + x] = cin && jj >= lo && jj <= hi ? D::load(__ldg(pk + (jj + Gi) * Wd + ii)) : D::zero();
+      }
     }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < nev * nA; idx += blockDim.x) {
-      const int q = divq(idx, dE), i = fe + 2 * (idx - q * nev), jj = r0 - ko + q;
-      const bool in = kin && jj >= lo && jj <= hi;
-      T *a = A + (i - r0) + nR * (jj - (r0 - ko));
-      T v = in ? pk[(jj + Gi) * Wd + (i + Gi)] : T(0);
-      if (NT) v = racc(v, U, a[-1] + a[1]);
-      *a = v;
+  };
+  auto used = [&](int kk) { return kk <= z1 + ko && ((kk >= z0 && kk <= z1) || !(kk & 1)); };
+  if (used(z0 - ko)) stage(z0 - ko);
+  __syncthreads();
+  int slot = 0;
+  for (int kk = z0 - ko; kk <= z1 + ko + 1; ++kk, slot = slot + 1 == R ? 0 : slot + 1) {
+    const bool in = used(kk);
+    // x pass: odd columns, then even columns
+    if (in) {
+#pragma unroll
+      for (int u = 0; u < K; ++u)
+        if (xo[u] >= 0) {
+          const int jr = xo[u] >> 16, x = xo[u] & 0xffff;
+          A[x + w * jr] = gsum(S + jr * wS + x + ko, 1);
+        }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < K; ++u)
+        if (xe[u] >= 0) {
+          const int jr = xe[u] >> 16, x = xe[u] & 0xffff;
+          E *a = A + x + w * jr;
+          const E v = S[jr * wS + x + ko];
+          if constexpr (NT != 0) *a = D::lift(v, a[-1], a[1]);
+          else *a = v;
+        }
+      __syncthreads();
+      // y pass into ring plane kk: odd rows, then even rows
+      E *rp = ring + slot * pl;
+      const E *Ay = A + w * ko;
+#pragma unroll
+      for (int u = 0; u < K; ++u)
+        if (yo[u] >= 0) rp[yo[u]] = gsum(Ay + yo[u], w);
+      if (used(kk + 1)) stage(kk + 1);
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < K; ++u)
+        if (ye[u] >= 0) {
+          E *r = rp + ye[u];
+          const E v = Ay[ye[u]];
+          if constexpr (NT != 0) *r = D::lift(v, r[-w], r[w]);
+          else *r = v;
+        }
+      __syncthreads();
+    } else {
+      if (used(kk + 1)) stage(kk + 1);
+      __syncthreads();
     }
-    __syncthreads();
-    // y pass into ring plane kk: odd rows, then even rows
-    T *rp = ring + slot * pl;
-    for (int idx = threadIdx.x; idx < nR * nodd; idx += blockDim.x) {
-      const int q = divq(idx, dR), ii = idx - q * nR, j = fo + 2 * q;
-      rp[ii + nR * (j - r0)] = gsum(A + ii + nR * (j - (r0 - ko)), nR);
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < nR * nev; idx += blockDim.x) {
-      const int q = divq(idx, dR), ii = idx - q * nR, j = fe + 2 * q;
-      T *r = rp + ii + nR * (j - r0);
-      T v = A[ii + nR * (j - (r0 - ko))];
-      if (NT) v = racc(v, U, r[-nR] + r[nR]);
-      *r = v;
-    }
-    __syncthreads();
     // z: odd plane k1 = kk - ko (planes k1-ko .. k1+ko are in the ring), then
     // the even plane k1 - 1 from its ring plane and the odd planes around it
     const int k1 = kk - ko;
-    if ((k1 & 1) && k1 >= r0 && k1 <= r1 + 1) {
-      const int s1 = (slot + ko + 1) % R;  // ring slot of plane k1
-      T *d1 = dz + (((k1 - fo) >> 1) & 1) * pl, *d0 = dz + ((((k1 - fo) >> 1) + 1) & 1) * pl;
-      if (k1 <= r1) {
-        for (int idx = threadIdx.x; idx < pl; idx += blockDim.x) {
-          const T *c = ring + idx;
-          T v = c[s1 * pl];
+    if ((k1 & 1) && k1 >= z0 && k1 <= z1 + 1) {
+      const int s1 = slot + ko + 1 >= R ? slot + ko + 1 - R : slot + ko + 1;  // ring slot of plane k1
+      const int s0 = s1 == 0 ? R - 1 : s1 - 1, k0 = k1 - 1, par = ((k1 - fz) >> 1) & 1;
+      E *d1 = dz + par * pl, *d0 = dz + (par ^ 1) * pl;
+      int so[N];  // offsets of the N even planes around k1
 #pragma unroll
-          for (int t = -ko; t <= ko; t += 2) {
-            int sl = s1 + t;
-            sl += sl < 0 ? R : 0;
-            sl -= sl >= R ? R : 0;
-            v = racc(v, T(-Wav<N, NT>::K(t)), c[sl * pl]);
-          }
-          d1[idx] = v;
-          const int q = divq(idx, dR);
-          emit(r0 + idx - q * nR, r0 + q, k1, idx, v);
-        }
+      for (int x = 0; x < N; ++x) {
+        int sl = s1 + 2 * x - ko;
+        sl += sl < 0 ? R : 0;
+        sl -= sl >= R ? R : 0;
+        so[x] = sl * pl;
       }
-      __syncthreads();
-      const int k0 = k1 - 1;
-      if (k0 >= r0 && k0 <= r1) {
-        const int s0 = s1 == 0 ? R - 1 : s1 - 1;
-        for (int idx = threadIdx.x; idx < pl; idx += blockDim.x) {
-          const int q = divq(idx, dR);
-          const int i = r0 + idx - q * nR, j = r0 + q;
-          T v = T(0);
+      const DivM dw = divm(w);
+      for (int idx = tid; idx < pl; idx += bd) {
+        const int q = divq(idx, dw), i = c0 + idx - q * w, j = r0 + q;
+        const bool mine = i >= B.lo[0] && i <= B.hi[0] && j >= B.lo[1] && j <= B.hi[1];
+        const E *c = ring + idx;
+        E v1 = D::zero();
+        if (k1 <= z1) {
+          v1 = c[s1 * pl];
+#pragma unroll
+          for (int x = 0; x < N; ++x) v1 = D::acc(v1, -W::K(2 * x - ko), c[so[x]]);
+          v1 = D::norm(v1);
+          if (NT) d1[idx] = v1;
+          if (mine && k1 >= B.lo[2] && k1 <= B.hi[2]) emit(i, j, k1, v1);
+        } else if (NT) {
+          v1 = d1[idx];
+        }
+        if (k0 >= B.lo[2] && k0 <= B.hi[2] && mine) {
+          E v = D::zero();
           if ((i | j) & 1) {
-            v = ring[s0 * pl + idx];
-            if (NT) v = racc(v, U, d0[idx] + d1[idx]);
+            v = c[s0 * pl];
+            if constexpr (NT != 0) v = D::lift(v, d0[idx], v1);
           }
-          emit(i, j, k0, idx, v);
+          emit(i, j, k0, v);
         }
       }
     }
-    __syncthreads();
   }
 }
 
-// detail_planes in float pairs (about 48 significant bits) on the FP32 pipe:
-// the same lifting-form passes in the same order, each FP64 input split
-// once into a pair when its plane is staged in shared memory; gamma reaches
-// emit as a double.  |error| <= a few 2^-47 of the largest input, far inside
-// the 1e-12 tolerance of the block norms.  Index arithmetic in 32 bits with
-// multiply-high divisions (the planes are the kernel's whole work).
-template <int N, int NT, typename F>
-__device__ __forceinline__ void detail_planes_f2(const double *__restrict__ Pb, int nb, int Gi, F2 *sm, F emit) {
-  using W = Wav<N, NT>;
-  constexpr int ko = N - 1, R = 2 * ko + 1;
-  constexpr float U = NT ? 0.25f : 0.0f;  // lifting update weight
-  const int Wd = nb + 2 * Gi;
-  const int r0 = -W::ext_f, r1 = nb - 1 + W::ext_b, nR = r1 - r0 + 1, nA = nR + 2 * ko;
-  const int lo = -Gi, hi = nb - 1 + Gi;
-  const int nodd = par_count(r0, r1 + 1, 1), nev = nR - nodd;
-  const int fo = par_first(r0, 1), fe = par_first(r0, 0);
-  const int pl = nR * nR;
-  const DivM dA = divm(nA), dO = divm(nodd), dE = divm(nev), dR = divm(nR);
-  F2 *ring = sm;             // [R][nR][nR]
-  F2 *dz = sm + R * pl;      // [2][nR][nR]
-  F2 *A = dz + 2 * pl;       // [nA][nR]
-  F2 *S = A + nA * nR;       // [nA][nA] the staged plane (rows, columns r0-ko .. r1+ko)
-  auto gsum = [](const F2 *v, int stride) {
-    F2 s = v[0];
-#pragma unroll
-    for (int t = -ko; t <= ko; t += 2) s = f2_acc(s, -float(Wav<N, NT>::K(t)), v[t * stride]);
-    return f2_norm(s);
+// column tiles of the extended region: tile q of nt is [i0, i1], cut before an
+// odd column
+__host__ __device__ __forceinline__ void det_cut(int r0, int r1, int q, int nt, int *i0, int *i1) {
+  auto at = [&](int x) {
+    const int c = r0 + x * (r1 - r0 + 1) / nt;
+    return x == 0 ? r0 : x == nt ? r1 + 1 : c | 1;
   };
-  auto lift = [](F2 v, F2 a, F2 b) { return NT ? f2_norm(f2_acc(v, U, f2_add(a, b))) : v; };
-  // first column / row of the staged plane inside the stored padded range
-  const int c0 = r0 - ko;
-  for (int kk = r0 - ko; kk <= r1 + ko + 1; ++kk) {
-    const int slot = (kk - (r0 - ko)) % R;
-    const bool kin = kk >= lo && kk <= hi;
-    const double *pk = Pb + (size_t)(kk + Gi) * Wd * Wd;
-    // stage rows jj = r0-ko .. r1+ko of the plane, columns r0-ko .. r1+ko
-    for (int idx = threadIdx.x; idx < nA * nA; idx += blockDim.x) {
-      const int jr = divq(idx, dA), ir = idx - jr * dA.d;
-      const int jj = c0 + jr, ii = c0 + ir;
-      const bool in = kin && jj >= lo && jj <= hi;
-      S[idx] = in ? f2_split(pk[(jj + Gi) * Wd + (ii + Gi)]) : F2{0.f, 0.f};
+  *i0 = at(q), *i1 = at(q + 1) - 1;
+}
+
+// fewest tiles whose shared memory leaves room for two CTAs on an SM and whose
+// passes have at most DET_ITEMS items per thread (24^3 with 6.2 in float pairs:
+// 72 KB and 384 threads 2.64 ms, 110 KB and 512 threads 2.25 ms)
+template <int N, int NT>
+static int det_tiles(int nb, size_t es, size_t *bytes) {
+  const int r0 = -Wav<N, NT>::ext_f, r1 = nb - 1 + Wav<N, NT>::ext_b;
+  for (int nt = 1;; ++nt) {
+    int w = 0;
+    for (int q = 0; q < nt; ++q) {
+      int i0, i1;
+      det_cut(r0, r1, q, nt, &i0, &i1);
+      w = std::max(w, det_tile<NT>(i0, i1).w);
     }
-    __syncthreads();
-    // x pass: odd columns, then even columns
-    for (int idx = threadIdx.x; idx < nodd * nA; idx += blockDim.x) {
-      const int jr = divq(idx, dO), i = fo + 2 * (idx - jr * dO.d);
-      A[(i - r0) + nR * jr] = gsum(S + jr * nA + (i - r0 + ko), 1);
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < nev * nA; idx += blockDim.x) {
-      const int jr = divq(idx, dE), i = fe + 2 * (idx - jr * dE.d);
-      F2 *a = A + (i - r0) + nR * jr;
-      *a = lift(S[jr * nA + (i - r0 + ko)], a[-1], a[1]);
-    }
-    __syncthreads();
-    // y pass into ring plane kk: odd rows, then even rows
-    F2 *rp = ring + slot * pl;
-    for (int idx = threadIdx.x; idx < nR * nodd; idx += blockDim.x) {
-      const int q = divq(idx, dR), ii = idx - q * nR, j = fo + 2 * q;
-      rp[ii + nR * (j - r0)] = gsum(A + ii + nR * (j - (r0 - ko)), nR);
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < nR * nev; idx += blockDim.x) {
-      const int q = divq(idx, dR), ii = idx - q * nR, j = fe + 2 * q;
-      F2 *r = rp + ii + nR * (j - r0);
-      *r = lift(A[ii + nR * (j - (r0 - ko))], r[-nR], r[nR]);
-    }
-    __syncthreads();
-    // z: odd plane k1 = kk - ko, then the even plane k1 - 1
-    const int k1 = kk - ko;
-    if ((k1 & 1) && k1 >= r0 && k1 <= r1 + 1) {
-      const int s1 = (slot + ko + 1) % R;
-      F2 *d1 = dz + (((k1 - fo) >> 1) & 1) * pl, *d0 = dz + ((((k1 - fo) >> 1) + 1) & 1) * pl;
-      if (k1 <= r1) {
-        for (int idx = threadIdx.x; idx < pl; idx += blockDim.x) {
-          const F2 *c = ring + idx;
-          F2 v = c[s1 * pl];
-#pragma unroll
-          for (int t = -ko; t <= ko; t += 2) {
-            int sl = s1 + t;
-            sl += sl < 0 ? R : 0;
-            sl -= sl >= R ? R : 0;
-            v = f2_acc(v, -float(Wav<N, NT>::K(t)), c[sl * pl]);
-          }
-          v = f2_norm(v);
-          d1[idx] = v;
-          const int q = divq(idx, dR);
-          emit(r0 + idx - q * nR, r0 + q, k1, idx, f2_dbl(v));
-        }
-      }
-      __syncthreads();
-      const int k0 = k1 - 1;
-      if (k0 >= r0 && k0 <= r1) {
-        const int s0 = s1 == 0 ? R - 1 : s1 - 1;
-        for (int idx = threadIdx.x; idx < pl; idx += blockDim.x) {
-          const int q = divq(idx, dR);
-          const int i = r0 + idx - q * nR, j = r0 + q;
-          double v = 0.0;
-          if ((i | j) & 1) v = f2_dbl(lift(ring[s0 * pl + idx], d0[idx], d1[idx]));
-          emit(i, j, k0, idx, v);
-        }
-      }
-    }
-    __syncthreads();
+    const int nR = r1 - r0 + 1, items = std::max(w * nR, (w + 1) / 2 * (nR + 2 * (N - 1)));
+    *bytes = es * det_elems<N>(nR, w);
+    if (*bytes <= 110 * 1024 && items <= DET_ITEMS * DET_THREADS) return nt;
   }
 }
 
 // Per leaf: max |gamma| over the extended region (Sec. 2.3, the block norm
-// that drives refinement and coarsening).
+// that drives refinement and coarsening).  One CTA per column tile; the norms
+// start at zero and take the maximum of the tiles' integer keys.
 template <int N, int NT, bool PAIRS>
-__global__ void __launch_bounds__(1024) k_criterion(Tree t, const double *__restrict__ P, int Gi,
-                                                   double *__restrict__ maxdet) {
-  const int b = blockIdx.x, nb = t.nb, Wd = nb + 2 * Gi;
+__global__ void __launch_bounds__(1024) k_criterion(int nb, const double *__restrict__ P, int Gi,
+                                                  unsigned long long *__restrict__ maxdet, int ntile) {
+  using E = typename DetOps<double, PAIRS>::E;
+  const int b = blockIdx.x / ntile, Wd = nb + 2 * Gi;
   extern __shared__ double sm[];
   unsigned long long mx = 0;  // max |gamma| as an integer key (integer pipe)
-  auto emit = [&](int, int, int, int, double g) { mx = max(mx, abs_key(g)); };
-  if constexpr (PAIRS)
-    detail_planes_f2<N, NT>(P + (size_t)b * Wd * Wd * Wd, nb, Gi, reinterpret_cast<F2 *>(sm), emit);
-  else
-    detail_planes<N, NT>(P + (size_t)b * Wd * Wd * Wd, nb, Gi, sm, emit);
-  // block max
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  __shared__ unsigned long long red[32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    unsigned long long v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0ULL;
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (threadIdx.x == 0) maxdet[b] = __longlong_as_double((long long)v);
+  const int r0 = -Wav<N, NT>::ext_f, r1 = nb - 1 + Wav<N, NT>::ext_b;
+  DetBox B{{r0, r0, r0}, {r1, r1, r1}};
+  det_cut(r0, r1, blockIdx.x - b * ntile, ntile, &B.lo[0], &B.hi[0]);
+  const double *Pb = P + (size_t)b * Wd * Wd * Wd;
+  if constexpr (PAIRS) {
+    // the largest pair by its high part's bits (a NaN above all), then its low
+    // part; one conversion at the end
+    unsigned kh = 0;
+    float kl = 0.f;
+    detail_planes<N, NT, PAIRS, double>(Pb, nb, Gi, B, reinterpret_cast<E *>(sm), [&](int, int, int, F2 g) {
+      const unsigned h = __float_as_uint(g.h) & 0x7fffffffu;
+      const float l = g.h < 0.f ? -g.l : g.l;
+      if (h > kh || (h == kh && l > kl)) kh = h, kl = l;
+    });
+    mx = abs_key(f2_dbl({__uint_as_float(kh), kl}));
+  } else {
+    detail_planes<N, NT, PAIRS, double>(Pb, nb, Gi, B, reinterpret_cast<E *>(sm),
+                                        [&](int, int, int, double g) { mx = max(mx, abs_key(g)); });
   }
-}
-
-// plane ring, z-detail ring and x-pass plane of detail_planes (elements of es bytes)
-template <int N, int NT>
-static size_t crit_smem(int nb, size_t es = sizeof(double)) {
-  using W = Wav<N, NT>;
-  const int nR = nb + W::ext_f + W::ext_b, ko = N - 1;
-  return es * ((size_t)(2 * ko + 3) * nR * nR + (size_t)nR * (nR + 2 * ko));
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((threadIdx.x & 31) == 0 && mx) atomicMax(maxdet + b, mx);
 }
 
 // FP32 grids evaluate the details in float pairs (FP32 pipe), FP64 grids in
 // FP64 (the plain form)
 template <int N, int NT, bool PAIRS>
 static int criterion_launch(mr_grid *g, const double *P, int Gi, double *maxdet) {
-  using W = Wav<N, NT>;
-  const int nR = g->desc.nb + W::ext_f + W::ext_b, nA = nR + 2 * (N - 1);
-  const size_t sm = crit_smem<N, NT>(g->desc.nb) + (PAIRS ? sizeof(F2) * (size_t)nA * nA : 0);
-  if (sm > 227 * 1024) return MR_ERR_UNSUPPORTED;
-  if (check_cuda(cudaFuncSetAttribute(k_criterion<N, NT, PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sm),
-                 "criterion smem"))
+  const int nb = g->desc.nb, n = g->nleaf;
+  size_t sm;
+  const int nt = det_tiles<N, NT>(nb, sizeof(double), &sm);
+  // (block sizes stay those whose whole planes fit an SM: 32^3 with 6.2 in float
+  // pairs is refused)
+  const int nR = nb + Wav<N, NT>::ext_f + Wav<N, NT>::ext_b, nA = nR + 2 * (N - 1);
+  if (8 * ((size_t)(2 * N + 1) * nR * nR + (size_t)nR * nA + (PAIRS ? (size_t)nA * nA : 0)) > 227 * 1024)
+    return MR_ERR_UNSUPPORTED;
+  const auto kc = k_criterion<N, NT, PAIRS>;
+  if (check_cuda(cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), "criterion smem") ||
+      check_cuda(cudaMemsetAsync(maxdet, 0, sizeof(double) * (size_t)n, g->stream), "criterion norms"))
     return MR_ERR_CUDA;
-  Tree t = tree_view(g);
-  static const int cc[2] = {1024, 512};
-  const int th = tune_threads(g, TuneKey{2, N, NT, g->desc.nb, PAIRS ? 5 : 8, Gi, 0}, cc, 2, [&](int thr) {
-    k_criterion<N, NT, PAIRS><<<g->nleaf, thr, sm, g->stream>>>(t, P, Gi, maxdet);
+  unsigned long long *md = reinterpret_cast<unsigned long long *>(maxdet);
+  // FP64: issue is limited by its own pipe, more warps hide its latency
+  static const int cc[2] = {PAIRS ? DET_THREADS : 2 * DET_THREADS, PAIRS ? 2 * DET_THREADS : DET_THREADS};
+  const int th = tune_threads(g, TuneKey{2, N, NT, nb, PAIRS ? 5 : 8, Gi, 0}, cc, 2, [&](int thr) {
+    kc<<<n * nt, thr, sm, g->stream>>>(nb, P, Gi, md, nt);
   });
-  MR_LAUNCH(g, MRK_CRITERION, k_criterion<N, NT, PAIRS><<<g->nleaf, th, sm, g->stream>>>(t, P, Gi, maxdet));
+  MR_LAUNCH(g, MRK_CRITERION, kc<<<n * nt, th, sm, g->stream>>>(nb, P, Gi, md, nt));
   return check_cuda(cudaGetLastError(), "k_criterion") ? MR_ERR_CUDA : MR_OK;
 }
 
@@ -449,80 +485,99 @@ __global__ void k_emit(int n, int M, const int8_t *st, const int *pos, const int
 
 // ------------------------------------------------------ interpolation
 // New leaf values: copy, zero-detail refinement of the parent's padded block
-// (J^s / K^s), or tensor H^a coarsening of the 8 children's padded blocks,
-// in the padded blocks' precision TP.
-// Child ch of a refined parent (Sec. 2.2.3, zero-detail refinement with
-// J^s / K^s of the parent's padded block Pp): the points of the child whose
-// local indices have parities (PX, PY, PZ).
-template <int N, int NT, bool PX, bool PY, bool PZ, typename TP, typename TO, typename PI>
-__device__ __forceinline__ void interp_class(const TP *Pp, int ch, int nb, PI pidx, TO *out) {
-  const int h = nb / 2, cnt = h * h * h;
-  for (int p = threadIdx.x; p < cnt; p += blockDim.x) {
-    const int r = p / h;
-    const int i = 2 * (p - r * h) + PX, j = 2 * (r % h) + PY, k = 2 * (r / h) + PZ;
-    const int f[3] = {(ch & 1) * nb + i, ((ch >> 1) & 1) * nb + j, ((ch >> 2) & 1) * nb + k};
-    const TP acc = refine_sum<N, NT, PX, PY, PZ, TP>([&](int ox, int oy, int oz) {
-      return Pp[pidx((f[0] + ox) / 2, (f[1] + oy) / 2, (f[2] + oz) / 2)];
-    });
-    out[i + nb * (j + nb * k)] = TO(acc);
-  }
+// (J^s / K^s), or tensor H^a coarsening of the 8 children's padded blocks, in
+// the padded blocks' precision TP.  Both sums are separable and run along
+// lines (wavelet_runs.cuh): 3 x 6 taps per child point at most instead of up
+// to 216 (43 on average with 6.x), 3 x 9 per parent point instead of 729.
+// Bound by shared-memory and issue slots; remeshing about 6 000 leaves of 24^3
+// with 6.2 and four fields spent 36 ms here with tensor sums per point, 4.3 ms now.
+
+// z-planes of a child per step, and the shared memory of its two passes
+constexpr int INTERP_Z = 8;
+static size_t interp_smem(int N, int nb, size_t es) {
+  const size_t m = nb / 2 + N - 1;
+  return es * INTERP_Z * (m * (m | 1) + (size_t)nb * (m | 1));
 }
 
 template <typename TO, typename TP, int N, int NT>
-__global__ void __launch_bounds__(512) k_interp(Tree to, const int *__restrict__ src,
-                                                const TP *__restrict__ P, int Gi,
+__global__ void __launch_bounds__(256) k_interp(int nb, const int *__restrict__ src, const TP *__restrict__ P, int Gi,
                                                 const TO *__restrict__ fold, TO *__restrict__ fnew) {
-  using W = Wav<N, NT>;
-  const int q = blockIdx.x, nb = to.nb, Wd = nb + 2 * Gi;
-  const size_t nb3 = (size_t)nb * nb * nb, np = (size_t)Wd * Wd * Wd;
+  using RS = RefSum<TP, TP>;
+  constexpr int h = N / 2;
+  const int q = blockIdx.x, Wd = nb + 2 * Gi, W2 = Wd * Wd, hb = nb / 2, tid = threadIdx.x, bd = blockDim.x;
+  const size_t nb3 = (size_t)nb * nb * nb, np = (size_t)Wd * W2;
   const int kind = src[2 * q], s = src[2 * q + 1];
   TO *out = fnew + (size_t)q * nb3;
-  auto pidx = [&](int i, int j, int k) {
-    return (size_t)(i + Gi) + Wd * ((size_t)(j + Gi) + (size_t)Wd * (k + Gi));
-  };
   if (kind == KIND_COPY) {
-    for (int p = threadIdx.x; p < (int)nb3; p += blockDim.x) out[p] = fold[(size_t)s * nb3 + p];
-  } else if (kind == KIND_CHILD) {
-    const int par = s >> 3, ch = s & 7;
-    const TP *Pp = P + (size_t)par * np;
-    // one parity class of the child's points at a time (the parity of the
-    // parent-grid index equals the child's, nb being even), so that every
-    // lane of a warp evaluates the same refinement sum
-    interp_class<N, NT, false, false, false>(Pp, ch, nb, pidx, out);
-    interp_class<N, NT, true, false, false>(Pp, ch, nb, pidx, out);
-    interp_class<N, NT, false, true, false>(Pp, ch, nb, pidx, out);
-    interp_class<N, NT, true, true, false>(Pp, ch, nb, pidx, out);
-    interp_class<N, NT, false, false, true>(Pp, ch, nb, pidx, out);
-    interp_class<N, NT, true, false, true>(Pp, ch, nb, pidx, out);
-    interp_class<N, NT, false, true, true>(Pp, ch, nb, pidx, out);
-    interp_class<N, NT, true, true, true>(Pp, ch, nb, pidx, out);
-  } else {
-    // children of the new parent in the old tree (level L = parent level + 1)
-    __shared__ int chs[8];
-    const int L = __ldg(to.lev + s);
-    if (threadIdx.x < 8) {
-      const int c = threadIdx.x;
-      int a[3];
-      for (int d = 0; d < 3; ++d) a[d] = __ldg(to.anc + 3 * s + d) + ((c >> d) & 1);
-      chs[c] = owner(to, L, a[0] * nb, a[1] * nb, a[2] * nb, s);
+    const float4 *f4 = reinterpret_cast<const float4 *>(fold + (size_t)s * nb3);  // nb^3 is a multiple of 8
+    float4 *o4 = reinterpret_cast<float4 *>(out);
+    const int n4 = (int)(nb3 * sizeof(TO) / 16);
+#pragma unroll 4
+    for (int p = tid; p < n4; p += bd) o4[p] = __ldg(f4 + p);
+    return;
+  }
+  if (kind != KIND_CHILD) return;  // parents: k_interp_parent
+  const int ch = s & 7;
+  const int cx = (ch & 1) * hb, cy = ((ch >> 1) & 1) * hb, cz = (ch >> 2) * hb;  // child's first coarse point
+  const TP *Pp = P + (size_t)(s >> 3) * np + Gi * (1 + Wd + (size_t)W2);
+  extern __shared__ double smi[];
+  const int m = hb + N - 1, mp = m | 1;        // coarse points per axis the child reads; pitch
+  TP *U1 = reinterpret_cast<TP *>(smi);        // [z][m][mp]: refined along z
+  TP *U2 = U1 + INTERP_Z * m * mp;             // [z][nb][mp]: and along y
+  const DivM dm = divm(m), dh = divm(hb), dnb = divm(nb);
+  const int nseg = (nb + 15) >> 4;
+  const DivM dl = divm(INTERP_Z * m);
+  for (int z0 = 0; z0 < nb; z0 += INTERP_Z) {
+    const int nz = min(INTERP_Z, nb - z0);
+    for (int idx = tid; idx < m * m; idx += bd) {
+      const int jy = divq(idx, dm), jx = idx - jy * m;
+      TP *d = U1 + jx + mp * jy;
+      refine_run<N, NT, RS>(Pp + (cx - h + 1 + jx) + Wd * (cy - h + 1 + jy), W2, 2 * cz + z0, nz,
+                            [&](int z, TP v) { d[z * m * mp] = v; });
     }
     __syncthreads();
-    for (int p = threadIdx.x; p < (int)nb3; p += blockDim.x) {
-      const int i = p % nb, j = (p / nb) % nb, k = p / (nb * nb);
-      const int f[3] = {2 * i, 2 * j, 2 * k};
-      int ch = 0, loc[3];
-      for (int d = 0; d < 3; ++d) {
-        const int cd = f[d] >= nb;
-        ch |= cd << d;
-        loc[d] = f[d] - cd * nb;
-      }
-      const TP *Pc = P + (size_t)chs[ch] * np;
-      const TP acc = coarsen_sum<N, NT, TP>([&](int tx, int ty, int tz) {
-        return Pc[pidx(loc[0] + tx, loc[1] + ty, loc[2] + tz)];
-      });
-      out[p] = TO(acc);
+    for (int idx = tid; idx < INTERP_Z * m * nseg; idx += bd) {
+      const int sg = divq(idx, dl), l = idx - sg * INTERP_Z * m, z = divq(l, dm), jx = l - z * m;
+      if (z >= nz) continue;
+      // (U1's row jy holds coarse point cy - h + 1 + jy)
+      const TP *r = U1 + z * m * mp + jx - (ptrdiff_t)(cy - h + 1) * mp;
+      TP *d = U2 + z * nb * mp + 16 * sg * mp + jx;
+      refine_run<N, NT, RS>(r, mp, 2 * cy + 16 * sg, min(16, nb - 16 * sg), [&](int y, TP v) { d[y * mp] = v; });
     }
+    __syncthreads();
+    // along x: one thread per (even, odd) pair, neighbouring threads write
+    // neighbouring points
+    for (int idx = tid; idx < nz * nb * hb; idx += bd) {
+      const int r = divq(idx, dh), px = idx - r * hb;  // r = y + nb z
+      const TP *w = U2 + r * mp + px;
+      TP v = TP(0);
+#pragma unroll
+      for (int x = 0; x < N; ++x) v = racc(v, TP(Wav<N, NT>::K(2 * x - (N - 1))), w[x]);
+      TO *o = out + (size_t)(z0 * nb + r) * nb + 2 * px;
+      o[0] = TO(w[h - 1]);
+      o[1] = TO(v);
+    }
+    __syncthreads();
   }
+}
+
+// One CTA per octant of a new parent: the child leaf's block coarsened.
+template <typename TO, typename TP, int N, int NT>
+__global__ void __launch_bounds__(256) k_interp_parent(Tree to, const int *__restrict__ src, const TP *__restrict__ P,
+                                                       int Gi, TO *__restrict__ fnew, int cap) {
+  const int q = blockIdx.x >> 3, c = blockIdx.x & 7, nb = to.nb, Wd = nb + 2 * Gi, hb = nb / 2;
+  if (src[2 * q] != KIND_PARENT) return;
+  // s: the new parent's first child in the old tree (level L = parent level + 1)
+  const int s = src[2 * q + 1], L = __ldg(to.lev + s);
+  int a[3];
+  for (int d = 0; d < 3; ++d) a[d] = (__ldg(to.anc + 3 * s + d) + ((c >> d) & 1)) * nb;
+  const int o = owner(to, L, a[0], a[1], a[2], s);
+  TO *out = fnew + (size_t)q * nb * nb * nb + hb * ((c & 1) + nb * (((c >> 1) & 1) + (size_t)nb * (c >> 2)));
+  extern __shared__ double smi[];
+  const int lo[3] = {0, 0, 0}, hi[3] = {hb, hb, hb};
+  coarsen_box<N, NT, TP>(P + (size_t)o * Wd * Wd * Wd + Gi * (1 + Wd + (size_t)Wd * Wd), Wd, lo, hi,
+                         reinterpret_cast<TP *>(smi), cap,
+                         [&](int x, int y, int z, TP v) { out[x + nb * (y + nb * z)] = TO(v); });
 }
 
 // ------------------------------------------------------------- update
@@ -548,26 +603,43 @@ __global__ void k_newmask(Tree tn, const int *src, int *nmask) {
   nmask[q] = mask;
 }
 
-// gamma over the extended region of every unchanged leaf F for the details
-// the coarsening discarded (in newly coarsened leaves, or in the new bands of
-// F or of its unchanged same-level neighbours), 0 elsewhere in the region.  Q
-// is indexed by F's old slot in the padded layout.  The 27 block-sized regions
-// around F are classified once: a newly coarsened leaf one level coarser owns
-// all of D in its region, an unchanged same-level leaf with newly coarsened
-// neighbours owns the part of its band next to them, finer leaves none.
+// A leaf's box of discarded details, packed: per axis the first and last pair of
+// points of the extended region (5 bits each; 43 points at most), bit 30 set.
+__device__ __forceinline__ int box_pack(const int *lo, const int *hi, int r0) {
+  int p = 1 << 30;
+  for (int d = 0; d < 3; ++d) p |= ((lo[d] - r0) >> 1) << (10 * d) | ((hi[d] - r0) >> 1) << (10 * d + 5);
+  return p;
+}
+__device__ __forceinline__ DetBox box_unpack(int p, int r0, int r1) {
+  DetBox B;
+  for (int d = 0; d < 3; ++d)
+    B.lo[d] = r0 + 2 * ((p >> (10 * d)) & 31), B.hi[d] = min(r0 + 2 * ((p >> (10 * d + 5)) & 31) + 1, r1);
+  return B;
+}
+
+// gamma for the details the coarsening discarded (in newly coarsened leaves, or
+// in the new bands of F or of its unchanged same-level neighbours) of every
+// unchanged leaf F, over the box of the extended region that holds them; 0 at
+// the box's other points.  Q is indexed by F's old slot in the padded layout.
+// The 27 block-sized regions around F are classified once: a newly coarsened
+// leaf one level coarser owns all of D in its region, an unchanged same-level
+// leaf with newly coarsened neighbours owns the part of its band next to them,
+// finer leaves none.  Most leaves discard next to one face, so the box is a
+// third of the region or less (the two update kernels together: 40.4 ms over
+// the whole region, 12.3 ms over the boxes, in that remeshing); the box goes to
+// hasD (0: nothing discarded).
 template <typename TP, int N, int NT>
-__global__ void __launch_bounds__(1024) k_update_gamma(Tree tn, const int *__restrict__ src,
-                                                      const int *__restrict__ nmask,
-                                                      const TP *__restrict__ P, int Gi,
-                                                      TP *__restrict__ Q, int *hasD) {
+__global__ void __launch_bounds__(DET_THREADS, sizeof(TP) == 4 ? 3 : 2) k_update_gamma(
+    Tree tn, const int *__restrict__ src, const int *__restrict__ nmask, const TP *__restrict__ P, int Gi,
+    TP *__restrict__ Q, int *hasD, int cap) {
   using W = Wav<N, NT>;
   const int q = blockIdx.x;
   if (src[2 * q] != KIND_COPY) return;
   const int s = src[2 * q + 1], L = __ldg(tn.lev + q), nb = tn.nb, Wd = nb + 2 * Gi;
-  const int ef = W::ext_f, eb = W::ext_b;
+  const int ef = W::ext_f, eb = W::ext_b, r0 = -ef, r1 = nb - 1 + eb;
   const size_t np = (size_t)Wd * Wd * Wd;
-  __shared__ int rD[27], any;
-  if (threadIdx.x == 0) any = 0;
+  __shared__ int rD[27], blo[3], bhi[3];
+  if (threadIdx.x < 3) blo[threadIdx.x] = 1 << 20, bhi[threadIdx.x] = -(1 << 20);
   __syncthreads();
   if (threadIdx.x < 27) {
     const int r = threadIdx.x;
@@ -582,104 +654,137 @@ __global__ void __launch_bounds__(1024) k_update_gamma(Tree tn, const int *__res
       else if (Lo == L && ko == KIND_COPY) v = nmask[o];
     }
     rD[r] = v;
-    if (v) atomicOr(&any, 1);
+    // box of D in this region: all of it, or the band next to each new neighbour m
+    for (int m = v == -1 ? 13 : 0; v && m < (v == -1 ? 14 : 27); ++m) {
+      if (v > 0 && !((v >> m) & 1)) continue;
+      const int md[3] = {m % 3 - 1, (m / 3) % 3 - 1, m / 9 - 1};
+      int lo[3], hi[3];
+      bool some = true;
+      for (int d = 0; d < 3; ++d) {
+        lo[d] = max(dd[d] * nb + (md[d] > 0 ? nb - ef : 0), r0);
+        hi[d] = min(dd[d] * nb + (md[d] < 0 ? eb : nb) - 1, r1);
+        some &= lo[d] <= hi[d];
+      }
+      if (some)
+        for (int d = 0; d < 3; ++d) atomicMin(&blo[d], lo[d]), atomicMax(&bhi[d], hi[d]);
+    }
   }
   __syncthreads();
-  if (!any) {
+  if (blo[0] > bhi[0]) {
     if (threadIdx.x == 0) hasD[q] = 0;
     return;
   }
+  const int packed = box_pack(blo, bhi, r0);
+  if (threadIdx.x == 0) hasD[q] = packed;
   TP *Qb = Q + (size_t)s * np;
   extern __shared__ double smd[];
-  TP *sm = reinterpret_cast<TP *>(smd);
-  detail_planes<N, NT, TP>(P + (size_t)s * np, nb, Gi, sm, [&](int i, int j, int k, int, TP g) {
-    if ((i | j | k) & 1) {
-      const int r = region_of(i, j, k, nb), v = rD[r];
-      bool inD = v == -1;
-      if (v > 0) {
-        const int dd[3] = {r % 3 - 1, (r / 3) % 3 - 1, r / 9 - 1};
-        inD = in_band_dev(v, i - dd[0] * nb, j - dd[1] * nb, k - dd[2] * nb, nb, ef, eb);
+  const DetBox B = box_unpack(packed, r0, r1);
+  // column tiles whose passes fit in shared memory and the threads' items
+  const int nR = det_tile<NT>(B.lo[1], B.hi[1]).w;
+  int wm = min(DET_ITEMS * DET_THREADS / nR, 2 * DET_ITEMS * DET_THREADS / (nR + 2 * (N - 1)) - 1);
+  while ((int)det_elems<N>(nR, wm) > cap) --wm;
+  const int step = max((wm - 1) & ~1, 2);  // (even: tiles start at the box's parity; one column more is computed)
+  for (int c = B.lo[0]; c <= B.hi[0]; c += step) {
+    DetBox T = B;
+    T.lo[0] = c, T.hi[0] = min(c + step - 1, B.hi[0]);
+    if (c != B.lo[0]) __syncthreads();
+    detail_planes<N, NT, false, TP>(P + (size_t)s * np, nb, Gi, T, reinterpret_cast<TP *>(smd),
+                                    [&](int i, int j, int k, TP g) {
+      if ((i | j | k) & 1) {
+        const int r = region_of(i, j, k, nb), v = rD[r];
+        bool inD = v == -1;
+        if (v > 0) {
+          const int dd[3] = {r % 3 - 1, (r / 3) % 3 - 1, r / 9 - 1};
+          inD = in_band_dev(v, i - dd[0] * nb, j - dd[1] * nb, k - dd[2] * nb, nb, ef, eb);
+        }
+        if (!inD) g = TP(0);
       }
-      if (!inD) g = TP(0);
-    }
-    Qb[(size_t)(i + Gi) + Wd * ((size_t)(j + Gi) + (size_t)Wd * (k + Gi))] = g;
-  });
-  if (threadIdx.x == 0) hasD[q] = 1;
+      Qb[(size_t)(i + Gi) + Wd * ((size_t)(j + Gi) + (size_t)Wd * (k + Gi))] = g;
+    });
+  }
 }
 
 // Subtract the synthesis of the discarded details (the J^s / K^s tensor taps
-// of the zero-detail refinement's complement) from the unchanged leaf:
-// separable, x then y then z, with the y-pass planes in a ring of
-// 2*hw(K^s)+1 shared-memory planes.  gamma is zero outside the extended region.
+// of the zero-detail refinement's complement) from the unchanged leaf, over the
+// points within reach of its box of details: separable, x then y then z, with
+// the y-pass planes in a ring of 2*hw(K^s)+1 shared-memory planes.  gamma is
+// zero outside the box.
 template <typename TO, typename TP, int N, int NT>
-__global__ void __launch_bounds__(256) k_update_apply(Tree tn, const int *__restrict__ src,
+__global__ void __launch_bounds__(256) k_update_apply(int nb, const int *__restrict__ src,
                                                       const int *__restrict__ hasD,
                                                       const TP *__restrict__ Q, int Gi,
                                                       TO *__restrict__ fnew) {
   using W = Wav<N, NT>;
   constexpr int hk = W::hwK, R = 2 * hk + 1;
-  const int q = blockIdx.x;
+  const int q = blockIdx.x, tid = threadIdx.x, bd = blockDim.x;
   if (src[2 * q] != KIND_COPY || !hasD[q]) return;
-  const int s = src[2 * q + 1], nb = tn.nb, Wd = nb + 2 * Gi;
-  const int r0 = -W::ext_f, r1 = nb - 1 + W::ext_b, nR = r1 - r0 + 1;
+  const int s = src[2 * q + 1], Wd = nb + 2 * Gi;
+  const DetBox B = box_unpack(hasD[q], -W::ext_f, nb - 1 + W::ext_b);
+  int o0[3], on[3];  // output points
+  for (int d = 0; d < 3; ++d) {
+    o0[d] = max(B.lo[d] - hk, 0);
+    on[d] = min(B.hi[d] + hk, nb - 1) - o0[d] + 1;
+  }
+  if (on[0] <= 0 || on[1] <= 0 || on[2] <= 0) return;
+  const int bx0 = B.lo[0], bx1 = B.hi[0], by0 = B.lo[1], by1 = B.hi[1], bz0 = B.lo[2], bz1 = B.hi[2];
+  const int nx = on[0], pl = nx * on[1], ny = by1 - by0 + 1;
   const TP *Qb = Q + (size_t)s * Wd * Wd * Wd;
   TO *v = fnew + (size_t)q * nb * nb * nb;
   extern __shared__ double smd[];
-  TP *ring = reinterpret_cast<TP *>(smd);   // [R][nb][nb]
-  TP *X = ring + (size_t)R * nb * nb;       // [nR][nb]: x pass of one plane
-  auto qidx = [&](int i, int j, int k) {
-    return (size_t)(i + Gi) + Wd * ((size_t)(j + Gi) + (size_t)Wd * (k + Gi));
-  };
-  for (int kk = r0; kk <= nb - 1 + hk; ++kk) {
-    const int slot = (kk - r0) % R;
-    if (kk <= r1) {
+  TP *ring = reinterpret_cast<TP *>(smd);  // [R][on1][nx]
+  TP *X = ring + (size_t)R * pl;           // [ny][nx]: x pass of one plane
+  const int xo = par_first(o0[0], 1), xe = par_first(o0[0], 0), nxo = par_count(o0[0], o0[0] + nx, 1), nxe = nx - nxo;
+  const DivM dxo = divm(max(nxo, 1)), dxe = divm(max(nxe, 1)), dx = divm(nx);
+  int slot = 0;
+  for (int kk = bz0; kk <= min(bz1 + hk, nb - 1) + hk; ++kk, slot = slot + 1 == R ? 0 : slot + 1) {
+    if (kk <= bz1) {
       // odd columns (K^s) first, then even ones (J^s): one filter per warp
-      const int hn = nb / 2;
-      for (int idx = threadIdx.x; idx < nb * nR; idx += blockDim.x) {
-        const bool od = idx < hn * nR;
-        const int q = od ? idx : idx - hn * nR;
-        const int i = 2 * (q % hn) + od, jj = r0 + q / hn;
-        const TP *p = Qb + qidx(i, jj, kk);
-        auto at = [&](int t) { return (i + t >= r0 && i + t <= r1) ? p[t] : TP(0); };
+      for (int idx = tid; idx < nx * ny; idx += bd) {
+        const bool od = idx < nxo * ny;
+        const int p0 = od ? idx : idx - nxo * ny, r = divq(p0, od ? dxo : dxe);
+        const int i = (od ? xo : xe) + 2 * (p0 - r * (od ? nxo : nxe)), jj = by0 + r;
+        const TP *p = Qb + (i + Gi) + Wd * ((jj + Gi) + (size_t)Wd * (kk + Gi));
+        auto at = [&](int t) { return (i + t >= bx0 && i + t <= bx1) ? p[t] : TP(0); };
         TP a = TP(0);
         if (od)
           for_taps<N, NT, FK_K>([&](int t, double w) { a = racc(a, TP(w), at(t)); });
         else
           for_taps<N, NT, FK_J>([&](int t, double w) { a = racc(a, TP(w), at(t)); });
-        X[i + nb * (jj - r0)] = a;
+        X[i - o0[0] + nx * r] = a;
       }
       __syncthreads();
-      for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
-        const int i = idx % nb, j = idx / nb;
-        auto at = [&](int t) { return (j + t >= r0 && j + t <= r1) ? X[i + nb * (j + t - r0)] : TP(0); };
+      for (int idx = tid; idx < pl; idx += bd) {
+        const int r = divq(idx, dx), x = idx - r * nx, j = o0[1] + r;
+        auto at = [&](int t) { return (j + t >= by0 && j + t <= by1) ? X[x + nx * (j + t - by0)] : TP(0); };
         TP a = TP(0);
         if (j & 1)
           for_taps<N, NT, FK_K>([&](int t, double w) { a = racc(a, TP(w), at(t)); });
         else
           for_taps<N, NT, FK_J>([&](int t, double w) { a = racc(a, TP(w), at(t)); });
-        ring[(size_t)slot * nb * nb + idx] = a;
+        ring[slot * pl + idx] = a;
       }
     }
     __syncthreads();
     // output plane k = kk - hk: its taps k+t with t in [-hk, hk] are planes
-    // kk-2hk .. kk, all in the ring (planes outside [r0, r1] read as 0)
+    // kk-2hk .. kk, all in the ring (planes outside the box read as 0)
     const int k = kk - hk;
-    if (k >= 0) {
-      const int sk = (slot + hk + 1) % R;
-      for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
+    if (k >= 0 && k < nb) {
+      const int sk = slot + hk + 1 >= R ? slot + hk + 1 - R : slot + hk + 1;
+      for (int idx = tid; idx < pl; idx += bd) {
         auto at = [&](int t) {
-          if (k + t < r0 || k + t > r1) return TP(0);
+          if (k + t < bz0 || k + t > bz1) return TP(0);
           int sl = sk + t;
           sl += sl < 0 ? R : 0;
           sl -= sl >= R ? R : 0;
-          return ring[(size_t)sl * nb * nb + idx];
+          return ring[sl * pl + idx];
         };
         TP a = TP(0);
         if (k & 1)
           for_taps<N, NT, FK_K>([&](int t, double w) { a = racc(a, TP(w), at(t)); });
         else
           for_taps<N, NT, FK_J>([&](int t, double w) { a = racc(a, TP(w), at(t)); });
-        const size_t p = idx + (size_t)nb * nb * k;
+        const int r = divq(idx, dx);
+        const size_t p = (size_t)(o0[0] + idx - r * nx) + nb * (o0[1] + r + (size_t)nb * k);
         if (a != TP(0)) v[p] = TO(Cvt<TP>::f(v[p]) - a);
       }
     }
@@ -771,15 +876,26 @@ static int interp_update(mr_grid *g, const Tree &to, const Tree &tn, const TP *P
   const int *src = g->newsrc;
   TP *Q = reinterpret_cast<TP *>(g->padQ64);
   const int tp = sizeof(TP) == 4 ? 4 : sizeof(TO) == 4 ? 5 : 8;
-  static const int ci[3] = {256, 128, 512};
-  const int thi = tune_threads(g, TuneKey{4, N, NT, g->desc.nb, tp, Gi, 0}, ci, 3, [&](int th) {
-    k_interp<TO, TP, N, NT><<<tn.nleaf, th, 0, g->stream>>>(to, src, P, Gi, (const TO *)field_ptr(g, fid),
-                                                            (TO *)next_field_ptr(g, fid));
+  const int nb = g->desc.nb;
+  const size_t smi = interp_smem(N, nb, sizeof(TP));
+  const int hH = Wav<N, NT>::hwH, fw = nb - 1 + 2 * hH;  // fine extent of a child's sums
+  const size_t smp = sizeof(TP) * 4 * (size_t)fw * (fw + nb / 2);
+  const auto ki = k_interp<TO, TP, N, NT>;
+  const auto kp = k_interp_parent<TO, TP, N, NT>;
+  if (check_cuda(cudaFuncSetAttribute(ki, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smi), "interp smem") ||
+      check_cuda(cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smp), "interp smem"))
+    return MR_ERR_CUDA;
+  const TO *fo = (const TO *)field_ptr(g, fid);
+  TO *fn = (TO *)next_field_ptr(g, fid);
+  static const int ci[2] = {256, 128};
+  const int thi = tune_threads(g, TuneKey{4, N, NT, nb, tp, Gi, 0}, ci, 2, [&](int th) {
+    ki<<<tn.nleaf, th, smi, g->stream>>>(nb, src, P, Gi, fo, fn);
   });
-  MR_LAUNCH(g, MRK_INTERP, k_interp<TO, TP, N, NT><<<tn.nleaf, thi, 0, g->stream>>>(
-                               to, src, P, Gi, (const TO *)field_ptr(g, fid), (TO *)next_field_ptr(g, fid)));
-  const size_t smg = crit_smem<N, NT>(g->desc.nb, sizeof(TP)), sma = apply_smem<N, NT>(g->desc.nb, sizeof(TP));
-  if (smg > 227 * 1024 || sma > 227 * 1024) return MR_ERR_UNSUPPORTED;
+  MR_LAUNCH(g, MRK_INTERP, ki<<<tn.nleaf, thi, smi, g->stream>>>(nb, src, P, Gi, fo, fn));
+  MR_LAUNCH(g, MRK_INTERP, kp<<<8 * tn.nleaf, 256, smp, g->stream>>>(to, src, P, Gi, fn, (int)(smp / sizeof(TP))));
+  const size_t smg = sizeof(TP) == 4 ? 72 * 1024 : 110 * 1024;  // three / two CTAs of 512 threads per SM
+  const size_t sma = apply_smem<N, NT>(nb, sizeof(TP));
+  if (sma > 227 * 1024) return MR_ERR_UNSUPPORTED;
   if (check_cuda(cudaFuncSetAttribute(k_update_gamma<TP, N, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)smg),
                  "update smem") ||
@@ -787,10 +903,10 @@ static int interp_update(mr_grid *g, const Tree &to, const Tree &tn, const TP *P
                                       (int)sma),
                  "update smem"))
     return MR_ERR_CUDA;
-  MR_LAUNCH(g, MRK_UPDATE, k_update_gamma<TP, N, NT><<<tn.nleaf, 1024, smg, g->stream>>>(tn, src, nmask, P, Gi,
-                                                                                       Q, hasD));
+  MR_LAUNCH(g, MRK_UPDATE, k_update_gamma<TP, N, NT><<<tn.nleaf, DET_THREADS, smg, g->stream>>>(
+                               tn, src, nmask, P, Gi, Q, hasD, (int)(smg / sizeof(TP))));
   MR_LAUNCH(g, MRK_UPDATE, k_update_apply<TO, TP, N, NT><<<tn.nleaf, 256, sma, g->stream>>>(
-                               tn, src, hasD, Q, Gi, (TO *)next_field_ptr(g, fid)));
+                               nb, src, hasD, Q, Gi, fn));
   return check_cuda(cudaGetLastError(), "interp/update") ? MR_ERR_CUDA : MR_OK;
 }
 

@@ -142,13 +142,14 @@ __device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
 // significant bits, l = the remainder truncated to 24 bits, so
 // |x - (h + l)| <= 2^-47 |x| + 2^-126 (values below the FP32 normal range
 // lose their remainder: an absolute error far below every tolerance here);
-// |x| >= 2^128, infinities and NaN go through the hardware conversion.
+// |x| >= 2^128 becomes an infinity, NaN stays NaN.
 __device__ __forceinline__ F2 f2_split(double x) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
   const unsigned hw = (unsigned)(u >> 32), sgn = hw & 0x80000000u;
   const int e = (int)((hw >> 20) & 0x7ffu) - 896;  // FP32 biased exponent
   if (e <= 0) return {__uint_as_float(sgn), 0.f};
-  if (e >= 255) return {(float)x, 0.f};
+  if (e >= 255)
+    return {__uint_as_float(sgn | (e == 1151 && ((hw << 12) | (unsigned)u) ? 0x7fc00000u : 0x7f800000u)), 0.f};
   const unsigned long long m = u & 0xfffffffffffffULL;  // 52 mantissa bits
   const unsigned hi = sgn | ((unsigned)e << 23) | (unsigned)(m >> 29);
   const unsigned r = (unsigned)(m & 0x1fffffffu);  // the 29 bits below: r * 2^(e - 179)
