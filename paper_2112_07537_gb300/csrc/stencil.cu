@@ -207,15 +207,18 @@ __global__ void k_field_set(Tree t, T *f, int kind, InitParams ip) {
   }
   for (int p = threadIdx.x; p < nb * nb * nb; p += blockDim.x) {
     const int rr = divq(p, t.dnb), k = divq(rr, t.dnb), i = p - rr * nb, j = rr - k * nb;
-    const double x[3] = {(a[0] * nb + i) * h, (a[1] * nb + j) * h, (a[2] * nb + k) * h};
     const double r2 = radial ? sq[0][i] + sq[1][j] + sq[2][k] : 0.0;
+    double x[3] = {0.0, 0.0, 0.0};
+    if (!radial) x[0] = (a[0] * nb + i) * h, x[1] = (a[1] * nb + j) * h, x[2] = (a[2] * nb + k) * h;
     double v = 0.0;
     if (kind == MR_INIT_GAUSSIAN) {
       v = ip.p[4] * exp(-r2 / (ip.p[3] * ip.p[3]));
     } else if (kind == MR_INIT_TANH_SPHERE) {
-      // tanh(x) rounds to +-1 from |x| = 19.1 on
+      // (1 - tanh y) / 2 = 1 / (1 + exp 2y): one exponential and one division,
+      // and no cancellation where tanh y nears 1; 0 and 1 from |y| = 19.07 on,
+      // where tanh y rounds to +-1 (the FP64 pipe bounds this kernel)
       const double y = (sqrt(r2) - ip.p[3]) / ip.p[4];
-      v = y > 22.0 ? 0.0 : y < -22.0 ? 1.0 : 0.5 * (1.0 - tanh(y));
+      v = y > 19.07 ? 0.0 : y < -19.07 ? 1.0 : 1.0 / (1.0 + exp(2.0 * y));
     } else if (kind == MR_INIT_GAUSSIAN_SUM || kind == MR_INIT_GAUSSIAN_SUM_ADD) {
       const int ng = (int)ip.p[0];
       for (int q = 0; q < ng; ++q) {
