@@ -24,7 +24,7 @@
 #include <algorithm>
 #include <cstdio>
 
-#include "mr_internal.cuh"
+#include "wavelet_runs.cuh"
 
 namespace mr {
 
@@ -181,9 +181,11 @@ __device__ TP refine_point(const Tree &t, const TI *phi, int L, int gx, int gy, 
 }
 
 // ---------------------------------------------------------------------------
-// The pre-pass of a leaf next to coarser ones: zero-detail refinement of the
-// coarser leaves' regions of its padded block (Part 1), substitution of the
-// band next to them, and Part 2 pushed to the coarser neighbours.
+// The padded block of a leaf: the gather, and next to coarser leaves the
+// zero-detail refinement of their regions (Part 1), the substitution of the band
+// next to them, and Part 2 pushed to the coarser neighbours.  A block is read
+// and written by its own CTA only, so the copy-bound gather of some leaves
+// overlaps the latency-bound phases of others.
 //
 // Coarser neighbours by parent: a leaf's coarser neighbours touch its parent
 // from outside, so they lie in the (up to) seven directions e = 1..7 of the
@@ -215,35 +217,34 @@ struct PrepTab {
 struct Boxes {
   int n, lo[7][3], hi[7][3];
 };
+// (by one warp, a lane per direction; faces first, then edges, then the corner)
 __device__ __forceinline__ void outward_boxes(Boxes &B, int ce, const int *s, int n, int dlo, int dhi) {
-  const int order[7] = {1, 2, 4, 3, 5, 6, 7};
-  int cnt = 0, kept = 0;
-  for (int q = 0; q < 7; ++q) {
-    const int e = order[q];
-    if (!((ce >> e) & 1)) continue;
-    bool inside = false;
-    for (int f = 1; f < 7; ++f) inside |= ((kept >> f) & 1) && (f & e) == f;
-    if (inside) continue;
-    int lo[3], hi[3];
-    for (int d = 0; d < 3; ++d) {
-      const bool on = (e >> d) & 1;
-      lo[d] = on && s[d] > 0 ? n - dhi : 0, hi[d] = on && s[d] < 0 ? dlo : n;
-    }
+  const int q = threadIdx.x & 31;
+  auto dir = [](int rank) { return (0x7653421 >> (4 * rank)) & 7; };
+  const int e = q < 7 ? dir(q) : 0;
+  bool keep = (ce >> e) & 1;  // not inside the box of a coarser neighbour across fewer axes
+  for (int f = 1; f < 7; ++f) keep = keep && !(((ce >> f) & 1) && f != e && (f & e) == f);
+  const unsigned kept = __ballot_sync(0xffffffffu, keep);
+  int lo[3], hi[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const bool on = (e >> d) & 1;
+    lo[d] = on && s[d] > 0 ? n - dhi : 0, hi[d] = on && s[d] < 0 ? dlo : n;
     // an earlier box (across the axes of f) covers this one along every axis
     // but the one of f that e does not have
-    for (int f = 1; f < 7; ++f)
-      if ((kept >> f) & 1)
-        for (int d = 0; d < 3; ++d)
-          if (((f & ~e) >> d) & 1) {
-            if (s[d] > 0) hi[d] = min(hi[d], n - dhi);
-            else lo[d] = max(lo[d], dlo);
-          }
-    kept |= 1 << e;
-    if (lo[0] >= hi[0] || lo[1] >= hi[1] || lo[2] >= hi[2]) continue;
-    for (int d = 0; d < 3; ++d) B.lo[cnt][d] = lo[d], B.hi[cnt][d] = hi[d];
-    ++cnt;
+    for (int r = 0; r < 6; ++r)
+      if (r < q && ((kept >> r) & 1) && (((dir(r) & ~e) >> d) & 1)) {
+        if (s[d] > 0) hi[d] = min(hi[d], n - dhi);
+        else lo[d] = max(lo[d], dlo);
+      }
   }
-  B.n = cnt;
+  keep = keep && lo[0] < hi[0] && lo[1] < hi[1] && lo[2] < hi[2];
+  const unsigned have = __ballot_sync(0xffffffffu, keep);
+  if (keep) {
+    const int at = __popc(have & ((1u << q) - 1u));
+    for (int d = 0; d < 3; ++d) B.lo[at][d] = lo[d], B.hi[at][d] = hi[d];
+  }
+  if (q == 0) B.n = __popc(have);
 }
 
 // level-Lq value (Lq = L or L - 1) at block-local point (i, j, k) through the
@@ -275,26 +276,65 @@ __device__ __noinline__ TI prep_fetch(const Tree &t, const PrepTab &T, const TI 
   return leaf_value(t, phi, o, Lq, g[0], g[1], g[2], err);
 }
 
-// Partial-sum type of the refinement: the block's, or float pairs for an FP32
-// field in an FP64 block (the K^s weights are dyadic, exact in FP32).
+// ---------------------------------------------------------------------------
+// The gather part of a leaf's padded block Pb (Alg. SM1): interior, the values
+// of same-level neighbours (copy) and the coincident values of finer neighbours
+// (their fine-to-coarse values are merged afterwards) -- everything but the
+// regions of coarser leaves.
+// One thread per (x, y) column of the padded block: along z the column crosses
+// at most three regions (a finer one in two halves), each of which is a run
+// of values a fixed stride apart in one leaf, so a point costs a load, a
+// store and two additions (a source index per point cost 113 instructions: 327
+// against 133 us for the 1 696 leaves next to coarser ones of a 3 424-leaf grid
+// of 24^3 blocks, shell 6).
+// ---------------------------------------------------------------------------
 template <typename TI, typename TP>
-struct RefSum {
-  using U = TP;
-  static __device__ __forceinline__ U zero() { return TP(0); }
-  static __device__ __forceinline__ U from(TI v) { return Cvt<TP>::f(v); }
-  static __device__ __forceinline__ U acc(U s, double w, U v) { return racc(s, TP(w), v); }
-  static __device__ __forceinline__ U norm(U s) { return s; }
-  static __device__ __forceinline__ TP value(U s) { return s; }
-};
-template <>
-struct RefSum<float, double> {
-  using U = F2;
-  static __device__ __forceinline__ U zero() { return f2_of(0.f); }
-  static __device__ __forceinline__ U from(float v) { return f2_of(v); }
-  static __device__ __forceinline__ U acc(U s, double w, U v) { return f2_acc(s, float(w), v); }
-  static __device__ __forceinline__ U norm(U s) { return f2_norm(s); }
-  static __device__ __forceinline__ double value(U s) { return f2_dbl(s); }
-};
+__device__ __forceinline__ void gather_block(const Tree &t, const PrepTab &T, const TI *__restrict__ phi, TP *Pb, int b,
+                                             int L, int Gi, int *err) {
+  const int nb = t.nb, Wd = nb + 2 * Gi, hb = nb / 2, W2 = Wd * Wd, nb2 = nb * nb;
+  const size_t nb3 = (size_t)nb * nb2;
+  const DivM dW = divm(Wd);
+  // n values st apart from src to padded planes from d on, four in flight
+  auto run = [&](TP *d, const TI *src, int st, int n) {
+    for (; n >= 4; n -= 4, d += 4 * W2, src += 4 * st) {
+      const TI v0 = ld(src), v1 = ld(src + st), v2 = ld(src + 2 * st), v3 = ld(src + 3 * st);
+      d[0] = Cvt<TP>::f(v0), d[W2] = Cvt<TP>::f(v1), d[2 * W2] = Cvt<TP>::f(v2), d[3 * W2] = Cvt<TP>::f(v3);
+    }
+    for (; n > 0; --n, d += W2, src += st) *d = Cvt<TP>::f(ld(src));
+  };
+  for (int c = threadIdx.x; c < W2; c += blockDim.x) {
+    const int row = divq(c, dW), i = c - row * Wd - Gi, j = row - Gi;
+    const int rx = i < 0 ? 0 : i >= nb ? 2 : 1, ry = j < 0 ? 0 : j >= nb ? 2 : 1;
+    const int ri = i - (rx - 1) * nb, rj = j - (ry - 1) * nb;  // region-local
+    TP *col = Pb + c + (size_t)W2 * Gi;                        // (i, j, 0)
+    for (int rz = 0; rz < 3; ++rz) {
+      const int r = rx + 3 * ry + 9 * rz, Lo = T.rlev[r];
+      if (Lo < L) continue;  // a coarser leaf's region: refined below
+      const int k0 = rz == 0 ? nb - Gi : 0, k1 = rz == 2 ? Gi : nb, z0 = (rz - 1) * nb;  // region-local planes
+      if (Lo == L) {
+        run(col + (ptrdiff_t)W2 * (z0 + k0), phi + (size_t)T.rslot[r] * nb3 + ri + nb * rj + nb2 * k0, nb2, k1 - k0);
+        continue;
+      }
+      const int hx = ri >= hb, hy = rj >= hb;
+      for (int hz = 0; hz < 2; ++hz) {
+        const int ka = hz ? max(k0, hb) : k0, kb = hz ? k1 : min(k1, hb);
+        if (ka >= kb) continue;
+        const int o2 = T.rsub[r][hx + 2 * hy + 4 * hz];
+        if (o2 >= 0) {
+          run(col + (ptrdiff_t)W2 * (z0 + ka),
+              phi + (size_t)o2 * nb3 + (2 * ri - hx * nb) + nb * (2 * rj - hy * nb) + nb2 * (2 * ka - hz * nb),
+              2 * nb2, kb - ka);
+        } else {  // two levels down (shells wider than half a block)
+          for (int k = ka; k < kb; ++k) {
+            const int gx = T.ranc[13][0] * nb + i, gy = T.ranc[13][1] * nb + j, gz = T.ranc[13][2] * nb + z0 + k;
+            const int ow = owner(t, L, gx, gy, gz, b);
+            col[(ptrdiff_t)W2 * (z0 + k)] = Cvt<TP>::f(leaf_value(t, phi, ow, L, gx, gy, gz, err));
+          }
+        }
+      }
+    }
+  }
+}
 
 // One box of a coarser leaf's region: expanded along the thin axis a, then b,
 // then c (b = x where it can, so that neighbouring threads are neighbours in
@@ -305,8 +345,16 @@ struct RefBox {
   int cb, cc, mb, mc;          // coarse range of the sums along b, c
   int mbp, nbp, S;             // pitches (odd: no bank conflicts)
   int off;                     // U1 at off, U2 at off + na * mbp * mc
-  unsigned dmb;                // reciprocal of mb
+  unsigned dmb, dna, dnb;      // reciprocals of mb, na, nb
+  unsigned dl2, dl3;           // and of the lines of pass 2 (na mc) and pass 3 (na nb)
 };
+
+// next start of the thread rotation after n items
+__device__ __forceinline__ int turn(int rot, int n, int bd) {
+  rot += n;
+  while (rot >= bd) rot -= bd;
+  return rot;
+}
 
 constexpr int SUB_RUN = 4;  // points of one item of the substitution
 
@@ -381,9 +429,13 @@ __device__ __forceinline__ void subst_run(const TP *src, int st, int n, bool cen
 #pragma unroll
   for (int m = 0; m < SUB_RUN; ++m) {
     if (m >= n) break;
-    TP acc = c[m];
+    // (the centre in its place among the taps: the partial sums stay small)
+    TP acc = TP(0);
 #pragma unroll
-    for (int x = 0; x < N; ++x) acc = racc(acc, TP(W::G(2 * x - hG)), e[m + x]);
+    for (int x = 0; x < N; ++x) {
+      if (x == N / 2) acc = radd(acc, c[m]);
+      acc = racc(acc, TP(W::G(2 * x - hG)), e[m + x]);
+    }
     put(m, acc);
   }
 }
@@ -402,7 +454,7 @@ __device__ __forceinline__ void subst_jobs(TP *Pb, int Wd, int Gi, const SubJob 
         const int n = J.it[s];
         int idx = (int)threadIdx.x - rot;
         if (idx < 0) idx += bd;
-        rot = (rot + n) & (bd - 1);
+        rot = turn(rot, n, bd);
         if (idx >= n) continue;
         const int st0 = J.st[s][0], st1 = J.st[s][1], st2 = J.st[s][2], sp1 = J.sp1[s];
         const int h0 = !(sp1 & 1), h1 = !(sp1 & 2), h2 = !(sp1 & 4);  // log2 of the steps
@@ -430,18 +482,21 @@ __device__ __forceinline__ void subst_jobs(TP *Pb, int Wd, int Gi, const SubJob 
               *c = subst_dispatch<N, NT, TP>(J.om & 1, J.om & 2, J.om & 4,
                                              [&](int tx, int ty, int tz) -> TP { return c[tx + Wd * ty + W2 * tz]; });
             }
-          } else if (s == 0) {
-            const int oth = J.om & ~(1 << d);
-            const bool keep0 = (oth & ~((p0 & 1) | ((p1 & 1) << 1) | ((p2 & 1) << 2))) != 0;
-            subst_run<N, NT>(pt, str, nr, keep0, put);
           } else {
-            // the previous pass summed another dimension; along this one it ran
-            // with step 1 from st[s-1], along the others its points are this pass's
-            const int k0 = J.cn[s - 1][0], k1 = k0 * J.cn[s - 1][1], ps = d == 0 ? 1 : d == 1 ? k0 : k1;
-            const int lead = J.st[s][d] - J.st[s - 1][d];
-            const TP *src = buf + J.off + (s == 2 ? J.n[0] : 0) + lead * ps + (d == 0 ? 2 * i0 : i0) +
-                            k0 * (d == 1 ? 2 * i1 : i1) + k1 * (d == 2 ? 2 * i2 : i2);
-            subst_run<N, NT>(src, ps, nr, true, put);
+            // pass 1 reads the block; a later one the previous pass's sums, which
+            // run with step 1 from st[s-1] along this dimension and hold this
+            // pass's points along the others
+            const int oth = J.om & ~(1 << d);
+            const bool centre = s > 0 || (oth & ~((p0 & 1) | ((p1 & 1) << 1) | ((p2 & 1) << 2))) != 0;
+            const TP *src = pt;
+            int ss = str;
+            if (s > 0) {
+              const int k0 = J.cn[s - 1][0], k1 = k0 * J.cn[s - 1][1];
+              ss = d == 0 ? 1 : d == 1 ? k0 : k1;
+              src = buf + J.off + (s == 2 ? J.n[0] : 0) + (J.st[s][d] - J.st[s - 1][d]) * ss +
+                    (d == 0 ? 2 * i0 : i0) + k0 * (d == 1 ? 2 * i1 : i1) + k1 * (d == 2 ? 2 * i2 : i2);
+            }
+            subst_run<N, NT>(src, ss, nr, centre, put);
           }
         }
       }
@@ -453,29 +508,15 @@ __device__ __forceinline__ void subst_jobs(TP *Pb, int Wd, int Gi, const SubJob 
 
 constexpr int PUSH_LAYERS = 4;
 
-// tensor H^a along one line: sum_t H^a(t) src[(2 m + t) st], m = 0 .. n - 1 <= M,
-// from one window of fine values; put(m, sum)
-template <int N, int NT, int M, typename TP, typename F>
-__device__ __forceinline__ void coarsen_run(const TP *src, int st, int n, F put) {
-  constexpr int hH = Wav<N, NT>::hwH, len = 2 * M - 1 + 2 * hH;
-  TP v[len];
-#pragma unroll
-  for (int x = 0; x < len; ++x) {
-    // (points that no sum with m < n reads are not loaded)
-    bool used = false;
-#pragma unroll
-    for (int m = 0; m < M; ++m)
-      if (x - hH - 2 * m >= -hH && x - hH - 2 * m <= hH && Wav<N, NT>::H(x - hH - 2 * m) != 0.0) used |= m < n;
-    v[x] = used ? src[(x - hH) * st] : TP(0);
-  }
-#pragma unroll
-  for (int m = 0; m < M; ++m) {
-    if (m >= n) break;
-    TP s = TP(0);
-    for_taps<N, NT, FK_H>([&](int t, double w) { s = racc(s, TP(w), v[2 * m + hH + t]); });
-    put(m, s);
-  }
-}
+// One box of coarse points to push: coarsened along the thinnest axis a, then b,
+// then c, layers layers of a at a time.
+struct PushBox {
+  int a, b, c;                 // axes
+  int na, nb, nc, fb, fc;      // coarse points per axis; fine extents along b, c
+  int la, layers, base;        // first layer; fine block index of (la, lo_b - h, lo_c - h); linear index of lo
+  int off, next;               // sums in shared memory; end of the batch this box opens
+  unsigned dfb, dfc, drb, dnb, dnc;  // reciprocals of fb, fc, ceil(nb / 4), nb, nc
+};
 
 // boxes, jobs and tables of the three phases (one set per CTA)
 struct PrepPlan {
@@ -484,6 +525,12 @@ struct PrepPlan {
   int nref, refnext[28];  // refinement boxes; end of the batch a box opens
   SubJob job[49];
   int job0[4];            // first job of each degree (job0[3]: end)
+  PushBox pbox[7];
+  int npb;
+  // coarser neighbours: direction, and the address in the side buffer of the
+  // leaf's coarse point (0, 0, 0) (every coordinate shifts by a constant)
+  int nq, qdir[7];
+  long long qbase[7];
 };
 
 // The boundary polynomial on the sums U1 of one box (beyond the domain along b
@@ -522,55 +569,28 @@ __device__ __noinline__ void bc_sums(const Tree &t, int Lc, const RefBox &B, int
   __syncthreads();
 }
 
-// planes of the sums along c: a chunk of twelve fine points (so that no leaf
+// planes of the sums along c: a chunk of eight fine points (so that no leaf
 // has more than 28 boxes), and on grids with physical boundaries the nodes of
 // the polynomial
-constexpr int prep_min_planes(int N, bool bounded) { return (N - 1) + 2 + 6 + (bounded ? N : 0); }
+constexpr int prep_min_planes(int N, bool bounded) { return (N - 1) + 2 + 4 + (bounded ? N : 0); }
 
-// Zero-detail refinement along one line: fine points f0 .. f0 + n - 1 (n <= 16)
-// from the coarse values src[q * st] (q: coarse index); put(m, v) receives
-// point f0 + m.  A register window of N coarse values moves along the line and
-// yields an even (coincident) and an odd (K^s) point per step.
-template <int N, int NT, typename RS, typename U, typename F>
-__device__ __forceinline__ void refine_run(const U *src, int st, int f0, int n, F put) {
-  using W = Wav<N, NT>;
-  constexpr int ko = N - 1, h = N / 2;
-  // window w[0..N-1] = coarse q-h+1 .. q+h around the odd point 2q + 1
-  const int q0 = f0 >> 1;
-  U w[N];
-#pragma unroll
-  for (int x = 0; x + 1 < N; ++x) w[x] = src[(q0 - h + 1 + x) * st];
-  const int par = f0 & 1;
-  // (the last value of a window is read only where its odd point exists)
-  w[N - 1] = par || n > 1 ? src[(q0 + h) * st] : w[0];
-  for (int m = -par; m < n; m += 2) {  // even point m, odd point m + 1
-    if (m >= 0) put(m, w[h - 1]);
-    if (m + 1 < n) {
-      U s = RS::acc(RS::zero(), W::K(-ko), w[0]);
-#pragma unroll
-      for (int x = 1; x < N; ++x) s = RS::acc(s, W::K(2 * x - ko), w[x]);
-      put(m + 1, s);
-    }
-    if (m + 2 < n) {
-#pragma unroll
-      for (int x = 0; x + 1 < N; ++x) w[x] = w[x + 1];
-      if (m + 3 < n) w[N - 1] = src[(q0 + (m + par) / 2 + 1 + h) * st];
-    }
-  }
-}
-
+// only_coarse: 0 every (needed) leaf, 1 the leaves next to coarser ones, 2 those
+// without the push
 template <typename TI, typename TP, int N, int NT, bool BND>
-__global__ void __launch_bounds__(256, sizeof(TP) == 4 ? 4 : 3) k_prep(Tree t, const TI *__restrict__ phi,
+__global__ void __launch_bounds__(sizeof(TP) == 4 ? 512 : 384, 2) k_prep(Tree t, const TI *__restrict__ phi,
                                                                      TP *__restrict__ P, TP *__restrict__ Q, int Gi,
                                                                      int Gpush, int only_coarse, int *cmask_out,
                                                                      int *err, const int *__restrict__ need,
-                                                                     int sum_bytes) {
+                                                                     int *__restrict__ pneed, int sum_bytes) {
   using W = Wav<N, NT>;
   using RS = RefSum<TI, TP>;
   using U = typename RS::U;
   constexpr int ko = N - 1;  // widest odd K^s tap
   const int b = blockIdx.x;
-  if (need && !need[b]) return;
+  if (need && !need[b]) {
+    if (threadIdx.x == 0) pneed[b] = 0;
+    return;
+  }
   const int nb = t.nb, Wd = nb + 2 * Gi, W2 = Wd * Wd, hb = nb / 2, tid = threadIdx.x, bd = blockDim.x;
   const size_t np = (size_t)Wd * W2, nb3 = (size_t)nb * nb * nb;
   const int L = __ldg(t.lev + b);
@@ -622,57 +642,126 @@ __global__ void __launch_bounds__(256, sizeof(TP) == 4 ? 4 : 3) k_prep(Tree t, c
   }
   __syncthreads();
   const int mask = T.cmask, ce = T.ce;
-  if (tid == 0 && cmask_out) cmask_out[b] = mask;
-  if (!mask) return;
-  // one thread per phase builds its boxes; the sub-blocks of finer regions (-1:
-  // refined further) are looked up meanwhile
-  if (tid == 0) {
-    int n = 0, used = 0, open = 0;
-    for (int e = 1; e < 8; ++e) {
-      if (!((ce >> e) & 1)) continue;
+  if (tid == 0) cmask_out[b] = mask, pneed[b] = mask ? 1 : 0;
+  if (only_coarse && !mask) return;
+  // one warp per phase builds its boxes (a lane per direction); the sub-blocks
+  // of finer regions (-1: refined further) are looked up meanwhile
+  if (!mask) {
+  } else if (tid < 32) {
+    const int e = tid;
+    const bool on = e < 8 && ((ce >> e) & 1);
+    RefBox B;
+    int nch = 0, step = 2, lc0 = 0, lenc = 0, plane = 0;
+    if (on) {
       int l[3], m[3];
       for (int d = 0; d < 3; ++d) {
-        const bool on = (e >> d) & 1;
-        l[d] = on ? (T.s[d] > 0 ? nb : -Gi) : (T.s[d] > 0 ? -Gi : 0);
-        m[d] = on ? Gi : nb + Gi;
+        const bool od = (e >> d) & 1;
+        l[d] = od ? (T.s[d] > 0 ? nb : -Gi) : (T.s[d] > 0 ? -Gi : 0);
+        m[d] = od ? Gi : nb + Gi;
       }
-      RefBox B;
       B.a = (e & 1) ? 0 : (e & 2) ? 1 : 2;
       B.b = B.a == 0 ? 1 : 0, B.c = 3 - B.a - B.b;
       B.la = l[B.a], B.na = m[B.a], B.lb = l[B.b], B.nb = m[B.b];
       B.cb = (B.lb - ko) >> 1, B.mb = ((B.lb + B.nb - 1 + ko) >> 1) - B.cb + 1;
-      B.mbp = B.mb | 1, B.nbp = B.nb | 1, B.dmb = divm(B.mb).m;
+      B.mbp = B.mb | 1, B.nbp = B.nb | 1;
       B.S = (B.a == 0 ? B.na * B.nb : B.na * B.nbp) | 1;
+      B.dmb = divm(B.mb).m, B.dna = divm(B.na).m, B.dnb = divm(B.nb).m, B.dl3 = divm(B.na * B.nb).m;
       // cut along c: mc planes of both sums
-      const int plane = B.na * B.mbp + B.S, most = capU / plane, ext = BND ? N : 0;
-      const int step = max(2 * (most - ko - 2 - ext), 2);
-      for (int c0 = 0; c0 < m[B.c]; c0 += step) {
-        B.lc = l[B.c] + c0, B.nc = min(step, m[B.c] - c0);
-        B.cc = (B.lc - ko) >> 1;
-        int ce1 = ((B.lc + B.nc - 1 + ko) >> 1) + 1;
-        if (BND) {  // the polynomial's nodes, where the chunk reaches beyond the domain
-          const int anc = (B.c == 0 ? ax : B.c == 1 ? ay : az) / 2;
-          const int first = bc_first(t, anc, B.c), end = bc_end(t, L - 1, anc, B.c);
-          if (B.cc < first) ce1 = max(ce1, first + N);
-          if (ce1 > end) B.cc = min(B.cc, end - N);
-        }
-        B.mc = ce1 - B.cc;
-        const int sz = plane * B.mc;
-        if (n && used + sz > capU) {
+      plane = B.na * B.mbp + B.S;
+      step = max(2 * (capU / plane - ko - 2 - (BND ? N : 0)), 2);
+      lc0 = l[B.c], lenc = m[B.c], nch = (lenc + step - 1) / step;
+    }
+    int pos = nch;  // first box of this direction
+    for (int w = 1; w < 8; w <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, pos, w);
+      if (tid >= w) pos += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, pos, 7);
+    pos -= nch;
+    for (int c0 = 0; c0 < lenc; c0 += step) {
+      B.lc = lc0 + c0, B.nc = min(step, lenc - c0);
+      B.cc = (B.lc - ko) >> 1;
+      int ce1 = ((B.lc + B.nc - 1 + ko) >> 1) + 1;
+      if (BND) {  // the polynomial's nodes, where the chunk reaches beyond the domain
+        const int anc = (B.c == 0 ? ax : B.c == 1 ? ay : az) / 2;
+        const int first = bc_first(t, anc, B.c), end = bc_end(t, L - 1, anc, B.c);
+        if (B.cc < first) ce1 = max(ce1, first + N);
+        if (ce1 > end) B.cc = min(B.cc, end - N);
+      }
+      B.mc = ce1 - B.cc;
+      B.dl2 = divm(B.na * B.mc).m;
+      B.off = plane * B.mc;  // (its size, until the batches are laid out)
+      plan.ref[pos++] = B;
+    }
+    __syncwarp();
+    if (tid == 0) {
+      int used = 0, open = 0;
+      for (int n = 0; n < total; ++n) {
+        const int sz = plan.ref[n].off;
+        if (n > open && used + sz > capU) {
           for (int q = open; q < n; ++q) plan.refnext[q] = n;
           open = n, used = 0;
         }
-        B.off = used, plan.ref[n++] = B;
-        used += sz;
+        plan.ref[n].off = used, used += sz;
+      }
+      for (int q = open; q < total; ++q) plan.refnext[q] = total;
+      plan.nref = total;
+    }
+  } else if (tid < 64) {
+    outward_boxes(plan.band, ce, T.s, nb, W::ext_b, W::ext_f);
+  } else if (tid < 96) {
+    const int gp = min(Gpush, hb), q = tid - 64;
+    outward_boxes(plan.push, ce, T.s, hb, gp, gp);
+    __syncwarp();
+    if constexpr (NT != 0) {
+      constexpr int hH = W::hwH;
+      if (q < plan.push.n) {
+        const int *lo = plan.push.lo[q], *hi = plan.push.hi[q];
+        const int e0 = hi[0] - lo[0], e1 = hi[1] - lo[1], e2 = hi[2] - lo[2];
+        PushBox B;
+        B.a = e0 <= e1 && e0 <= e2 ? 0 : e1 <= e2 ? 1 : 2, B.b = B.a == 0 ? 1 : 0, B.c = 3 - B.a - B.b;
+        B.na = hi[B.a] - lo[B.a], B.nb = hi[B.b] - lo[B.b], B.nc = hi[B.c] - lo[B.c], B.la = lo[B.a];
+        B.fb = 2 * B.nb - 1 + 2 * hH, B.fc = 2 * B.nc - 1 + 2 * hH;
+        B.layers = max(1, min(min(B.na, PUSH_LAYERS), capP / (B.fc * (B.fb + B.nb))));
+        const int sA = B.a == 0 ? 1 : B.a == 1 ? Wd : W2, sB = B.b == 0 ? 1 : Wd, sC = B.c == 1 ? Wd : W2;
+        B.base = (2 * B.la + Gi) * sA + (2 * lo[B.b] - hH + Gi) * sB + (2 * lo[B.c] - hH + Gi) * sC;
+        B.dfb = divm(B.fb).m, B.dfc = divm(B.fc).m, B.drb = divm((B.nb + 3) >> 2).m, B.dnb = divm(B.nb).m;
+        B.dnc = divm(B.nc).m;
+        B.off = B.layers * B.fc * (B.fb + B.nb);  // (its size, until the batches are laid out)
+        plan.pbox[q] = B;
+      }
+      // the neighbour in direction f holds point p at p - hb or p + nb along the
+      // axes of f, in the leaf's half along the others
+      if (q >= 8 && q < 16) {
+        const int f = q - 8;
+        const bool on = f && ((ce >> f) & 1);
+        const unsigned have = __ballot_sync(0x0000ff00u, on);
+        if (on) {
+          int r2 = 13, st = 1;
+          long long x = 0;
+          for (int d = 0; d < 3; ++d, st *= Wd) {
+            const bool od = (f >> d) & 1;
+            if (od) r2 += T.s[d] * (d == 0 ? 1 : d == 1 ? 3 : 9);
+            x += (long long)st * ((od ? (T.s[d] > 0 ? -hb : nb) : T.odd[d] * hb) + Gi);
+          }
+          const int at = __popc(have & ((1u << q) - 1u));
+          plan.qdir[at] = f, plan.qbase[at] = (long long)T.rslot[r2] * (long long)np + x;
+        }
+        if (q == 15) plan.nq = __popc(have);
+      }
+      __syncwarp();
+      if (q == 0) {
+        const int n = plan.push.n;
+        int used = 0, open = 0;
+        for (int e = 0; e < n; ++e) {
+          const int sz = plan.pbox[e].off;
+          if (e > open && used + sz > capP) plan.pbox[open].next = e, open = e, used = 0;
+          plan.pbox[e].off = used, used += sz;
+        }
+        if (n) plan.pbox[open].next = n;
+        plan.npb = n;
       }
     }
-    for (int q = open; q < n; ++q) plan.refnext[q] = n;
-    plan.nref = n;
-  } else if (tid == 32) {
-    outward_boxes(plan.band, ce, T.s, nb, W::ext_b, W::ext_f);
-  } else if (tid == 64) {
-    const int gp = min(Gpush, hb);
-    outward_boxes(plan.push, ce, T.s, hb, gp, gp);
   }
   for (int q = tid; q < 216; q += bd) {
     const int r = q >> 3, h = q & 7;
@@ -687,6 +776,9 @@ __global__ void __launch_bounds__(256, sizeof(TP) == 4 ? 4 : 3) k_prep(Tree t, c
     T.rsub[r][h] = o2;
   }
   __syncthreads();
+  TP *Pb = P + (size_t)b * np;
+  gather_block(t, T, phi, Pb, b, L, Gi, err);
+  if (!mask) return;
   // substitution jobs: one thread each (degree 1: classes x, y, z; 2: xy, xz,
   // yz; 3: xyz), then one thread lays out their sums
   {
@@ -697,7 +789,28 @@ __global__ void __launch_bounds__(256, sizeof(TP) == 4 ? 4 : 3) k_prep(Tree t, c
       sub_job_build(plan.job[tid], plan.band.lo[e], plan.band.hi[e], cls[k], W::hwG);
     }
   }
-  TP *Pb = P + (size_t)b * np;
+  // layout of the substitution sums: batches within a degree (by one thread,
+  // while the others refine)
+  auto sub_layout = [&]() {
+    const int nbx = plan.band.n;
+    int j = 0;
+    for (int deg = 1; deg <= 3; ++deg) {
+      const int end = j + (deg < 3 ? 3 : 1) * nbx;
+      plan.job0[deg - 1] = j;
+      int used = 0, open = j;
+      for (; j < end; ++j) {
+        SubJob &J = plan.job[j];
+        const int sz = deg == 1 ? 0 : J.n[0] + (deg == 3 ? J.n[1] : 0);
+        if (j > open && used + sz > capP) {
+          plan.job[open].next = j;
+          open = j, used = 0;
+        }
+        J.off = used, used += sz;
+      }
+      if (open < end) plan.job[open].next = end;
+    }
+    plan.job0[3] = j;
+  };
   const long long lin1 = nb, lin2 = (long long)nb * nb;
   // coarse values beyond a physical boundary (the leaf's own parent range or
   // its lateral ghosts): the polynomial is applied to the sums along b and c;
@@ -705,6 +818,8 @@ __global__ void __launch_bounds__(256, sizeof(TP) == 4 ? 4 : 3) k_prep(Tree t, c
   const bool cbc = BND && bc_touches(t, L, ax, ay, az, -Gi - ko - 1, nb + Gi + ko + 1);
   bool bad = false;  // a refined value is NaN: one flag per CTA, set below
   if (BND && cbc && sizeof(TI) != sizeof(TP)) {
+    __syncthreads();
+    if (tid == bd - 1) sub_layout();
     for (int e = 0; e < plan.nref; ++e) {
       const RefBox &B = plan.ref[e];
       const DivM dna = divm(B.na), dnb = divm(B.nb);
@@ -733,7 +848,7 @@ __global__ void __launch_bounds__(256, sizeof(TP) == 4 ? 4 : 3) k_prep(Tree t, c
         const int pitch = B.mbp;
         int idx = tid - rot;
         if (idx < 0) idx += bd;
-        rot = (rot + ncol) & (bd - 1);
+        rot = turn(rot, ncol, bd);
         for (; idx < ncol; idx += bd) {
           const int kc = divq(idx, DivM{B.dmb, B.mb}), jb = idx - kc * B.mb;
           int q[3];
@@ -798,6 +913,7 @@ __global__ void __launch_bounds__(256, sizeof(TP) == 4 ? 4 : 3) k_prep(Tree t, c
         }
       }
       __syncthreads();
+      if (e0 == 0 && tid == bd - 1) sub_layout();
       if constexpr (BND && sizeof(TI) == sizeof(TP))
         if (cbc)
           for (int e = e0; e < e1; ++e)
@@ -808,13 +924,13 @@ __global__ void __launch_bounds__(256, sizeof(TP) == 4 ? 4 : 3) k_prep(Tree t, c
       for (int e = e0; e < e1; ++e) {
         const RefBox &B = plan.ref[e];
         const int na = B.na, lines = na * B.mc, nseg = (B.nb + 15) >> 4, n = lines * nseg;
-        const DivM dl = divm(lines), dna = divm(na);
+        const DivM dl{B.dl2, lines}, dna{B.dna, na};
         const int sb = B.a == 0 ? na : 1, sa = B.a == 0 ? 1 : B.nbp;
         const U *U1 = UB + B.off;
         U *U2 = UB + B.off + na * B.mbp * B.mc;
         int idx = tid - rot;
         if (idx < 0) idx += bd;
-        rot = (rot + n) & (bd - 1);
+        rot = turn(rot, n, bd);
         for (; idx < n; idx += bd) {
           const int sg = divq(idx, dl), ln = idx - sg * lines, kc = divq(ln, dna), ia = ln - kc * na;
           const int f0 = B.lb + 16 * sg, n1 = min(16, B.nb - 16 * sg);
@@ -830,14 +946,14 @@ __global__ void __launch_bounds__(256, sizeof(TP) == 4 ? 4 : 3) k_prep(Tree t, c
         const RefBox &B = plan.ref[e];
         const int na = B.na, lines = na * B.nb, nseg = (B.nc + 15) >> 4, n = lines * nseg;
         const int n1d = B.a == 0 ? na : B.nb;  // dimension that varies fastest over threads
-        const DivM dl = divm(lines), df = divm(n1d);
+        const DivM dl{B.dl3, lines}, df{B.a == 0 ? B.dna : B.dnb, n1d};
         const int sb = B.a == 0 ? na : 1, sa = B.a == 0 ? 1 : B.nbp;
         const int psa = B.a == 0 ? 1 : B.a == 1 ? Wd : W2, psb = B.b == 0 ? 1 : B.b == 1 ? Wd : W2,
                   psc = B.c == 0 ? 1 : B.c == 1 ? Wd : W2;
         const U *U2 = UB + B.off + na * B.mbp * B.mc;
         int idx = tid - rot;
         if (idx < 0) idx += bd;
-        rot = (rot + n) & (bd - 1);
+        rot = turn(rot, n, bd);
         for (; idx < n; idx += bd) {
           const int sg = divq(idx, dl), ln = idx - sg * lines, hi = divq(ln, df), lo = ln - hi * n1d;
           const int ia = B.a == 0 ? lo : hi, ib = B.a == 0 ? hi : lo;
@@ -854,28 +970,6 @@ __global__ void __launch_bounds__(256, sizeof(TP) == 4 ? 4 : 3) k_prep(Tree t, c
       e0 = e1;
     }
   }
-  // layout of the substitution sums: batches within a degree
-  __syncthreads();
-  if (tid == 0) {
-    const int nbx = plan.band.n;
-    int j = 0;
-    for (int deg = 1; deg <= 3; ++deg) {
-      const int end = j + (deg < 3 ? 3 : 1) * nbx;
-      plan.job0[deg - 1] = j;
-      int used = 0, open = j;
-      for (; j < end; ++j) {
-        SubJob &J = plan.job[j];
-        const int sz = deg == 1 ? 0 : J.n[0] + (deg == 3 ? J.n[1] : 0);
-        if (j > open && used + sz > capP) {
-          plan.job[open].next = j;
-          open = j, used = 0;
-        }
-        J.off = used, used += sz;
-      }
-      if (open < end) plan.job[open].next = end;
-    }
-    plan.job0[3] = j;
-  }
   if (__syncthreads_or(bad) && tid == 0) atomicOr(err, 2);
   if (BND && bc_touches(t, L, ax, ay, az, -Gi, nb + Gi))
     bc_box<N>(t, L, ax, ay, az, Pb + Gi * (1 + Wd + W2), Wd, W2, -Gi, -Gi, -Gi, Wd, Wd, Wd);
@@ -887,169 +981,79 @@ __global__ void __launch_bounds__(256, sizeof(TP) == 4 ? 4 : 3) k_prep(Tree t, c
   // coincident values the gather took are already the coarsened ones)
   if (only_coarse == 2 || NT == 0) return;
   // Part 2: H^a coarsening of the padded block at the coarse points of the push
-  // boxes, thinnest axis a first (then b, c), up to PUSH_LAYERS layers of a at a
-  // time: one thread loads a fine column along a and sums every layer from it;
-  // along b and c a thread sums four points from one window.  Each value goes to
-  // the side buffer of every coarser neighbour in whose shell the point lies.
+  // boxes: one thread loads a fine column along a and sums every layer from it;
+  // along b a thread sums four points from one window; along c one point, which
+  // goes to the side buffer of every coarser neighbour in whose shell it lies.
   if constexpr (NT != 0) {
     constexpr int hH = W::hwH;
-    const int gp = min(Gpush, hb);
-    for (int e = 0; e < plan.push.n; ++e) {
-      const int *lo = plan.push.lo[e];
-      const int n3[3] = {plan.push.hi[e][0] - lo[0], plan.push.hi[e][1] - lo[1], plan.push.hi[e][2] - lo[2]};
-      const int a = n3[0] <= n3[1] && n3[0] <= n3[2] ? 0 : n3[1] <= n3[2] ? 1 : 2, bx = a == 0 ? 1 : 0,
-                c = 3 - a - bx;
-      const int na = n3[a], nbb = n3[bx], nc = n3[c], fb = 2 * nbb - 1 + 2 * hH, fc = 2 * nc - 1 + 2 * hH;
-      const int sA = a == 0 ? 1 : a == 1 ? Wd : W2, sB = bx == 0 ? 1 : Wd, sC = c == 1 ? Wd : W2;
-      const int layers = max(1, min(min(na, PUSH_LAYERS), capP / (fc * (fb + nbb))));
-      const int rb = (nbb + 3) >> 2, rc = (nc + 3) >> 2;  // runs of four points along b, c
-      const DivM dfb = divm(fb), dfc = divm(fc), drb = divm(rb), dnb = divm(nbb), drc = divm(rc);
-      const int q0 = 2 * lo[bx] - hH + Gi, q1 = 2 * lo[c] - hH + Gi;
-      for (int l0 = 0; l0 < na; l0 += layers) {
-        const int nl = min(layers, na - l0);
-        TP *A = reinterpret_cast<TP *>(smraw), *Bf = A + nl * fc * fb;  // [l][fc][fb], [l][fc][nbb]
-        const TP *src0 = Pb + (2 * (lo[a] + l0) + Gi) * sA + q0 * sB + q1 * sC;
-        for (int idx = tid; idx < fc * fb; idx += bd) {
-          const int ic = divq(idx, dfb), ib = idx - ic * fb;
-          coarsen_run<N, NT, PUSH_LAYERS>(src0 + ib * sB + ic * sC, sA, nl,
-                                          [&](int l, TP v) { A[l * fc * fb + idx] = v; });
-        }
-        __syncthreads();
-        for (int idx = tid; idx < nl * fc * rb; idx += bd) {
-          const int r = divq(idx, drb), ib = 4 * (idx - r * rb);
-          TP *d = Bf + r * nbb + ib;
-          coarsen_run<N, NT, 4>(A + r * fb + 2 * ib + hH, 1, min(4, nbb - ib), [&](int m, TP v) { d[m] = v; });
-        }
-        __syncthreads();
-        for (int idx = tid; idx < nl * rc * nbb; idx += bd) {
-          const int r = divq(idx, dnb), l = divq(r, drc), ib = idx - r * nbb, ic = 4 * (r - l * rc);
-          coarsen_run<N, NT, 4>(Bf + (l * fc + 2 * ic + hH) * nbb + ib, nbb, min(4, nc - ic), [&](int m, TP sv) {
-            int p[3], inb = 0;
-            p[a] = lo[a] + l0 + l, p[bx] = lo[bx] + ib, p[c] = lo[c] + ic + m;
-            for (int d = 0; d < 3; ++d) inb |= (T.s[d] > 0 ? p[d] >= hb - gp : p[d] < gp) << d;
-            for (int f = 1; f < 8; ++f) {
-              if (!((ce >> f) & 1) || (f & ~inb)) continue;
-              // position in the neighbour: beyond its face along the axes of f,
-              // in the leaf's half along the others
-              int r2 = 13, x[3];
-              for (int d = 0; d < 3; ++d) {
-                const bool on = (f >> d) & 1;
-                if (on) r2 += T.s[d] * (d == 0 ? 1 : d == 1 ? 3 : 9);
-                x[d] = (on ? (T.s[d] > 0 ? p[d] - hb : nb + p[d]) : p[d] + T.odd[d] * hb) + Gi;
-              }
-              Q[(size_t)T.rslot[r2] * np + x[0] + Wd * (x[1] + (size_t)Wd * x[2])] = sv;
-            }
-          });
-        }
-        __syncthreads();
-      }
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// The gather part of every leaf's padded block (Alg. SM1): interior, the
-// values of same-level neighbours (copy) and the coincident values of finer
-// neighbours (their fine-to-coarse values are merged afterwards, as for every
-// leaf) -- everything but the regions of coarser leaves.  A leaf with a
-// coarser neighbour is flagged in pneed for the full pre-pass (refinement of
-// the coarse regions, substitution, Part-2 push).
-// Finer regions are resolved through the owners of their eight one-level-
-// finer sub-blocks (one lookup per sub-block, not per point).
-// One thread per (x, y) column of the padded block: along z the column crosses
-// at most three regions (a finer one in two halves), each of which is a run
-// of values a fixed stride apart in one leaf, so a point costs a load, a
-// store and two additions.
-// ---------------------------------------------------------------------------
-template <typename TI, typename TP>
-__global__ void __launch_bounds__(512) k_fill_plain(Tree t, const TI *__restrict__ phi, TP *__restrict__ P,
-                                                    int Gi, const int *__restrict__ need,
-                                                    int *__restrict__ pneed, int *__restrict__ cmask_out,
-                                                    int *err, int coarse_only) {
-  const int b = blockIdx.x;
-  if (need && !need[b]) {
-    if (threadIdx.x == 0) pneed[b] = 0;
-    return;
-  }
-  const int nb = t.nb, Wd = nb + 2 * Gi, hb = nb / 2;
-  const size_t np = (size_t)Wd * Wd * Wd, nb3 = (size_t)nb * nb * nb;
-  const int L = __ldg(t.lev + b);
-  __shared__ int rslot[27], rlev[27], rsub[27][8];
-  __shared__ int coarse;
-  if (threadIdx.x == 0) coarse = 0;
-  __syncthreads();
-  if (threadIdx.x < 27) {
-    const int r = threadIdx.x;
-    const int dd[3] = {r % 3 - 1, (r / 3) % 3 - 1, r / 9 - 1};
-    int g[3];
-    for (int d = 0; d < 3; ++d) g[d] = __ldg(t.anc + 3 * b + d) * nb + (dd[d] < 0 ? -1 : dd[d] > 0 ? nb : 0);
-    const int o = beyond3(t, L, g) ? b : owner(t, L, g[0], g[1], g[2], b);
-    const int Lo = __ldg(t.lev + o);
-    rslot[r] = o, rlev[r] = Lo;
-    if (r != 13 && Lo < L) atomicOr(&coarse, 1);
-  }
-  __syncthreads();
-  // a leaf with a coarser neighbour: its coarser regions and everything
-  // after the gather are the full pre-pass's (which also writes its cmask)
-  if (threadIdx.x == 0) {
-    pneed[b] = coarse ? 1 : 0;
-    if (!coarse) cmask_out[b] = 0;
-  }
-  if (coarse_only && !coarse) return;  // the caller needs the pre-pass's leaves only
-  for (int q = threadIdx.x; q < 216; q += blockDim.x) {
-    const int r = q >> 3, h = q & 7;
-    int o2 = -1;
-    if (rlev[r] == L + 1 && L < t.M) {
-      const int dd[3] = {r % 3 - 1, (r / 3) % 3 - 1, r / 9 - 1};
-      int g[3];
-      for (int d = 0; d < 3; ++d) g[d] = 2 * (__ldg(t.anc + 3 * b + d) + dd[d]) * nb + ((h >> d) & 1) * nb;
-      o2 = owner(t, L + 1, g[0], g[1], g[2], b);
-      if (o2 < 0 || o2 >= t.nleaf || __ldg(t.lev + o2) != L + 1) o2 = -1;
-    }
-    rsub[r][h] = o2;
-  }
-  __syncthreads();
-  const int ax = __ldg(t.anc + 3 * b) * nb, ay = __ldg(t.anc + 3 * b + 1) * nb, az = __ldg(t.anc + 3 * b + 2) * nb;
-  const int W2 = Wd * Wd, nb2 = nb * nb;
-  const DivM dW = divm(Wd);
-  // n values st apart from src to padded planes from d on, four in flight
-  auto run = [&](TP *d, const TI *src, int st, int n) {
-    for (; n >= 4; n -= 4, d += 4 * W2, src += 4 * st) {
-      const TI v0 = ld(src), v1 = ld(src + st), v2 = ld(src + 2 * st), v3 = ld(src + 3 * st);
-      d[0] = Cvt<TP>::f(v0), d[W2] = Cvt<TP>::f(v1), d[2 * W2] = Cvt<TP>::f(v2), d[3 * W2] = Cvt<TP>::f(v3);
-    }
-    for (; n > 0; --n, d += W2, src += st) *d = Cvt<TP>::f(ld(src));
-  };
-  for (int c = threadIdx.x; c < W2; c += blockDim.x) {
-    const int row = divq(c, dW), i = c - row * Wd - Gi, j = row - Gi;
-    const int rx = i < 0 ? 0 : i >= nb ? 2 : 1, ry = j < 0 ? 0 : j >= nb ? 2 : 1;
-    const int ri = i - (rx - 1) * nb, rj = j - (ry - 1) * nb;  // region-local
-    TP *col = P + (size_t)b * np + c + (size_t)W2 * Gi;        // (i, j, 0)
-    for (int rz = 0; rz < 3; ++rz) {
-      const int r = rx + 3 * ry + 9 * rz, Lo = rlev[r];
-      if (Lo < L) continue;  // a coarser leaf's region: refined by the pre-pass
-      const int k0 = rz == 0 ? nb - Gi : 0, k1 = rz == 2 ? Gi : nb, z0 = (rz - 1) * nb;  // region-local planes
-      if (Lo == L) {
-        run(col + (ptrdiff_t)W2 * (z0 + k0), phi + (size_t)rslot[r] * nb3 + ri + nb * rj + nb2 * k0, nb2, k1 - k0);
-        continue;
-      }
-      const int hx = ri >= hb, hy = rj >= hb;
-      for (int hz = 0; hz < 2; ++hz) {
-        const int ka = hz ? max(k0, hb) : k0, kb = hz ? k1 : min(k1, hb);
-        if (ka >= kb) continue;
-        const int o2 = rsub[r][hx + 2 * hy + 4 * hz];
-        if (o2 >= 0) {
-          run(col + (ptrdiff_t)W2 * (z0 + ka),
-              phi + (size_t)o2 * nb3 + (2 * ri - hx * nb) + nb * (2 * rj - hy * nb) + nb2 * (2 * ka - hz * nb),
-              2 * nb2, kb - ka);
-        } else {  // two levels down (shells wider than half a block)
-          for (int k = ka; k < kb; ++k) {
-            const int gx = ax + i, gy = ay + j, gz = az + z0 + k;
-            const int ow = owner(t, L, gx, gy, gz, b);
-            col[(ptrdiff_t)W2 * (z0 + k)] = Cvt<TP>::f(leaf_value(t, phi, ow, L, gx, gy, gz, err));
+    const int gp = min(Gpush, hb), npb = plan.npb, nq = plan.nq;
+    TP *buf = reinterpret_cast<TP *>(smraw);
+    for (int e0 = 0; e0 < npb;) {
+      const int e1 = plan.pbox[e0].next;
+      bool more = true;
+      for (int it = 0; more; ++it) {
+        more = false;
+        int rot = 0;
+        for (int e = e0; e < e1; ++e) {
+          const PushBox &B = plan.pbox[e];
+          const int l0 = it * B.layers, nl = min(B.layers, B.na - l0), n = B.fc * B.fb;
+          more |= l0 + B.layers < B.na;
+          if (nl <= 0) continue;
+          int idx = tid - rot;
+          if (idx < 0) idx += bd;
+          rot = turn(rot, n, bd);
+          const int sA = B.a == 0 ? 1 : B.a == 1 ? Wd : W2, sB = B.b == 0 ? 1 : Wd, sC = B.c == 1 ? Wd : W2;
+          TP *A = buf + B.off;  // [l][fc][fb]
+          for (; idx < n; idx += bd) {
+            const int ic = divq(idx, DivM{B.dfb, B.fb}), ib = idx - ic * B.fb;
+            coarsen_run<N, NT, PUSH_LAYERS>(Pb + B.base + 2 * l0 * sA + ib * sB + ic * sC, sA, nl,
+                                            [&](int l, TP v) { A[l * n + idx] = v; });
           }
         }
+        __syncthreads();
+        rot = 0;
+        for (int e = e0; e < e1; ++e) {
+          const PushBox &B = plan.pbox[e];
+          const int nl = min(B.layers, B.na - it * B.layers), rb = (B.nb + 3) >> 2, n = nl * B.fc * rb;
+          if (nl <= 0) continue;
+          int idx = tid - rot;
+          if (idx < 0) idx += bd;
+          rot = turn(rot, n, bd);
+          const TP *A = buf + B.off + hH;
+          TP *D = buf + B.off + B.layers * B.fc * B.fb;  // [l][fc][nb]
+          for (; idx < n; idx += bd) {
+            const int r = divq(idx, DivM{B.drb, rb}), ib = 4 * (idx - r * rb);
+            TP *d = D + r * B.nb + ib;
+            coarsen_run<N, NT, 4>(A + r * B.fb + 2 * ib, 1, min(4, B.nb - ib), [&](int m, TP v) { d[m] = v; });
+          }
+        }
+        __syncthreads();
+        rot = 0;
+        for (int e = e0; e < e1; ++e) {
+          const PushBox &B = plan.pbox[e];
+          const int l0 = it * B.layers, nl = min(B.layers, B.na - l0), n = nl * B.nc * B.nb;
+          if (nl <= 0) continue;
+          int idx = tid - rot;
+          if (idx < 0) idx += bd;
+          rot = turn(rot, n, bd);
+          const TP *D = buf + B.off + B.layers * B.fc * B.fb;
+          const int lob = plan.push.lo[e][B.b], loc = plan.push.lo[e][B.c];
+          for (; idx < n; idx += bd) {
+            const int r = divq(idx, DivM{B.dnb, B.nb}), l = divq(r, DivM{B.dnc, B.nc}), ib = idx - r * B.nb,
+                      ic = r - l * B.nc;
+            const TP sv = tap_sum<N, NT, FK_H>(D + (l * B.fc + 2 * ic + hH) * B.nb + ib, B.nb);
+            const int va = B.la + l0 + l, vb = lob + ib, vc = loc + ic;
+            const int px = B.a == 0 ? va : vb, py = B.a == 0 ? vb : B.a == 1 ? va : vc, pz = B.a == 2 ? va : vc;
+            const int inb = (T.s[0] > 0 ? px >= hb - gp : px < gp) | (T.s[1] > 0 ? py >= hb - gp : py < gp) << 1 |
+                            (T.s[2] > 0 ? pz >= hb - gp : pz < gp) << 2;
+            const int lin = px + Wd * py + W2 * pz;
+            for (int f = 0; f < nq; ++f)
+              if (!(plan.qdir[f] & ~inb)) Q[plan.qbase[f] + lin] = sv;
+          }
+        }
+        __syncthreads();
       }
+      e0 = e1;
     }
   }
 }
@@ -1169,37 +1173,21 @@ int ghost_impl(mr_grid *g, const TI *phi_in, TI *phi_out, int G, TP *P, TP *Q, i
   if (check_cuda(cudaFuncSetAttribute(prep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
                  "k_prep smem"))
     return MR_ERR_CUDA;
-  // The plain gather writes every region but the coarser leaves' of the
-  // padded block (of every needed leaf in a full fill, of the leaves with a
-  // coarser neighbour in the pre-pass-only modes); the pre-pass then takes
-  // the leaves with a coarser neighbour (pneed) from that prefilled block.
   const int tp = sizeof(TP) == 4 ? 4 : sizeof(TI) == 4 ? 5 : 8;
-  const int co = only_coarse ? 1 : 0;
-  {
-    static const int cf[3] = {256, 128, 512};
-    const int thr = tune_threads(g, TuneKey{0, N, NT, nb, tp, Gi, co}, cf, 3, [&](int th) {
-      k_fill_plain<TI, TP><<<n, th, 0, g->stream>>>(t, phi_in, P, Gi, need, g->pneed, g->cmask, err, co);
-    });
-    MR_LAUNCH(g, MRK_PART2, k_fill_plain<TI, TP><<<n, thr, 0, g->stream>>>(t, phi_in, P, Gi, need, g->pneed,
-                                                                          g->cmask, err, co));
-    if (check_cuda(cudaGetLastError(), "k_fill_plain")) return MR_ERR_CUDA;
-    if (!only_coarse) {  // (pre-pass-only modes: the pre-pass counts its leaves)
-      const double wd = nb + 2.0 * G;  // the requested shell (not the internal one)
-      count_units(g, MRK_PART2, need, n,
-                  (wd * wd * wd - (double)nb * nb * nb) * (double)(sizeof(TI) + sizeof(TP)), g->pneed);
-    }
-  }
-  const int *need_prep = g->pneed;
-  static const int cp[2] = {256, 128};
+  // 256 threads per leaf; more where the grid does not fill the chip (a leaf's
+  // phases are latency-bound: 120 leaves of 16^3 with 4.2)
+  const int big = sizeof(TP) == 4 ? 512 : 384, cp[2] = {n > 2 * 152 ? 256 : big, n > 2 * 152 ? 128 : 256};
   const int thp = tune_threads(g, TuneKey{1, N, NT, nb, tp, Gi, only_coarse}, cp, 2, [&](int th) {
-    prep<<<n, th, sm, g->stream>>>(t, phi_in, P, Q, Gi, G, only_coarse, g->cmask, err, need_prep, (int)sm);
+    prep<<<n, th, sm, g->stream>>>(t, phi_in, P, Q, Gi, G, only_coarse, g->cmask, err, need, g->pneed, (int)sm);
   });
-  MR_LAUNCH(g, MRK_PART1, prep<<<n, thp, sm, g->stream>>>(t, phi_in, P, Q, Gi, G, only_coarse, g->cmask, err,
-                                                          need_prep, (int)sm));
+  MR_LAUNCH(g, MRK_PART1, prep<<<n, thp, sm, g->stream>>>(t, phi_in, P, Q, Gi, G, only_coarse, g->cmask, err, need,
+                                                          g->pneed, (int)sm));
   if (check_cuda(cudaGetLastError(), "k_prep")) return MR_ERR_CUDA;
   if (only_coarse != 2) {  // the substitution-only pass fills no shell
-    const double wd = nb + 2.0 * G;
-    count_units(g, MRK_PART1, need_prep, n, (wd * wd * wd - (double)nb * nb * nb) * (double)(sizeof(TI) + sizeof(TP)));
+    const double wd = nb + 2.0 * G;  // the requested shell (not the internal one)
+    const double bytes = (wd * wd * wd - (double)nb * nb * nb) * (double)(sizeof(TI) + sizeof(TP));
+    count_units(g, MRK_PART1, g->pneed, n, bytes);
+    if (!only_coarse) count_units(g, MRK_PART2, need, n, bytes, g->pneed);  // leaves that only gather
   }
   if (only_coarse) return MR_OK;
   static const int cm[3] = {256, 128, 512};
