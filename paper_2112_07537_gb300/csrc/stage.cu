@@ -68,6 +68,11 @@ __device__ __forceinline__ const float *face_ptr(const FaceSrc &s, int ax, int i
   return s.base[(p >= hb) + 2 * (q >= hb)] + 2 * (i + nb * (j + nb * k));
 }
 
+// step from one z-plane to the next behind a face
+__device__ __forceinline__ int face_step(const FaceSrc &s, int nb, int Wd) {
+  return s.kind == 1 ? Wd * Wd : (nb * nb) << (s.kind == 2);
+}
+
 // one float from global to shared memory, asynchronously
 __device__ __forceinline__ void copy_async(float *dst, const float *src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
@@ -86,49 +91,52 @@ struct StageArgs {
   const float *vpad;  // ghost-filled velocity components (shell 3) or null
   float nu, vscale;
   int diff;
+  DivM dws;     // nb + 6
+  float cu, cv;  // the stage: cu u^n + cv (phi + dt r)
 };
 
-// RK3-TVD stage (or the bare rhs r) of one cell with value c
+// RK3-TVD stage (or the bare rhs r) of one cell with value c (uo: 0 in stage 0)
 __device__ __forceinline__ float stage_value(const StageArgs &s, float c, float r, float uo) {
-  if (s.rhs_only) return r;
-  const float v = c + s.dt * r;
-  return s.stage == 0 ? v : s.stage == 1 ? 0.75f * uo + 0.25f * v : (1.0f / 3) * uo + (2.0f / 3) * v;
+  return s.rhs_only ? r : fmaf(s.cv, fmaf(s.dt, r, c), s.cu * uo);
 }
 
 // ---------------------------------------------------------------------------
-// k_fused: one CTA per slab of nz z-planes.  Shared memory (floats):
+// k_fused: one CTA per slab of at most nz z-planes (the block is cut evenly, at
+// least three planes to a slab).  Shared memory (floats):
 //   T  [nz][nb+6][nb+7]  the slab's planes with their x and y ghosts
-//   H  [6][nb][nb]       three planes below and above the slab
 //   X  [nz][nb][nb+7]    half velocity u_x on the x rows (velocity fields);
 //                        each row's walk leaves its flux differences there
 //   Y  [nz][nb+6][nb]    likewise u_y on the y columns
 // (odd row pitch: threads on neighbouring x rows hit different banks).  The x
 // and y lines of the slab are walked first, one thread each with the same
-// code, then the z lines, whose thread finishes its cells (u_z and u^n are
-// read once, along x, straight from memory).  Bound by issued instructions
-// (ncu: 390 per point with velocity fields, issue slots 61 % busy, DRAM 27 %),
-// so every difference and smoothness term is evaluated once along a line;
-// slabs of a quarter block keep three CTAs (27 warps at nb = 24) on an SM, the
-// z walks' extra interface per slab costs 5 %.  Measured against the whole
-// block in one CTA (WENO-Z5, 6.2 ghosts): 3 424 leaves of 24^3 with velocity
-// fields 1 660 -> 755 us per launch, 42 400 leaves with a constant velocity
-// 15.35 -> 6.06 ms, 11 019 leaves of 16^3 with velocity fields 1 333 -> 843 us.
-// k_march takes 1 070 us, 8.5 ms and 1 047 us there.
+// code, then the z lines, whose thread finishes its cells.  What one thread
+// alone reads (the three values beyond each end of a z line, u_z, u^n) goes
+// straight to its registers, and copies advance by pointer increments: bound by
+// issued instructions (ncu), of which the flux arithmetic is about half.
+// Every difference and smoothness term is evaluated once along a line; slabs of
+// a quarter block keep three CTAs (27 warps at nb = 24) on an SM, the z walks'
+// extra interface per slab costs 5 %.  Measured against the whole block in one
+// CTA (WENO-Z5, 6.2 ghosts): 3 424 leaves of 24^3 with velocity fields 1 660 ->
+// 532 us per launch, 42 400 leaves with a constant velocity 15.35 -> 4.97 ms,
+// 11 019 leaves of 16^3 with velocity fields 1 333 -> 596 us (742 us, 6.02 ms and
+// 836 us with the planes around a slab in shared memory and an index per copy).
+// k_march takes 1 070 us, 8.5 ms and 1 047 us there; x and y walks in code of their
+// own are slower (590 us: the instruction cache).
 // ---------------------------------------------------------------------------
 __host__ __device__ constexpr int fused_smem_floats(int nb, int nz, bool vel) {
-  return nz * (nb + 6) * (nb + 7) + 6 * nb * nb + (vel ? nz * nb * (nb + 7) + nz * (nb + 6) * nb
-                                                        : nz * nb * (nb + 1) + nz * nb * nb);
+  return nz * (nb + 6) * (nb + 7) + (vel ? nz * nb * (nb + 7) + nz * (nb + 6) * nb : nz * nb * (nb + 1) + nz * nb * nb);
 }
 
 template <int SCHEME, bool VEL, bool LAP>
 __global__ void __launch_bounds__(288, 3) k_fused(Tree t, StageArgs s, int nz, int nslab) {
-  const int b = blockIdx.x / nslab, k0 = (blockIdx.x - b * nslab) * nz;
-  const int nb = t.nb, nb2 = nb * nb, Ws = nb + 6, RS = nb + 7, Wd = nb + 2 * s.Gi, nzs = min(nz, nb - k0);
-  const int tid = threadIdx.x, bd = blockDim.x;
+  const int b = blockIdx.x / nslab, sl = blockIdx.x - b * nslab;
+  const int nb = t.nb, nb2 = nb * nb, Ws = nb + 6, W2 = Ws * Ws, RS = nb + 7, Wd = nb + 2 * s.Gi;
+  const int k0 = sl * nb / nslab, nzs = (sl + 1) * nb / nslab - k0;
+  const int tid = threadIdx.x, bd = blockDim.x, tst = Ws * RS;
   const int L = __ldg(t.lev + b);
   const int a[3] = {__ldg(t.anc + 3 * b) * nb, __ldg(t.anc + 3 * b + 1) * nb, __ldg(t.anc + 3 * b + 2) * nb};
   extern __shared__ float sm[];
-  float *T = sm, *H = T + nz * Ws * RS, *X = H + 6 * nb2, *Y = X + nz * nb * (VEL ? RS : nb + 1);
+  float *T = sm, *X = T + nz * tst, *Y = X + nz * nb * (VEL ? RS : nb + 1);
   __shared__ FaceSrc fs[6];
   face_sources(t, b, L, a, s.phi, s.P, s.Q, s.Gi, s.lifted, fs);
   const DivM dnb = t.dnb;
@@ -137,59 +145,48 @@ __global__ void __launch_bounds__(288, 3) k_fused(Tree t, StageArgs s, int nz, i
   // Every value goes to shared memory by an asynchronous copy of its own (all
   // in flight at once; nothing waits for memory before the barrier).  Each
   // thread keeps its (x, y) and steps through the planes.
-  // Interior planes of the slab and of its z neighbourhood inside the leaf:
-  // the field, or the substituted block that the pre-pass wrote.
-  {
-    const int ka = max(k0 - 3, 0), kb = min(k0 + nzs + 3, nb);
-    const bool pad = s.cmask[b] != 0;
-    const int sy = pad ? Wd : nb, sz = pad ? Wd * Wd : nb2;
-    const float *src = (pad ? s.P + (size_t)b * Wd * Wd * Wd + s.Gi * (1 + Wd + Wd * Wd)
-                            : s.phi + (size_t)b * nb2 * nb) + (size_t)ka * sz;
-    for (int c = tid; c < nb2; c += bd) {
-      const int j = divq(c, dnb), i = c - j * nb;
-      const float *p = src + i + sy * j;
-      float *tp = T + (j + 3) * RS + i + 3, *hp = H + c;
-      for (int z = ka - k0; z < kb - k0; ++z, p += sz)
-        copy_async(z < 0 ? hp + (z + 3) * nb2 : z < nzs ? tp + z * Ws * RS : hp + (z - nzs + 3) * nb2, p);
-    }
+  // Interior of the leaf: the field, or the substituted block that the pre-pass wrote.
+  const bool pad = s.cmask[b] != 0;
+  const int sy = pad ? Wd : nb, sz = sy * sy;
+  const float *src = (pad ? s.P + (size_t)b * Wd * sz + s.Gi * (1 + Wd + sz) : s.phi + (size_t)b * nb2 * nb) + k0 * sz;
+  for (int c = tid; c < nb2; c += bd) {
+    const int j = divq(c, dnb), i = c - j * nb;
+    const float *p = src + i + sy * j;
+    float *tp = T + (j + 3) * RS + i + 3;
+#pragma unroll 2
+    for (int k = 0; k < nzs; ++k, p += sz, tp += tst) copy_async(tp, p);
   }
   const float hscale = 0.5f * s.vscale;
-  const size_t vblk = (size_t)Ws * Ws * Ws;
-  const float *vb = VEL ? s.vpad + (size_t)b * vblk : nullptr;
+  const size_t vblk = (size_t)W2 * Ws;
+  const float *vb = VEL ? s.vpad + (size_t)b * vblk + k0 * W2 : nullptr;
   const size_t vcomp = (size_t)t.nleaf * vblk;
   if (VEL) {
-    const DivM dws = divm(Ws);
-    const float *vx = vb + (size_t)Ws * Ws * (k0 + 3) + 3 * Ws, *vy = vb + vcomp + (size_t)Ws * Ws * (k0 + 3) + 3;
+    const float *vx = vb + 3 * W2 + 3 * Ws, *vy = vb + vcomp + 3 * W2 + 3;
     for (int c = tid; c < nb * Ws; c += bd) {
-      const int j = divq(c, dws), x = c - j * Ws, jy = divq(c, dnb), i = c - jy * nb;
+      const int j = divq(c, s.dws), x = c - j * Ws, jy = divq(c, dnb), i = c - jy * nb;
       float *xp = X + j * RS + x, *yp = Y + c;
       const float *px = vx + c, *py = vy + i + Ws * jy;
-      for (int k = 0; k < nzs; ++k) {
-        copy_async(xp + k * nb * RS, px + k * Ws * Ws);
-        copy_async(yp + k * Ws * nb, py + k * Ws * Ws);
+      for (int k = 0; k < nzs; ++k, xp += nb * RS, yp += Ws * nb, px += W2, py += W2) {
+        copy_async(xp, px);
+        copy_async(yp, py);
       }
     }
   }
   __syncthreads();  // fs
-  // ghosts: x and y of the slab's planes, z planes beyond the leaf
-  for (int c = tid; c < nb * 6; c += bd) {
-    const int j = c / 6, m = c - 6 * j, i = m < 3 ? m - 3 : nb + m - 3;
-    const FaceSrc &f = fs[m < 3 ? 0 : 1];
+  // x and y ghosts of the slab's planes
+  for (int c = tid; c < 12 * nb; c += bd) {
+    const bool yd = c >= 6 * nb;
+    const int cc = yd ? c - 6 * nb : c, q = yd ? divq(cc, dnb) : cc / 6, r = cc - q * (yd ? nb : 6);
+    const int m = yd ? q : r, o = m < 3 ? m - 3 : nb + m - 3;  // ghost layer
+    const int i = yd ? r : o, j = yd ? o : q;
+    const FaceSrc &f = fs[2 * yd + (m >= 3)];
     float *tp = T + (j + 3) * RS + i + 3;
-    for (int k = 0; k < nzs; ++k) copy_async(tp + k * Ws * RS, face_ptr(f, 0, i, j, k0 + k, nb, Wd));
-  }
-  for (int c = tid; c < 6 * nb; c += bd) {
-    const int m = divq(c, dnb), i = c - m * nb, j = m < 3 ? m - 3 : nb + m - 3;
-    const FaceSrc &f = fs[m < 3 ? 2 : 3];
-    float *tp = T + (j + 3) * RS + i + 3;
-    for (int k = 0; k < nzs; ++k) copy_async(tp + k * Ws * RS, face_ptr(f, 1, i, j, k0 + k, nb, Wd));
-  }
-  for (int h = 0; h < 6; ++h) {
-    const int z = h < 3 ? k0 + h - 3 : k0 + nzs + h - 3;
-    if (z >= 0 && z < nb) continue;
-    for (int c = tid; c < nb2; c += bd) {
-      const int j = divq(c, dnb), i = c - j * nb;
-      copy_async(H + h * nb2 + c, face_ptr(fs[z < 0 ? 4 : 5], 2, i, j, z, nb, Wd));
+    const float *p = face_ptr(f, yd, i, j, k0, nb, Wd);
+    const int st = face_step(f, nb, Wd);
+    const bool two = f.kind == 2;
+    for (int k = 0; k < nzs; ++k, p += st, tp += tst) {
+      if (two && k0 + k == nb / 2) p = face_ptr(f, yd, i, j, k0 + k, nb, Wd);  // the next finer leaf
+      copy_async(tp, p);
     }
   }
   copy_wait();
@@ -226,44 +223,82 @@ __global__ void __launch_bounds__(288, 3) k_fused(Tree t, StageArgs s, int nz, i
           [&](int m, float dF, float, float lap) { ve[m * d * sv] = LAP ? fmaf(-lk, lap, dF) : dF; });
     }
   }
+  // z lines.  The three values beyond either end of the slab: the leaf's own
+  // planes or the ghosts behind its z faces, loaded for the thread's first line
+  // before the barrier.
+  const bool down = !VEL && s.uz < 0.f;  // walk direction
+  const int e = down ? nzs - 1 : 0, d = down ? -1 : 1;
+  float lo[3], hi[3];  // in walk order
+  auto ends = [&](int c) {
+    const int j = divq(c, dnb), i = c - j * nb;
+    auto line = [&](bool top, float *v) {
+      const int z = top ? nzs : -3;
+      const FaceSrc &f = fs[4 + top];
+      const bool own = top ? k0 + nzs < nb : k0 > 0;
+      const float *p = own ? src + i + sy * j + z * sz : face_ptr(f, 2, i, j, k0 + z, nb, Wd);
+      const int st = own ? sz : face_step(f, nb, Wd);
+      const float v0 = __ldg(p), v1 = __ldg(p + st), v2 = __ldg(p + 2 * st);
+      v[0] = down ? v2 : v0, v[1] = v1, v[2] = down ? v0 : v2;
+    };
+    line(down, lo), line(!down, hi);
+  };
+  if (tid < nb2) ends(tid);
   __syncthreads();
   const bool rk_u = !s.rhs_only && s.stage > 0;
+  const float k2 = -2.f * invh;
+  const int xst = (VEL ? nb * RS : nb * (nb + 1)) * d, yst = (VEL ? Ws * nb : nb2) * d;
+  const ptrdiff_t gst = d * nb2;
   for (int c = tid; c < nb2; c += bd) {
     const int j = divq(c, dnb), i = c - j * nb;
-    const float *tp = T + (j + 3) * RS + i + 3, *hp = H + c;
-    const int tst = Ws * RS;
-    const float *xp = VEL ? X + j * RS + i + 3 : X + j * (nb + 1) + i;
-    const float *yp = VEL ? Y + (j + 3) * nb + i : Y + c;
-    const int xst = VEL ? nb * RS : nb * (nb + 1), yst = VEL ? Ws * nb : nb2;
-    const size_t q0 = (size_t)b * nb2 * nb + (size_t)k0 * nb2 + c;
+    const float *tp = T + (j + 3) * RS + i + 3 + e * tst;
+    const float *xp = (VEL ? X + j * RS + i + 3 : X + j * (nb + 1) + i) + e * d * xst;
+    const float *yp = (VEL ? Y + (j + 3) * nb + i : Y + c) + e * d * yst;
+    const size_t q0 = (size_t)b * nb2 * nb + (k0 + e) * nb2 + c;
     const float *up = s.u + q0;
-    auto phi = [&](int m) { return m < 0 ? hp[(m + 3) * nb2] : m < nzs ? tp[m * tst] : hp[(m - nzs + 3) * nb2]; };
-    const int e = !VEL && s.uz < 0.f ? nzs - 1 : 0, d = !VEL && s.uz < 0.f ? -1 : 1;  // walk direction
-    float un = rk_u ? up[(size_t)e * nb2] : 0.f;  // u^n one cell ahead
-    auto finish = [&](int m, float dF, float ph, float lap) {
-      const float uo = un;
-      const int z = e + d * m;
-      if (rk_u && m + 1 < nzs) un = up[(size_t)(z + d) * nb2];
+    float *op = s.out + q0;
+    const int pst = d * tst;
+    float uo = rk_u ? *up : 0.f;  // u^n of the current cell
+    auto finish = [&](float dF, float ph, float lap) {
       float acc = LAP ? fmaf(-lk, lap, dF) : dF;
-      acc = (xon ? xp[z * xst] : 0.f) + (yon ? yp[z * yst] : 0.f) + acc;
-      s.out[q0 + (size_t)z * nb2] = stage_value(s, ph, -2.f * (acc * invh), uo);
+      acc = (xon ? *xp : 0.f) + (yon ? *yp : 0.f) + acc;
+      *op = stage_value(s, ph, acc * k2, uo);
+      xp += xst, yp += yst, op += gst;
     };
-    if (VEL) {
-      const float *vz = vb + 2 * vcomp + (size_t)Ws * Ws * k0 + Ws * (j + 3) + i + 3;  // plane k0 - 3
-      float nxt = __ldg(vz);
-      auto hv = [&](int m) {
-        const float v = nxt;
-        if (m + 1 < nzs + 3) nxt = __ldg(vz + (size_t)Ws * Ws * (m + 4));  // one plane ahead
-        return rmul(hscale, v);
-      };
-      walk_line<float, SCHEME, LAP, false>(nzs, s.diff, phi, hv, finish);
-    } else if (zon) {
+    if (zon) {
+      const float *vp = vb + 2 * vcomp + Ws * (j + 3) + i + 3;  // plane k0 - 3
+      float vz[7];
+#pragma unroll
+      for (int x = 0; x < 7; ++x, vp += W2) vz[x] = VEL ? __ldg(vp) : 0.f;
       const float hu = 0.5f * fabsf(s.uz);
-      walk_line<float, SCHEME, LAP, true>(nzs, s.diff, [&](int m) { return phi(e + d * m); },
-                                          [&](int) { return hu; }, finish);
+      auto half = [&](float v) { return VEL ? rmul(hscale, v) : hu; };
+      Walk<float, SCHEME, LAP, !VEL> w;
+      w.start([&](int m) { return m < 0 ? lo[m + 3] : tp[m * pst]; }, [&](int m) { return half(vz[m + 3]); });
+      float vn = vz[6];  // one plane ahead
+      tp += 3 * pst;
+      auto cell = [&](float an, bool more) {
+        const float v = vn, un = uo;
+        if (more) {  // the next cell's velocity and u^n
+          if (VEL) vn = __ldg(vp), vp += W2;
+          up += gst;
+          if (rk_u) uo = *up;
+        }
+        const float nx = uo;
+        uo = un;
+        w.step(0, s.diff, an, half(v), [&](int, float dF, float ph, float lap) { finish(dF, ph, lap); });
+        uo = nx;
+      };
+#pragma unroll 3
+      for (int m = 3; m < nzs; ++m, tp += pst) cell(*tp, true);
+      cell(hi[0], true);
+      cell(hi[1], true);
+      cell(hi[2], false);
     } else {
-      for (int m = 0; m < nzs; ++m) finish(m, 0.f, phi(e + d * m), 0.f);
+      for (int m = 0; m < nzs; ++m, tp += pst, up += gst) {
+        if (rk_u) uo = *up;
+        finish(0.f, *tp, 0.f);
+      }
     }
+    if (c + bd < nb2) ends(c + bd);
   }
 }
 
@@ -507,7 +542,8 @@ int launch_fused(mr_grid *g, const void *phi, const void *P, const void *Q, int 
   }
   StageArgs s{(const float *)phi, (const float *)P, (const float *)Q, Gi, NT != 0, g->cmask, (const float *)u,
               (float *)out, stage, rhs_only ? 1 : 0, (float)dt, (float)uc[0], (float)uc[1], (float)uc[2],
-              (const float *)vpad, (float)g->diff_nu, (float)g->vel_scale, g->diff_order};
+              (const float *)vpad, (float)g->diff_nu, (float)g->vel_scale, g->diff_order, divm(nb + 6),
+              stage == 0 ? 0.f : stage == 1 ? 0.75f : 1.0f / 3, stage == 0 ? 1.f : stage == 1 ? 0.25f : 2.0f / 3};
   const bool march_ok = nb >= 12 && nb * nb <= 576;
   const size_t smm = sizeof(float) * (size_t)march_smem_floats(nb, vel);
   // slab heights: a quarter of the block (at least four planes), or four planes
@@ -527,7 +563,7 @@ int launch_fused(mr_grid *g, const void *phi, const void *P, const void *Q, int 
       return MR_ERR_CUDA;
     const int mode = 2 * scheme + (vel ? 1 : 0);
     auto fused = [&](int th) {
-      const int nz = th == cand[0] ? hq : ht, ns = (nb + nz - 1) / nz;
+      const int ns = (nb + (th == cand[0] ? hq : ht) - 1) / (th == cand[0] ? hq : ht), nz = (nb + ns - 1) / ns;
       kf<<<g->nleaf * ns, th, sizeof(float) * fused_smem_floats(nb, nz, vel), g->stream>>>(t, s, nz, ns);
     };
     auto march = [&]() { km<<<g->nleaf, nb * nb, smm, g->stream>>>(t, s); };
