@@ -78,7 +78,17 @@ __device__ __forceinline__ void copy_async(float *dst, const float *src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
                : "memory");
 }
+// two floats (both addresses multiples of 8)
+__device__ __forceinline__ void copy_async2(float *dst, const float *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
 __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// n floats from global memory into the L2 cache (16-byte multiples)
+__device__ __forceinline__ void prefetch_l2(const float *p, int n) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(4 * n) : "memory");
+}
 
 struct StageArgs {
   const float *phi, *P, *Q;
@@ -103,73 +113,102 @@ __device__ __forceinline__ float stage_value(const StageArgs &s, float c, float 
 // ---------------------------------------------------------------------------
 // k_fused: one CTA per slab of at most nz z-planes (the block is cut evenly, at
 // least three planes to a slab).  Shared memory (floats):
-//   T  [nz][nb+6][nb+7]  the slab's planes with their x and y ghosts
-//   X  [nz][nb][nb+7]    half velocity u_x on the x rows (velocity fields);
+//   T  [nz][nb+6][RS]    the slab's planes with their x and y ghosts
+//   X  [nz][nb][XS]      half velocity u_x on the x rows (velocity fields);
 //                        each row's walk leaves its flux differences there
 //   Y  [nz][nb+6][nb]    likewise u_y on the y columns
-// (odd row pitch: threads on neighbouring x rows hit different banks).  The x
-// and y lines of the slab are walked first, one thread each with the same
-// code, then the z lines, whose thread finishes its cells.  What one thread
-// alone reads (the three values beyond each end of a z line, u_z, u^n) goes
-// straight to its registers, and copies advance by pointer increments: bound by
-// issued instructions (ncu), of which the flux arithmetic is about half.
-// Every difference and smoothness term is evaluated once along a line; slabs of
-// a quarter block keep three CTAs (27 warps at nb = 24) on an SM, the z walks'
-// extra interface per slab costs 5 %.  Measured against the whole block in one
-// CTA (WENO-Z5, 6.2 ghosts): 3 424 leaves of 24^3 with velocity fields 1 660 ->
-// 532 us per launch, 42 400 leaves with a constant velocity 15.35 -> 4.97 ms,
-// 11 019 leaves of 16^3 with velocity fields 1 333 -> 596 us (742 us, 6.02 ms and
-// 836 us with the planes around a slab in shared memory and an index per copy).
-// k_march takes 1 070 us, 8.5 ms and 1 047 us there; x and y walks in code of their
-// own are slower (590 us: the instruction cache).
+// The x and y lines of the slab are walked first, a pair of lines per thread
+// with the same code, then the z lines (pairs of neighbours in x), whose thread
+// finishes its cells.  What one thread alone reads (the three values beyond each
+// end of a z line, u_z, u^n) goes straight to its registers.  Bound by issued
+// instructions and by the latency of the copies: the packed walk issues 243
+// instructions per point (velocity fields) where one line per thread issued 323
+// and an index per copy and planes around the slab in shared memory 388; the
+// copies alone take 40 to 57 % of the time, overlapped with the walks of the
+// other CTAs.  Slabs of a quarter block (half of a block of at most 16) keep
+// three CTAs on an SM with velocity fields (more would spill), four without; the
+// z walks' extra interface per slab costs 5 %.  Measured per launch (WENO-Z5,
+// 6.2 ghosts): 3 424 leaves of 24^3 with velocity fields 1 660 us (whole block per
+// CTA), 742 (slabs), 530 (fewer copies), 527 (packed); 42 400 leaves with a
+// constant velocity 15.35 ms, 6.02, 4.97, 3.99; 11 019 leaves of 16^3 with velocity
+// fields 1 333 us, 836, 596, 476; 1 272 leaves with diffusion 104 us, 89, 74.
+// k_march takes 1 070 us, 8.5 ms and 1 047 us in the first three.  Separate code for
+// x and y walks, or unrolled z walks, is slower by a tenth (instruction cache).
 // ---------------------------------------------------------------------------
+// row pitch for n floats per row: twice an odd number (two-way bank conflicts at
+// worst where neighbouring threads walk neighbouring rows)
+__host__ __device__ constexpr int fused_pitch(int n) { return n + (n % 4 == 0 ? 2 : 0); }
 __host__ __device__ constexpr int fused_smem_floats(int nb, int nz, bool vel) {
-  return nz * (nb + 6) * (nb + 7) + (vel ? nz * nb * (nb + 7) + nz * (nb + 6) * nb : nz * nb * (nb + 1) + nz * nb * nb);
+  return nz * (nb + 6) * fused_pitch(nb + 6) + 2 + nz * nb * fused_pitch(vel ? nb + 6 : nb) +
+         nz * (vel ? nb + 6 : nb) * nb;
 }
 
 template <int SCHEME, bool VEL, bool LAP>
-__global__ void __launch_bounds__(288, 3) k_fused(Tree t, StageArgs s, int nz, int nslab) {
+__global__ void __launch_bounds__(160, VEL ? 3 : 4) k_fused(Tree t, StageArgs s, int nz, int nslab) {
   const int b = blockIdx.x / nslab, sl = blockIdx.x - b * nslab;
-  const int nb = t.nb, nb2 = nb * nb, Ws = nb + 6, W2 = Ws * Ws, RS = nb + 7, Wd = nb + 2 * s.Gi;
+  const int nb = t.nb, nb2 = nb * nb, Ws = nb + 6, W2 = Ws * Ws, RS = fused_pitch(nb + 6),
+            XS = VEL ? RS : fused_pitch(nb), Wd = nb + 2 * s.Gi;
   const int k0 = sl * nb / nslab, nzs = (sl + 1) * nb / nslab - k0;
   const int tid = threadIdx.x, bd = blockDim.x, tst = Ws * RS;
   const int L = __ldg(t.lev + b);
   const int a[3] = {__ldg(t.anc + 3 * b) * nb, __ldg(t.anc + 3 * b + 1) * nb, __ldg(t.anc + 3 * b + 2) * nb};
-  extern __shared__ float sm[];
-  float *T = sm, *X = T + nz * tst, *Y = X + nz * nb * (VEL ? RS : nb + 1);
+  extern __shared__ __align__(16) float sm[];
+  // (x = -3 is column 1 of a row, x = nb + 2 the first float of the next one)
+  float *T = sm, *X = T + nz * tst + 2, *Y = X + nz * nb * XS;
   __shared__ FaceSrc fs[6];
   face_sources(t, b, L, a, s.phi, s.P, s.Q, s.Gi, s.lifted, fs);
   const DivM dnb = t.dnb;
   __shared__ float sh_h;
-  if (tid == 32) sh_h = (float)(t.tree_len / ((double)nb * (double)(1 << L)));
-  // Every value goes to shared memory by an asynchronous copy of its own (all
-  // in flight at once; nothing waits for memory before the barrier).  Each
-  // thread keeps its (x, y) and steps through the planes.
+  if (tid == bd - 1) sh_h = (float)(t.tree_len / ((double)nb * (double)(1 << L)));
+  // Values go to shared memory by asynchronous copies (all in flight at once;
+  // nothing waits for memory before the barrier), two floats each where the
+  // source allows it.  Each thread keeps its (x, y) and steps through the planes.
   // Interior of the leaf: the field, or the substituted block that the pre-pass wrote.
   const bool pad = s.cmask[b] != 0;
   const int sy = pad ? Wd : nb, sz = sy * sy;
   const float *src = (pad ? s.P + (size_t)b * Wd * sz + s.Gi * (1 + Wd + sz) : s.phi + (size_t)b * nb2 * nb) + k0 * sz;
-  for (int c = tid; c < nb2; c += bd) {
-    const int j = divq(c, dnb), i = c - j * nb;
-    const float *p = src + i + sy * j;
-    float *tp = T + (j + 3) * RS + i + 3;
+  if (!pad || !(s.Gi & 1)) {  // rows at even addresses
+    for (int c = tid; c < nb2 / 2; c += bd) {
+      const int j = divq(2 * c, dnb), i = 2 * c - j * nb;
+      const float *p = src + i + sy * j;
+      float *tp = T + (j + 3) * RS + i + 4;
 #pragma unroll 2
-    for (int k = 0; k < nzs; ++k, p += sz, tp += tst) copy_async(tp, p);
+      for (int k = 0; k < nzs; ++k, p += sz, tp += tst) copy_async2(tp, p);
+    }
+  } else {
+    for (int c = tid; c < nb2; c += bd) {
+      const int j = divq(c, dnb), i = c - j * nb;
+      const float *p = src + i + sy * j;
+      float *tp = T + (j + 3) * RS + i + 4;
+      for (int k = 0; k < nzs; ++k, p += sz, tp += tst) copy_async(tp, p);
+    }
   }
   const float hscale = 0.5f * s.vscale;
   const size_t vblk = (size_t)W2 * Ws;
   const float *vb = VEL ? s.vpad + (size_t)b * vblk + k0 * W2 : nullptr;
   const size_t vcomp = (size_t)t.nleaf * vblk;
+  // u_z and u^n are read one plane ahead of the z walks: less than memory's
+  // latency, more than that of the L2 cache
+  const bool rk_u = !s.rhs_only && s.stage > 0;
+  if (tid == bd - 1) {
+    if (VEL) prefetch_l2(vb + 2 * vcomp, (nzs + 6) * W2);
+    if (rk_u) prefetch_l2(s.u + (size_t)b * nb2 * nb + k0 * nb2, nzs * nb2);
+  }
   if (VEL) {
     const float *vx = vb + 3 * W2 + 3 * Ws, *vy = vb + vcomp + 3 * W2 + 3;
+    for (int c = tid; c < nb * Ws / 2; c += bd) {
+      const int j = divq(2 * c, s.dws), x = 2 * c - j * Ws;
+      float *xp = X + j * XS + x;
+      const float *px = vx + 2 * c;
+#pragma unroll 2
+      for (int k = 0; k < nzs; ++k, xp += nb * XS, px += W2) copy_async2(xp, px);
+    }
     for (int c = tid; c < nb * Ws; c += bd) {
-      const int j = divq(c, s.dws), x = c - j * Ws, jy = divq(c, dnb), i = c - jy * nb;
-      float *xp = X + j * RS + x, *yp = Y + c;
-      const float *px = vx + c, *py = vy + i + Ws * jy;
-      for (int k = 0; k < nzs; ++k, xp += nb * RS, yp += Ws * nb, px += W2, py += W2) {
-        copy_async(xp, px);
-        copy_async(yp, py);
-      }
+      const int j = divq(c, dnb), i = c - j * nb;
+      float *yp = Y + c;
+      const float *py = vy + i + Ws * j;
+#pragma unroll 2
+      for (int k = 0; k < nzs; ++k, yp += Ws * nb, py += W2) copy_async(yp, py);
     }
   }
   __syncthreads();  // fs
@@ -180,7 +219,7 @@ __global__ void __launch_bounds__(288, 3) k_fused(Tree t, StageArgs s, int nz, i
     const int m = yd ? q : r, o = m < 3 ? m - 3 : nb + m - 3;  // ghost layer
     const int i = yd ? r : o, j = yd ? o : q;
     const FaceSrc &f = fs[2 * yd + (m >= 3)];
-    float *tp = T + (j + 3) * RS + i + 3;
+    float *tp = T + (j + 3) * RS + i + 4;
     const float *p = face_ptr(f, yd, i, j, k0, nb, Wd);
     const int st = face_step(f, nb, Wd);
     const bool two = f.kind == 2;
@@ -194,111 +233,123 @@ __global__ void __launch_bounds__(288, 3) k_fused(Tree t, StageArgs s, int nz, i
   const float invh = 1.0f / sh_h;
   const float lk = LAP ? 0.5f * s.nu * invh : 0.f;  // rhs = -2/h (dF - lk lap)
   const bool xon = VEL || LAP || s.ux != 0.f, yon = VEL || LAP || s.uy != 0.f, zon = VEL || LAP || s.uz != 0.f;
-  // x lines, then y lines: base and pitch of the line in T and in X / Y.  A
-  // constant velocity u < 0 is walked in the other direction with |u|: the
-  // right-biased flux of u phi is minus the left-biased one of |u| phi on the
-  // mirrored line, and the order of the difference reverses with it.  So
-  // neither sign selects an upwind side.
-  const int nl = nb * nzs;
-  for (int idx = tid; idx < 2 * nl; idx += bd) {
-    const bool yd = idx >= nl;
+  // Pairs of x lines, then of y lines: line q and line q + np, which lie os and
+  // ov floats apart in T and in X / Y (y lines: neighbours, np = 1).  A constant
+  // velocity u < 0 is walked in the other direction with |u|: the right-biased
+  // flux of u phi is minus the left-biased one of |u| phi on the mirrored line,
+  // and the order of the difference reverses with it.  So neither sign selects
+  // an upwind side.
+  const int np = nb * nzs / 2;
+  for (int idx = tid; idx < 2 * np; idx += bd) {
+    const bool yd = idx >= np;
     if (yd ? !yon : !xon) continue;
-    const int q = yd ? idx - nl : idx, k = divq(q, dnb), l = q - k * nb;
-    const float *p = T + (yd ? (k * Ws + 3) * RS + l + 3 : (k * Ws + l + 3) * RS + 3);
-    const int st = yd ? RS : 1;
-    if (VEL) {
-      float *v = yd ? Y + (k * Ws + 3) * nb + l : X + q * RS + 3;
-      const int sv = yd ? nb : 1;
-      walk_line<float, SCHEME, LAP, false>(
-          nb, s.diff, [&](int m) { return p[m * st]; }, [&](int m) { return rmul(hscale, v[m * sv]); },
-          [&](int m, float dF, float, float lap) { v[m * sv] = LAP ? fmaf(-lk, lap, dF) : dF; });
-    } else {
-      float *v = yd ? Y + k * nb2 + l : X + q * (nb + 1);
-      const float uu = yd ? s.uy : s.ux, hu = 0.5f * fabsf(uu);
-      const int e = uu >= 0.f ? 0 : nb - 1, sv = yd ? nb : 1, d = uu >= 0.f ? 1 : -1;
-      const float *pe = p + e * st;
-      float *ve = v + e * sv;
-      walk_line<float, SCHEME, LAP, true>(
-          nb, s.diff, [&](int m) { return pe[m * d * st]; }, [&](int) { return hu; },
-          [&](int m, float dF, float, float lap) { ve[m * d * sv] = LAP ? fmaf(-lk, lap, dF) : dF; });
+    const int q = yd ? 2 * (idx - np) : idx, k = divq(q, dnb), l = q - k * nb;
+    const int q2 = yd ? q + 1 : q + np, k2 = divq(q2, dnb), l2 = q2 - k2 * nb;
+    const float *p = T + (yd ? (k * Ws + 3) * RS + l + 4 : (k * Ws + l + 3) * RS + 4);
+    const int st = yd ? RS : 1, os = yd ? 1 : ((k2 - k) * Ws + l2 - l) * RS, ov = yd ? 1 : np * XS;
+    // (the differences of an x row go one float further than its velocities: to
+    // even addresses, and never ahead of the velocities still to be read)
+    float *v = yd ? Y + (VEL ? (k * Ws + 3) * nb : k * nb2) + l : X + q * XS + (VEL ? 3 : -1);
+    const int sv = yd ? nb : 1, oe = yd ? 0 : 1;
+    const float uu = VEL ? 0.f : yd ? s.uy : s.ux, hu = 0.5f * fabsf(uu);
+    const bool rev = !VEL && uu < 0.f;
+    const int dst = rev ? -st : st, dsv = rev ? -sv : sv;
+    p += rev ? (nb - 1) * st : 0;
+    float *w = v + oe + (rev ? (nb - 1) * sv : 0);
+    auto phi = [&](int m) { return make_float2(p[m * dst], p[m * dst + os]); };
+    auto hv = [&](int m) {
+      return VEL ? pmul(both(hscale), make_float2(v[m * sv], v[m * sv + ov])) : both(hu);
+    };
+    Walk2<SCHEME, LAP, !VEL> wk;
+    wk.start(phi, hv);
+#pragma unroll 4
+    for (int m = 0; m < nb; ++m) {
+      const float2 vn = hv(m + 3), an = phi(m + 3);
+      wk.step(s.diff, an, vn, [&](float2 dF, float2, float2 lap) {
+        if (LAP) dF = pfma(-lk, lap, dF);
+        w[m * dsv] = dF.x, w[m * dsv + ov] = dF.y;
+      });
     }
   }
-  // z lines.  The three values beyond either end of the slab: the leaf's own
-  // planes or the ghosts behind its z faces, loaded for the thread's first line
-  // before the barrier.
+  // z lines, pairs of neighbours in x.  The three values beyond either end of the
+  // slab: the leaf's own planes or the ghosts behind its z faces, loaded for the
+  // thread's first pair before the barrier.
   const bool down = !VEL && s.uz < 0.f;  // walk direction
   const int e = down ? nzs - 1 : 0, d = down ? -1 : 1;
-  float lo[3], hi[3];  // in walk order
+  float2 lo[3], hi[3];  // in walk order
   auto ends = [&](int c) {
-    const int j = divq(c, dnb), i = c - j * nb;
-    auto line = [&](bool top, float *v) {
+    const int j = divq(2 * c, dnb), i = 2 * c - j * nb;
+    auto line = [&](bool top, float2 *v) {
       const int z = top ? nzs : -3;
       const FaceSrc &f = fs[4 + top];
       const bool own = top ? k0 + nzs < nb : k0 > 0;
       const float *p = own ? src + i + sy * j + z * sz : face_ptr(f, 2, i, j, k0 + z, nb, Wd);
       const int st = own ? sz : face_step(f, nb, Wd);
-      const float v0 = __ldg(p), v1 = __ldg(p + st), v2 = __ldg(p + 2 * st);
+      // (the two points of a pair lie in the same quadrant of a face: nb / 2 odd
+      // is the exception)
+      const float *p2 = own || f.kind != 2 ? p + 1 : face_ptr(f, 2, i + 1, j, k0 + z, nb, Wd);
+      const float2 v0 = make_float2(__ldg(p), __ldg(p2)), v1 = make_float2(__ldg(p + st), __ldg(p2 + st)),
+                   v2 = make_float2(__ldg(p + 2 * st), __ldg(p2 + 2 * st));
       v[0] = down ? v2 : v0, v[1] = v1, v[2] = down ? v0 : v2;
     };
     line(down, lo), line(!down, hi);
   };
-  if (tid < nb2) ends(tid);
+  const int nc = nb2 / 2;
+  if (tid < nc) ends(tid);
   __syncthreads();
-  const bool rk_u = !s.rhs_only && s.stage > 0;
   const float k2 = -2.f * invh;
-  const int xst = (VEL ? nb * RS : nb * (nb + 1)) * d, yst = (VEL ? Ws * nb : nb2) * d;
+  const int xst = nb * XS * d, yst = (VEL ? Ws * nb : nb2) * d, pst = d * tst;
   const ptrdiff_t gst = d * nb2;
-  for (int c = tid; c < nb2; c += bd) {
-    const int j = divq(c, dnb), i = c - j * nb;
-    const float *tp = T + (j + 3) * RS + i + 3 + e * tst;
-    const float *xp = (VEL ? X + j * RS + i + 3 : X + j * (nb + 1) + i) + e * d * xst;
-    const float *yp = (VEL ? Y + (j + 3) * nb + i : Y + c) + e * d * yst;
-    const size_t q0 = (size_t)b * nb2 * nb + (k0 + e) * nb2 + c;
+  auto ld2 = [](const float *p) { return *reinterpret_cast<const float2 *>(p); };
+  for (int c = tid; c < nc; c += bd) {
+    const int j = divq(2 * c, dnb), i = 2 * c - j * nb;
+    const float *tp = T + (j + 3) * RS + i + 4 + e * tst;
+    const float *xp = X + j * XS + i + (VEL ? 4 : 0) + e * d * xst;
+    const float *yp = (VEL ? Y + (j + 3) * nb + i : Y + 2 * c) + e * d * yst;
+    const size_t q0 = (size_t)b * nb2 * nb + (k0 + e) * nb2 + 2 * c;
     const float *up = s.u + q0;
     float *op = s.out + q0;
-    const int pst = d * tst;
-    float uo = rk_u ? *up : 0.f;  // u^n of the current cell
-    auto finish = [&](float dF, float ph, float lap) {
-      float acc = LAP ? fmaf(-lk, lap, dF) : dF;
-      acc = (xon ? *xp : 0.f) + (yon ? *yp : 0.f) + acc;
-      *op = stage_value(s, ph, acc * k2, uo);
+    float2 uo = rk_u ? ld2(up) : both(0.f);  // u^n of the current cell
+    auto finish = [&](float2 dF, float2 ph, float2 lap, float2 un) {
+      const float2 acc = padd(padd(xon ? ld2(xp) : both(0.f), yon ? ld2(yp) : both(0.f)), LAP ? pfma(-lk, lap, dF) : dF);
+      float2 r = pmul(acc, both(k2));
+      if (!s.rhs_only) r = pfma(s.cv, pfma(s.dt, r, ph), pmul(both(s.cu), un));
+      *reinterpret_cast<float2 *>(op) = r;
       xp += xst, yp += yst, op += gst;
     };
     if (zon) {
       const float *vp = vb + 2 * vcomp + Ws * (j + 3) + i + 3;  // plane k0 - 3
-      float vz[7];
+      float2 vz[7];
 #pragma unroll
-      for (int x = 0; x < 7; ++x, vp += W2) vz[x] = VEL ? __ldg(vp) : 0.f;
+      for (int x = 0; x < 7; ++x, vp += W2) vz[x] = VEL ? make_float2(__ldg(vp), __ldg(vp + 1)) : both(0.f);
       const float hu = 0.5f * fabsf(s.uz);
-      auto half = [&](float v) { return VEL ? rmul(hscale, v) : hu; };
-      Walk<float, SCHEME, LAP, !VEL> w;
-      w.start([&](int m) { return m < 0 ? lo[m + 3] : tp[m * pst]; }, [&](int m) { return half(vz[m + 3]); });
-      float vn = vz[6];  // one plane ahead
+      auto half = [&](float2 v) { return VEL ? pmul(both(hscale), v) : both(hu); };
+      Walk2<SCHEME, LAP, !VEL> w;
+      w.start([&](int m) { return m < 0 ? lo[m + 3] : ld2(tp + m * pst); }, [&](int m) { return half(vz[m + 3]); });
+      float2 vn = vz[6];  // one plane ahead
       tp += 3 * pst;
-      auto cell = [&](float an, bool more) {
-        const float v = vn, un = uo;
+      auto cell = [&](float2 an, bool more) {
+        const float2 v = half(vn), un = uo;
         if (more) {  // the next cell's velocity and u^n
-          if (VEL) vn = __ldg(vp), vp += W2;
+          if (VEL) vn = make_float2(__ldg(vp), __ldg(vp + 1)), vp += W2;
           up += gst;
-          if (rk_u) uo = *up;
+          if (rk_u) uo = ld2(up);
         }
-        const float nx = uo;
-        uo = un;
-        w.step(0, s.diff, an, half(v), [&](int, float dF, float ph, float lap) { finish(dF, ph, lap); });
-        uo = nx;
+        w.step(s.diff, an, v, [&](float2 dF, float2 ph, float2 lap) { finish(dF, ph, lap, un); });
       };
-#pragma unroll 3
-      for (int m = 3; m < nzs; ++m, tp += pst) cell(*tp, true);
+      // (unrolled, the kernel falls out of the instruction cache)
+#pragma unroll 1
+      for (int m = 3; m < nzs; ++m, tp += pst) cell(ld2(tp), true);
       cell(hi[0], true);
       cell(hi[1], true);
       cell(hi[2], false);
     } else {
       for (int m = 0; m < nzs; ++m, tp += pst, up += gst) {
-        if (rk_u) uo = *up;
-        finish(0.f, *tp, 0.f);
+        if (rk_u) uo = ld2(up);
+        finish(both(0.f), ld2(tp), both(0.f), uo);
       }
     }
-    if (c + bd < nb2) ends(c + bd);
+    if (c + bd < nc) ends(c + bd);
   }
 }
 
@@ -546,10 +597,9 @@ int launch_fused(mr_grid *g, const void *phi, const void *P, const void *Q, int 
               stage == 0 ? 0.f : stage == 1 ? 0.75f : 1.0f / 3, stage == 0 ? 1.f : stage == 1 ? 0.25f : 2.0f / 3};
   const bool march_ok = nb >= 12 && nb * nb <= 576;
   const size_t smm = sizeof(float) * (size_t)march_smem_floats(nb, vel);
-  // slab heights: a quarter of the block (at least four planes), or four planes
-  // of a large and half of a small block
-  const int hq = nb > 16 ? (nb + 3) / 4 : 4, ht = nb > 16 ? 4 : std::max(6, nb / 2);
-  auto threads_of = [&](int nz) { return std::min(288, (2 * nb * nz + 31) / 32 * 32); };
+  // slab heights: a quarter of a large and half of a small block, or four planes
+  const int hq = nb > 16 ? (nb + 3) / 4 : nb / 2, ht = 4;
+  auto threads_of = [&](int nz) { return std::min(160, (nb * nz + 31) / 32 * 32); };
   const int cand[2] = {threads_of(hq), threads_of(ht)};
   const int ncand = cand[0] != cand[1] ? 2 : 1;
   const int vcand[2] = {1, 2};

@@ -180,6 +180,106 @@ __device__ __forceinline__ void walk_line(int n, int diff, FP phi, FV hv, FE emi
   }
 }
 
+// ---------------------------------------------------------------------------
+// Two FP32 lines at once.  A thread walks a pair of lines in lockstep with packed
+// arithmetic (one instruction per pair of sums, products or fused multiply-adds,
+// each half rounded like the scalar instruction), so a kernel bound by issued
+// instructions issues about half of them; selects, minima and reciprocals have
+// no packed form.  Operation for operation the values of the scalar code above.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 pfma(float a, float2 b, float2 c) { return __ffma2_rn(both(a), b, c); }
+__device__ __forceinline__ float2 psub(float2 a, float2 b) { return __ffma2_rn(both(-1.f), b, a); }
+
+__device__ __forceinline__ float2 weno_v(float2 hm, float2 hp) {
+  const float2 g = psub(hp, hm);
+  return pfma(pmul(both(13.0f / 3), g), g, both((float)WenoC<float>::eps));
+}
+
+__device__ __forceinline__ float2 weno_corr(float2 c0, float2 c1, float2 c2, float2 n0, float2 n1, float2 n2) {
+  const float cap = float(WenoC<float>::rcap);
+  const float2 tau = psub(c0, c2);
+  auto ratio = [&](float2 c) {
+    const float2 r = pmul(tau, make_float2(rcp_approx(c.x), rcp_approx(c.y)));
+    return make_float2(fminf(fabsf(r.x), cap), fminf(fabsf(r.y), cap));
+  };
+  const float2 r0 = ratio(c0), r1 = ratio(c1), r2 = ratio(c2), one = both(1.f);
+  const float2 a0 = pfma(r0, r0, one), a1 = pfma(r1, r1, one), a2 = pfma(r2, r2, one);
+  const float2 den = pfma(6.f, a1, pfma(3.f, a2, a0));
+  return pmul(pfma(a2, n2, pfma(a1, n1, pmul(a0, n0))), make_float2(rcp_approx(den.x), rcp_approx(den.y)));
+}
+
+// half_flux of a pair; lx, ly: the side of either line (LEFT: left of both)
+template <int SCHEME, bool LEFT>
+__device__ __forceinline__ float2 half_flux2(float2 w2, float2 w3, float2 h0, float2 h1, float2 h2, float2 h3,
+                                             float2 h4, float2 v0, float2 v1, float2 v2, float2 v3, bool lx, bool ly) {
+  auto up = [&](float2 l, float2 r) { return LEFT ? l : make_float2(lx ? l.x : r.x, ly ? l.y : r.y); };
+  const float2 c = up(w2, w3), e2 = up(h1, h3);
+  float2 s;
+  if (SCHEME == MR_CONS3) {
+    s = pfma(1.0f / 3, h2, pmul(both(1.0f / 6), e2));
+  } else {
+    const float2 e1 = up(h0, h4), e4 = up(h3, h1);
+    if (SCHEME == MR_CONS5) {
+      s = pfma(11.0f / 60, e2, pfma(-1.0f / 30, e1, pfma(2.0f / 5, h2, pmul(both(-1.0f / 20), e4))));
+    } else {
+      // (t_0, t_2 with the sign changed: they are squared)
+      const float2 t0 = pfma(-3.f, e2, e1), t1 = padd(e2, h2), t2 = pfma(-3.f, h2, e4);
+      const float2 c0 = pfma(t0, t0, up(v0, v3)), c1 = pfma(t1, t1, up(v1, v2)), c2 = pfma(t2, t2, up(v2, v1));
+      const float2 n0 = pfma(5.0f / 6, e2, pmul(both(-1.0f / 3), e1)), n1 = pfma(2.f, h2, e2),
+                   n2 = pfma(2.f, h2, pmul(both(-0.5f), e4));
+      s = weno_corr(c0, c1, c2, n0, n1, n2);
+    }
+  }
+  return LEFT ? padd(c, s) : pfma(make_float2(lx ? 1.f : -1.f, ly ? 1.f : -1.f), s, c);
+}
+
+// Walk of a pair of lines (see Walk)
+template <int SCHEME, bool LAP, bool LEFT>
+struct Walk2 {
+  float2 am, a0, a1, a2, a3, va, vb, vc;
+  float2 w2, w3, w4, w5, h0, h1, h2, h3, h4, v0, v1, v2, v3, Fm;
+  __device__ __forceinline__ float2 flux(float2 ul, float2 ur) {
+    const float2 u = LEFT ? ul : padd(ul, ur);
+    return half_flux2<SCHEME, LEFT>(w2, w3, h0, h1, h2, h3, h4, v0, v1, v2, v3, u.x >= 0.f, u.y >= 0.f);
+  }
+  template <typename FP, typename FV>
+  __device__ __forceinline__ void start(FP phi, FV hv) {
+    const float2 wa = pmul(hv(-3), phi(-3));
+    am = phi(-2);
+    const float2 wb = pmul(hv(-2), am), vl = hv(-1);
+    a0 = phi(-1), w2 = pmul(vl, a0);
+    va = hv(0), a1 = phi(0), w3 = pmul(va, a1);
+    vb = hv(1), a2 = phi(1), w4 = pmul(vb, a2);
+    vc = hv(2), a3 = phi(2), w5 = pmul(vc, a3);
+    h0 = psub(wb, wa), h1 = psub(w2, wb), h2 = psub(w3, w2), h3 = psub(w4, w3), h4 = psub(w5, w4);
+    v0 = v1 = v2 = v3 = both(0.f);
+    if (SCHEME == MR_WENOZ5) v0 = weno_v(h0, h1), v1 = weno_v(h1, h2), v2 = weno_v(h2, h3), v3 = weno_v(h3, h4);
+    Fm = flux(vl, va);
+  }
+  // an, vn: values and half velocities at cell m + 3; emit(dF, c, lap)
+  template <typename FE>
+  __device__ __forceinline__ void step(int diff, float2 an, float2 vn, FE emit) {
+    const float2 wn = pmul(vn, an);
+    w2 = w3, w3 = w4, w4 = w5;
+    h0 = h1, h1 = h2, h2 = h3, h3 = h4, h4 = psub(wn, w5);
+    w5 = wn;
+    if (SCHEME == MR_WENOZ5) v0 = v1, v1 = v2, v2 = v3, v3 = weno_v(h3, h4);
+    const float2 Fp = flux(va, vb);
+    emit(psub(Fp, Fm), a1,
+         LAP ? make_float2(lap_term<float>(am.x, a0.x, a1.x, a2.x, a3.x, diff),
+                           lap_term<float>(am.y, a0.y, a1.y, a2.y, a3.y, diff))
+             : both(0.f));
+    Fm = Fp;
+    va = vb, vb = vc, vc = vn;
+    if (LAP) am = a0, a0 = a1;
+    a1 = a2, a2 = a3, a3 = an;
+  }
+};
+
 // Central Laplacian at *c: sum over the three directions of lap_term.
 template <typename T>
 __device__ __forceinline__ T lap_at(const T *c, const int *stride, int diff) {
