@@ -287,10 +287,15 @@ __device__ __noinline__ TI prep_fetch(const Tree &t, const PrepTab &T, const TI 
 // store and two additions (a source index per point cost 113 instructions: 327
 // against 133 us for the 1 696 leaves next to coarser ones of a 3 424-leaf grid
 // of 24^3 blocks, shell 6).
+// LEAN (passes whose blocks are read in their interior and next to coarser
+// leaves alone): beside the interior only the points within reach of a coarser
+// neighbour, the layers that the substitution and the push read -- a third of the
+// ghosts is left out where one face borders on a coarser leaf (the pre-pass of
+// the grid above 390 -> 376 us, of 42 400 leaves of 24^3 2.56 -> 2.42 ms).
 // ---------------------------------------------------------------------------
-template <typename TI, typename TP>
+template <bool LEAN, typename TI, typename TP>
 __device__ __forceinline__ void gather_block(const Tree &t, const PrepTab &T, const TI *__restrict__ phi, TP *Pb, int b,
-                                             int L, int Gi, int *err) {
+                                             int L, int Gi, int reach, int *err) {
   const int nb = t.nb, Wd = nb + 2 * Gi, hb = nb / 2, W2 = Wd * Wd, nb2 = nb * nb;
   const size_t nb3 = (size_t)nb * nb2;
   const DivM dW = divm(Wd);
@@ -302,15 +307,38 @@ __device__ __forceinline__ void gather_block(const Tree &t, const PrepTab &T, co
     }
     for (; n > 0; --n, d += W2, src += st) *d = Cvt<TP>::f(ld(src));
   };
+  // bit m of all / some: a column near the outward sides m (bit 0: x, 1: y) lies
+  // within reach of a coarser neighbour everywhere / near the outward side of z
+  unsigned all = 0, some = 0;
+  for (int m = 0; m < 4 && LEAN; ++m)
+    for (int e = 1; e < 8; ++e)
+      if (((T.ce >> e) & 1) && !(e & 3 & ~m)) (e & 4 ? some : all) |= 1u << m;
+  auto near = [&](int x, int d) { return T.s[d] > 0 ? x >= nb - reach : x < reach; };
   for (int c = threadIdx.x; c < W2; c += blockDim.x) {
     const int row = divq(c, dW), i = c - row * Wd - Gi, j = row - Gi;
+    int za = -Gi, zb = nb + Gi;  // planes wanted of this column
+    if (LEAN) {
+      const int m = (near(i, 0) ? 1 : 0) | (near(j, 1) ? 2 : 0);
+      const bool in = i >= 0 && i < nb && j >= 0 && j < nb;
+      if (!((all >> m) & 1)) {
+        const bool zn = (some >> m) & 1;
+        if (!zn && !in) continue;
+        za = !zn ? 0 : T.s[2] < 0 ? -Gi : in ? min(0, nb - reach) : nb - reach;
+        zb = !zn ? nb : T.s[2] > 0 ? nb + Gi : in ? max(nb, reach) : reach;
+      }
+    }
     const int rx = i < 0 ? 0 : i >= nb ? 2 : 1, ry = j < 0 ? 0 : j >= nb ? 2 : 1;
     const int ri = i - (rx - 1) * nb, rj = j - (ry - 1) * nb;  // region-local
     TP *col = Pb + c + (size_t)W2 * Gi;                        // (i, j, 0)
     for (int rz = 0; rz < 3; ++rz) {
       const int r = rx + 3 * ry + 9 * rz, Lo = T.rlev[r];
       if (Lo < L) continue;  // a coarser leaf's region: refined below
-      const int k0 = rz == 0 ? nb - Gi : 0, k1 = rz == 2 ? Gi : nb, z0 = (rz - 1) * nb;  // region-local planes
+      const int z0 = (rz - 1) * nb;  // region-local planes
+      int k0 = rz == 0 ? nb - Gi : 0, k1 = rz == 2 ? Gi : nb;
+      if (LEAN) {
+        k0 = max(k0, za - z0), k1 = min(k1, zb - z0);
+        if (k0 >= k1) continue;
+      }
       if (Lo == L) {
         run(col + (ptrdiff_t)W2 * (z0 + k0), phi + (size_t)T.rslot[r] * nb3 + ri + nb * rj + nb2 * k0, nb2, k1 - k0);
         continue;
@@ -777,7 +805,13 @@ __global__ void __launch_bounds__(sizeof(TP) == 4 ? 512 : 384, 2) k_prep(Tree t,
   }
   __syncthreads();
   TP *Pb = P + (size_t)b * np;
-  gather_block(t, T, phi, Pb, b, L, Gi, err);
+  // The band is ext_b or ext_f layers deep and reads hwG further; the push starts
+  // 2 Gpush layers from the side and reads hwH further.  In blocks less than twice
+  // as wide the tests cost more than they leave out (11 019 leaves of 16^3 with
+  // 4.2, reach 10: 738 -> 766 us).
+  const int reach = max(max(W::ext_b, W::ext_f) + W::hwG, only_coarse == 1 && NT ? 2 * min(Gpush, hb) + W::hwH : 0);
+  if (!BND && sizeof(TP) == 4 && only_coarse && 2 * reach <= nb) gather_block<true>(t, T, phi, Pb, b, L, Gi, reach, err);
+  else gather_block<false>(t, T, phi, Pb, b, L, Gi, 0, err);
   if (!mask) return;
   // substitution jobs: one thread each (degree 1: classes x, y, z; 2: xy, xz,
   // yz; 3: xyz), then one thread lays out their sums
