@@ -635,7 +635,7 @@ def main():
                    "scheme": args.scheme, "precision": args.precision,
                    "diffusion": f"DIFF-{args.diffusion}, nu={args.nu}" if args.diffusion else None},
         "roofline": {"bound": "hbm",
-                     "kernel": "ghost_fill (k_prep + k_fill_plain)" if name == "ghost_fill" else name,
+                     "kernel": "ghost_fill (k_prep)" if name == "ghost_fill" else name,
                      "achieved": achieved, "peak": hbm, "unit": "GB/s",
                      "frac": achieved / hbm if achieved else None, "peak_source": src,
                      "traffic": None, "alg_bytes_per_launch": per_launch,

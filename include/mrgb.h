@@ -127,8 +127,8 @@ typedef struct {
  * Condition (default: extrapolation through the N nearest points):
  * MR_GRID_BC_DIRICHLET0 -- zero value: through 0 at the boundary and the
  * N-1 nearest points off it; MR_GRID_BC_ZERO -- plain zeros.  Such grids run
- * a general point-wise ghost path (one thread per padded point, the tensor
- * sums of Alg. SM1/SM2 evaluated directly) and the per-block stage kernel;
+ * the same ghost kernels with the polynomial added, the stage kernel that reads
+ * padded blocks (in FP32, too) and a criterion of their own;
  * the criterion's extended region stops at the boundary, neighbours and the
  * update step never reach beyond it, and every adaptation iteration
  * ghost-fills every field in full with FP64 padded blocks.
@@ -319,8 +319,8 @@ int mr_autotune_clear(void);
 /* Which kernel runs the FP32 stage (ghost faces + rhs + RK3 stage, the
  * supplement's "Finite differences" and "Time integration" schemes) of
  * mr_step, mr_step_vel, mr_step_vel_scaled, mr_rhs_advect and
- * mr_rhs_advect_vel: 1 = k_fused (the ghost-extended block in shared memory,
- * one thread per grid line), 2 = k_march (the block traversed plane by plane,
+ * mr_rhs_advect_vel: 1 = k_fused (slabs of a block with their ghosts in shared
+ * memory, one thread per pair of grid lines), 2 = k_march (the block traversed plane by plane,
  * one thread per grid column, two CTAs per SM), 0 = chosen by the autotuner
  * on grids with mr_autotune enabled (the faster of the two for that
  * configuration), else k_fused (the default).  k_march
@@ -406,7 +406,8 @@ int mr_profile_read(mr_grid *grid, int kid, double *total_ms, int *nlaunch, cons
 int mr_launch_count(mr_grid *grid, long long *n);
 /* Algorithmic bytes of the recorded launches of kernel kid (the roofline
  * numerator), accumulated on the device while profiling is on.  Defined for
- * the ghost pre-pass (kid 0) and the ghost gather (kid 1): every point of the
+ * the ghost fill, whose leaves next to coarser ones count as the pre-pass (kid 0)
+ * and the others as plain gathers (kid 1, no launch of its own): every point of the
  * requested shell G of each leaf the launch reconstructs is written once and
  * its source value read once, ((nb + 2G)^3 - nb^3) * (source + padded
  * element size) per leaf -- the internal shell the kernels also fill (wider

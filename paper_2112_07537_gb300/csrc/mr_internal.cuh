@@ -276,28 +276,6 @@ __device__ __forceinline__ TP refine_dispatch(bool ox, bool oy, bool oz, F val) 
   }
 }
 
-// tensor H^a: sum over nonzero (tx, ty, tz) of H(tx)H(ty)H(tz) val(tx,ty,tz)
-template <int N, int NT, typename TP, typename F>
-__device__ __forceinline__ TP coarsen_sum(F val) {
-  using W = Wav<N, NT>;
-  TP s = TP(0);
-#pragma unroll
-  for (int tz = -W::hwH; tz <= W::hwH; ++tz) {
-    if (W::H(tz) == 0.0) continue;
-#pragma unroll
-    for (int ty = -W::hwH; ty <= W::hwH; ++ty) {
-      if (W::H(ty) == 0.0) continue;
-#pragma unroll
-      for (int tx = -W::hwH; tx <= W::hwH; ++tx) {
-        if (W::H(tx) == 0.0) continue;
-        const TP wgt = TP(W::H(tx)) * TP(W::H(ty)) * TP(W::H(tz));
-        s = racc(s, wgt, val(tx, ty, tz));
-      }
-    }
-  }
-  return s;
-}
-
 // substitution: -sum over t != 0 (t only along odd dims) of prod G^a
 template <int N, int NT, bool OX, bool OY, bool OZ, typename TP, typename F>
 __device__ __forceinline__ TP subst_sum(F val) {
@@ -342,44 +320,11 @@ struct Cls {
   static constexpr int x = X, y = Y, z = Z;
 };
 
-// up to 27 disjoint boxes [lo, hi) of block-local points
-struct BoxList {
-  int n;
-  int lo[27][3], hi[27][3];
-};
-
 // first point of parity par at or after lo; number of such points in [lo, hi)
 __device__ __forceinline__ int par_first(int lo, int par) { return lo + ((lo ^ par) & 1); }
 __device__ __forceinline__ int par_count(int lo, int hi, int par) {
   const int f = par_first(lo, par);
   return f < hi ? (hi - f + 1) >> 1 : 0;
-}
-
-// f(i, j, k) for every point of parity class (OX, OY, OZ) in the boxes, as
-// one flat index space spread over the CTA (each thread walks the boxes
-// forward, so locating a point's box costs O(1) amortised)
-template <int OX, int OY, int OZ, typename F>
-__device__ __forceinline__ void for_class_points(const BoxList &bl, F f) {
-  auto cnt3 = [&](int e, int &nx, int &ny) {
-    nx = par_count(bl.lo[e][0], bl.hi[e][0], OX);
-    ny = par_count(bl.lo[e][1], bl.hi[e][1], OY);
-    return nx * ny * par_count(bl.lo[e][2], bl.hi[e][2], OZ);
-  };
-  int total = 0, nx, ny;
-  for (int e = 0; e < bl.n; ++e) total += cnt3(e, nx, ny);
-  if (!total) return;
-  int e = 0, base = 0, cnt = cnt3(0, nx, ny);
-  DivM dx = divm(nx > 0 ? nx : 1), dy = divm(ny > 0 ? ny : 1);
-  for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-    while (idx >= base + cnt) {
-      base += cnt;
-      cnt = cnt3(++e, nx, ny);
-      dx = divm(nx > 0 ? nx : 1), dy = divm(ny > 0 ? ny : 1);
-    }
-    const int q = idx - base, r = divq(q, dx), qz = divq(r, dy), qx = q - r * nx, qy = r - qz * ny;
-    f(par_first(bl.lo[e][0], OX) + 2 * qx, par_first(bl.lo[e][1], OY) + 2 * qy,
-      par_first(bl.lo[e][2], OZ) + 2 * qz);
-  }
 }
 
 // region index (0..26) of a block-local point within the +-1 neighbour ring
@@ -530,10 +475,10 @@ struct mr_grid {
   int *refined2;
   int *scan;              // capacity + 1
   int *newsrc;            // 8*capacity: source mapping of new leaves
-  int *counter;           // device words: [0] changed count, [1] error bits, [2..] scratch
+  int *counter;           // device words: [0] changed count, [1] error bits, [8] leaves in the list, rest scratch
   double *dscratch;       // reduction scratch
   int *cmask;             // per-leaf coarse-direction masks (ghost fill), then new-band masks
-  int *hasD;              // per new leaf: the update step has discarded details
+  int *hasD;              // per new leaf: box of the details the update discards; in FP32 steps: list of leaves next to coarser ones
   int *pneed;             // per leaf: 1 = left to the full ghost pre-pass (has a coarser neighbour)
   double *mdlast;         // block norms the last adaptation iteration decided with
   int nleaf_last;         // leaves of the tree mdlast belongs to
@@ -609,7 +554,7 @@ int check_cuda(cudaError_t e, const char *where);
 void *field_ptr(mr_grid *g, int fid);      // fid >= nfields: temporaries
 void *next_field_ptr(mr_grid *g, int fid);
 
-// tune.cu: launch-shape autotuner (kid: 0 k_fill_plain, 1 k_prep,
+// tune.cu: launch-shape autotuner (kid: 1 k_prep,
 // 2 k_criterion, 3 k_fused, 4 k_interp, 5 k_merge, 6 the FP32 stage kernel
 // variant (candidates 1 k_fused, 2 k_march); tp: 4 FP32, 5 FP32 field with
 // FP64 padded blocks, 8 FP64)
@@ -634,6 +579,7 @@ int launch_ghost(mr_grid *g, const void *phi_in, void *phi_out, int G, bool fp64
 int launch_crop(mr_grid *g, const void *P, int Gi, void *out, int G, bool fp64_src);
 int launch_crop64(mr_grid *g, const double *P, int Gi, double *out, int G);
 int launch_prep32(mr_grid *g, const void *phi, int *Gi);
+int launch_coarse_list(mr_grid *g);
 int launch_writeback32(mr_grid *g, int Gi, void *phi);
 int launch_substitute(mr_grid *g, void *phi, const int *need = nullptr, bool in_side_buffer = false,
                       bool f32 = false);

@@ -124,59 +124,35 @@ __device__ __forceinline__ T lap_term(T m2, T m1, T c, T p1, T p2, int diff) {
   return (T(16) * (m1 + p1) - (m2 + p2) - T(30) * c) * T(1.0 / 12);
 }
 
-// State of a walk along one grid line: step() moves one cell on and hands
-// emit(m, dF, c, lap) the halved flux difference F_{m+1/2}/2 - F_{m-1/2}/2 of
-// cell m, its value c = phi(m) and (LAP) its Laplacian term along the line.  The
-// velocities of the two points of an interface pick its upwind side, or (LEFT: a
-// constant velocity along the walk) it is the left one throughout.  The point
-// fluxes are rounded products (never contracted into a sum), so a flux does not
-// depend on where its line starts.
-template <typename T, int SCHEME, bool LAP, bool LEFT>
-struct Walk {
-  T am, a0, a1, a2, a3, va, vb, vc;  // phi(m-2 .. m+2), half velocities at m .. m+2
-  T w2, w3, w4, w5, h0, h1, h2, h3, h4, v0, v1, v2, v3, Fm;
-  // phi(m), hv(m): value and half velocity at cells -3 .. 2
-  template <typename FP, typename FV>
-  __device__ __forceinline__ void start(FP phi, FV hv) {
-    const T wa = rmul(hv(-3), phi(-3));
-    am = phi(-2);
-    const T wb = rmul(hv(-2), am), vl = hv(-1);
-    a0 = phi(-1), w2 = rmul(vl, a0);
-    va = hv(0), a1 = phi(0), w3 = rmul(va, a1);
-    vb = hv(1), a2 = phi(1), w4 = rmul(vb, a2);
-    vc = hv(2), a3 = phi(2), w5 = rmul(vc, a3);
-    h0 = wb - wa, h1 = w2 - wb, h2 = w3 - w2, h3 = w4 - w3, h4 = w5 - w4;
-    v0 = v1 = v2 = v3 = T(0);
-    if (SCHEME == MR_WENOZ5) v0 = weno_v(h0, h1), v1 = weno_v(h1, h2), v2 = weno_v(h2, h3), v3 = weno_v(h3, h4);
-    Fm = half_flux<T, SCHEME>(w2, w3, h0, h1, h2, h3, h4, v0, v1, v2, v3, LEFT || vl + va >= T(0));
-  }
-  // an, vn: value and half velocity at cell m + 3
-  template <typename FE>
-  __device__ __forceinline__ void step(int m, int diff, T an, T vn, FE emit) {
-    const T wn = rmul(vn, an);
+// Walks n cells of one grid line and hands emit(m, dF, c) the halved flux
+// difference F_{m+1/2}/2 - F_{m-1/2}/2 of every cell m and its value c = phi(m).
+// phi(m), hv(m): value and half velocity at cell m (-3 <= m < n + 3, called once
+// each in ascending order); the velocities of the two points of an interface pick
+// its upwind side.  The point fluxes are rounded products (never contracted into
+// a sum), so a flux does not depend on where its line starts.
+template <typename T, int SCHEME, typename FP, typename FV, typename FE>
+__device__ __forceinline__ void walk_line(int n, FP phi, FV hv, FE emit) {
+  const T wa = rmul(hv(-3), phi(-3)), wb = rmul(hv(-2), phi(-2));
+  T vl = hv(-1), w2 = rmul(vl, phi(-1));
+  T va = hv(0), a1 = phi(0), w3 = rmul(va, a1);
+  T vb = hv(1), a2 = phi(1), w4 = rmul(vb, a2);
+  T vc = hv(2), a3 = phi(2), w5 = rmul(vc, a3);
+  T h0 = wb - wa, h1 = w2 - wb, h2 = w3 - w2, h3 = w4 - w3, h4 = w5 - w4;
+  T v0 = T(0), v1 = T(0), v2 = T(0), v3 = T(0);
+  if (SCHEME == MR_WENOZ5) v0 = weno_v(h0, h1), v1 = weno_v(h1, h2), v2 = weno_v(h2, h3), v3 = weno_v(h3, h4);
+  T Fm = half_flux<T, SCHEME>(w2, w3, h0, h1, h2, h3, h4, v0, v1, v2, v3, vl + va >= T(0));
+#pragma unroll(sizeof(T) == 4 ? 4 : 2)
+  for (int m = 0; m < n; ++m) {
+    const T vn = hv(m + 3), an = phi(m + 3), wn = rmul(vn, an);
     w2 = w3, w3 = w4, w4 = w5;
     h0 = h1, h1 = h2, h2 = h3, h3 = h4, h4 = wn - w5;
     w5 = wn;
     if (SCHEME == MR_WENOZ5) v0 = v1, v1 = v2, v2 = v3, v3 = weno_v(h3, h4);
-    const T Fp = half_flux<T, SCHEME>(w2, w3, h0, h1, h2, h3, h4, v0, v1, v2, v3, LEFT || va + vb >= T(0));
-    emit(m, Fp - Fm, a1, LAP ? lap_term<T>(am, a0, a1, a2, a3, diff) : T(0));
+    const T Fp = half_flux<T, SCHEME>(w2, w3, h0, h1, h2, h3, h4, v0, v1, v2, v3, va + vb >= T(0));
+    emit(m, Fp - Fm, a1);
     Fm = Fp;
     va = vb, vb = vc, vc = vn;
-    if (LAP) am = a0, a0 = a1;
     a1 = a2, a2 = a3, a3 = an;
-  }
-};
-
-// Walks the n cells of one line.  phi(m), hv(m): value and half velocity at cell
-// m (-3 <= m < n + 3, called once each in ascending order).
-template <typename T, int SCHEME, bool LAP, bool LEFT, typename FP, typename FV, typename FE>
-__device__ __forceinline__ void walk_line(int n, int diff, FP phi, FV hv, FE emit) {
-  Walk<T, SCHEME, LAP, LEFT> w;
-  w.start(phi, hv);
-#pragma unroll(sizeof(T) == 4 ? 4 : 2)
-  for (int m = 0; m < n; ++m) {
-    const T vn = hv(m + 3), an = phi(m + 3);
-    w.step(m, diff, an, vn, emit);
   }
 }
 
@@ -237,15 +213,18 @@ __device__ __forceinline__ float2 half_flux2(float2 w2, float2 w3, float2 h0, fl
   return LEFT ? padd(c, s) : pfma(make_float2(lx ? 1.f : -1.f, ly ? 1.f : -1.f), s, c);
 }
 
-// Walk of a pair of lines (see Walk)
+// Walk of a pair of lines: walk_line a cell at a time, with (LAP) the Laplacian
+// term along the line and (LEFT: a constant velocity along the walk) the left side
+// throughout.
 template <int SCHEME, bool LAP, bool LEFT>
 struct Walk2 {
-  float2 am, a0, a1, a2, a3, va, vb, vc;
+  float2 am, a0, a1, a2, a3, va, vb, vc;  // phi(m-2 .. m+2), half velocities at m .. m+2
   float2 w2, w3, w4, w5, h0, h1, h2, h3, h4, v0, v1, v2, v3, Fm;
   __device__ __forceinline__ float2 flux(float2 ul, float2 ur) {
     const float2 u = LEFT ? ul : padd(ul, ur);
     return half_flux2<SCHEME, LEFT>(w2, w3, h0, h1, h2, h3, h4, v0, v1, v2, v3, u.x >= 0.f, u.y >= 0.f);
   }
+  // phi(m), hv(m): values and half velocities at cells -3 .. 2
   template <typename FP, typename FV>
   __device__ __forceinline__ void start(FP phi, FV hv) {
     const float2 wa = pmul(hv(-3), phi(-3));

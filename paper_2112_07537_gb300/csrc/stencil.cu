@@ -19,7 +19,7 @@ namespace mr {
 // rounded products and the sums of walk_line leave nothing to contract, so a
 // flux does not depend on where its line was cut.  Measured (WENO-Z5, velocity
 // fields, 1 408 leaves of 24^3 = 19.5 M points): 23.9 ms per launch with both
-// fluxes of every point evaluated per thread and four divisions each, 6.35 ms
+// fluxes of every point evaluated per thread and four divisions each, 6.08 ms
 // so (the FP64 pipe's floor for 147 instructions a point is 4.6 ms); 15 leaves
 // of 16^3: 680 us in 15 CTAs, 39 us.
 template <typename T, int SCHEME>
@@ -39,12 +39,11 @@ __global__ void __launch_bounds__(256) k_rhs_stage(Tree t, const T *__restrict__
   auto walk = [&](int d, const T *p, const T *v, int st, int sv, int n, auto emit) {
     if (vpad) {
       v += d * vcomp;
-      walk_line<T, SCHEME, false, false>(
-          n, 0, [&](int m) { return p[m * st]; }, [&](int m) { return rmul(hscale, v[m * sv]); }, emit);
+      walk_line<T, SCHEME>(
+          n, [&](int m) { return p[m * st]; }, [&](int m) { return rmul(hscale, v[m * sv]); }, emit);
     } else {
       const T hu = T(0.5) * (d == 0 ? ux : d == 1 ? uy : uz);
-      walk_line<T, SCHEME, false, false>(
-          n, 0, [&](int m) { return p[m * st]; }, [&](int) { return hu; }, emit);
+      walk_line<T, SCHEME>(n, [&](int m) { return p[m * st]; }, [&](int) { return hu; }, emit);
     }
   };
   const bool xon = vpad || ux != T(0), yon = vpad || uy != T(0), zon = vpad || uz != T(0);
@@ -60,7 +59,7 @@ __global__ void __launch_bounds__(256) k_rhs_stage(Tree t, const T *__restrict__
     T *rr = (yd ? R1 : R0) + i + RS * (j + nb * k);
     const int rs = yd ? RS : 1;
     walk(yd ? 1 : 0, Pb + o, Vb + (vpad ? ov : 0), yd ? Wd : 1, yd ? Wv : 1, n,
-         [&](int m, T dF, T, T) { rr[m * rs] = dF; });
+         [&](int m, T dF, T) { rr[m * rs] = dF; });
   }
   __syncthreads();
   const T h = T(t.tree_len / ((double)nb * (double)(1 << __ldg(t.lev + b)))), inv2 = T(2) / h, invh2 = T(1) / (h * h);
@@ -69,7 +68,7 @@ __global__ void __launch_bounds__(256) k_rhs_stage(Tree t, const T *__restrict__
     const int j = c / nb, i = c - j * nb;
     const T *p = Pb + i + Wd * j;
     const size_t q0 = (size_t)b * nb * nb * nb + c + (size_t)nb * nb * k0;
-    auto finish = [&](int m, T dz, T ph, T) {
+    auto finish = [&](int m, T dz, T ph) {
       const int ro = i + RS * (j + nb * m);
       T acc = T(0);
       if (xon) acc = R0[ro];
@@ -93,7 +92,7 @@ __global__ void __launch_bounds__(256) k_rhs_stage(Tree t, const T *__restrict__
     if (zon)
       walk(2, p, Vb + (vpad ? i + Wv * j : 0), Wd * Wd, Wv * Wv, nzs, finish);
     else
-      for (int m = 0; m < nzs; ++m) finish(m, T(0), p[(size_t)m * Wd * Wd], T(0));
+      for (int m = 0; m < nzs; ++m) finish(m, T(0), p[(size_t)m * Wd * Wd]);
   }
 }
 

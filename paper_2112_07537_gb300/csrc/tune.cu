@@ -34,7 +34,7 @@ std::mutex g_mu;
 std::map<TuneKey, Entry> g_table;
 
 const char *tune_kernel_name(int kid) {
-  static const char *names[] = {"k_fill_plain", "k_prep", "k_criterion", "k_fused", "k_interp", "k_merge",
+  static const char *names[] = {"?", "k_prep", "k_criterion", "k_fused", "k_interp", "k_merge",
                                 "stage kernel (1 k_fused, 2 k_march)"};
   return kid >= 0 && kid < (int)(sizeof names / sizeof names[0]) ? names[kid] : "?";
 }
