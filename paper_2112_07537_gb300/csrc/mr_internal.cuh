@@ -475,10 +475,10 @@ struct mr_grid {
   int *refined2;
   int *scan;              // capacity + 1
   int *newsrc;            // 8*capacity: source mapping of new leaves
-  int *counter;           // device words: [0] changed count, [1] error bits, [8] leaves in the list, rest scratch
+  int *counter;           // device words: [0] changed count, [1] error bits, [2..] scratch
   double *dscratch;       // reduction scratch
   int *cmask;             // per-leaf coarse-direction masks (ghost fill), then new-band masks
-  int *hasD;              // per new leaf: box of the details the update discards; in FP32 steps: list of leaves next to coarser ones
+  int *hasD;              // per new leaf: box of the details the update discards (0: none)
   int *pneed;             // per leaf: 1 = left to the full ghost pre-pass (has a coarser neighbour)
   double *mdlast;         // block norms the last adaptation iteration decided with
   int nleaf_last;         // leaves of the tree mdlast belongs to
@@ -579,7 +579,6 @@ int launch_ghost(mr_grid *g, const void *phi_in, void *phi_out, int G, bool fp64
 int launch_crop(mr_grid *g, const void *P, int Gi, void *out, int G, bool fp64_src);
 int launch_crop64(mr_grid *g, const double *P, int Gi, double *out, int G);
 int launch_prep32(mr_grid *g, const void *phi, int *Gi);
-int launch_coarse_list(mr_grid *g);
 int launch_writeback32(mr_grid *g, int Gi, void *phi);
 int launch_substitute(mr_grid *g, void *phi, const int *need = nullptr, bool in_side_buffer = false,
                       bool f32 = false);
