@@ -219,6 +219,7 @@ struct PrepTab {
 // dhi on the + side) next to the coarser neighbours ce
 struct Boxes {
   int n, lo[7][3], hi[7][3];
+  int flat[7];  // axes along which the neighbour does not lie across a side (bit per axis)
 };
 // (by one warp, a lane per direction; faces first, then edges, then the corner)
 __device__ __forceinline__ void outward_boxes(Boxes &B, int ce, const int *s, int n, int dlo, int dhi) {
@@ -246,6 +247,7 @@ __device__ __forceinline__ void outward_boxes(Boxes &B, int ce, const int *s, in
   if (keep) {
     const int at = __popc(have & ((1u << q) - 1u));
     for (int d = 0; d < 3; ++d) B.lo[at][d] = lo[d], B.hi[at][d] = hi[d];
+    B.flat[at] = 7 & ~e;
   }
   if (q == 0) B.n = __popc(have);
 }
@@ -389,12 +391,26 @@ __device__ __forceinline__ int turn(int rot, int n, int bd) {
 
 constexpr int SUB_RUN = 4;  // points of one item of the substitution
 
+// Flat axes are used where arithmetic counts: FP64 blocks (ghost fills of 1 408
+// leaves of 24^3 with 6.2, shell 6: 637 -> 546 us, of 2 080 with shell 11 1 770 ->
+// 1 693 us); with FP32 blocks the listed coordinates cost more than the sums they
+// save (42 400 leaves 2.42 -> 2.56 ms).
+template <typename TP>
+constexpr bool sub_flat = sizeof(TP) == 8;
+
+// Points of a band box along a flat axis (sub_coord): even ones below lo from e0
+// on, odd ones of [lo, hi) from o0 on, even ones above from e1 on
+struct SubAxes {
+  short lo[3], hi[3], e0[3], o0[3], e1[3], nlo[3], nod[3];
+};
+
 // One parity class (odd dimensions om) of degree deg over one band box: summed
 // one odd dimension at a time (o[0] first), as walked by subst_sep.
 struct SubJob {
   int om, deg, o[3];
   short st[3][3], cn[3][3];  // per pass: first point, count per axis
   int sp1[3];              // per pass: axes walked with step 1 (others 2)
+  short fl[3], flat, box;  // per pass: axes walked by sub_coord; flat axes of the box; the box
   unsigned d0[3], d1[3];   // reciprocals of the item counts along axes 0, 1
   int n[3], it[3];         // points per pass; items (runs of SUB_RUN points along o[pass])
   int off, next;           // sums in shared memory; end of the batch this job opens
@@ -405,9 +421,14 @@ struct SubJob {
 // o_deg becomes -S(p), S(p) = sum over t != 0 (t along the odd dimensions) of
 // prod_d G^a(t_d) P(p + t).  S is summed one odd dimension at a time, thinnest
 // box side first, with the partial sums of each (box, class) job in shared
-// memory: pass 1 reads the padded block at every point the later passes need
-// (odd dimensions not yet summed span the box plus the G^a half-width), the
-// last pass writes -S into the block.  Pass 1 drops its t = 0 term where every
+// memory: pass 1 reads the padded block at every point the later passes need, the
+// last pass writes -S into the block.  Odd dimensions not yet summed span the box
+// plus the G^a half-width; along a flat axis (the band goes on to both ends of the
+// box) only the box's odd points and the even ones beyond it: a band point has no
+// detail along the odd dimensions it shares with the class, so the terms at even
+// points inside add up to zero over the other dimensions and are left out, and
+// away from the ends S is the sum of the pass before (half the points of a face
+// box).  Pass 1 drops its t = 0 term where every
 // other odd coordinate is odd -- exactly at the class points, which no other
 // term of any pass reads -- so the product over all t leaves out t = 0.
 // Points of one degree read lower degrees only, so all jobs of a degree run
@@ -416,8 +437,25 @@ struct SubJob {
 // dimension: their taps share a window of even points, loaded together (13
 // loads in flight for four points instead of 28 in four dependent rounds).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void sub_job_build(SubJob &J, const int *lo, const int *hi, int om, int hG) {
-  J.om = om, J.deg = __popc(om);
+// coordinate of index q along flat axis d
+__device__ __forceinline__ int sub_coord(const SubAxes &J, int d, int q) {
+  const int a = J.nlo[d], b = a + J.nod[d];
+  return 2 * q + (q < a ? J.e0[d] : q < b ? J.o0[d] - 2 * a : J.e1[d] - 2 * b);
+}
+
+__device__ __forceinline__ void sub_job_build(SubJob &J, SubAxes *ax, int box, const int *lo, const int *hi, int om,
+                                              int hG, int flat) {
+  J.om = om, J.deg = __popc(om), J.flat = (short)flat, J.box = (short)box;
+  int nall[3];
+  for (int d = 0; d < 3; ++d) {
+    const int nlo = par_count(lo[d] - hG, lo[d], 0), nod = par_count(lo[d], hi[d], 1);
+    nall[d] = nlo + nod + par_count(hi[d], hi[d] + hG, 0);
+    if (flat && om == 7) {  // (one job per box)
+      SubAxes &A = ax[box];
+      A.lo[d] = (short)lo[d], A.hi[d] = (short)hi[d], A.nlo[d] = (short)nlo, A.nod[d] = (short)nod;
+      A.e0[d] = (short)par_first(lo[d] - hG, 0), A.o0[d] = (short)par_first(lo[d], 1), A.e1[d] = (short)par_first(hi[d], 0);
+    }
+  }
   int o[3], n = 0;
   for (int d = 0; d < 3; ++d)
     if ((om >> d) & 1) o[n++] = d;
@@ -432,10 +470,11 @@ __device__ __forceinline__ void sub_job_build(SubJob &J, const int *lo, const in
     J.n[s] = J.it[s] = 0;
     if (s >= n) continue;
     summed |= 1 << o[s];
-    J.sp1[s] = om & ~summed;
+    J.sp1[s] = om & ~summed & ~flat, J.fl[s] = (short)(om & ~summed & flat);
     for (int d = 0; d < 3; ++d) {
       const int odd = (om >> d) & 1;
-      if ((J.sp1[s] >> d) & 1) J.st[s][d] = (short)(lo[d] - hG), J.cn[s][d] = (short)(hi[d] - lo[d] + 2 * hG);
+      if ((J.fl[s] >> d) & 1) J.st[s][d] = 0, J.cn[s][d] = (short)nall[d];
+      else if ((J.sp1[s] >> d) & 1) J.st[s][d] = (short)(lo[d] - hG), J.cn[s][d] = (short)(hi[d] - lo[d] + 2 * hG);
       else J.st[s][d] = (short)par_first(lo[d], odd), J.cn[s][d] = (short)par_count(lo[d], hi[d], odd);
     }
     J.n[s] = J.cn[s][0] * J.cn[s][1] * J.cn[s][2];
@@ -471,9 +510,44 @@ __device__ __forceinline__ void subst_run(const TP *src, int st, int n, bool cen
   }
 }
 
+// the same along flat axis d, for its odd points i .. i + n - 1: the line src holds
+// the sums at the coordinates of sub_coord, the even points inside count as 0
+template <int N, int NT, typename TP, typename F>
+__device__ __forceinline__ void subst_ends(const TP *src, int st, const SubAxes &J, int d, int i, int n, F put) {
+  using W = Wav<N, NT>;
+  constexpr int hG = W::hwG;
+  const int lo = J.lo[d], hi = J.hi[d], y = J.o0[d] + 2 * i, a = J.nlo[d], b = a + J.nod[d], e0 = J.e0[d],
+            e1 = J.e1[d] - 2 * b;
+  const TP *c = src + (a + i) * st;
+  if (y - hG >= lo && y + 2 * (n - 1) + hG < hi) {
+#pragma unroll
+    for (int m = 0; m < SUB_RUN; ++m)
+      if (m < n) put(m, c[m * st]);
+    return;
+  }
+  TP e[N - 1 + SUB_RUN];
+#pragma unroll
+  for (int x = 0; x < N - 1 + SUB_RUN; ++x) {
+    const int v = y + 2 * x - hG;
+    e[x] = x < N - 1 + n && (v < lo || v >= hi) ? src[((v - (v < lo ? e0 : e1)) >> 1) * st] : TP(0);
+  }
+#pragma unroll
+  for (int m = 0; m < SUB_RUN; ++m) {
+    if (m >= n) break;
+    TP acc = TP(0);
+#pragma unroll
+    for (int x = 0; x < N; ++x) {
+      if (x == N / 2) acc = radd(acc, c[m * st]);
+      acc = racc(acc, TP(W::G(2 * x - hG)), e[m + x]);
+    }
+    put(m, acc);
+  }
+}
+
 template <int N, int NT, typename TP>
-__device__ __forceinline__ void subst_jobs(TP *Pb, int Wd, int Gi, const SubJob *jobs, int j0, int jend, TP *buf,
-                                           int cap) {
+__device__ __forceinline__ void subst_jobs(TP *Pb, int Wd, int Gi, const SubJob *jobs, const SubAxes *axes, int j0,
+                                           int jend, TP *buf, int cap) {
+  constexpr bool FLAT = sub_flat<TP>;
   const int W2 = Wd * Wd, bd = blockDim.x;
   while (j0 < jend) {
     const int j1 = jobs[j0].next, deg = jobs[j0].deg;
@@ -482,12 +556,13 @@ __device__ __forceinline__ void subst_jobs(TP *Pb, int Wd, int Gi, const SubJob 
       int rot = 0;  // the items of a job continue the thread rotation of the previous one
       for (int j = j0; j < j1; ++j) {
         const SubJob &J = jobs[j];
+        const SubAxes &A = axes[J.box];
         const int n = J.it[s];
         int idx = (int)threadIdx.x - rot;
         if (idx < 0) idx += bd;
         rot = turn(rot, n, bd);
         if (idx >= n) continue;
-        const int st0 = J.st[s][0], st1 = J.st[s][1], st2 = J.st[s][2], sp1 = J.sp1[s];
+        const int st0 = J.st[s][0], st1 = J.st[s][1], st2 = J.st[s][2], sp1 = J.sp1[s], fl = J.fl[s];
         const int h0 = !(sp1 & 1), h1 = !(sp1 & 2), h2 = !(sp1 & 4);  // log2 of the steps
         const int d = J.o[s], cd = J.cn[s][d];
         const int c0 = J.cn[s][0], c1 = J.cn[s][1];
@@ -500,7 +575,9 @@ __device__ __forceinline__ void subst_jobs(TP *Pb, int Wd, int Gi, const SubJob 
           const int r = divq(idx, dc0), q2 = divq(r, dc1), q0 = idx - r * m0, q1 = r - q2 * m1;
           const int i0 = d == 0 ? q0 * SUB_RUN : q0, i1 = d == 1 ? q1 * SUB_RUN : q1, i2 = d == 2 ? q2 * SUB_RUN : q2;
           const int nr = min(SUB_RUN, cd - (d == 0 ? i0 : d == 1 ? i1 : i2));  // points of this run
-          const int p0 = st0 + (i0 << h0), p1 = st1 + (i1 << h1), p2 = st2 + (i2 << h2);
+          const int p0 = FLAT && fl & 1 ? sub_coord(A, 0, i0) : st0 + (i0 << h0),
+                    p1 = FLAT && fl & 2 ? sub_coord(A, 1, i1) : st1 + (i1 << h1),
+                    p2 = FLAT && fl & 4 ? sub_coord(A, 2, i2) : st2 + (i2 << h2);
           TP *pt = Pb + (p0 + Gi) + Wd * (p1 + Gi) + W2 * (p2 + Gi);
           TP *out = dst + i0 + c0 * (i1 + c1 * i2);
           auto put = [&](int m, TP acc) {
@@ -524,6 +601,12 @@ __device__ __forceinline__ void subst_jobs(TP *Pb, int Wd, int Gi, const SubJob 
             if (s > 0) {
               const int k0 = J.cn[s - 1][0], k1 = k0 * J.cn[s - 1][1];
               ss = d == 0 ? 1 : d == 1 ? k0 : k1;
+              if (FLAT && ((J.flat >> d) & 1)) {
+                subst_ends<N, NT>(buf + J.off + (s == 2 ? J.n[0] : 0) + (d == 0 ? 0 : i0) + k0 * (d == 1 ? 0 : i1) +
+                                      k1 * (d == 2 ? 0 : i2),
+                                  ss, A, d, d == 0 ? i0 : d == 1 ? i1 : i2, nr, put);
+                continue;
+              }
               src = buf + J.off + (s == 2 ? J.n[0] : 0) + (J.st[s][d] - J.st[s - 1][d]) * ss +
                     (d == 0 ? 2 * i0 : i0) + k0 * (d == 1 ? 2 * i1 : i1) + k1 * (d == 2 ? 2 * i2 : i2);
             }
@@ -555,6 +638,7 @@ struct PrepPlan {
   RefBox ref[28];
   int nref, refnext[28];  // refinement boxes; end of the batch a box opens
   SubJob job[49];
+  SubAxes axes[7];
   int job0[4];            // first job of each degree (job0[3]: end)
   PushBox pbox[7];
   int npb;
@@ -823,7 +907,7 @@ __global__ void __launch_bounds__(sizeof(TP) == 4 ? 512 : 384, 2) k_prep(Tree t,
     if (tid < 7 * nbx) {
       const int k = tid < 3 * nbx ? tid % 3 : tid < 6 * nbx ? 3 + (tid - 3 * nbx) % 3 : 6;
       const int e = tid < 3 * nbx ? tid / 3 : tid < 6 * nbx ? (tid - 3 * nbx) / 3 : tid - 6 * nbx;
-      sub_job_build(plan.job[tid], plan.band.lo[e], plan.band.hi[e], cls[k], W::hwG);
+      sub_job_build(plan.job[tid], plan.axes, e, plan.band.lo[e], plan.band.hi[e], cls[k], W::hwG, sub_flat<TP> ? plan.band.flat[e] : 0);
     }
   }
   // layout of the substitution sums: batches within a degree (by one thread,
@@ -1013,7 +1097,7 @@ __global__ void __launch_bounds__(sizeof(TP) == 4 ? 512 : 384, 2) k_prep(Tree t,
   // substitution, degree by degree (a point of degree d reads lower degrees
   // only, so the classes of one degree are independent)
   for (int deg = 1; deg <= 3; ++deg)
-    subst_jobs<N, NT, TP>(Pb, Wd, Gi, plan.job, plan.job0[deg - 1], plan.job0[deg], reinterpret_cast<TP *>(smraw), capP);
+    subst_jobs<N, NT, TP>(Pb, Wd, Gi, plan.job, plan.axes, plan.job0[deg - 1], plan.job0[deg], reinterpret_cast<TP *>(smraw), capP);
   // (N.0: H^a is the identity and even points are never substituted, so the
   // coincident values the gather took are already the coarsened ones)
   if (only_coarse == 2 || NT == 0) return;
