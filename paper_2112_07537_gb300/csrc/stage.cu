@@ -131,7 +131,8 @@ __device__ __forceinline__ float stage_value(const StageArgs &s, float c, float 
 // 6.2 ghosts): 3 424 leaves of 24^3 with velocity fields 1 660 us (whole block per
 // CTA), 742 (slabs), 530 (fewer copies), 527 (packed); 42 400 leaves with a
 // constant velocity 15.35 ms, 6.02, 4.97, 3.99; 11 019 leaves of 16^3 with velocity
-// fields 1 333 us, 836, 596, 476; 1 272 leaves with diffusion 104 us, 89, 74.
+// fields 1 333 us, 836, 596, 476 (4.2); 1 272 leaves of 20^3 with diffusion 104 us,
+// 89 and 72 (2.2; from the slabs on).
 // k_march takes 1 070 us, 8.5 ms and 1 047 us in the first three.  Separate code for
 // x and y walks, or unrolled z walks, is slower by a tenth (instruction cache).
 // ---------------------------------------------------------------------------
