@@ -58,22 +58,27 @@ __device__ __forceinline__ float weno_corr(float c0, float c1, float c2, float n
 // the four divisions become one: a_k times (c_0 c_1 c_2)^2 is
 // (c_0 c_1 c_2)^2 + (tau c_i c_j)^2.  Where that product could leave the
 // exponent range (c above 1e45, infinities, NaN) or the cap could act (tau
-// above 2^49 c, checked on the exponent words), the quotients are taken one by
-// one.
+// above 2^49 c), the quotients are taken one by one.  Where tau is below 2^-26
+// of every c, r_k^2 < 2^-53 and each a_k is 1 to rounding: it is taken as 1, for
+// the scaled weights of a field so small that every c is eps are 1e-180 and their
+// products with N_k would underflow (from differences of 1e-128 down).  All
+// three tests are on the exponent words, whose difference is at most 0.1 off the
+// logarithm of the ratio.
 __device__ __forceinline__ double weno_corr(double c0, double c1, double c2, double n0, double n1, double n2) {
   const double tau = fabs(c0 - c2);
   const unsigned k0 = (unsigned)__double2hiint(c0), k1 = (unsigned)__double2hiint(c1),
                  k2 = (unsigned)__double2hiint(c2);
   const unsigned hi = max(max(k0, k1), k2), lo = min(min(k0, k1), k2);
-  double a0, a1, a2;
-  if (hi > 0x49466bb7u || (int)lo <= __double2hiint(tau) - (49 << 20)) {
+  const int above = (int)lo - __double2hiint(tau);  // c over tau, in exponent words
+  double a0 = 1.0, a1 = 1.0, a2 = 1.0;
+  if (hi > 0x49466bb7u || above <= -(49 << 20)) {
     const double cap = WenoC<double>::rcap;
     double r0 = tau / c0, r1 = tau / c1, r2 = tau / c2;
     r0 = r0 > cap ? cap : r0;
     r1 = r1 > cap ? cap : r1;
     r2 = r2 > cap ? cap : r2;
     a0 = fma(r0, r0, 1.0), a1 = fma(r1, r1, 1.0), a2 = fma(r2, r2, 1.0);
-  } else {
+  } else if (above < (27 << 20)) {
     const double q0 = c1 * c2, q1 = c0 * c2, q2 = c0 * c1, pr = q0 * c0, p2 = pr * pr;
     const double e0 = tau * q0, e1 = tau * q1, e2 = tau * q2;
     a0 = fma(e0, e0, p2), a1 = fma(e1, e1, p2), a2 = fma(e2, e2, p2);
