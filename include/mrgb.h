@@ -230,7 +230,8 @@ int mr_ghost_fill_static(mr_grid *grid, int fid, int G, void *padded);
 
 /* Wait for the grid's stream and report device-side errors recorded by the
  * kernels since the last check (MR_ERR_BALANCE: a ghost point was owned by
- * a leaf more than one level away, or a shell exceeded the stored padding). */
+ * a leaf more than one level away, or a shell exceeded the stored padding;
+ * on periodic grids also a NaN among the refined ghosts of a coarser leaf). */
 int mr_sync(mr_grid *grid);
 
 /* rhs = -sum_d (F_{i+1/2} - F_{i-1/2}) / h for d(phi)/dt + div(u phi) = 0,

@@ -213,6 +213,7 @@ struct PrepTab {
   int rmul[27];
   int cmask, ce;  // coarser directions (bit region), coarser neighbours (bit e)
   int s[3], odd[3];  // outward side per axis (+-1), anchor parity
+  int miss;          // prep_fetch met a point that no leaf holds
 };
 
 // up to 7 disjoint boxes over [0, n) per axis, the layers (dlo on the - side,
@@ -253,9 +254,10 @@ __device__ __forceinline__ void outward_boxes(Boxes &B, int ce, const int *s, in
 }
 
 // level-Lq value (Lq = L or L - 1) at block-local point (i, j, k) through the
-// region tables, or through the owner map beyond the neighbouring regions
+// region tables, or through the owner map beyond the neighbouring regions; NaN,
+// and T.miss set, where no leaf holds the point
 template <typename TI>
-__device__ __noinline__ TI prep_fetch(const Tree &t, const PrepTab &T, const TI *phi, int b, int L, int Lq, int i, int j,
+__device__ __noinline__ TI prep_fetch(const Tree &t, PrepTab &T, const TI *phi, int b, int L, int Lq, int i, int j,
                                       int k, int *err) {
   const int nb = t.nb, hb = nb / 2, sc = Lq == L ? 1 : 2;
   const size_t nb3 = (size_t)nb * nb * nb;
@@ -277,7 +279,10 @@ __device__ __noinline__ TI prep_fetch(const Tree &t, const PrepTab &T, const TI 
   int g[3];
   for (int d = 0; d < 3; ++d) g[d] = (Lq == L ? T.ranc[13][d] * nb : T.ranc[13][d] * nb / 2) + (d == 0 ? i : d == 1 ? j : k);
   const int o = owner(t, Lq, g[0], g[1], g[2], b);
-  if (__ldg(t.lev + o) < Lq) return TI(__int_as_float(0x7fc00000));
+  if (__ldg(t.lev + o) < Lq) {
+    T.miss = 1;
+    return TI(__int_as_float(0x7fc00000));
+  }
   return leaf_value(t, phi, o, Lq, g[0], g[1], g[2], err);
 }
 
@@ -714,7 +719,7 @@ __global__ void __launch_bounds__(sizeof(TP) == 4 ? 512 : 384, 2) k_prep(Tree t,
   __shared__ PrepPlan plan;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int capU = sum_bytes / (int)sizeof(U), capP = sum_bytes / (int)sizeof(TP);
-  if (tid == 0) T.cmask = 0, T.ce = 0;
+  if (tid == 0) T.cmask = 0, T.ce = 0, T.miss = 0;
   __syncthreads();
   // owners of the 27 block-sized regions around b (same or coarser leaves own
   // a whole region); regions beyond a physical boundary count as the block
@@ -1091,7 +1096,8 @@ __global__ void __launch_bounds__(sizeof(TP) == 4 ? 512 : 384, 2) k_prep(Tree t,
       e0 = e1;
     }
   }
-  if (__syncthreads_or(bad) && tid == 0) atomicOr(err, 2);
+  // (a NaN of the field itself is no error on grids with physical boundaries)
+  if (__syncthreads_or(bad) && (!BND || T.miss) && tid == 0) atomicOr(err, 2);
   if (BND && bc_touches(t, L, ax, ay, az, -Gi, nb + Gi))
     bc_box<N>(t, L, ax, ay, az, Pb + Gi * (1 + Wd + W2), Wd, W2, -Gi, -Gi, -Gi, Wd, Wd, Wd);
   // substitution, degree by degree (a point of degree d reads lower degrees
