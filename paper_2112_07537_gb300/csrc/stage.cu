@@ -233,6 +233,8 @@ __global__ void __launch_bounds__(160, VEL ? 3 : 4) k_fused(Tree t, StageArgs s,
   __syncthreads();
   const float invh = 1.0f / sh_h;
   const float lk = LAP ? 0.5f * s.nu * invh : 0.f;  // rhs = -2/h (dF - lk lap)
+  // (axes walked for the Laplacian alone add no flux: 0 times an infinity or NaN
+  // would reach the whole stencil)
   const bool xon = VEL || LAP || s.ux != 0.f, yon = VEL || LAP || s.uy != 0.f, zon = VEL || LAP || s.uz != 0.f;
   // Pairs of x lines, then of y lines: line q and line q + np, which lie os and
   // ov floats apart in T and in X / Y (y lines: neighbours, np = 1).  A constant
@@ -267,7 +269,7 @@ __global__ void __launch_bounds__(160, VEL ? 3 : 4) k_fused(Tree t, StageArgs s,
     for (int m = 0; m < nb; ++m) {
       const float2 vn = hv(m + 3), an = phi(m + 3);
       wk.step(s.diff, an, vn, [&](float2 dF, float2, float2 lap) {
-        if (LAP) dF = pfma(-lk, lap, dF);
+        if (LAP) dF = pfma(-lk, lap, VEL || uu != 0.f ? dF : both(0.f));
         w[m * dsv] = dF.x, w[m * dsv + ov] = dF.y;
       });
     }
@@ -312,6 +314,7 @@ __global__ void __launch_bounds__(160, VEL ? 3 : 4) k_fused(Tree t, StageArgs s,
     float *op = s.out + q0;
     float2 uo = rk_u ? ld2(up) : both(0.f);  // u^n of the current cell
     auto finish = [&](float2 dF, float2 ph, float2 lap, float2 un) {
+      if (LAP && !VEL && s.uz == 0.f) dF = both(0.f);
       const float2 acc = padd(padd(xon ? ld2(xp) : both(0.f), yon ? ld2(yp) : both(0.f)), LAP ? pfma(-lk, lap, dF) : dF);
       float2 r = pmul(acc, both(k2));
       if (!s.rhs_only) r = pfma(s.cv, pfma(s.dt, r, ph), pmul(both(s.cu), un));
