@@ -105,7 +105,7 @@ static size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 static int layout(const mr_grid_desc *d, Layout *L, int *shell_rk, int *shell_ad, size_t *map_cells,
                   int *M) {
   if (!d) return MR_ERR_INVALID;
-  if (d->nb < 8 || d->nb > 32 || (d->nb & 1)) return MR_ERR_INVALID;
+  if (d->nb < 8 || d->nb > MAX_NB || (d->nb & 1)) return MR_ERR_INVALID;
   if (!((d->wav_N == 2 || d->wav_N == 4 || d->wav_N == 6) && (d->wav_Nt == 0 || d->wav_Nt == 2)))
     return MR_ERR_INVALID;
   if (d->precision != MR_F32 && d->precision != MR_F64) return MR_ERR_INVALID;

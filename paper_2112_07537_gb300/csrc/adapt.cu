@@ -74,6 +74,7 @@ __host__ __device__ __forceinline__ size_t det_elems(int nR, int w) {
 // threads of a CTA, and items per thread and pass (det_tiles cuts accordingly):
 // the index arithmetic of a pass is done once, not once per plane
 constexpr int DET_THREADS = 512, DET_ITEMS = 2;
+constexpr size_t DET_BYTES = 110 * 1024;  // shared memory: two CTAs on an SM
 
 template <int N, int NT, bool PAIRS, typename TP, typename F>
 __device__ __forceinline__ void detail_planes(const TP *__restrict__ Pb, int nb, int Gi, const DetBox &B,
@@ -258,7 +259,7 @@ static int det_tiles(int nb, size_t es, size_t *bytes) {
     }
     const int nR = r1 - r0 + 1, items = std::max(w * nR, (w + 1) / 2 * (nR + 2 * (N - 1)));
     *bytes = es * det_elems<N>(nR, w);
-    if (*bytes <= 110 * 1024 && items <= DET_ITEMS * DET_THREADS) return nt;
+    if (*bytes <= DET_BYTES && items <= DET_ITEMS * DET_THREADS) return nt;
   }
 }
 
@@ -308,7 +309,7 @@ static int criterion_launch(mr_grid *g, const double *P, int Gi, double *maxdet)
   if (8 * ((size_t)(2 * N + 1) * nR * nR + (size_t)nR * nA + (PAIRS ? (size_t)nA * nA : 0)) > 227 * 1024)
     return MR_ERR_UNSUPPORTED;
   const auto kc = k_criterion<N, NT, PAIRS>;
-  if (check_cuda(cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), "criterion smem") ||
+  if (smem_limit(kc, DET_BYTES, "criterion smem") ||
       check_cuda(cudaMemsetAsync(maxdet, 0, sizeof(double) * (size_t)n, g->stream), "criterion norms"))
     return MR_ERR_CUDA;
   unsigned long long *md = reinterpret_cast<unsigned long long *>(maxdet);
@@ -497,6 +498,11 @@ constexpr int INTERP_Z = 8;
 static size_t interp_smem(int N, int nb, size_t es) {
   const size_t m = nb / 2 + N - 1;
   return es * INTERP_Z * (m * (m | 1) + (size_t)nb * (m | 1));
+}
+// sums of four layers of a new parent's octant (fine extent: a child's and the H^a half-widths)
+static size_t parent_smem(int hH, int nb, size_t es) {
+  const size_t fw = nb - 1 + 2 * hH;
+  return es * 4 * fw * (fw + nb / 2);
 }
 
 template <typename TO, typename TP, int N, int NT>
@@ -878,12 +884,12 @@ static int interp_update(mr_grid *g, const Tree &to, const Tree &tn, const TP *P
   const int tp = sizeof(TP) == 4 ? 4 : sizeof(TO) == 4 ? 5 : 8;
   const int nb = g->desc.nb;
   const size_t smi = interp_smem(N, nb, sizeof(TP));
-  const int hH = Wav<N, NT>::hwH, fw = nb - 1 + 2 * hH;  // fine extent of a child's sums
-  const size_t smp = sizeof(TP) * 4 * (size_t)fw * (fw + nb / 2);
+  constexpr int hH = Wav<N, NT>::hwH;
+  const size_t smp = parent_smem(hH, nb, sizeof(TP));
   const auto ki = k_interp<TO, TP, N, NT>;
   const auto kp = k_interp_parent<TO, TP, N, NT>;
-  if (check_cuda(cudaFuncSetAttribute(ki, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smi), "interp smem") ||
-      check_cuda(cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smp), "interp smem"))
+  if (smem_limit(ki, interp_smem(N, MAX_NB, sizeof(TP)), "interp smem") ||
+      smem_limit(kp, parent_smem(hH, MAX_NB, sizeof(TP)), "interp smem"))
     return MR_ERR_CUDA;
   const TO *fo = (const TO *)field_ptr(g, fid);
   TO *fn = (TO *)next_field_ptr(g, fid);
@@ -895,12 +901,9 @@ static int interp_update(mr_grid *g, const Tree &to, const Tree &tn, const TP *P
   MR_LAUNCH(g, MRK_INTERP, kp<<<8 * tn.nleaf, 256, smp, g->stream>>>(to, src, P, Gi, fn, (int)(smp / sizeof(TP))));
   const size_t smg = sizeof(TP) == 4 ? 72 * 1024 : 110 * 1024;  // three / two CTAs of 512 threads per SM
   const size_t sma = apply_smem<N, NT>(nb, sizeof(TP));
-  if (sma > 227 * 1024) return MR_ERR_UNSUPPORTED;
-  if (check_cuda(cudaFuncSetAttribute(k_update_gamma<TP, N, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smg),
-                 "update smem") ||
-      check_cuda(cudaFuncSetAttribute(k_update_apply<TO, TP, N, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sma),
+  if (sma > MAX_SMEM) return MR_ERR_UNSUPPORTED;
+  if (smem_limit(k_update_gamma<TP, N, NT>, smg, "update smem") ||
+      smem_limit(k_update_apply<TO, TP, N, NT>, std::min(apply_smem<N, NT>(MAX_NB, sizeof(TP)), MAX_SMEM),
                  "update smem"))
     return MR_ERR_CUDA;
   MR_LAUNCH(g, MRK_UPDATE, k_update_gamma<TP, N, NT><<<tn.nleaf, DET_THREADS, smg, g->stream>>>(

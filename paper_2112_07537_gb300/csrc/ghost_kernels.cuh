@@ -1294,12 +1294,9 @@ int ghost_impl(mr_grid *g, const TI *phi_in, TI *phi_out, int G, TP *P, TP *Q, i
   const auto prep = t.bnd ? k_prep<TI, TP, N, NT, true> : k_prep<TI, TP, N, NT, false>;
   const auto merge = t.bnd ? k_merge<TI, TP, N, NT, true> : k_merge<TI, TP, N, NT, false>;
   const size_t sm = prep_sum_bytes(N, nb, Gi, sizeof(TP), t.bnd != 0);
-  if (sm > 200 * 1024) return MR_ERR_UNSUPPORTED;
-  // (set on every launch: the kernel's static shared memory counts against
-  // the 48 KB that needs no opt-in)
-  if (check_cuda(cudaFuncSetAttribute(prep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
-                 "k_prep smem"))
-    return MR_ERR_CUDA;
+  constexpr size_t most = 200 * 1024;  // leaves room for the kernel's static tables
+  if (sm > most) return MR_ERR_UNSUPPORTED;
+  if (smem_limit(prep, most, "k_prep smem")) return MR_ERR_CUDA;
   const int tp = sizeof(TP) == 4 ? 4 : sizeof(TI) == 4 ? 5 : 8;
   // 256 threads per leaf; more where the grid does not fill the chip (a leaf's
   // phases are latency-bound: 120 leaves of 16^3 with 4.2)

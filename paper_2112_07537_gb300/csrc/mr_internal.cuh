@@ -551,6 +551,18 @@ void kt_end(mr_grid *g);
 mr::Tree tree_view(const mr_grid *g);
 int set_error(const char *msg);
 int check_cuda(cudaError_t e, const char *where);
+
+// Dynamic shared memory a kernel may be launched with.  The limit belongs to the
+// function, not to a grid, so every call for a function passes the same number, the
+// most that any accepted grid asks for: with each launch's own size, a host thread
+// working on a smaller grid could lower it between another thread's call and its
+// launch.
+constexpr int MAX_NB = 32;  // largest block that mr_grid_create accepts
+constexpr size_t MAX_SMEM = 227 * 1024;  // of an SM
+template <typename K>
+int smem_limit(K kernel, size_t most, const char *where) {
+  return check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most), where);
+}
 void *field_ptr(mr_grid *g, int fid);      // fid >= nfields: temporaries
 void *next_field_ptr(mr_grid *g, int fid);
 

@@ -144,6 +144,10 @@ __host__ __device__ constexpr int fused_smem_floats(int nb, int nz, bool vel) {
          nz * (vel ? nb + 6 : nb) * nb;
 }
 
+// largest block, and its slabs: a quarter of a large and half of a small one
+constexpr int FUSED_MAX_NB = 26;
+__host__ __device__ constexpr int fused_height(int nb) { return nb > 16 ? (nb + 3) / 4 : nb / 2; }
+
 template <int SCHEME, bool VEL, bool LAP>
 __global__ void __launch_bounds__(160, VEL ? 3 : 4) k_fused(Tree t, StageArgs s, int nz, int nslab) {
   const int b = blockIdx.x / nslab, sl = blockIdx.x - b * nslab;
@@ -377,6 +381,7 @@ __global__ void __launch_bounds__(160, VEL ? 3 : 4) k_fused(Tree t, StageArgs s,
 // rounded products in both, never contracted; where the compiler fuses another
 // multiply-add differently the two may differ in the last bit).
 // ---------------------------------------------------------------------------
+constexpr int MARCH_MAX_NB = 24;
 // faces, XP..FY, PH[3], and (velocity fields) UX[2], UY[2]
 __host__ __device__ constexpr int march_smem_floats(int nb, bool vel) {
   return 18 * nb * nb + 4 * nb * (nb + 1) + (vel ? 11 : 7) * (nb + 6) * (nb + 6);
@@ -591,7 +596,7 @@ int launch_fused(mr_grid *g, const void *phi, const void *P, const void *Q, int 
   Tree t = tree_view(g);
   const bool vel = vpad != nullptr;
   const int nb = g->desc.nb, N = g->desc.wav_N, NT = g->desc.wav_Nt;
-  if (nb > 26) {  // the block with its ghosts and flux differences exceeds an SM's shared memory
+  if (nb > FUSED_MAX_NB) {
     set_error("FP32 stage: blocks of more than 26 points per edge");
     return MR_ERR_CUDA;
   }
@@ -599,23 +604,21 @@ int launch_fused(mr_grid *g, const void *phi, const void *P, const void *Q, int 
               (float *)out, stage, rhs_only ? 1 : 0, (float)dt, (float)uc[0], (float)uc[1], (float)uc[2],
               (const float *)vpad, (float)g->diff_nu, (float)g->vel_scale, g->diff_order, divm(nb + 6),
               stage == 0 ? 0.f : stage == 1 ? 0.75f : 1.0f / 3, stage == 0 ? 1.f : stage == 1 ? 0.25f : 2.0f / 3};
-  const bool march_ok = nb >= 12 && nb * nb <= 576;
+  const bool march_ok = nb >= 12 && nb <= MARCH_MAX_NB;
   const size_t smm = sizeof(float) * (size_t)march_smem_floats(nb, vel);
-  // slab heights: a quarter of a large and half of a small block, or four planes
+  // slab heights: fused_height, or four planes
   // (four instead of eight at 16^3: 613 against 500 us for 11 019 leaves; instead
   // of six at 24^3: 4.88 against 4.44 ms for 42 400)
-  const int hq = nb > 16 ? (nb + 3) / 4 : nb / 2, ht = 4;
+  const int hq = fused_height(nb), ht = 4;
   auto threads_of = [&](int nz) { return std::min(160, (nb * nz + 31) / 32 * 32); };
   const int cand[2] = {threads_of(hq), threads_of(ht)};
   const int ncand = cand[0] != cand[1] ? 2 : 1;
   const int vcand[2] = {1, 2};
   const bool can_tune = rhs_only || stage == 0;
   auto run = [&](auto kf, auto km) -> int {
-    const int smf_max = (int)sizeof(float) * fused_smem_floats(nb, std::max(hq, ht), vel);
-    if (check_cuda(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, smf_max), "fused smem"))
+    if (smem_limit(kf, sizeof(float) * fused_smem_floats(FUSED_MAX_NB, fused_height(FUSED_MAX_NB), vel), "fused smem"))
       return MR_ERR_CUDA;
-    if (march_ok &&
-        check_cuda(cudaFuncSetAttribute(km, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smm), "march smem"))
+    if (march_ok && smem_limit(km, sizeof(float) * march_smem_floats(MARCH_MAX_NB, vel), "march smem"))
       return MR_ERR_CUDA;
     const int mode = 2 * scheme + (vel ? 1 : 0);
     auto fused = [&](int th) {

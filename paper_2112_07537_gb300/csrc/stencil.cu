@@ -118,8 +118,7 @@ static int rhs_dispatch(mr_grid *g, const T *P, int Gi, const T *u, T *out, int 
     while (seg > 4 && 2 * nb * nz * ((nb + seg - 1) / seg) < 256) seg = (seg + 1) / 2;
   const size_t sm = 2 * sizeof(T) * (size_t)nz * nb * (nb + 1);
   auto go = [&](auto kern) -> int {
-    if (check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), "rhs smem"))
-      return MR_ERR_CUDA;
+    if (smem_limit(kern, 2 * sizeof(T) * 8 * MAX_NB * (MAX_NB + 1), "rhs smem")) return MR_ERR_CUDA;
     MR_LAUNCH(g, MRK_RHS, kern<<<n * nslab, 256, sm, g->stream>>>(t, P, Gi, u, out, stage, T(dt), ux, uy, uz, rhs_only,
                                                                   vpad, T(g->diff_nu), g->diff_order, T(g->vel_scale),
                                                                   nz, nslab, seg));
