@@ -1300,8 +1300,9 @@ int ghost_impl(mr_grid *g, const TI *phi_in, TI *phi_out, int G, TP *P, TP *Q, i
   const int tp = sizeof(TP) == 4 ? 4 : sizeof(TI) == 4 ? 5 : 8;
   // 256 threads per leaf; more where the grid does not fill the chip (a leaf's
   // phases are latency-bound: 120 leaves of 16^3 with 4.2)
-  const int big = sizeof(TP) == 4 ? 512 : 384, cp[2] = {n > 2 * 152 ? 256 : big, n > 2 * 152 ? 128 : 256};
-  const int thp = tune_threads(g, TuneKey{1, N, NT, nb, tp, Gi, only_coarse}, cp, 2, [&](int th) {
+  const int big = sizeof(TP) == 4 ? 512 : 384, many = n > 2 * 152, cp[2] = {many ? 256 : big, many ? 128 : 256};
+  const int bnd = t.bnd != 0;
+  const int thp = tune_threads(g, TuneKey{1, N, NT, nb, tp, Gi, only_coarse + 4 * many + 8 * bnd}, cp, 2, [&](int th) {
     prep<<<n, th, sm, g->stream>>>(t, phi_in, P, Q, Gi, G, only_coarse, g->cmask, err, need, g->pneed, (int)sm);
   });
   MR_LAUNCH(g, MRK_PART1, prep<<<n, thp, sm, g->stream>>>(t, phi_in, P, Q, Gi, G, only_coarse, g->cmask, err, need,
@@ -1315,7 +1316,7 @@ int ghost_impl(mr_grid *g, const TI *phi_in, TI *phi_out, int G, TP *P, TP *Q, i
   }
   if (only_coarse) return MR_OK;
   static const int cm[3] = {256, 128, 512};
-  const int thm = tune_threads(g, TuneKey{5, N, NT, nb, tp, Gi, 0}, cm, 3, [&](int th) {
+  const int thm = tune_threads(g, TuneKey{5, N, NT, nb, tp, Gi, 8 * bnd}, cm, 3, [&](int th) {
     merge<<<n, th, 0, g->stream>>>(t, P, Q, Gi, G, g->cmask, phi_out, need);
   });
   MR_LAUNCH(g, MRK_MERGE, merge<<<n, thm, 0, g->stream>>>(t, P, Q, Gi, G, g->cmask, phi_out, need));

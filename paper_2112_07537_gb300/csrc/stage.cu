@@ -620,7 +620,7 @@ int launch_fused(mr_grid *g, const void *phi, const void *P, const void *Q, int 
       return MR_ERR_CUDA;
     if (march_ok && smem_limit(km, sizeof(float) * march_smem_floats(MARCH_MAX_NB, vel), "march smem"))
       return MR_ERR_CUDA;
-    const int mode = 2 * scheme + (vel ? 1 : 0);
+    const int mode = 2 * scheme + (vel ? 1 : 0) + (g->diff_order ? 8 : 0);
     auto fused = [&](int th) {
       const int ns = (nb + (th == cand[0] ? hq : ht) - 1) / (th == cand[0] ? hq : ht), nz = (nb + ns - 1) / ns;
       kf<<<g->nleaf * ns, th, sizeof(float) * fused_smem_floats(nb, nz, vel), g->stream>>>(t, s, nz, ns);

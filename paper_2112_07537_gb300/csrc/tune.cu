@@ -3,7 +3,8 @@
 // the first time a key is met on a grid with autotuning enabled, each
 // candidate is launched on the grid's own data (once to warm up, then timed
 // with CUDA events on the grid's stream) and the fastest is kept in a
-// process-wide table that every later launch with that key reads.  Only
+// process-wide table that every later launch with that key reads, on this grid or
+// another: whatever selects the kernel or its candidates is part of the key.  Only
 // launches that give the same result when repeated are tuned (they read
 // their inputs and overwrite their outputs), so tuning changes no value:
 // every kernel computes each output point with the same arithmetic whatever
