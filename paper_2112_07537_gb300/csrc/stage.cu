@@ -596,10 +596,6 @@ int launch_fused(mr_grid *g, const void *phi, const void *P, const void *Q, int 
   Tree t = tree_view(g);
   const bool vel = vpad != nullptr;
   const int nb = g->desc.nb, N = g->desc.wav_N, NT = g->desc.wav_Nt;
-  if (nb > FUSED_MAX_NB) {
-    set_error("FP32 stage: blocks of more than 26 points per edge");
-    return MR_ERR_CUDA;
-  }
   StageArgs s{(const float *)phi, (const float *)P, (const float *)Q, Gi, NT != 0, g->cmask, (const float *)u,
               (float *)out, stage, rhs_only ? 1 : 0, (float)dt, (float)uc[0], (float)uc[1], (float)uc[2],
               (const float *)vpad, (float)g->diff_nu, (float)g->vel_scale, g->diff_order, divm(nb + 6),
@@ -616,6 +612,10 @@ int launch_fused(mr_grid *g, const void *phi, const void *P, const void *Q, int 
   const int vcand[2] = {1, 2};
   const bool can_tune = rhs_only || stage == 0;
   auto run = [&](auto kf, auto km) -> int {
+    if (nb > FUSED_MAX_NB) {
+      set_error("FP32 stage: blocks of more than 26 points per edge");
+      return MR_ERR_CUDA;
+    }
     if (smem_limit(kf, sizeof(float) * fused_smem_floats(FUSED_MAX_NB, fused_height(FUSED_MAX_NB), vel), "fused smem"))
       return MR_ERR_CUDA;
     if (march_ok && smem_limit(km, sizeof(float) * march_smem_floats(MARCH_MAX_NB, vel), "march smem"))
