@@ -694,9 +694,19 @@ __device__ __noinline__ void bc_sums(const Tree &t, int Lc, const RefBox &B, int
 // the polynomial
 constexpr int prep_min_planes(int N, bool bounded) { return (N - 1) + 2 + 4 + (bounded ? N : 0); }
 
+// Blocks so narrow that coarse columns of the refinement leave the neighbouring
+// regions, where values are looked up through the owner map: 8^3 with 6.0, 8^3 and
+// 10^3 with 6.2.  Their kernel (NARROW) looks every value of such a column up once
+// (fills of 576 leaves of 8^3 with 6.2, shell 3: FP32 384 -> 206 us, FP64 426 -> 265;
+// of 55 leaves, FP64: 212 -> 149).  In the other blocks only columns that meet a finer
+// leaf are looked up; there the tap-by-tap form stays, since the window costs every
+// column registers (fill and crop of 2 080 leaves of 24^3 with 6.2, FP32: 488 us so, 492
+// with it).
+__host__ __device__ constexpr bool prep_narrow(int N, int nb, int Gi) { return (Gi + N) / 2 * 2 > nb; }
+
 // only_coarse: 0 every (needed) leaf, 1 the leaves next to coarser ones, 2 those
 // without the push
-template <typename TI, typename TP, int N, int NT, bool BND>
+template <typename TI, typename TP, int N, int NT, bool BND, bool NARROW>
 __global__ void __launch_bounds__(sizeof(TP) == 4 ? 512 : 384, 2) k_prep(Tree t, const TI *__restrict__ phi,
                                                                      TP *__restrict__ P, TP *__restrict__ Q, int Gi,
                                                                      int Gpush, int only_coarse, int *cmask_out,
@@ -992,7 +1002,15 @@ __global__ void __launch_bounds__(sizeof(TP) == 4 ? 512 : 384, 2) k_prep(Tree t,
           const int r0 = rr + (B.la < 0 ? 0 : 1) * ra, r1 = r0 + ra;
           if (ok) ok = T.rmul[r0] && T.rmul[r1];
           U *d = UB + B.off + jb + pitch * na * kc;
-          if (!ok) {  // a finer leaf or a region beyond the neighbours: point by point
+          if (!ok && NARROW) {  // a finer leaf or a region beyond the neighbours
+            auto at = [&](int qa) {
+              q[a] = qa;
+              return RS::from(prep_fetch<TI>(t, T, phi, b, L, L - 1, q[0], q[1], q[2], err));
+            };
+            refine_run<N, NT, RS>(at, B.la, na, [&](int ia, U v) { d[pitch * ia] = RS::norm(v); });
+            continue;
+          }
+          if (!ok) {
             for (int ia = 0; ia < na; ++ia) {
               U s = RS::zero();
               const int f = B.la + ia;
@@ -1291,7 +1309,9 @@ int ghost_impl(mr_grid *g, const TI *phi_in, TI *phi_out, int G, TP *P, TP *Q, i
   int *err = g->counter + 1;
   // (bounded grids have their own instantiations: their out-of-line calls would
   // cost the others registers)
-  const auto prep = t.bnd ? k_prep<TI, TP, N, NT, true> : k_prep<TI, TP, N, NT, false>;
+  auto prep = t.bnd ? k_prep<TI, TP, N, NT, true, false> : k_prep<TI, TP, N, NT, false, false>;
+  if constexpr (N == 6)  // (shorter filters never reach that far)
+    if (!t.bnd && prep_narrow(N, nb, Gi)) prep = k_prep<TI, TP, N, NT, false, true>;
   const auto merge = t.bnd ? k_merge<TI, TP, N, NT, true> : k_merge<TI, TP, N, NT, false>;
   const size_t sm = prep_sum_bytes(N, nb, Gi, sizeof(TP), t.bnd != 0);
   constexpr size_t most = 200 * 1024;  // leaves room for the kernel's static tables

@@ -28,21 +28,22 @@ struct RefSum<float, double> {
 };
 
 // Zero-detail refinement along one line: fine points f0 .. f0 + n - 1 (n <= 16)
-// from the coarse values src[q * st] (q: coarse index); put(m, v) receives
-// point f0 + m.  A register window of N coarse values moves along the line and
-// yields an even (coincident) and an odd (K^s) point per step.
-template <int N, int NT, typename RS, typename U, typename F>
-__device__ __forceinline__ void refine_run(const U *src, int st, int f0, int n, F put) {
+// from the coarse values at(q) (q: coarse index, each called once); put(m, v)
+// receives point f0 + m.  A register window of N coarse values moves along the
+// line and yields an even (coincident) and an odd (K^s) point per step.
+template <int N, int NT, typename RS, typename A, typename F>
+__device__ __forceinline__ void refine_run(A at, int f0, int n, F put) {
   using W = Wav<N, NT>;
+  using U = typename RS::U;
   constexpr int ko = N - 1, h = N / 2;
   // window w[0..N-1] = coarse q-h+1 .. q+h around the odd point 2q + 1
   const int q0 = f0 >> 1;
   U w[N];
 #pragma unroll
-  for (int x = 0; x + 1 < N; ++x) w[x] = src[(q0 - h + 1 + x) * st];
+  for (int x = 0; x + 1 < N; ++x) w[x] = at(q0 - h + 1 + x);
   const int par = f0 & 1;
   // (the last value of a window is read only where its odd point exists)
-  w[N - 1] = par || n > 1 ? src[(q0 + h) * st] : w[0];
+  w[N - 1] = par || n > 1 ? at(q0 + h) : w[0];
   for (int m = -par; m < n; m += 2) {  // even point m, odd point m + 1
     if (m >= 0) put(m, w[h - 1]);
     if (m + 1 < n) {
@@ -54,9 +55,14 @@ __device__ __forceinline__ void refine_run(const U *src, int st, int f0, int n, 
     if (m + 2 < n) {
 #pragma unroll
       for (int x = 0; x + 1 < N; ++x) w[x] = w[x + 1];
-      if (m + 3 < n) w[N - 1] = src[(q0 + (m + par) / 2 + 1 + h) * st];
+      if (m + 3 < n) w[N - 1] = at(q0 + (m + par) / 2 + 1 + h);
     }
   }
+}
+// the same from the coarse values src[q * st]
+template <int N, int NT, typename RS, typename U, typename F>
+__device__ __forceinline__ void refine_run(const U *src, int st, int f0, int n, F put) {
+  refine_run<N, NT, RS>([&](int q) { return src[q * st]; }, f0, n, put);
 }
 
 // tensor H^a along one line: sum_t H^a(t) src[(2 m + t) st], m = 0 .. n - 1 <= M,
