@@ -71,12 +71,13 @@ __host__ __device__ __forceinline__ size_t det_elems(int nR, int w) {
   return (size_t)(2 * ko + 3) * nR * w + (size_t)nA * w + (size_t)nA * (w + 2 * ko);
 }
 
-// threads of a CTA, and items per thread and pass (det_tiles cuts accordingly):
-// the index arithmetic of a pass is done once, not once per plane
+// Threads of a CTA, and items per thread and pass (det_tiles cuts accordingly):
+// with KEEP the index arithmetic of a pass is done once, not once per plane (see
+// criterion_impl).
 constexpr int DET_THREADS = 512, DET_ITEMS = 2;
 constexpr size_t DET_BYTES = 110 * 1024;  // shared memory: two CTAs on an SM
 
-template <int N, int NT, bool PAIRS, typename TP, typename F>
+template <int N, int NT, bool PAIRS, bool KEEP, typename TP, typename F>
 __device__ __forceinline__ void detail_planes(const TP *__restrict__ Pb, int nb, int Gi, const DetBox &B,
                                               typename DetOps<TP, PAIRS>::E *sm, F emit) {
   using W = Wav<N, NT>;
@@ -102,27 +103,44 @@ __device__ __forceinline__ void detail_planes(const TP *__restrict__ Pb, int nb,
     return q < nR ? ko + q : q < nR + eb ? (r0 & 1 ? ko - 1 : ko - 2) - 2 * (q - nR)
                                          : ko + nR + (r1 & 1 ? 0 : 1) + 2 * (q - nR - eb);
   };
-  // the thread's items of every pass, the same on all planes (-1: none).  x
-  // passes: (row, column) of A, packed; y and z passes: offset in a plane
-  int xo[K], xe[K], yo[K], ye[K];
+  // items of the passes, the same on all planes.  x passes: (row, column) of A,
+  // packed (-1: a row that is left out); y and z passes: offset in a plane
   const int fz = par_first(z0, 1);  // first odd plane
-  {
-    const int fo = par_first(c0, 1), nxo = par_count(c0, c0 + w, 1);
-    // even columns: those whose odd neighbours are computed (N.0: all)
-    const int fe = NT && par_first(c0, 0) == c0 ? c0 + 2 : par_first(c0, 0);
-    const int nxe = par_count(fe, NT ? c0 + w - 1 : c0 + w, 0);
-    const int fy = par_first(r0, 1), ge = par_first(r0, 0), nyo = par_count(r0, r1 + 1, 1), nye = nR - nyo;
-    const DivM dxo = divm(nxo > 0 ? nxo : 1), dxe = divm(nxe > 0 ? nxe : 1), dw = divm(w);
+  const int fo = par_first(c0, 1), nxo = par_count(c0, c0 + w, 1);
+  // even columns: those whose odd neighbours are computed (N.0: all)
+  const int fe = NT && par_first(c0, 0) == c0 ? c0 + 2 : par_first(c0, 0);
+  const int nxe = par_count(fe, NT ? c0 + w - 1 : c0 + w, 0);
+  const int fy = par_first(r0, 1), ge = par_first(r0, 0), nyo = par_count(r0, r1 + 1, 1), nye = nR - nyo;
+  const DivM dxo = divm(nxo > 0 ? nxo : 1), dxe = divm(nxe > 0 ? nxe : 1), dw = divm(w);
+  auto at_x = [&](int idx, DivM d, int n, int first) {
+    const int q = divq(idx, d), r = row(q);
+    return r >= 0 && r < nA ? r << 16 | (first - c0 + 2 * (idx - q * n)) : -1;
+  };
+  auto at_xo = [&](int idx) { return at_x(idx, dxo, nxo, fo); };
+  auto at_xe = [&](int idx) { return at_x(idx, dxe, nxe, fe); };
+  auto at_yo = [&](int idx) { const int q = divq(idx, dw); return idx - q * w + w * (fy - r0 + 2 * q); };
+  auto at_ye = [&](int idx) { const int q = divq(idx, dw); return idx - q * w + w * (ge - r0 + 2 * q); };
+  int xo[K], xe[K], yo[K], ye[K];
+  if constexpr (KEEP) {
 #pragma unroll
     for (int u = 0; u < K; ++u) {
-      const int idx = tid + u * bd, qo = divq(idx, dxo), qe = divq(idx, dxe), qw = divq(idx, dw);
-      const int ro = row(qo), re = row(qe);
-      xo[u] = idx < nxo * nE && ro >= 0 && ro < nA ? ro << 16 | (fo - c0 + 2 * (idx - qo * nxo)) : -1;
-      xe[u] = idx < nxe * nE && re >= 0 && re < nA ? re << 16 | (fe - c0 + 2 * (idx - qe * nxe)) : -1;
-      yo[u] = idx < w * nyo ? idx - qw * w + w * (fy - r0 + 2 * qw) : -1;
-      ye[u] = idx < w * nye ? idx - qw * w + w * (ge - r0 + 2 * qw) : -1;
+      const int idx = tid + u * bd;
+      xo[u] = idx < nxo * nE ? at_xo(idx) : -1, xe[u] = idx < nxe * nE ? at_xe(idx) : -1;
+      yo[u] = idx < w * nyo ? at_yo(idx) : -1, ye[u] = idx < w * nye ? at_ye(idx) : -1;
     }
   }
+  auto each = [&](const int *kept, int n, auto at, auto f) {
+    if constexpr (KEEP) {
+#pragma unroll
+      for (int u = 0; u < K; ++u)
+        if (kept[u] >= 0) f(kept[u]);
+    } else {
+      for (int idx = tid; idx < n; idx += bd) {
+        const int o = at(idx);
+        if (o >= 0) f(o);
+      }
+    }
+  };
   // G^a output: v[0] - sum_{t odd} K(t) v[t*stride]
   auto gsum = [](const E *v, int stride) {
     E s = v[0];
@@ -152,39 +170,31 @@ __device__ __forceinline__ void detail_planes(const TP *__restrict__ Pb, int nb,
     const bool in = used(kk);
     // x pass: odd columns, then even columns
     if (in) {
-#pragma unroll
-      for (int u = 0; u < K; ++u)
-        if (xo[u] >= 0) {
-          const int jr = xo[u] >> 16, x = xo[u] & 0xffff;
-          A[x + w * jr] = gsum(S + jr * wS + x + ko, 1);
-        }
+      each(xo, nxo * nE, at_xo, [&](int o) {
+        const int jr = o >> 16, x = o & 0xffff;
+        A[x + w * jr] = gsum(S + jr * wS + x + ko, 1);
+      });
       __syncthreads();
-#pragma unroll
-      for (int u = 0; u < K; ++u)
-        if (xe[u] >= 0) {
-          const int jr = xe[u] >> 16, x = xe[u] & 0xffff;
-          E *a = A + x + w * jr;
-          const E v = S[jr * wS + x + ko];
-          if constexpr (NT != 0) *a = D::lift(v, a[-1], a[1]);
-          else *a = v;
-        }
+      each(xe, nxe * nE, at_xe, [&](int o) {
+        const int jr = o >> 16, x = o & 0xffff;
+        E *a = A + x + w * jr;
+        const E v = S[jr * wS + x + ko];
+        if constexpr (NT != 0) *a = D::lift(v, a[-1], a[1]);
+        else *a = v;
+      });
       __syncthreads();
       // y pass into ring plane kk: odd rows, then even rows
       E *rp = ring + slot * pl;
       const E *Ay = A + w * ko;
-#pragma unroll
-      for (int u = 0; u < K; ++u)
-        if (yo[u] >= 0) rp[yo[u]] = gsum(Ay + yo[u], w);
+      each(yo, w * nyo, at_yo, [&](int o) { rp[o] = gsum(Ay + o, w); });
       if (used(kk + 1)) stage(kk + 1);
       __syncthreads();
-#pragma unroll
-      for (int u = 0; u < K; ++u)
-        if (ye[u] >= 0) {
-          E *r = rp + ye[u];
-          const E v = Ay[ye[u]];
-          if constexpr (NT != 0) *r = D::lift(v, r[-w], r[w]);
-          else *r = v;
-        }
+      each(ye, w * nye, at_ye, [&](int o) {
+        E *r = rp + o;
+        const E v = Ay[o];
+        if constexpr (NT != 0) *r = D::lift(v, r[-w], r[w]);
+        else *r = v;
+      });
       __syncthreads();
     } else {
       if (used(kk + 1)) stage(kk + 1);
@@ -205,7 +215,6 @@ __device__ __forceinline__ void detail_planes(const TP *__restrict__ Pb, int nb,
         sl -= sl >= R ? R : 0;
         so[x] = sl * pl;
       }
-      const DivM dw = divm(w);
       for (int idx = tid; idx < pl; idx += bd) {
         const int q = divq(idx, dw), i = c0 + idx - q * w, j = r0 + q;
         const bool mine = i >= B.lo[0] && i <= B.hi[0] && j >= B.lo[1] && j <= B.hi[1];
@@ -245,9 +254,9 @@ __host__ __device__ __forceinline__ void det_cut(int r0, int r1, int q, int nt, 
 }
 
 // fewest tiles whose shared memory leaves room for two CTAs on an SM and whose
-// passes have at most DET_ITEMS items per thread (24^3 with 6.2 in float pairs:
+// passes (KEEP) have at most DET_ITEMS items per thread (24^3 with 6.2 in float pairs:
 // 72 KB and 384 threads 2.64 ms, 110 KB and 512 threads 2.25 ms)
-template <int N, int NT>
+template <int N, int NT, bool KEEP>
 static int det_tiles(int nb, size_t es, size_t *bytes) {
   const int r0 = -Wav<N, NT>::ext_f, r1 = nb - 1 + Wav<N, NT>::ext_b;
   for (int nt = 1;; ++nt) {
@@ -259,16 +268,16 @@ static int det_tiles(int nb, size_t es, size_t *bytes) {
     }
     const int nR = r1 - r0 + 1, items = std::max(w * nR, (w + 1) / 2 * (nR + 2 * (N - 1)));
     *bytes = es * det_elems<N>(nR, w);
-    if (*bytes <= DET_BYTES && items <= DET_ITEMS * DET_THREADS) return nt;
+    if (*bytes <= DET_BYTES && (!KEEP || items <= DET_ITEMS * DET_THREADS)) return nt;
   }
 }
 
 // Per leaf: max |gamma| over the extended region (Sec. 2.3, the block norm
 // that drives refinement and coarsening).  One CTA per column tile; the norms
 // start at zero and take the maximum of the tiles' integer keys.
-template <int N, int NT, bool PAIRS>
-__global__ void __launch_bounds__(1024) k_criterion(int nb, const double *__restrict__ P, int Gi,
-                                                  unsigned long long *__restrict__ maxdet, int ntile) {
+template <int N, int NT, bool PAIRS, bool KEEP>
+__global__ void __launch_bounds__(1024, KEEP ? 1 : 2) k_criterion(int nb, const double *__restrict__ P, int Gi,
+                                                                unsigned long long *__restrict__ maxdet, int ntile) {
   using E = typename DetOps<double, PAIRS>::E;
   const int b = blockIdx.x / ntile, Wd = nb + 2 * Gi;
   extern __shared__ double sm[];
@@ -282,40 +291,38 @@ __global__ void __launch_bounds__(1024) k_criterion(int nb, const double *__rest
     // part; one conversion at the end
     unsigned kh = 0;
     float kl = 0.f;
-    detail_planes<N, NT, PAIRS, double>(Pb, nb, Gi, B, reinterpret_cast<E *>(sm), [&](int, int, int, F2 g) {
+    detail_planes<N, NT, PAIRS, KEEP, double>(Pb, nb, Gi, B, reinterpret_cast<E *>(sm), [&](int, int, int, F2 g) {
       const unsigned h = __float_as_uint(g.h) & 0x7fffffffu;
       const float l = g.h < 0.f ? -g.l : g.l;
       if (h > kh || (h == kh && l > kl)) kh = h, kl = l;
     });
     mx = abs_key(f2_dbl({__uint_as_float(kh), kl}));
   } else {
-    detail_planes<N, NT, PAIRS, double>(Pb, nb, Gi, B, reinterpret_cast<E *>(sm),
-                                        [&](int, int, int, double g) { mx = max(mx, abs_key(g)); });
+    detail_planes<N, NT, PAIRS, KEEP, double>(Pb, nb, Gi, B, reinterpret_cast<E *>(sm),
+                                              [&](int, int, int, double g) { mx = max(mx, abs_key(g)); });
   }
   for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if ((threadIdx.x & 31) == 0 && mx) atomicMax(maxdet + b, mx);
 }
 
-// FP32 grids evaluate the details in float pairs (FP32 pipe), FP64 grids in
-// FP64 (the plain form)
-template <int N, int NT, bool PAIRS>
+template <int N, int NT, bool PAIRS, bool KEEP>
 static int criterion_launch(mr_grid *g, const double *P, int Gi, double *maxdet) {
   const int nb = g->desc.nb, n = g->nleaf;
   size_t sm;
-  const int nt = det_tiles<N, NT>(nb, sizeof(double), &sm);
+  const int nt = det_tiles<N, NT, KEEP>(nb, sizeof(double), &sm);
   // (block sizes stay those whose whole planes fit an SM: 32^3 with 6.2 in float
   // pairs is refused)
   const int nR = nb + Wav<N, NT>::ext_f + Wav<N, NT>::ext_b, nA = nR + 2 * (N - 1);
   if (8 * ((size_t)(2 * N + 1) * nR * nR + (size_t)nR * nA + (PAIRS ? (size_t)nA * nA : 0)) > 227 * 1024)
     return MR_ERR_UNSUPPORTED;
-  const auto kc = k_criterion<N, NT, PAIRS>;
+  const auto kc = k_criterion<N, NT, PAIRS, KEEP>;
   if (smem_limit(kc, DET_BYTES, "criterion smem") ||
       check_cuda(cudaMemsetAsync(maxdet, 0, sizeof(double) * (size_t)n, g->stream), "criterion norms"))
     return MR_ERR_CUDA;
   unsigned long long *md = reinterpret_cast<unsigned long long *>(maxdet);
   // FP64: issue is limited by its own pipe, more warps hide its latency
   static const int cc[2] = {PAIRS ? DET_THREADS : 2 * DET_THREADS, PAIRS ? 2 * DET_THREADS : DET_THREADS};
-  const int th = tune_threads(g, TuneKey{2, N, NT, nb, PAIRS ? 5 : 8, Gi, 0}, cc, 2, [&](int thr) {
+  const int th = tune_threads(g, TuneKey{2, N, NT, nb, PAIRS ? 5 : 8, Gi, KEEP ? 0 : 4}, cc, 2, [&](int thr) {
     kc<<<n * nt, thr, sm, g->stream>>>(nb, P, Gi, md, nt);
   });
   MR_LAUNCH(g, MRK_CRITERION, kc<<<n * nt, th, sm, g->stream>>>(nb, P, Gi, md, nt));
@@ -324,8 +331,17 @@ static int criterion_launch(mr_grid *g, const double *P, int Gi, double *maxdet)
 
 template <int N, int NT>
 static int criterion_impl(mr_grid *g, const double *P, int Gi, double *maxdet) {
-  return g->desc.precision == MR_F32 ? criterion_launch<N, NT, true>(g, P, Gi, maxdet)
-                                     : criterion_launch<N, NT, false>(g, P, Gi, maxdet);
+  // FP32 grids evaluate the details in float pairs (FP32 pipe), FP64 grids in FP64.
+  // There the kept indices cost 62 registers, one CTA of 1 024 threads to an SM: they
+  // pay where every tile has an SM to itself (55 leaves of 24^3 with 6.2: 177 us
+  // against 192), and two CTAs of 32 registers elsewhere (576 leaves: 1 451 against
+  // 1 080 us; of 16^3 with 4.2 342 and 258; of 32^3 with 2.0, which the kept indices cut
+  // into two tiles, 655 and 317).
+  if (g->desc.precision == MR_F32) return criterion_launch<N, NT, true, true>(g, P, Gi, maxdet);
+  size_t sm;
+  return g->nleaf * det_tiles<N, NT, true>(g->desc.nb, sizeof(double), &sm) <= 152
+             ? criterion_launch<N, NT, false, true>(g, P, Gi, maxdet)
+             : criterion_launch<N, NT, false, false>(g, P, Gi, maxdet);
 }
 
 int launch_criterion(mr_grid *g, const double *P, int Gi, double *maxdet) {
@@ -694,7 +710,7 @@ __global__ void __launch_bounds__(DET_THREADS, sizeof(TP) == 4 ? 3 : 2) k_update
     DetBox T = B;
     T.lo[0] = c, T.hi[0] = min(c + step - 1, B.hi[0]);
     if (c != B.lo[0]) __syncthreads();
-    detail_planes<N, NT, false, TP>(P + (size_t)s * np, nb, Gi, T, reinterpret_cast<TP *>(smd),
+    detail_planes<N, NT, false, true, TP>(P + (size_t)s * np, nb, Gi, T, reinterpret_cast<TP *>(smd),
                                     [&](int i, int j, int k, TP g) {
       if ((i | j | k) & 1) {
         const int r = region_of(i, j, k, nb), v = rD[r];

@@ -571,8 +571,8 @@ void *next_field_ptr(mr_grid *g, int fid);
 // variant (candidates 1 k_fused, 2 k_march); tp: 4 FP32, 5 FP32 field with
 // FP64 padded blocks, 8 FP64; mode: what else selects the kernel or its
 // candidates -- k_prep: which leaves it takes (only_coarse), + 4 on grids of many
-// leaves, + 8 with physical boundaries, as k_merge; stage kernels: 2 * scheme, + 1
-// with velocity fields, + 8 with diffusion)
+// leaves, + 8 with physical boundaries, as k_merge; k_criterion: 4 on FP64 grids of
+// many leaves; stage kernels: 2 * scheme, + 1 with velocity fields, + 8 with diffusion)
 struct TuneKey {
   int kid, N, Nt, nb, tp, shell, mode;
 };

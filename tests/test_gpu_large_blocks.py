@@ -1,6 +1,7 @@
 """Calls on the largest blocks of FP32 grids: what is refused, with which code, and
-the block norms of the largest accepted one (float pairs, 41^3 extended regions;
-1e-12 of the field maximum, as in test_gpu_adapt_tiles.py)."""
+the block norms of the largest accepted one (float pairs, 41^3 extended regions); and
+the norms of FP64 grids of many leaves.  Norms within 1e-12 of the field maximum, as
+in test_gpu_adapt_tiles.py."""
 import numpy as np
 import pytest
 
@@ -57,3 +58,22 @@ def test_largest_float_pair_norms(mr, oracle_mod):
     big = _grid(mr, nb, 6, 2)
     big.field_copy_in(0, phi)
     assert _code(mr, big.criterion, 0, md) == UNSUPPORTED
+
+
+@pytest.mark.parametrize("nb,N,Nt,n", [(8, 2, 2, 6), (18, 4, 0, 6), (26, 4, 2, 5), (32, 2, 0, 5)])
+def test_fp64_norms_of_many_leaves(mr, oracle_mod, nb, N, Nt, n):
+    """FP64 grids of more tiles than SMs, among them regions of more points per plane
+    than a CTA has threads."""
+    import torch
+    nt = (n, n, n)
+    lev, anc = I.uniform_leaves(nt, 0)
+    lev, anc = I.refine_leaves(lev, anc, np.all(anc == 0, axis=1))
+    g = mr.Grid(nt, 0.5, nb, 0, 1, N, Nt, lev, anc, precision=mr.F64)
+    lev, anc, _ = g.leaves()
+    phi = np.random.default_rng(nb).uniform(-1, 1, (g.nleaf, nb, nb, nb))
+    g.field_copy_in(0, phi)
+    md = torch.empty(g.nleaf, dtype=torch.float64, device="cuda")
+    g.criterion(0, md)
+    g.sync()
+    ref = oracle_mod.block_maxdet(oracle_mod.Grid(nt, 0.5, nb, N, Nt, 0, 1, lev, anc), phi)
+    assert np.abs(md.cpu().numpy() - ref).max() <= 1e-12 * np.abs(phi).max()
