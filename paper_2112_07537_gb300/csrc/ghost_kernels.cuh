@@ -213,7 +213,7 @@ struct PrepTab {
   int rmul[27];
   int cmask, ce;  // coarser directions (bit region), coarser neighbours (bit e)
   int s[3], odd[3];  // outward side per axis (+-1), anchor parity
-  int miss;          // prep_fetch met a point that no leaf holds
+  int miss;          // bounded grids: prep_fetch met a point that no leaf holds
 };
 
 // up to 7 disjoint boxes over [0, n) per axis, the layers (dlo on the - side,
@@ -254,9 +254,9 @@ __device__ __forceinline__ void outward_boxes(Boxes &B, int ce, const int *s, in
 }
 
 // level-Lq value (Lq = L or L - 1) at block-local point (i, j, k) through the
-// region tables, or through the owner map beyond the neighbouring regions; NaN,
-// and T.miss set, where no leaf holds the point
-template <typename TI>
+// region tables, or through the owner map beyond the neighbouring regions; NaN where
+// no leaf holds the point (BND: and T.miss set)
+template <bool BND, typename TI>
 __device__ __noinline__ TI prep_fetch(const Tree &t, PrepTab &T, const TI *phi, int b, int L, int Lq, int i, int j,
                                       int k, int *err) {
   const int nb = t.nb, hb = nb / 2, sc = Lq == L ? 1 : 2;
@@ -280,7 +280,7 @@ __device__ __noinline__ TI prep_fetch(const Tree &t, PrepTab &T, const TI *phi, 
   for (int d = 0; d < 3; ++d) g[d] = (Lq == L ? T.ranc[13][d] * nb : T.ranc[13][d] * nb / 2) + (d == 0 ? i : d == 1 ? j : k);
   const int o = owner(t, Lq, g[0], g[1], g[2], b);
   if (__ldg(t.lev + o) < Lq) {
-    T.miss = 1;
+    if (BND) T.miss = 1;
     return TI(__int_as_float(0x7fc00000));
   }
   return leaf_value(t, phi, o, Lq, g[0], g[1], g[2], err);
@@ -729,7 +729,8 @@ __global__ void __launch_bounds__(sizeof(TP) == 4 ? 512 : 384, 2) k_prep(Tree t,
   __shared__ PrepPlan plan;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int capU = sum_bytes / (int)sizeof(U), capP = sum_bytes / (int)sizeof(TP);
-  if (tid == 0) T.cmask = 0, T.ce = 0, T.miss = 0;
+  if (tid == 0) T.cmask = 0, T.ce = 0;
+  if (BND && tid == 0) T.miss = 0;
   __syncthreads();
   // owners of the 27 block-sized regions around b (same or coarser leaves own
   // a whole region); regions beyond a physical boundary count as the block
@@ -1005,7 +1006,7 @@ __global__ void __launch_bounds__(sizeof(TP) == 4 ? 512 : 384, 2) k_prep(Tree t,
           if (!ok && NARROW) {  // a finer leaf or a region beyond the neighbours
             auto at = [&](int qa) {
               q[a] = qa;
-              return RS::from(prep_fetch<TI>(t, T, phi, b, L, L - 1, q[0], q[1], q[2], err));
+              return RS::from(prep_fetch<BND, TI>(t, T, phi, b, L, L - 1, q[0], q[1], q[2], err));
             };
             refine_run<N, NT, RS>(at, B.la, na, [&](int ia, U v) { d[pitch * ia] = RS::norm(v); });
             continue;
@@ -1017,7 +1018,7 @@ __global__ void __launch_bounds__(sizeof(TP) == 4 ? 512 : 384, 2) k_prep(Tree t,
               for (int o = (f & 1) ? -ko : 0; o <= ((f & 1) ? ko : 0); o += 2) {
                 q[a] = (f + o) >> 1;
                 s = RS::acc(s, (f & 1) ? W::K(o) : 1.0,
-                            RS::from(prep_fetch<TI>(t, T, phi, b, L, L - 1, q[0], q[1], q[2], err)));
+                            RS::from(prep_fetch<BND, TI>(t, T, phi, b, L, L - 1, q[0], q[1], q[2], err)));
               }
               d[pitch * ia] = RS::norm(s);
             }
