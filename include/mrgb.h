@@ -298,8 +298,8 @@ int mr_graph_replays(mr_grid *grid, long long *n);
 /* Launch-shape autotuner.  With enable = 1, the first launch of each tunable
  * kernel configuration (kernel, wavelet, nb, precision, shell, mode) on this
  * grid times every candidate CTA size on the grid's own data -- the ghost
- * gather, pre-pass and merge, the criterion, the interpolation, and the fused
- * stage kernel (one grid line per thread or two), each only on launches that
+ * fill and merge, the criterion, the interpolation, and the fused stage kernel
+ * (slab heights), each only on launches that
  * overwrite their outputs from unchanged inputs, so repeating them changes
  * nothing -- and keeps the fastest in a table shared by every grid of the
  * process (later launches of that configuration use it whether or not their

@@ -51,7 +51,7 @@ struct DetOps<double, true> {
 // the y pass runs.  A block is cut into column tiles so that two or three CTAs
 // share an SM and one computes while another waits at a barrier.  Bound by issued
 // instructions of the FP32 pipe (float pairs) and by the barriers: 2 080 leaves
-// of 24^3, 6.2, took 2.79 ms whole (163 KB, one CTA per SM), 2.25 ms in tiles.
+// of 24^3, 6.2, took 2.79 ms whole (163 KB, one CTA per SM), 2.23 ms in tiles.
 // emit(i, j, k, gamma) is called once per point of the box (gamma unconverted).
 struct DetBox {  // inclusive
   int lo[3], hi[3];
@@ -310,8 +310,8 @@ static int criterion_launch(mr_grid *g, const double *P, int Gi, double *maxdet)
   const int nb = g->desc.nb, n = g->nleaf;
   size_t sm;
   const int nt = det_tiles<N, NT, KEEP>(nb, sizeof(double), &sm);
-  // (block sizes stay those whose whole planes fit an SM: 32^3 with 6.2 in float
-  // pairs is refused)
+  // (accepted are the block sizes whose untiled planes would fit an SM: of all,
+  // 32^3 with 6.2 in float pairs is refused, although its tiles would fit)
   const int nR = nb + Wav<N, NT>::ext_f + Wav<N, NT>::ext_b, nA = nR + 2 * (N - 1);
   if (8 * ((size_t)(2 * N + 1) * nR * nR + (size_t)nR * nA + (PAIRS ? (size_t)nA * nA : 0)) > 227 * 1024)
     return MR_ERR_UNSUPPORTED;
@@ -956,8 +956,8 @@ int adapt_iteration(mr_grid *g, int crit, double er, double ec, int flags, int *
   int e = launch_ghost(g, field_ptr(g, crit), field_ptr(g, crit), G, true, &Pv, &Gi);
   if (e) return e;
   const double *P = (const double *)Pv;
-  // grids with physical boundaries take the general point-wise paths: the
-  // bounded criterion, and full ghost fills (with write-back) of every field
+  // grids with physical boundaries take the bounded criterion, and full ghost
+  // fills (with write-back) of every field
   const bool bnd = grid_bounded(g);
   e = bnd ? launch_criterion_bounded(g, P, Gi, g->maxdet) : launch_criterion(g, P, Gi, g->maxdet);
   if (e) return e;

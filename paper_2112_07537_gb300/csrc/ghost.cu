@@ -1,7 +1,6 @@
 // ghost.cu -- ghost reconstruction (Alg. SM1 / SM2): the launchers of the
-// ghost kernels (the kernels and their instantiations are in
-// ghost_kernels.cuh and ghost_ff.cu / ghost_fd.cu / ghost_dd.cu), the crop
-// and write-back kernels, and the allocation-free ghost fill.
+// ghost kernels (the kernels are in ghost_kernels.cuh, instantiated in
+// ghost_i_*.cu), the write-back kernel, and the allocation-free ghost fill.
 #include <algorithm>
 #include <cstdio>
 

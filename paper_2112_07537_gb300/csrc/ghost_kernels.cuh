@@ -397,8 +397,8 @@ __device__ __forceinline__ int turn(int rot, int n, int bd) {
 constexpr int SUB_RUN = 4;  // points of one item of the substitution
 
 // Flat axes are used where arithmetic counts: FP64 blocks (ghost fills of 1 408
-// leaves of 24^3 with 6.2, shell 6: 637 -> 546 us, of 2 080 with shell 11 1 770 ->
-// 1 693 us); with FP32 blocks the listed coordinates cost more than the sums they
+// leaves of 24^3 with 6.2, shell 6: 637 -> 563 us, of 2 080 with shell 11 1 770 ->
+// 1 672 us); with FP32 blocks the listed coordinates cost more than the sums they
 // save (42 400 leaves 2.42 -> 2.56 ms).
 template <typename TP>
 constexpr bool sub_flat = sizeof(TP) == 8;
@@ -433,7 +433,9 @@ struct SubJob {
 // detail along the odd dimensions it shares with the class, so the terms at even
 // points inside add up to zero over the other dimensions and are left out, and
 // away from the ends S is the sum of the pass before (half the points of a face
-// box).  Pass 1 drops its t = 0 term where every
+// box).  (A NaN or infinity at such a point therefore reaches the degree-1 points
+// around it, but not every point of higher degree that has it among its taps.)
+// Pass 1 drops its t = 0 term where every
 // other odd coordinate is odd -- exactly at the class points, which no other
 // term of any pass reads -- so the product over all t leaves out t = 0.
 // Points of one degree read lower degrees only, so all jobs of a degree run
@@ -1207,9 +1209,9 @@ __global__ void __launch_bounds__(sizeof(TP) == 4 ? 512 : 384, 2) k_prep(Tree t,
 // Shared memory of the pre-pass's sums, or what a chunk of the largest box
 // takes.  Four CTAs of 256 threads per SM with FP32 blocks, three with FP64
 // ones; the sums stay small enough that the L1 cache keeps a share of the SM's
-// memory, since the block is read back through it: at 3 424 leaves of 24^3 with
-// 6.2 the pre-pass takes 312 us with 27 or 34 KB, 417 us with 42 KB (L1 almost
-// gone) and 323 us with 54 KB (three CTAs).
+// memory, since the block is read back through it: without the gather the kernel took
+// 312 us at 3 424 leaves of 24^3 with 6.2 with 27 or 34 KB, 417 with 42 KB (L1 almost
+// gone) and 323 with 54 KB (three CTAs).
 static size_t prep_sum_bytes(int N, int nb, int Gi, size_t es, bool bounded) {
   const int ko = N - 1, m = nb + Gi, mb = ((m - 1 + 2 * ko) >> 1) + 2;
   const size_t plane = (size_t)Gi * (mb | 1) + ((size_t)Gi * (m | 1) | 1);

@@ -1,6 +1,9 @@
 // stage.cu -- the FP32 stage kernels: ghost faces + advection right-hand side
 // + RK3 stage in one launch.  Two kernels compute the same values with the
-// same arithmetic; the autotuner picks the faster:
+// same arithmetic.  k_fused runs unless mr_set_stage_kernel or the autotuner, which
+// times both, says otherwise; k_march took twice its time wherever both were timed
+// (3 424 leaves of 24^3 with velocity fields 1 070 against 526 us, 42 400 with a
+// constant velocity 8.5 against 3.99 ms, 11 019 of 16^3 1 047 against 477 us):
 //   k_fused  one CTA per slab of a leaf: the slab with its ghosts in shared
 //            memory, one thread per pair of grid lines;
 //   k_march  one CTA per leaf marching through the block's z-planes: the six
@@ -121,20 +124,17 @@ __device__ __forceinline__ float stage_value(const StageArgs &s, float c, float 
 // with the same code, then the z lines (pairs of neighbours in x), whose thread
 // finishes its cells.  What one thread alone reads (the three values beyond each
 // end of a z line, u_z, u^n) goes straight to its registers.  Bound by issued
-// instructions and by the latency of the copies: the packed walk issues 243
-// instructions per point (velocity fields) where one line per thread issued 323
-// and an index per copy and planes around the slab in shared memory 388; the
-// copies alone take 40 to 57 % of the time, overlapped with the walks of the
-// other CTAs.  Slabs of a quarter block (half of a block of at most 16) keep
-// three CTAs on an SM with velocity fields (more would spill), four without; the
-// z walks' extra interface per slab costs 5 %.  Measured per launch (WENO-Z5,
-// 6.2 ghosts): 3 424 leaves of 24^3 with velocity fields 1 660 us (whole block per
-// CTA), 742 (slabs), 530 (fewer copies), 527 (packed); 42 400 leaves with a
-// constant velocity 15.35 ms, 6.02, 4.97, 3.99; 11 019 leaves of 16^3 with velocity
-// fields 1 333 us, 836, 596, 476 (4.2); 1 272 leaves of 20^3 with diffusion 104 us,
-// 89 and 72 (2.2; from the slabs on).
-// k_march takes 1 070 us, 8.5 ms and 1 047 us in the first three.  Separate code for
-// x and y walks, or unrolled z walks, is slower by a tenth (instruction cache).
+// instructions (243 per point with velocity fields; 323 with one line per thread)
+// and by the latency of the copies, which alone take 40 to 57 % of the time,
+// overlapped with the walks of the other CTAs.  Slabs of a quarter block (half of a
+// block of at most 16) keep three CTAs on an SM with velocity fields (more would
+// spill), four without; the z walks' extra interface per slab costs 5 %.  Per launch
+// (WENO-Z5): 3 424 leaves of 24^3 with velocity fields and 6.2 526 us (the block in
+// shared memory as a whole, one line per thread: 1 660); 42 400 leaves with a constant
+// velocity 3.99 ms (15.35); 11 019 leaves of 16^3 with velocity fields and 4.2 477 us
+// (1 333); 1 272 leaves of 20^3 with diffusion and 2.2 74 us (104 in slabs of one line
+// per thread).  Separate code for x and y walks, or unrolled z walks, is slower by a
+// tenth (instruction cache).
 // ---------------------------------------------------------------------------
 // row pitch for n floats per row: twice an odd number (two-way bank conflicts at
 // worst where neighbouring threads walk neighbouring rows)
@@ -144,7 +144,8 @@ __host__ __device__ constexpr int fused_smem_floats(int nb, int nz, bool vel) {
          nz * (vel ? nb + 6 : nb) * nb;
 }
 
-// largest block, and its slabs: a quarter of a large and half of a small one
+// largest block accepted (the slabs of 28^3 to 32^3 would fit an SM, too: 84 to 121 KB
+// with velocity fields), and its slabs: a quarter of a large and half of a small one
 constexpr int FUSED_MAX_NB = 26;
 __host__ __device__ constexpr int fused_height(int nb) { return nb > 16 ? (nb + 3) / 4 : nb / 2; }
 

@@ -19,9 +19,9 @@ namespace mr {
 // rounded products and the sums of walk_line leave nothing to contract, so a
 // flux does not depend on where its line was cut.  Measured (WENO-Z5, velocity
 // fields, 1 408 leaves of 24^3 = 19.5 M points): 23.9 ms per launch with both
-// fluxes of every point evaluated per thread and four divisions each, 6.08 ms
-// so (the FP64 pipe's floor for 147 instructions a point is 4.6 ms); 15 leaves
-// of 16^3: 680 us in 15 CTAs, 39 us.
+// fluxes of every point evaluated per thread and four divisions each, 5.88 ms
+// so (the FP64 pipe's floor for 147 instructions a point is 4.6 ms; flat parts of
+// a field skip some, see weno_corr); 15 leaves of 16^3: 680 us in 15 CTAs, 38 us.
 template <typename T, int SCHEME>
 __global__ void __launch_bounds__(256) k_rhs_stage(Tree t, const T *__restrict__ P, int Gi, const T *u, T *out,
                                                    int stage, T dt, T ux, T uy, T uz, int rhs_only,
